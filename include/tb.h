@@ -67,7 +67,7 @@ extern "C" {
                                            bind then stages the blob through page-locked memory of the batch */
 
 /* tb_batch_set_flags */
-#define TB_FLAG_GENERAL_KERNELS 1       /* always use the general decode kernel (any layout), never a pipelined one */
+#define TB_FLAG_GENERAL_KERNELS 1       /* always use the general decode kernel (any layout), never a pipelined or two-step one */
 #define TB_FLAG_ONE_BLOCK_PER_STREAM 2  /* pipelined greedy decode: never the segmented kernel, one block per stream */
 #define TB_FLAG_LOG_SOFTMAX 8           /* tb_greedy_decode and tb_stream_chunk (RNNT rows) score every visited row by its log-softmax:
                                            L = m + log(sum_v exp(x_v - m)) over the row's vocab+1 entries, computed in float inside
@@ -88,7 +88,9 @@ extern "C" {
                                            TB_STATUS_WAIT_TIMEOUT is set, the outputs of that call are undefined */
 
 /* tb_batch_last_greedy_kernel */
-#define TB_KERNEL_GENERAL 1     /* one block per stream, a block-wide argmax per visited row */
+#define TB_KERNEL_GENERAL 1     /* any layout: the rows reduced to summaries by one launch and decided by a second (token stride 1,
+                                   S <= 4), else -- or with TB_FLAG_GENERAL_KERNELS -- one block per stream with a block-wide
+                                   argmax per visited row */
 #define TB_KERNEL_PIPELINED 2   /* one block per stream: rows staged in shared memory, at most two segments */
 #define TB_KERNEL_SEGMENTED 3   /* streams cut into segments decoded by many small pipelines on all SMs, then stitched */
 
@@ -323,7 +325,8 @@ int tb_batch_bind_models(tb_batch *b, int32_t n, const int32_t *slots, const int
  * tb_greedy_decode picks a pipelined kernel whenever the call fits it (bf16 logits, token
  * stride 1, the S rows of a frame contiguous, vocab <= 2048, S <= 4) -- the segmented one when every
  * bound graph carries resolved lists that fit a block's shared memory, else the one-block-per-stream
- * one -- and the general kernel otherwise; all give identical results.  The paper has no counterpart
+ * one -- and the general kernels otherwise, or when the lists are walked or larger than 48 KB a stream; all give
+ * identical results.  The paper has no counterpart
  * of this call.
  * Errors: TB_ERR_INVALID_ARG (unknown bits).
  */

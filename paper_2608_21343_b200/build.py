@@ -18,6 +18,7 @@ NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
     "--fmad=false",  # the arithmetic contract forbids fusing x + lambda*bonus
     "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off", "-shared", "-cudart", "static",
+    "-t", "0",  # the files are compiled side by side
 ]
 
 

@@ -199,6 +199,75 @@ bool tb_pinned_free(void* p, size_t bytes) {
   return false;
 }
 
+// ---- working memory that outlives a batch -----------------------------------------------------------------------
+// Decode calls need working memory whose size depends on the call (a cudaMalloc of tens of MB takes 1 to 20 ms).  A batch
+// takes it on its first call and keeps it; when the batch is destroyed -- which waits for the device, so nothing reads
+// the memory any more -- its blocks go to this pool (at most kScratchPoolMax), where the next batch finds them.  With
+// the last batch of the process the pool is emptied.
+namespace {
+constexpr size_t kScratchPoolMax = static_cast<size_t>(256) << 20;
+struct ScratchPool {
+  struct Block { int device; void* mem; size_t bytes; };
+  std::mutex mu;
+  std::vector<Block> free_blocks;
+  size_t total = 0;
+  int batches = 0;
+};
+ScratchPool& scratch_pool() {
+  static ScratchPool* pool = new ScratchPool();
+  return *pool;
+}
+// A block of at least `want` bytes on the current device (= device), or null.
+void* scratch_take(int device, size_t want, size_t* got) {
+  {
+    ScratchPool& pool = scratch_pool();
+    std::lock_guard<std::mutex> lock(pool.mu);
+    int best = -1;
+    for (int i = 0; i < static_cast<int>(pool.free_blocks.size()); ++i) {
+      const ScratchPool::Block& k = pool.free_blocks[i];
+      if (k.device == device && k.bytes >= want && (best < 0 || k.bytes < pool.free_blocks[best].bytes)) best = i;
+    }
+    if (best >= 0) {
+      const ScratchPool::Block k = pool.free_blocks[best];
+      pool.free_blocks.erase(pool.free_blocks.begin() + best);
+      pool.total -= k.bytes;
+      *got = k.bytes;
+      return k.mem;
+    }
+  }
+  void* mem = nullptr;
+  if (cudaMalloc(&mem, want) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+  *got = want;
+  return mem;
+}
+void scratch_give(int device, void* mem, size_t bytes) {
+  if (!mem) return;
+  {
+    ScratchPool& pool = scratch_pool();
+    std::lock_guard<std::mutex> lock(pool.mu);
+    if (pool.total + bytes <= kScratchPoolMax) {
+      pool.free_blocks.push_back({device, mem, bytes});
+      pool.total += bytes;
+      return;
+    }
+  }
+  cudaFree(mem);
+}
+void scratch_count_batch(int by) {
+  ScratchPool& pool = scratch_pool();
+  std::vector<ScratchPool::Block> drop;
+  {
+    std::lock_guard<std::mutex> lock(pool.mu);
+    pool.batches += by;
+    if (pool.batches == 0) { drop.swap(pool.free_blocks); pool.total = 0; }
+  }
+  int prev = -1;
+  if (!drop.empty()) cudaGetDevice(&prev);
+  for (const ScratchPool::Block& k : drop) { cudaSetDevice(k.device); cudaFree(k.mem); }
+  if (prev >= 0) cudaSetDevice(prev);
+}
+}  // namespace
+
 struct tb_batch {
   int device = 0;
   int32_t vocab = 0, n_classes = 0, n_slots = 0, max_beam = 0, max_tree_steps = 0;
@@ -248,6 +317,10 @@ struct tb_batch {
   size_t sg_scratch_bytes = 0;
   int32_t sg_shape[4] = {0, 0, 0, 0};   // streams, frames, rows per frame, segments of the layout in place
   bool sg_captured = false;
+  // working memory of the two-step kernels (tb_rows.cu), grown on demand like the others: what an offline decode needs,
+  // and the room for long lists of streaming slots without resolved lists
+  void* rows_scratch = nullptr; size_t rows_scratch_bytes = 0;
+  void* chunk_spill = nullptr; size_t chunk_spill_bytes = 0;
   int32_t plan_G = 0, plan_H = 0, plan_NB = 0;   // tb_batch_set_greedy_plan (0: automatic)
   int32_t last_kernel = 0, last_NB = 0, last_G = 0;
   int32_t n_sm = 0, max_smem = 0;
@@ -258,7 +331,10 @@ static void destroy_batch(tb_batch* b) {
   if (!b) return;
   cudaDeviceSynchronize();
   cudaFree(b->arena); cudaFree(b->d_slots); cudaFree(b->d_sstate); cudaFree(b->d_cls);
-  cudaFree(b->d_status); cudaFree(b->d_tree); cudaFree(b->seg_scratch); cudaFree(b->sg_scratch); cudaFree(b->d_hyp_hash); cudaFree(b->d_hyp_len); cudaFree(b->d_model_recs); cudaFree(b->d_slot_pos); cudaFree(b->d_top);
+  cudaFree(b->d_status); cudaFree(b->d_tree); cudaFree(b->d_hyp_hash); cudaFree(b->d_hyp_len); cudaFree(b->d_model_recs); cudaFree(b->d_slot_pos);
+  scratch_give(b->device, b->seg_scratch, b->seg_scratch_bytes); scratch_give(b->device, b->sg_scratch, b->sg_scratch_bytes);
+  scratch_give(b->device, b->rows_scratch, b->rows_scratch_bytes); scratch_give(b->device, b->chunk_spill, b->chunk_spill_bytes);
+  scratch_give(b->device, b->d_top, b->d_top_bytes);
   for (auto& s : b->staging) {
     if (s.held) tb_graph_free(s.held);
     for (tb_graph* h : s.held_more) tb_graph_free(h);
@@ -267,6 +343,7 @@ static void destroy_batch(tb_batch* b) {
   }
   cudaGetLastError();
   delete b;
+  scratch_count_batch(-1);
 }
 
 extern "C" int tb_batch_create(int32_t vocab, const int32_t* case_class, int32_t n_slots, int32_t max_beam,
@@ -287,6 +364,7 @@ extern "C" int tb_batch_create(int32_t vocab, const int32_t* case_class, int32_t
   if (!guard.ok) return TB_ERR_CUDA;
   tb_batch* b = new (std::nothrow) tb_batch();
   if (!b) return TB_ERR_OOM;
+  scratch_count_batch(1);
   b->device = device; b->vocab = vocab; b->n_classes = n_classes; b->n_slots = n_slots;
   b->max_beam = max_beam; b->max_tree_steps = max_tree_steps;
   b->class_map_hash = tb_hash_class_map(case_class, vocab);
@@ -784,6 +862,38 @@ extern "C" int tb_batch_status(tb_batch* b, int32_t* device_status, void* stream
   return st == 0 ? TB_OK : TB_ERR_DEVICE_STATUS;
 }
 
+// Working memory of at least `want` bytes; never allocated while the caller's stream is being captured into a graph
+// (growing frees the old block first, which waits for earlier work: one decode per batch at a time).
+static bool grow_scratch(tb_batch* b, void** mem, size_t* have, size_t want, bool capturing) {
+  if (want <= *have) return true;
+  if (capturing || want > (static_cast<size_t>(4) << 30)) return false;
+  cudaFree(*mem);
+  *have = 0;
+  *mem = scratch_take(b->device, want, have);
+  return *mem != nullptr;
+}
+static bool is_capturing(cudaStream_t stream) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) { cudaGetLastError(); return false; }
+  return cap != cudaStreamCaptureStatusNone;
+}
+static void query_device(tb_batch* b) {
+  if (b->n_sm != 0) return;
+  cudaDeviceGetAttribute(&b->n_sm, cudaDevAttrMultiProcessorCount, b->device);
+  cudaDeviceGetAttribute(&b->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device);
+  cudaGetLastError();
+}
+struct SlotSummary { int32_t max_cache = 0, max_states = 0, all_resolved = 1; };
+static SlotSummary slot_summary(const tb_batch* b, int32_t n) {
+  SlotSummary r;
+  for (int32_t i = 0; i < n; ++i) {
+    r.max_cache = b->slot_cache_bytes[i] > r.max_cache ? b->slot_cache_bytes[i] : r.max_cache;
+    r.max_states = b->slot_n_states[i] > r.max_states ? b->slot_n_states[i] : r.max_states;
+    if (!b->slot_resolved[i]) r.all_resolved = 0;
+  }
+  return r;
+}
+
 static int fill_decode_params(tb_batch* b, const void* logits, int dtype, int32_t n, int32_t frames, int32_t S,
                               int32_t n_dur, const int64_t* strides, TbDecodeParams* p) {
   if (!b || !logits || !strides || (dtype != TB_BF16 && dtype != TB_F32)) return TB_ERR_INVALID_ARG;
@@ -815,23 +925,25 @@ extern "C" int tb_greedy_decode(tb_batch* b, const void* logits, int dtype, int3
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
   p.normalize = (b->flags & TB_FLAG_LOG_SOFTMAX) ? 1 : 0;
   if (!(b->flags & TB_FLAG_GENERAL_KERNELS)) {
-    int32_t max_cache = 0, max_states = 0, all_resolved = 1;
-    for (int32_t i = 0; i < B; ++i) {
-      max_cache = b->slot_cache_bytes[i] > max_cache ? b->slot_cache_bytes[i] : max_cache;
-      max_states = b->slot_n_states[i] > max_states ? b->slot_n_states[i] : max_states;
-      if (!b->slot_resolved[i]) all_resolved = 0;
-    }
+    const SlotSummary sl = slot_summary(b, B);
+    const int32_t max_cache = sl.max_cache, max_states = sl.max_states, all_resolved = sl.all_resolved;
     // Working memory is never allocated while the caller's stream is being captured into a graph (allocation is
     // not allowed there): the decode then runs with the block it has, or on a path that needs none.
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusNone; }
-    const bool capturing = cap != cudaStreamCaptureStatusNone;
+    const bool capturing = is_capturing(stream);
+    query_device(b);
+    TbRowsPlan rplan;
+    auto run_rows = [&]() -> bool {
+      if (!tb_rows_plan(p, max_cache, max_states, all_resolved, b->n_sm, b->max_smem, &rplan)) return false;
+      if (!grow_scratch(b, &b->rows_scratch, &b->rows_scratch_bytes, rplan.scratch_bytes, capturing)) return false;
+      rc = tb_launch_rows(p, rplan, b->n_sm, b->rows_scratch, stream);
+      if (rc == TB_OK) { b->last_kernel = TB_KERNEL_GENERAL; b->last_NB = 1; b->last_G = 0; }
+      return true;
+    };
+    // Lists that are walked or too large for the pipelined kernels' caches (48 KB): in two steps, many stretches of a stream
+    // at once, each reading its lists from L2.
+    if (b->plan_G == 0 && !(b->flags & (TB_FLAG_ONE_BLOCK_PER_STREAM | TB_FLAG_TEST_WAIT_TIMEOUT)) && (!all_resolved || max_cache > (48 << 10)))
+      if (run_rows()) return rc;
     if (!(b->flags & TB_FLAG_ONE_BLOCK_PER_STREAM)) {
-      if (b->n_sm == 0) {
-        cudaDeviceGetAttribute(&b->n_sm, cudaDevAttrMultiProcessorCount, b->device);
-        cudaDeviceGetAttribute(&b->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device);
-        cudaGetLastError();
-      }
       TbSegPlan plan;
       plan.force_G = b->plan_G; plan.force_H = b->plan_H; plan.force_NB = b->plan_NB;
       plan.test_timeout = (b->flags & TB_FLAG_TEST_WAIT_TIMEOUT) ? 1 : 0;
@@ -841,13 +953,8 @@ extern "C" int tb_greedy_decode(tb_batch* b, const void* logits, int dtype, int3
         const size_t want = tb_greedy_seg_scratch_bytes(B, T, S, nseg);
         bool ok = true;
         if (want > b->sg_scratch_bytes) {
-          ok = !capturing && !b->sg_captured && want <= (static_cast<size_t>(4) << 30);
-          if (ok) {
-            cudaFree(b->sg_scratch);                    // (waits for earlier work: one decode per batch at a time)
-            b->sg_scratch = nullptr; b->sg_scratch_bytes = 0; b->sg_shape[0] = 0;
-            if (cudaMalloc(&b->sg_scratch, want) == cudaSuccess) b->sg_scratch_bytes = want;
-            else { cudaGetLastError(); ok = false; }
-          }
+          ok = !b->sg_captured && grow_scratch(b, &b->sg_scratch, &b->sg_scratch_bytes, want, capturing);
+          b->sg_shape[0] = 0;
         }
         if (ok && (b->sg_shape[0] != B || b->sg_shape[1] != T || b->sg_shape[2] != S || b->sg_shape[3] != nseg)) {
           // another layout: what the last one left (launch numbers, records) would be misread
@@ -865,15 +972,11 @@ extern "C" int tb_greedy_decode(tb_batch* b, const void* logits, int dtype, int3
     // the two-segment decode keeps what its second segment produces in scratch memory of the batch; growing it
     // frees the old block first (cudaFree waits for earlier work), so one decode per batch at a time
     const size_t want = tb_greedy_fast_scratch_bytes(B, T, S);
-    if (!capturing && want > b->seg_scratch_bytes && want <= (static_cast<size_t>(1) << 30)) {
-      cudaFree(b->seg_scratch);
-      b->seg_scratch = nullptr; b->seg_scratch_bytes = 0;
-      if (cudaMalloc(&b->seg_scratch, want) == cudaSuccess) b->seg_scratch_bytes = want;
-      else cudaGetLastError();
-    }
+    grow_scratch(b, &b->seg_scratch, &b->seg_scratch_bytes, want, capturing);
     rc = tb_launch_greedy_fast(p, max_cache, max_states, all_resolved, b->seg_scratch, b->seg_scratch_bytes, stream);
     if (rc == TB_OK) { b->last_kernel = TB_KERNEL_PIPELINED; b->last_NB = 1; b->last_G = 0; }
     if (rc != 1) return rc;
+    if (run_rows()) return rc;
   }
   rc = tb_launch_decode_general(p, stream);
   if (rc == TB_OK) { b->last_kernel = TB_KERNEL_GENERAL; b->last_NB = 1; b->last_G = 0; }
@@ -934,6 +1037,18 @@ static int stream_chunk_params(tb_batch* b, const void* logits, int dtype, int32
   return TB_OK;
 }
 
+static int launch_chunk(tb_batch* b, const TbDecodeParams& p, cudaStream_t stream, const TbInlineBinds* binds) {
+  if (!(b->flags & TB_FLAG_GENERAL_KERNELS)) {
+    query_device(b);
+    const SlotSummary sl = slot_summary(b, p.n_streams);
+    if (p.n_streams <= b->n_sm) if (sl.all_resolved || grow_scratch(b, &b->chunk_spill, &b->chunk_spill_bytes, tb_chunk_rows_spill_bytes(p), is_capturing(stream))) {
+      const int rc = tb_launch_chunk_rows(p, sl.max_states, b->n_sm, b->max_smem, sl.all_resolved ? nullptr : b->chunk_spill, stream, binds);
+      if (rc != 1) return rc;
+    }
+  }
+  return tb_launch_decode_general(p, stream, binds);
+}
+
 extern "C" int tb_stream_chunk(tb_batch* b, const void* logits, int dtype, int32_t n_slots, int32_t chunk,
                                int32_t S, int32_t n_dur, const int64_t* strides, const int32_t* valid_frames,
                                int32_t* out_tokens, int32_t* out_frames, int32_t* out_durs, int32_t* out_counts,
@@ -945,7 +1060,7 @@ extern "C" int tb_stream_chunk(tb_batch* b, const void* logits, int dtype, int32
   if (rc != TB_OK) return rc;
   DeviceGuard guard(b->device);
   if (!guard.ok) return TB_ERR_CUDA;
-  return tb_launch_decode_general(p, static_cast<cudaStream_t>(stream_));
+  return launch_chunk(b, p, static_cast<cudaStream_t>(stream_), nullptr);
 }
 
 extern "C" int tb_stream_chunk_binds(tb_batch* b, int32_t n_binds, const int32_t* bind_slots, const tb_graph* const* bind_graphs,
@@ -972,7 +1087,7 @@ extern "C" int tb_stream_chunk_binds(tb_batch* b, int32_t n_binds, const int32_t
     std::vector<tb_graph*> let_go;
     if (in_chunk && !(b->flags & TB_FLAG_COPIED_BINDS) &&
         prepare_pulled_binds(b, n_binds, bind_slots, bind_graphs, stream, &ib, &used, &let_go)) {
-      rc = tb_launch_decode_general(p, stream, &ib);
+      rc = launch_chunk(b, p, stream, &ib);
       if (rc == TB_OK && cudaEventRecord(used->done, stream) == cudaSuccess) used->pending = true;
       else if (rc == TB_OK) { cudaGetLastError(); cudaStreamSynchronize(stream); }   // (no event: the graphs are let go only after the launch is done)
       if (rc != TB_OK) {
@@ -993,7 +1108,7 @@ extern "C" int tb_stream_chunk_binds(tb_batch* b, int32_t n_binds, const int32_t
     if (rc != TB_OK) return rc;
     b->n_copied_binds += n_binds;
   }
-  return tb_launch_decode_general(p, stream);
+  return launch_chunk(b, p, stream, nullptr);
 }
 
 extern "C" int tb_batch_bind_counts(const tb_batch* b, int64_t* out_pulled, int64_t* out_copied) {
@@ -1013,14 +1128,11 @@ static void beam_prepass(tb_batch* b, TbBeamParams* p, int32_t T, int32_t E, int
   if (2 * (b->vocab + 1) > (1 << TB_RS_TOK_BITS) || b->vocab > 0xFFFE) return;   // (the steps' token view has the same limit)
   const int32_t M = 2 * p->K + 8;
   const size_t want = static_cast<size_t>(p->B) * T * E * (M + 1) * sizeof(TbTopEnt);
-  if (want > b->d_top_bytes) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) { cudaGetLastError(); return; }
-    if (cap != cudaStreamCaptureStatusNone || want > (static_cast<size_t>(2) << 30)) return;
-    cudaFree(b->d_top);
-    b->d_top = nullptr; b->d_top_bytes = 0;
-    if (cudaMalloc(&b->d_top, want) != cudaSuccess) { cudaGetLastError(); return; }
-    b->d_top_bytes = want;
+  {
+    void* mem = b->d_top;
+    const bool ok = grow_scratch(b, &mem, &b->d_top_bytes, want, want > b->d_top_bytes && is_capturing(stream));
+    b->d_top = static_cast<TbTopEnt*>(mem);
+    if (!ok) return;
   }
   if (tb_launch_beam_topm(p->logits, p->dtype, p->B, T, E, p->V, p->C, p->stream_stride, frame_stride, row_stride, n_frames,
                           b->d_slots, b->arena, b->d_cls, M, b->d_top, stream) != TB_OK)

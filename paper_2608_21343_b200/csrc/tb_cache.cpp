@@ -18,7 +18,7 @@
 namespace {
 
 constexpr uint32_t kMagic = 0x31474254u;   // "TBG1"
-constexpr uint32_t kVersion = 4;
+constexpr uint32_t kVersion = 5;
 
 // FNV-1a style checksum over 8-byte words (the tail byte by byte): detects damage, is not cryptographic
 uint64_t fnv1a(const void* p, size_t n, uint64_t h = 1469598103934665603ull) {
@@ -195,7 +195,8 @@ extern "C" int tb_graph_load(const char* path, tb_graph** out) {
         in = static_cast<int32_t>(te.tok_cls & 0xffffu) < h.vocab && te.dst >= 0 && te.dst < Ns;
       }
       if (Re >= 0) {
-        in = in && Re <= TB_RS_MAX_ENTRIES && h.vocab + 1 <= (1 << (TB_RS_TOK_BITS - 1));
+        in = in && Re <= TB_RS_MAX_ENTRIES;
+        const int tb = tb_rs_tok_bits(h.vocab);
         for (int64_t u = 0; in && u < Ns; ++u) {
           TbRsRec rr;
           std::memcpy(&rr, bl + g->off_rsrec + 16 * u, 16);
@@ -204,7 +205,7 @@ extern "C" int tb_graph_load(const char* path, tb_graph** out) {
         for (int64_t e = 0; in && e < Re; ++e) {
           TbRsEnt re;
           std::memcpy(&re, bl + g->off_rsent + 8 * e, 8);
-          const uint32_t tok2 = re.dst_tok & ((1u << TB_RS_TOK_BITS) - 1), dst = re.dst_tok >> TB_RS_TOK_BITS;
+          const uint32_t tok2 = re.dst_tok & ((1u << tb) - 1), dst = re.dst_tok >> tb;
           in = tok2 <= 2u * static_cast<uint32_t>(h.vocab) && (tok2 & 1u) == 0 && dst < static_cast<uint32_t>(Ns);
         }
       }

@@ -95,7 +95,8 @@ static void finalize_graph(tb_graph* g, const int32_t* case_class, int32_t vocab
     std::vector<TbRsRec> rrecs(N);
     std::vector<TbRsEnt> rents;
     std::vector<int32_t> seen(n_classes, -1);   // class -> state that listed it during the current walk
-    bool fits = 2 * (vocab + 1) <= (1 << TB_RS_TOK_BITS) && N < (1 << (32 - TB_RS_TOK_BITS));
+    const int tb = tb_rs_tok_bits(vocab);
+    bool fits = N < (1 << (32 - tb));
     g->d_max = 0.0f;
     for (int32_t s = 0; s < N; ++s) {
       float acc = 0.0f;
@@ -109,7 +110,7 @@ static void finalize_graph(tb_graph* g, const int32_t* case_class, int32_t vocab
             const float bonus = acc + g->arc_w[a];
             const float lb = lambda * bonus;
             for (int32_t j = ctb[c]; j < ctb[c + 1]; ++j)
-              rents.push_back({(static_cast<uint32_t>(g->arc_dst[a]) << TB_RS_TOK_BITS) | static_cast<uint32_t>(2 * ctk[j]), lb});
+              rents.push_back({(static_cast<uint32_t>(g->arc_dst[a]) << tb) | static_cast<uint32_t>(2 * ctk[j]), lb});
           }
           if (rents.size() > TB_RS_MAX_ENTRIES) fits = false;
         }
@@ -117,8 +118,8 @@ static void finalize_graph(tb_graph* g, const int32_t* case_class, int32_t vocab
       }
       g->d_max = std::max(g->d_max, std::fabs(acc));
       if (fits) {
-        std::sort(rents.begin() + first, rents.end(), [](const TbRsEnt& x, const TbRsEnt& y) {
-          return (x.dst_tok & ((1u << TB_RS_TOK_BITS) - 1)) < (y.dst_tok & ((1u << TB_RS_TOK_BITS) - 1));
+        std::sort(rents.begin() + first, rents.end(), [tb](const TbRsEnt& x, const TbRsEnt& y) {
+          return (x.dst_tok & ((1u << tb) - 1)) < (y.dst_tok & ((1u << tb) - 1));
         });
         while ((rents.size() - first) % 4 != 0)   // sentinels: the blank column with lb = -inf
           rents.push_back({static_cast<uint32_t>(2 * vocab), -std::numeric_limits<float>::infinity()});

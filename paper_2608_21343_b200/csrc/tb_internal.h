@@ -116,6 +116,12 @@ struct TbRsEnt {
 static_assert(sizeof(TbRsRec) == 16 && sizeof(TbRsEnt) == 8, "record sizes");
 #define TB_RS_MAX_ENTRIES (1 << 18)
 #define TB_RS_TOK_BITS 12   /* 2 * token < 4096, i.e. vocab + 1 <= 2048 */
+// Larger vocabularies (read by the general and the two-step kernels only): 15 bits of 2 * token, 17 of the target state.
+#define TB_RS_TOK_BITS_WIDE 15
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int tb_rs_tok_bits(int32_t vocab) { return 2 * (vocab + 1) <= (1 << TB_RS_TOK_BITS) ? TB_RS_TOK_BITS : TB_RS_TOK_BITS_WIDE; }
 
 uint64_t tb_hash_class_map(const int32_t* case_class, int32_t vocab);
 

@@ -98,6 +98,19 @@ bool tb_greedy_seg_plan(const TbDecodeParams& p, int32_t max_cache_bytes, int32_
 size_t tb_greedy_seg_scratch_bytes(int32_t n_streams, int32_t frames, int32_t S, int32_t nseg_max);
 int tb_launch_greedy_seg(const TbDecodeParams& p, int32_t max_cache_bytes, const TbSegPlan& plan, void* scratch,
                          cudaStream_t stream);
+// The two-step kernels (tb_rows.cu): any vocabulary, fp32 or bf16, any strides with contiguous tokens, S <= 4.
+struct TbRowsPlan {
+  int32_t nseg = 0, cache_bytes = 0, smem = 0, all_resolved = 0;
+  size_t scratch_bytes = 0;
+};
+bool tb_rows_plan(const TbDecodeParams& p, int32_t max_cache_bytes, int32_t max_states, int32_t all_resolved, int32_t n_sm,
+                  int32_t max_smem, TbRowsPlan* plan);
+int tb_launch_rows(const TbDecodeParams& p, const TbRowsPlan& plan, int32_t n_sm, void* scratch, cudaStream_t stream);
+// One streaming chunk.  spill: device memory of tb_chunk_rows_spill_bytes, needed when a slot's graph has no resolved
+// lists (else null).  Returns 1 when the call is outside what the kernel covers.
+size_t tb_chunk_rows_spill_bytes(const TbDecodeParams& p);
+int tb_launch_chunk_rows(const TbDecodeParams& p, int32_t max_states, int32_t n_sm, int32_t max_smem, void* spill, cudaStream_t stream,
+                         const TbInlineBinds* binds);
 int tb_launch_beam_step(const TbBeamParams& p, cudaStream_t stream);
 int tb_launch_beam_frames(const TbBeamParams& p, int32_t T, int32_t E, int64_t frame_stride, int64_t row_stride,
                           cudaStream_t stream);

@@ -1,0 +1,757 @@
+// Device code of the two-step greedy decode (tb_rows.cu): rows of any vocabulary, fp32 or bf16, any strides with
+// contiguous tokens, reduced to 32-byte summaries, and the decider that walks a stretch of one stream from summaries.
+//
+// Step 1 (frames_summary, one warp per row, independent of the graph state): the row's best root-boosted token, a bound on
+// all others, its blank logit, and -- where asked for -- its log-softmax normaliser or its best duration.
+// Step 2 (decide, one warp per stretch): the sequential part.  A round looks at the rows (t, k), (t+1, 0), (t+2, 0),
+// (t+3, 0) under the current graph state at once: the lanes share out the state's list of boosted tokens, every lane
+// gathers its tokens' logits from the four rows, two warp-wide integer reductions per row find the best listed token
+// (largest value, then lowest token), lane r compares it with row r's summary, and one ballot gives the run of leading
+// blanks and the row that ends it.  What bounds it is the chain state -> list -> logits -> token -> state: a trip to
+// shared memory or L2 for each arrow and about 200 dependent instructions.
+//
+// The code is kept small on purpose (no register-resident lists, loops not unrolled beyond what keeps loads in flight,
+// options as uniform branches instead of instantiations): a chunk or a short utterance runs through it a few dozen times
+// only, and a first version of 130-250 KB spent most of its time fetching instructions (a 100-frame utterance: 83 us,
+// the same at 2 and at 16 stretches).
+//
+// Exactness: as in tb_greedy_fast.cu.  A summary's winner is accepted only when it clears every other token by a margin
+// that dominates all roundings, or when no token that is not listed can reach the best of {blank, listed tokens}; else
+// the row is evaluated exactly (exact_row).
+#ifndef TB_ROWS_CUH_
+#define TB_ROWS_CUH_
+
+#include <cuda_bf16.h>
+
+#include "tb_device.cuh"
+
+namespace {
+
+constexpr int kRowsPerFrame = 4;      // rows per frame (S) the summaries are laid out for
+constexpr int kWalkBuf = 256;         // entries of a list put together by walking that are kept in shared memory
+
+struct RowSum {      // 32 bytes, read as two 16-byte halves
+  float y1;          // best root-boosted token value of the row (ties: lowest id)
+  float y2b;         // upper bound on the root-boosted value of every other token
+  float xb;          // blank logit
+  float x1;          // raw logit of the best token
+  float rootcw1;     // root arc weight of the best token's class (0 if none)
+  int32_t rootdst1;  // root arc target of the best token's class (0 if none)
+  uint32_t packed;   // id1 | kRsOvf | kRsGap | duration << 24
+  float extra;       // the row's normaliser (log-softmax), or the logit of its best duration (TDT)
+};
+static_assert(sizeof(RowSum) == 32, "two 16-byte halves");
+constexpr uint32_t kRsIdMask = 0x3FFFu, kRsOvf = 1u << 16, kRsGap = 1u << 17, kRsAbsent = 1u << 18;
+
+// Order-preserving map float -> uint32 (-0 is folded into +0 first, so equal floats get equal keys).
+__device__ __forceinline__ uint32_t order_key(float v) {
+  const uint32_t u = __float_as_uint(v + 0.0f);
+  return u ^ ((u >> 31) ? 0xFFFFFFFFu : 0x80000000u);
+}
+__device__ __forceinline__ float order_key_inv(uint32_t k) {
+  return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xFFFFFFFFu));
+}
+
+// ---- the graph's root in shared memory: weight and arc per class -------------------------------------------------
+struct RootTab {
+  float* w;          // [C] root arc weight (0 if none)
+  uint16_t* arc;     // [C] root arc + 1 (0 if none)
+  float* stats;      // beta_min, beta_max, largest |w|
+};
+__host__ __device__ inline size_t root_tab_bytes(int C) {
+  return ((static_cast<size_t>(C) * 4 + 15) & ~size_t(15)) + ((static_cast<size_t>(C) * 2 + 15) & ~size_t(15)) + 16;
+}
+__device__ __forceinline__ RootTab root_tab_at(unsigned char* mem, int C) {
+  RootTab r;
+  r.w = reinterpret_cast<float*>(mem);
+  mem += (static_cast<size_t>(C) * 4 + 15) & ~size_t(15);
+  r.arc = reinterpret_cast<uint16_t*>(mem);
+  mem += (static_cast<size_t>(C) * 2 + 15) & ~size_t(15);
+  r.stats = reinterpret_cast<float*>(mem);
+  return r;
+}
+// Block-wide (three barriers); part: 3 floats per warp of scratch shared memory.
+__device__ inline void root_tab_fill(const RootTab& r, const GraphPtrs& g, bool bound, float lam, int C, float* part) {
+  const int tid = threadIdx.x, n = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarps = (n + 31) >> 5;
+#pragma unroll 1
+  for (int c = tid; c < C; c += n) { r.w[c] = 0.0f; r.arc[c] = 0; }
+  __syncthreads();
+  float bmin = 0.0f, bmax = 0.0f, R = 0.0f;
+  if (bound) {
+    const int a0 = g.arc_begin[0], e = g.arc_begin[1];
+#pragma unroll 1
+    for (int a = a0 + tid; a < e; a += n) {
+      const int c = g.arc_cls[a];
+      const float wv = __fadd_rn(0.0f, g.arc_w[a]);          // the walk's fl(acc + w) with acc = 0
+      const float cb = __fmul_rn(lam, wv);
+      if (c >= 0 && c < C) { r.w[c] = wv; r.arc[c] = static_cast<uint16_t>(a - a0 + 1); }
+      bmin = fminf(bmin, cb); bmax = fmaxf(bmax, cb); R = fmaxf(R, fabsf(wv));
+    }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    bmin = fminf(bmin, __shfl_xor_sync(0xffffffffu, bmin, off));
+    bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, off));
+    R = fmaxf(R, __shfl_xor_sync(0xffffffffu, R, off));
+  }
+  if (lane == 0) { part[3 * warp] = bmin; part[3 * warp + 1] = bmax; part[3 * warp + 2] = R; }
+  __syncthreads();
+  if (tid == 0) {
+#pragma unroll 1
+    for (int w2 = 1; w2 < nwarps; ++w2) {
+      bmin = fminf(bmin, part[3 * w2]); bmax = fmaxf(bmax, part[3 * w2 + 1]); R = fmaxf(R, part[3 * w2 + 2]);
+    }
+    r.stats[0] = bmin; r.stats[1] = bmax; r.stats[2] = R;
+  }
+  __syncthreads();
+}
+
+// ---- step 1: one row -> summary -----------------------------------------------------------------------------------
+struct RowCtx {
+  const float* rootw; const uint16_t* rootarc;   // RootTab
+  const int32_t* cls;                            // device [V] token -> class
+  const float* arc_w; const int32_t* arc_dst;    // the root's arcs
+  float lam, beta_min, beta_max, bmag_max;       // bmag_max: bound on |lambda| * (|D(s)| + largest root weight) over all states s
+  bool boosts, norm;                             // the root has arcs; the row's normaliser is wanted
+  int V, n_dur;
+};
+
+// G 16-byte blocks per lane: one group of a row is 32 * G blocks.
+template <typename LT> struct RowBlock;
+template <> struct RowBlock<uint16_t> {          // eight bf16 each
+  static constexpr int E = 8;
+  static constexpr uint32_t kNone = 0xFF80FF80u;   // -inf
+  static __device__ __forceinline__ __nv_bfloat162 h2(uint32_t w) { __nv_bfloat162 r; *reinterpret_cast<uint32_t*>(&r) = w; return r; }
+  template <int G> static __device__ __forceinline__ float max(const uint4 (&q)[G]) {
+    __nv_bfloat162 m = h2(kNone);
+#pragma unroll
+    for (int u = 0; u < G; ++u) m = __hmax2(m, __hmax2(__hmax2(h2(q[u].x), h2(q[u].y)), __hmax2(h2(q[u].z), h2(q[u].w))));
+    const uint32_t w = *reinterpret_cast<const uint32_t*>(&m);
+    return fmaxf(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+  }
+  static __device__ __forceinline__ float threshold(float t) { return __bfloat162float(__float2bfloat16_rd(t)); }
+  // one bit per element of blocks u0 .. u0 + 3 at or above t (a value of `threshold`): bit 4 u + i + 16 h is half h of word i
+  static constexpr int kUnits = 4;
+  template <int G> static __device__ __forceinline__ uint32_t hits(const uint4 (&q)[G], int u0, float t) {
+    const __nv_bfloat162 t2 = __float2bfloat162_rn(t);
+    uint32_t r = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      r |= __hge2_mask(h2(q[u0 + u].x), t2) & (0x00010001u << (4 * u));
+      r |= __hge2_mask(h2(q[u0 + u].y), t2) & (0x00010001u << (4 * u + 1));
+      r |= __hge2_mask(h2(q[u0 + u].z), t2) & (0x00010001u << (4 * u + 2));
+      r |= __hge2_mask(h2(q[u0 + u].w), t2) & (0x00010001u << (4 * u + 3));
+    }
+    return r;
+  }
+  static __device__ __forceinline__ int unit(int bit) { return (bit & 15) >> 2; }
+  static __device__ __forceinline__ int elem(int bit) { return (bit & 3) * 2 + (bit >> 4); }
+  template <typename F> static __device__ __forceinline__ void each2(const uint4& q, F f) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { const uint32_t w = (&q.x)[i]; f(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
+  }
+};
+template <> struct RowBlock<float> {             // four floats each
+  static constexpr int E = 4;
+  static constexpr uint32_t kNone = 0xFF800000u;
+  template <int G> static __device__ __forceinline__ float max(const uint4 (&q)[G]) {
+    float m = -INFINITY;
+#pragma unroll
+    for (int u = 0; u < G; ++u)
+      m = fmaxf(m, fmaxf(fmaxf(__uint_as_float(q[u].x), __uint_as_float(q[u].y)), fmaxf(__uint_as_float(q[u].z), __uint_as_float(q[u].w))));
+    return m;
+  }
+  static __device__ __forceinline__ float threshold(float t) { return t; }
+  static constexpr int kUnits = 8;
+  template <int G> static __device__ __forceinline__ uint32_t hits(const uint4 (&q)[G], int, float t) {
+    uint32_t r = 0;
+#pragma unroll
+    for (int u = 0; u < G; ++u)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) r |= __uint_as_float((&q[u].x)[i]) >= t ? 1u << (4 * u + i) : 0u;
+    return r;
+  }
+  static __device__ __forceinline__ int unit(int bit) { return bit >> 2; }
+  static __device__ __forceinline__ int elem(int bit) { return bit & 3; }
+  template <typename F> static __device__ __forceinline__ void each2(const uint4& q, F f) {
+    f(__uint_as_float(q.x), __uint_as_float(q.y)); f(__uint_as_float(q.z), __uint_as_float(q.w));
+  }
+};
+__device__ __forceinline__ float exp2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// The rows of up to 32 frames by one warp: frames f0, f0 + step, ... (n of them), row k of a frame only when row k - 1 is
+// likely to select a token (its best root-boosted token reaches the blank less a margin); a row left out is marked
+// kRsAbsent, and a decider that gets there after all evaluates it exactly.  About half the rows of three per frame are
+// never visited, and fewer still are read here.  sums: the summary of row 0 of frame 0.
+//
+// One row: a pass over its groups of 32 * G aligned 16-byte blocks for the maximum, then a pass for the few candidates --
+// over the last group, still in registers, and from L1 over the groups before it.  The elements before the first and
+// after the last aligned block are one per lane; nothing outside the row is read.  The next row's blocks are requested
+// before a row's candidates are looked at, where a row is one group.  What is the same for all lanes is kept by lane i
+// for frame i and finished for all frames of a pass at once (root arcs, normalisers, durations, the store).
+template <typename LT, int G>
+__device__ __forceinline__ void frames_summary(const RowCtx& h, const LT* base, int64_t st, int64_t ss, int S, int f0, int step, int n,
+                                               RowSum* sums, int fmask, int lane) {
+  using RB = RowBlock<LT>;
+  constexpr int E = RB::E;
+  const int V = h.V;
+  const float kL2e = 1.4426950408889634f;
+  unsigned todo = n >= 32 ? 0xFFFFFFFFu : (1u << n) - 1u;
+  const float margin = 0.5f * h.beta_max;
+#pragma unroll 1
+  for (int k = 0; k < S; ++k) {
+    // this lane's frame: what the warp finds out about its row
+    float m_y1 = -INFINITY, m_y2 = -INFINITY, m_M = 0.0f, m_acc = 0.0f;
+    int m_id = 0x7FFFFFFF;
+    const LT* row0 = base + static_cast<int64_t>(f0) * st + static_cast<int64_t>(k) * ss;
+    const int64_t fstep = static_cast<int64_t>(step) * st;
+    uint4 q[G];
+    float xs;
+    const LT* row = nullptr;
+    int hd = 0, nb = 0, sidx = 0;
+    bool sok = false;
+    auto begin = [&](int i) {                                  // geometry and first group of frame i's row
+      row = row0 + static_cast<int64_t>(i) * fstep;
+      hd = min(V, static_cast<int>((16u - static_cast<uint32_t>(reinterpret_cast<uintptr_t>(row) & 15)) & 15u) / static_cast<int>(sizeof(LT)));
+      nb = (V - hd) / E;
+      sidx = lane < hd ? lane : nb * E + lane;                 // this lane's element outside the blocks
+      sok = sidx < V && lane < 2 * E;
+      xs = -INFINITY;
+      if (sok) xs = LogitLoad<LT>::at(row + sidx);
+    };
+    auto load = [&](int g) {
+      const uint4* blk = reinterpret_cast<const uint4*>(row + hd) + lane;
+#pragma unroll
+      for (int u = 0; u < G; ++u) {
+        q[u] = make_uint4(RB::kNone, RB::kNone, RB::kNone, RB::kNone);
+        if (g + 32 * u + lane < nb) q[u] = __ldg(blk + g + 32 * u);
+      }
+    };
+    unsigned left = todo;
+    int i = __ffs(left) - 1;
+    if (i >= 0) { begin(i); load(0); }
+#pragma unroll 1
+    while (left) {
+      left &= left - 1u;
+      const LT* rowi = row;
+      const int hdi = hd, nbi = nb, si = sidx;
+      const bool soki = sok;
+      const float xsi = xs;
+      const int inext = __ffs(left) - 1;
+      float m = fmaxf(xsi, RB::template max<G>(q));
+      int g_last = 0;
+#pragma unroll 1
+      for (int g = 32 * G; g < nb; g += 32 * G) { load(g); m = fmaxf(m, RB::template max<G>(q)); g_last = g; }
+      const float mf = order_key_inv(__reduce_max_sync(0xffffffffu, order_key(m)));
+      // every token whose root-boosted value can reach that of the raw maximum has x >= m - (beta_max - beta_min); gamma
+      // keeps a strict margin over all roundings
+      const float gamma = (fabsf(mf) + fabsf(h.beta_max) + fabsf(h.beta_min)) * 0.0009765625f + 1e-30f;
+      const float thr = RB::threshold(__fsub_rn(__fsub_rn(mf, __fsub_rn(h.beta_max, h.beta_min)), gamma));
+      // L = M + log(sum_v exp(x_v - M)): one fused multiply-add and one exponential per entry, see tb_fast_common.cuh
+      float M = 0.0f, acc0 = 0.0f, acc1 = 0.0f;
+      if (h.norm) M = fmaxf(mf, LogitLoad<LT>::at(rowi + V));
+      const float nc = -__fmul_rn(M, kL2e);
+      ValId b{-INFINITY, INT32_MAX};
+      float sec = -INFINITY;
+      auto offer = [&](int idx) {
+        const float cb = h.boosts ? __fmul_rn(h.lam, h.rootw[__ldg(h.cls + idx)]) : 0.0f;
+        const ValId c{__fadd_rn(LogitLoad<LT>::at(rowi + idx), cb), idx};
+        if (better(c, b)) { sec = fmaxf(sec, b.v); b = c; } else { sec = fmaxf(sec, c.v); }
+      };
+#pragma unroll 1
+      for (int g = g_last; g >= 0; g -= 32 * G) {
+        if (g != g_last) load(g);
+        if (h.norm) {
+#pragma unroll
+          for (int u = 0; u < G; ++u)
+            RB::each2(q[u], [&](float x0, float x1) {
+              acc0 = __fadd_rn(acc0, exp2_approx(__fmaf_rn(x0, kL2e, nc)));
+              acc1 = __fadd_rn(acc1, exp2_approx(__fmaf_rn(x1, kL2e, nc)));
+            });
+        }
+        uint32_t hits = RB::template hits<G>(q, 0, thr), hits2 = 0u;
+        if constexpr (RB::kUnits < G) hits2 = RB::template hits<G>(q, RB::kUnits, thr);
+        if (g == 0 && inext >= 0) {                            // (q is free: the next row is on its way from here on)
+          begin(inext);
+          load(0);
+        }
+        int ub = g + lane;
+#pragma unroll 1
+        for (;;) {
+          if (hits == 0u) {
+            if (hits2 == 0u) break;
+            hits = hits2; hits2 = 0u; ub += 32 * RB::kUnits;
+          }
+          const int bit = __ffs(hits) - 1;
+          hits &= hits - 1u;
+          const int bi = ub + 32 * RB::unit(bit);
+          if (bi < nbi) offer(hdi + bi * E + RB::elem(bit));   // (places without a block pass only a threshold of -inf)
+        }
+      }
+      if (soki && xsi >= thr) offer(si);
+      if (h.norm) {
+        float acc = __fadd_rn(acc0, acc1);
+        if (soki) acc = __fadd_rn(acc, exp2_approx(__fmaf_rn(xsi, kL2e, nc)));
+        if (lane == 0) acc = __fadd_rn(acc, exp2_approx(__fmaf_rn(LogitLoad<LT>::at(rowi + V), kL2e, nc)));
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) acc = __fadd_rn(acc, __shfl_xor_sync(0xffffffffu, acc, off));
+        if (lane == i) { m_M = M; m_acc = acc; }
+      }
+      // across the warp: best (value, lowest id) and the runner-up value; tokens that are not candidates have x < thr,
+      // hence a root-boosted value <= fl(thr + beta_max)
+      const uint32_t key = order_key(b.v);
+      const uint32_t kmax = __reduce_max_sync(0xffffffffu, key);
+      const int idmin = static_cast<int>(__reduce_min_sync(0xffffffffu, key == kmax ? static_cast<uint32_t>(b.i) : 0x7FFFFFFFu));
+      const uint32_t k2 = __reduce_max_sync(0xffffffffu, order_key((key == kmax && b.i == idmin) ? sec : b.v));
+      if (lane == i) { m_y1 = order_key_inv(kmax); m_id = idmin; m_y2 = fmaxf(order_key_inv(k2), __fadd_rn(thr, h.beta_max)); }
+      i = inext;
+    }
+    // ---- lane i finishes frame i's row
+    bool need = false;
+    if (lane < n) {
+      const int f = f0 + lane * step;
+      uint4* o = reinterpret_cast<uint4*>(sums + (f & fmask) * S + k);
+      uint4 w0 = make_uint4(0u, 0u, 0u, 0u), w1 = make_uint4(0u, 0u, kRsAbsent, 0u);
+      if ((todo >> lane) & 1u) {
+        const LT* r = row0 + static_cast<int64_t>(lane) * fstep;
+        const bool ovf = m_id >= V;                            // no candidate at all (cannot happen with finite logits)
+        const int id1 = ovf ? 0 : m_id;
+        const int a1 = h.boosts ? h.rootarc[__ldg(h.cls + id1)] : 0;
+        const float x1 = LogitLoad<LT>::at(r + id1), xb = LogitLoad<LT>::at(r + V);
+        float cw = 0.0f, extra = 0.0f;
+        int cd = 0, dur = 0;
+        if (a1) { cw = __fadd_rn(0.0f, h.arc_w[a1 - 1]); cd = h.arc_dst[a1 - 1]; }
+        if (h.norm && m_M != -INFINITY) {
+          const float c_lo = __fmaf_rn(m_M, kL2e, -__fmul_rn(m_M, kL2e));      // what the rounding of M * log2(e) left out, exactly
+          extra = __fadd_rn(m_M, __fsub_rn(logf(m_acc), __fmul_rn(c_lo, 0.6931471805599453f)));
+        }
+#pragma unroll 4
+        for (int d = 0; d < h.n_dur; ++d) {                    // the row's best duration (lowest on ties)
+          const float xd = LogitLoad<LT>::at(r + V + 1 + d);
+          if (d == 0 || xd > extra) { extra = xd; dur = d; }
+        }
+        // the same margin as the decider's, with the largest scale any state can have
+        const float tau = (fabsf(m_y1) + 4.0f * h.bmag_max) * 1.9073486328125e-6f + 1e-30f;
+        w0 = make_uint4(__float_as_uint(m_y1), __float_as_uint(m_y2), __float_as_uint(xb), __float_as_uint(x1));
+        w1 = make_uint4(__float_as_uint(cw), static_cast<uint32_t>(cd),
+                        static_cast<uint32_t>(id1) | (ovf ? kRsOvf : 0u) | ((m_y1 - m_y2 > tau) ? kRsGap : 0u) | (static_cast<uint32_t>(dur) << 24),
+                        __float_as_uint(extra));
+        // (a row whose duration moves the cursor on has no row after it; normalisers are wanted for every row)
+        need = h.norm || ((ovf || !(m_y1 + margin < xb)) && dur == 0);
+      }
+      o[0] = w0; o[1] = w1;
+    }
+    todo = __ballot_sync(0xffffffffu, need);
+  }
+  __syncwarp();
+}
+
+// ---- step 2: the decider -------------------------------------------------------------------------------------------
+__device__ __forceinline__ uint4 lds128(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t shared_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
+
+// What a decider needs to know about its stream's graph and rows; the same for all lanes.
+template <typename LT>
+struct DecideCtx {
+  const LT* base;                  // row (frame 0 of the call, row 0) of the stream
+  int64_t st, ss;                  // element strides: frame, row in frame
+  int V, S, n_dur, tb;             // tb: bits of 2 * token in a list entry (tb_rs_tok_bits)
+  bool bound, resolved, norm;
+  int n_states, max_depth;
+  float lam, R;                    // lambda; largest |root arc weight|
+  const TbRsRec* rsrec;            // resolved lists, in the arena or in shared memory
+  const TbRsEnt* rsent;
+  const TbStateRec* strec;         // without resolved lists: what the suffix-chain walk reads
+  const TbTokEnt* tokent;
+  RootTab root;
+  const int32_t* cls; const float* arc_w; const int32_t* arc_dst;
+  uint32_t* bitmap;                // [(V + 32) / 32] shared memory of this warp, zero between uses
+  TbRsEnt* walk_buf;               // [kWalkBuf] shared memory of this warp, and
+  TbRsEnt* spill;                  // [V + 32] global memory: lists put together by walking (null: the lists are resolved)
+  int32_t* status;
+};
+
+// The tokens boosted by the non-root part of the current state's suffix chain: entries {target << tb | 2 * token, lb},
+// lb = fl(lambda * fl(acc + w)).  Resolved lists are read where they lie.
+struct TokList {
+  const TbRsEnt* ent;
+  int n;
+  float D, bmag;
+};
+// {target << tb | 2 token} -> {2 token | target}: an integer minimum finds the lowest token and its target at once
+__device__ __forceinline__ uint32_t td_pack(uint32_t dst_tok, int tb) { return __funnelshift_r(dst_tok, dst_tok, tb); }
+__device__ __forceinline__ int td_tok(uint32_t td, int tb) { return static_cast<int>(td >> (33 - tb)); }
+__device__ __forceinline__ int td_dst(uint32_t td, int tb) { return static_cast<int>(td & (0xFFFFFFFFu >> tb)); }
+
+// The list of state s (warp-wide).
+template <typename LT>
+__device__ __forceinline__ TokList list_of(const DecideCtx<LT>& c, int s, int lane) {
+  TokList L;
+  if (c.resolved) {
+    L.ent = c.rsent; L.n = 0; L.D = 0.0f; L.bmag = fabsf(c.lam) * c.R;
+    if (s > 0) {                                              // (the root's list is empty)
+      const uint4 r = *reinterpret_cast<const uint4*>(c.rsrec + s);
+      L.ent += r.x; L.n = static_cast<int>(r.y); L.D = __uint_as_float(r.z); L.bmag = __uint_as_float(r.w);
+    }
+    return L;
+  }
+  // Chain walk: the chain state closest to s first; a token whose class a closer state lists is in the bitmap already.
+  // acc = suffix-link weights crossed so far, in walk order.
+  int n = 0;
+  float acc = 0.0f;
+  int u = s > 0 ? s : 0;
+  uint4 rec = make_uint4(0u, 0u, 0u, 0u);                     // TbStateRec
+  if (u != 0) rec = *reinterpret_cast<const uint4*>(c.strec + u);
+#pragma unroll 1
+  for (int it = 0; u != 0; ++it) {
+    if (it > c.max_depth + 1) { if (lane == 0) atomicOr(c.status, TB_STATUS_WALK_TOO_DEEP); break; }
+    // the next chain state's record is requested before this state's arcs are: the two trips to L2 overlap
+    const int nu = (static_cast<int>(rec.z) > 0 && static_cast<int>(rec.z) < c.n_states) ? static_cast<int>(rec.z) : 0;
+    uint4 nrec = rec;
+    if (nu > 0) nrec = *reinterpret_cast<const uint4*>(c.strec + nu);
+    const int e1 = static_cast<int>(rec.y);
+#pragma unroll 2
+    for (int e = static_cast<int>(rec.x) + lane; __any_sync(0xffffffffu, e < e1); e += 32) {
+      uint4 ent = make_uint4(0u, 0u, 0u, 0u);                 // TbTokEnt
+      if (e < e1) ent = *reinterpret_cast<const uint4*>(c.tokent + e);
+      const int tk = static_cast<int>(ent.x & 0xFFFFu);
+      const bool fresh = e < e1 && !((c.bitmap[tk >> 5] >> (tk & 31)) & 1u);
+      const unsigned mask = __ballot_sync(0xffffffffu, fresh);
+      if (fresh) {
+        atomicOr(&c.bitmap[tk >> 5], 1u << (tk & 31));
+        TbRsEnt o;
+        o.dst_tok = (ent.z << c.tb) | (2u * static_cast<uint32_t>(tk));
+        o.lb = __fmul_rn(c.lam, __fadd_rn(acc, __uint_as_float(ent.y)));
+        const int at = n + __popc(mask & ((1u << lane) - 1u));
+        c.spill[at] = o;
+        if (at < kWalkBuf) c.walk_buf[at] = o;
+      }
+      n += __popc(mask);
+    }
+    __syncwarp();
+    acc = __fadd_rn(acc, __uint_as_float(rec.w));
+    u = nu;
+    rec = nrec;
+  }
+  L.n = n; L.D = acc; L.bmag = fabsf(c.lam) * (fabsf(acc) + c.R);
+  L.ent = n <= kWalkBuf ? c.walk_buf : c.spill;
+#pragma unroll 1
+  for (int i = lane; i < n; i += 32) c.bitmap[(L.ent[i].dst_tok & ((1u << c.tb) - 1u)) >> 6] = 0u;
+  __syncwarp();
+  return L;
+}
+
+struct RowPick { float val; int tok, next, dur; float xdur; };   // tok == V: blank
+
+// Exact evaluation of one row under the current state by the whole warp.
+template <typename LT>
+__device__ __forceinline__ RowPick exact_row(const DecideCtx<LT>& c, const TokList& L, const LT* row, int s, int lane) {
+  ValId best{LogitLoad<LT>::at(row + c.V), c.V};
+  int bn = s;
+#pragma unroll 1
+  for (int i = lane; i < L.n; i += 32) {
+    const TbRsEnt e = L.ent[i];
+    const int tk = static_cast<int>((e.dst_tok & ((1u << c.tb) - 1u)) >> 1);
+    if (tk >= c.V) continue;                                   // (padding)
+    atomicOr(&c.bitmap[tk >> 5], 1u << (tk & 31));
+    const ValId o{__fadd_rn(LogitLoad<LT>::at(row + tk), e.lb), tk};
+    if (better(o, best)) { best = o; bn = static_cast<int>(e.dst_tok >> c.tb); }
+  }
+  __syncwarp();
+#pragma unroll 4
+  for (int tk = lane; tk < c.V; tk += 32) {
+    const float x = LogitLoad<LT>::at(row + tk);
+    float v = x;
+    int nx = -1;
+    if (c.bound) {
+      const int cl = __ldg(c.cls + tk);
+      v = __fadd_rn(x, __fmul_rn(c.lam, __fadd_rn(L.D, c.root.w[cl])));
+      nx = c.root.arc[cl];
+      nx = nx ? -1 - nx : 0;                                   // (the arc's target is looked up for the winner only)
+    }
+    const ValId o{v, tk};
+    if (!((c.bitmap[tk >> 5] >> (tk & 31)) & 1u) && better(o, best)) { best = o; bn = nx; }
+  }
+  __syncwarp();
+#pragma unroll 1
+  for (int i = lane; i < L.n; i += 32) c.bitmap[(L.ent[i].dst_tok & ((1u << c.tb) - 1u)) >> 6] = 0u;
+  __syncwarp();
+  const uint32_t key = order_key(best.v);
+  const uint32_t kmax = __reduce_max_sync(0xffffffffu, key);
+  const uint32_t idmin = __reduce_min_sync(0xffffffffu, key == kmax ? static_cast<uint32_t>(best.i) : 0xFFFFFFFFu);
+  const unsigned who = __ballot_sync(0xffffffffu, key == kmax && static_cast<uint32_t>(best.i) == idmin);
+  const int src = __ffs(who) - 1;
+  RowPick pk;
+  pk.dur = 0; pk.xdur = 0.0f;
+#pragma unroll 1
+  for (int d = 0; d < c.n_dur; ++d) {                          // the row's best duration (lowest on ties)
+    const float xd = LogitLoad<LT>::at(row + c.V + 1 + d);
+    if (d == 0 || xd > pk.xdur) { pk.xdur = xd; pk.dur = d; }
+  }
+  pk.val = __shfl_sync(0xffffffffu, best.v, src);
+  pk.tok = static_cast<int>(idmin);
+  pk.next = __shfl_sync(0xffffffffu, bn, src);
+  if (pk.tok == c.V) pk.next = s;
+  else if (!c.bound) pk.next = -1;
+  else if (pk.next < 0) pk.next = c.arc_dst[-pk.next - 2];     // -1 - (arc + 1) -> arc
+  return pk;
+}
+
+// Where a decider stands.
+struct Cursor {
+  int t, k, s;          // frame, row in frame, graph state
+  int n_out, nv;        // tokens emitted, row values logged
+  bool stable;          // the last token left the state unchanged
+  bool failed;
+  int met;              // frame start at which it met a later stretch of the stream (-1: none)
+  bool listed;          // list is that of state s
+  TokList list;
+};
+// Where its results go.
+struct DecideOut {
+  int32_t* tok; int32_t* frm; int32_t* dur;   // emitted tokens, their frames, durations (dur may be null)
+  float* vals;                                // value of every visited row, in order
+  int cap;                                    // places in tok / frm
+  // a stretch of an offline decode (SEG): the graph state at every frame start it answers for, [first, next), and how
+  // much it had logged there; past `next` it stops where its state is the one recorded there
+  volatile int32_t* trace; int2* trace_aux;
+  int first, next;
+  bool is_last, prefetch;
+};
+
+// Decides the rows from the cursor on, up to frame `end` (exclusive).  Summaries of row k of frame f are at shared
+// address sum_a + (((f - f0) & mask) * S + k) * 32; SEG: that is a ring of mask + 1 frames which the decider fills itself
+// from gsum (the summary of row 0 of frame 0), else they are all in place.  f0: the frame the rows (c.base) start at.
+template <typename LT, bool SEG>
+__device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const DecideOut& o, const RowSum* gsum,
+                                       uint32_t sum_a, int mask, int f0, int end, int lane) {
+  const int S = c.S, V = c.V, tb = c.tb;
+  const bool tdt = !SEG && c.n_dur > 0;
+  int t = cu.t, k = cu.k, s = cu.s, n_out = cu.n_out, nv = cu.nv;
+  bool stable = cu.stable, no_grid = false, listed = cu.listed;
+  TokList L = cu.list;
+  const uint32_t none = (2u * static_cast<uint32_t>(V)) << (32 - tb), tmask = (1u << tb) - 1u;
+  // what a row adds to the score: its value less its normaliser, or plus its duration's logit
+  auto adjust = [&](float v, float extra) { return c.norm ? __fsub_rn(v, extra) : tdt ? __fadd_rn(v, extra) : v; };
+  auto trace = [&](int fs, int st_, int n_tok, int n_val) {
+    if (SEG && fs >= o.first && fs < o.next) { o.trace_aux[fs] = make_int2(n_tok, n_val); o.trace[fs] = st_; }
+  };
+  if (SEG && lane == 0 && k == 0) trace(t, s, n_out, nv);
+  int loaded = t & ~3, refill = t;            // SEG: frames up to `loaded` have been asked for; the next group is due at frame `refill`
+  const int max_rounds = (end - t) * (S + 1) + 8;
+#pragma unroll 1
+  for (int it = 0; t < end; ++it) {
+    if (it >= max_rounds) { if (lane == 0) atomicOr(c.status, TB_STATUS_STEP_LIMIT); cu.failed = true; break; }
+    if (SEG) {
+      if (k == 0 && t >= o.next && !o.is_last) {
+        if (!c.bound || o.trace[t] == s) { cu.met = t; break; }     // (unbound: no graph state, the owner's decode from here is this one's)
+      }
+      // the ring, in groups of four frames: those up to 12 frames ahead are in place, the next group is on its way; the
+      // rows of the next frames are asked into L2, which this stretch's rows have long left when the call's logits are
+      // larger than it
+      if (t >= refill) {
+        do {
+          if (loaded < end) {
+            const int nq = min(4, end - loaded) * S * 2;
+            const uint4* src = reinterpret_cast<const uint4*>(gsum + static_cast<int64_t>(loaded) * S);
+            const uint32_t dst = sum_a + static_cast<uint32_t>((loaded & mask) * S) * 32u;
+            if (lane < nq) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16u * lane), "l"(src + lane) : "memory");
+          }
+          asm volatile("cp.async.commit_group;" ::: "memory");
+          loaded += 4;
+        } while (loaded < t + 16);
+        refill = (t & ~3) + 4;
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        if (o.prefetch && lane < 4 * S) {
+          const int f = refill + 4 + lane / S;
+          if (f < end) {
+            const unsigned char* pr = reinterpret_cast<const unsigned char*>(c.base + static_cast<int64_t>(f) * c.st + static_cast<int64_t>(lane % S) * c.ss);
+            const uintptr_t p0 = (reinterpret_cast<uintptr_t>(pr) + 15) & ~static_cast<uintptr_t>(15);
+            const uint32_t bytes = static_cast<uint32_t>(V) * sizeof(LT) - 16u & ~15u;
+            if (V * sizeof(LT) > 64) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p0), "r"(bytes) : "memory");
+          }
+        }
+        __syncwarp();
+      }
+    }
+    if (!listed) { L = list_of(c, s, lane); listed = true; }
+    // Two kinds of round.  List round: the eight lanes 8 r .. 8 r + 7 take row r of {(t, k), (t + 1, 0), (t + 2, 0),
+    // (t + 3, 0)} and share out the list.  Grid round (no boosted tokens, or a state that just repeated itself): lane
+    // 4 q + j resolves row (t + q, j) on its own, and the walk goes through tokens too while they leave the state unchanged.
+    const bool grid = !tdt && !no_grid && (L.n == 0 || (stable && L.n <= 64));
+    no_grid = false;
+    const int left = end - 1 - t;              // frames after the current one
+    const int r = grid ? lane >> 2 : lane >> 3;
+    const int rk = grid ? min(lane & 3, S - 1) : r == 0 ? k : 0;
+    const bool valid = r <= left;
+    const LT* row = c.base + static_cast<int64_t>(t - f0 + min(r, left)) * c.st + static_cast<int64_t>(rk) * c.ss;
+    const uint32_t a = sum_a + static_cast<uint32_t>(((t + r - f0) & mask) * S + rk) * 32u;
+    const uint4 q1 = lds128(a + 16u), q0 = lds128(a);
+    const uint32_t id1x2 = 2u * (q1.z & kRsIdMask);
+    float lv = -INFINITY;
+    uint32_t lt = none;
+    bool in_deep = false;
+    {
+      const int step = grid ? 1 : 8;
+#pragma unroll 1
+      for (int i0 = grid ? 0 : lane & 7; i0 < L.n; i0 += 4 * step) {
+        uint2 e[4];
+        float x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          e[u] = make_uint2(2u * static_cast<uint32_t>(V), 0xFF800000u);
+          if (i0 + u * step < L.n) e[u] = *reinterpret_cast<const uint2*>(L.ent + i0 + u * step);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = LogitLoad<LT>::at(row + ((e[u].x & tmask) >> 1));
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const uint32_t td = td_pack(e[u].x, tb);
+          const float v = __fadd_rn(x[u], __uint_as_float(e[u].y));
+          if (v > lv || (v == lv && td < lt)) { lv = v; lt = td; }
+          in_deep |= (e[u].x & tmask) == id1x2;
+        }
+      }
+    }
+    if (!grid) {
+      // the group's best (largest value, then lowest token), in all its lanes
+#pragma unroll
+      for (int off = 1; off <= 4; off <<= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, lv, off);
+        const uint32_t ot = __shfl_xor_sync(0xffffffffu, lt, off);
+        if (ov > lv || (ov == lv && ot < lt)) { lv = ov; lt = ot; }
+      }
+      in_deep = ((__ballot_sync(0xffffffffu, in_deep) >> (8 * r)) & 0xFFu) != 0u;
+    }
+    // the row's pick: the best plain token is exact when the summary's winner is not listed and clears the others by the
+    // rounding margin (at the root it is exact by construction); else it is bounded from above
+    const float y1 = __uint_as_float(q0.x), y2b = __uint_as_float(q0.y), xb = __uint_as_float(q0.z), x1 = __uint_as_float(q0.w);
+    const float extra = __uint_as_float(q1.w);
+    const int id1 = static_cast<int>(id1x2 >> 1), dur = static_cast<int>(q1.z >> 24);
+    float wv = lv;
+    int wtok = td_tok(lt, tb), wnext = td_dst(lt, tb);
+    bool rescan = (q1.z & (kRsOvf | kRsAbsent)) != 0;
+    {
+      const bool plain_ok = !in_deep && ((q1.z & kRsGap) != 0 || s <= 0);
+      const float nd = __fadd_rn(x1, __fmul_rn(c.lam, __fadd_rn(L.D, __uint_as_float(q1.x))));
+      const float ub = (in_deep ? y2b : y1) + c.lam * L.D;
+      const float tau = (fabsf(y1) + 4.0f * L.bmag) * 3.814697265625e-6f + 1e-30f;
+      rescan = rescan || (!plain_ok && !(fmaxf(wv, xb) > ub + tau));
+      if (plain_ok && (nd > wv || (nd == wv && id1 < wtok))) { wv = nd; wtok = id1; wnext = c.bound ? static_cast<int>(q1.y) : -1; }
+    }
+    const bool blank = !(wv >= xb);                            // (a tie with blank goes to the token)
+
+    int tok = V, tnext = s;                                    // the token that ends the round (V: none) and where it leads
+    if (grid) {
+      const bool ready = (lane & 3) < S && (r > 0 || (lane & 3) >= k) && valid && !rescan;
+      const unsigned ready_all = __ballot_sync(0xffffffffu, ready);
+      const unsigned blank_all = __ballot_sync(0xffffffffu, ready && blank);
+      const unsigned keep_all = __ballot_sync(0xffffffffu, wnext == s);
+      // Which rows the decode visits follows from the blank / token pattern alone while the state stays what it is: in a
+      // frame, row j is visited when rows 0 .. j-1 selected tokens (bit 4 q + j: row j of frame t + q).
+      const unsigned m1 = 0x11111111u;
+      const unsigned smask = S >= 4 ? 0xFFFFFFFFu : (m1 << S) - m1;
+      const unsigned pre = (1u << k) - 1u;
+      const unsigned tok_all = ready_all & ~blank_all;
+      const unsigned tokx = tok_all | pre;
+      const unsigned a0 = tokx & m1, a1 = (tokx >> 1) & m1, a2 = (tokx >> 2) & m1;
+      const unsigned vis = (m1 | (a0 << 1) | ((a0 & a1) << 2) | ((a0 & a1 & a2) << 3)) & smask & ~pre;
+      // the walk ends before a row that is not ready (or needs the exact evaluation) and after a token that changes the state
+      const unsigned bad = vis & (~ready_all | (tok_all & ~keep_all));
+      const int pb = bad ? __ffs(bad) - 1 : 32;
+      const bool last_tok = pb < 32 && ((tok_all >> (pb & 31)) & 1u);
+      const unsigned cm = (vis & (pb < 32 ? (1u << (pb & 31)) - 1u : 0xFFFFFFFFu)) | (last_tok ? 1u << (pb & 31) : 0u);
+      if (cm == 0u) { no_grid = true; continue; }              // (the current row needs the exact evaluation: a list round)
+      const unsigned tm = cm & tok_all, bm = cm & blank_all;
+      // frames closed: by a blank, or by a token in the frame's last row
+      const unsigned cl = bm | (tm & (m1 << (S - 1)));
+      const unsigned clf = (cl | (cl >> 1) | (cl >> 2) | (cl >> 3)) & m1;
+      const int fcl = __popc(clf);
+      const int pos = fcl < 8 ? __popc(((tm | (fcl == 0 ? pre : 0u)) >> (4 * (fcl & 7))) & 0xFu) : 0;
+      const unsigned upto = 0xFFFFFFFFu >> (31 - lane);
+      const bool mine_t = (tm >> lane) & 1u;
+      const int ntok = n_out + __popc(tm & upto), nval = nv + __popc(cm & upto);
+      if (last_tok) { tok = __shfl_sync(0xffffffffu, wtok, pb & 31); tnext = __shfl_sync(0xffffffffu, wnext, pb & 31); }
+      if ((cm >> lane) & 1u) o.vals[nval - 1] = adjust(mine_t ? wv : xb, extra);
+      if (mine_t && ntok <= o.cap) {
+        o.tok[ntok - 1] = wtok; o.frm[ntok - 1] = t + r;
+        if (!SEG && o.dur) o.dur[ntok - 1] = 0;
+      }
+      if ((cl >> lane) & 1u) trace(t + r + 1, (last_tok && lane == pb) ? tnext : s, ntok, nval);
+      nv += __popc(cm);
+      n_out += __popc(tm);
+      k = pos;
+      t += fcl;
+      if (last_tok) stable = false;
+    } else {
+      const unsigned m8 = 0x01010101u;                         // (bit 8 r: row r)
+      const unsigned valid_m = __ballot_sync(0xffffffffu, valid) & m8;
+      const unsigned blank_m = __ballot_sync(0xffffffffu, valid && !rescan && blank) & m8;
+      const unsigned resc_m = __ballot_sync(0xffffffffu, rescan) & m8;
+      // the blank rows visited (vm), and the row after them (frame t + j)
+      unsigned vm = 0u;
+      int j = 0;
+      if (!tdt) { const unsigned stop = ~blank_m & m8; j = stop ? (__ffs(stop) - 1) >> 3 : 4; vm = m8 & ((1u << (8 * j - (j == 4 ? 1 : 0))) - 1u); }
+      else
+#pragma unroll 1
+        while (j < 4 && ((blank_m >> (8 * j)) & 1u)) { vm |= 1u << (8 * j); j += max(__shfl_sync(0xffffffffu, dur, 8 * j), 1); }
+      const bool took = j < 4 && ((valid_m >> (8 * j)) & 1u);
+      const int jl = 8 * min(j, 3);
+      tok = took ? __shfl_sync(0xffffffffu, wtok, jl) : V;
+      tnext = took ? __shfl_sync(0xffffffffu, wnext, jl) : s;
+      float val = __shfl_sync(0xffffffffu, wv, jl);
+      float j_extra = __shfl_sync(0xffffffffu, extra, jl);
+      int j_dur = tdt ? __shfl_sync(0xffffffffu, dur, jl) : 0;
+      if (took && ((resc_m >> jl) & 1u)) {
+        const RowPick pk = exact_row(c, L, c.base + static_cast<int64_t>(t - f0 + j) * c.st + (j == 0 ? static_cast<int64_t>(k) * c.ss : 0), s, lane);
+        tok = pk.tok; tnext = pk.next; val = pk.val;
+        if (tdt) { j_dur = pk.dur; j_extra = pk.xdur; }
+      }
+      if ((vm >> lane) & 1u) {
+        o.vals[nv + __popc(vm & ((1u << lane) - 1u))] = adjust(xb, extra);
+        trace(t + r + 1, s, n_out, nv + r + 1);
+      }
+      nv += __popc(vm);
+      t += j;
+      if (j > 0) k = 0;
+      if (took) {
+        if (lane == 0) o.vals[nv] = adjust(val, j_extra);
+        ++nv;
+        bool closed = false;
+        if (tok == V) {                        // blank after all (exact evaluation)
+          t += tdt ? max(j_dur, 1) : 1;
+          k = 0; closed = true;
+        } else {
+          if (lane == 0 && n_out < o.cap) {
+            o.tok[n_out] = tok; o.frm[n_out] = t;
+            if (!SEG && o.dur) o.dur[n_out] = j_dur;
+          }
+          ++n_out;
+          if (tdt && j_dur > 0) { t += j_dur; k = 0; }
+          else if (++k == S) { ++t; k = 0; closed = true; }
+          stable = tnext == s;
+        }
+        if (closed && lane == 0) trace(t, tnext, n_out, nv);
+      }
+    }
+    if (tok != V && tnext != s && c.bound) {
+      if (tnext < 0 || tnext >= c.n_states) { if (lane == 0) atomicOr(c.status, TB_STATUS_BAD_STATE); tnext = 0; }
+      s = tnext;
+      listed = false;
+    }
+  }
+  if (SEG) asm volatile("cp.async.wait_all;" ::: "memory");
+  cu.t = t; cu.k = k; cu.s = s; cu.n_out = n_out; cu.nv = nv; cu.stable = stable; cu.listed = listed; cu.list = L;
+}
+
+}  // namespace
+
+#endif  // TB_ROWS_CUH_

@@ -1,0 +1,129 @@
+"""GPU parity of the two-step greedy decode (rows reduced to summaries, then decided) and of the chunk kernel built from the
+same parts, against the CPU oracle: vocabularies and alignments at the edges of a warp's blocks, padded and reordered
+layouts, every number of rows per frame, long lists, ties, blank-only and token-only rows."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+from paper_2608_21343_b200 import workloads as W
+from helpers import SCORE_TOL, check_greedy, make_batch, oracle_graph, to_device, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(seed, B, T, S, V, dtype, n_phrases=40, n_dur=0, levels=None, **over):
+    w = W.get_workload(2, seed=seed, B=B, T=T, S=S, V=V, dtype=dtype, n_phrases=n_phrases, n_plants=min(6, T // 4), n_dur=n_dur, **over)
+    data = W.batch_inputs(w)
+    if levels:                                    # coarse logits: ties between tokens, and with the blank, are frequent
+        x = data["logits"] if dtype == "f32" else W.bf16_bits_to_f32(data["logits"])
+        data["logits"] = W.to_storage(np.round(x * levels) / levels, dtype)
+    return w, data
+
+
+def _check(tb, w, data, logits=None, lengths=None, lists=None, what="", flags=0):
+    lists = data["phrases"] if lists is None else lists
+    batch, _ = make_batch(tb, w, lists)
+    logits = to_device(data["logits"]) if logits is None else logits
+    dl = None if lengths is None else torch.tensor(lengths, dtype=torch.int32, device="cuda:0")
+    for _ in range(2):                            # what the first call leaves in the working memory must not matter
+        out = to_host(tb.tb_greedy_decode(batch, logits, lengths=dl))
+    assert tb.tb_batch_status(batch) == 0
+    for i, p in enumerate(lists):
+        check_greedy(out, i, O.greedy_rnnt(oracle_graph(w, p), data["logits"][i], None if lengths is None else lengths[i]), what)
+    return out
+
+
+@pytest.mark.parametrize("dtype,V", [("f32", 1), ("f32", 3), ("f32", 31), ("f32", 511), ("f32", 512), ("f32", 513), ("f32", 1024), ("f32", 2049),
+                                      ("f32", 8192), ("bf16", 2047), ("bf16", 2048), ("bf16", 2055), ("bf16", 4099), ("bf16", 8192)])
+def test_vocabularies(tb, dtype, V):
+    w, data = _inputs(V, 4, 60, 3, V, dtype, n_phrases=30 if V > 8 else 3, len_hi=6 if V > 8 else 2)
+    lists = list(data["phrases"])
+    lists[1] = None
+    _check(tb, w, data, lists=lists, lengths=[60, 59, 1, 0], what=f"V {V}")
+
+
+@pytest.mark.parametrize("S", [1, 2, 4])
+@pytest.mark.parametrize("T", [1, 7, 33, 250])
+def test_rows_per_frame_and_lengths(tb, S, T):
+    w, data = _inputs(10 * S + T, 3, T, S, 130, "f32")
+    _check(tb, w, data, lengths=[T, max(0, T - 1), T // 2], what=f"S {S} T {T}")
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_layouts_that_are_not_packed(tb, dtype):
+    w, data = _inputs(3, 3, 50, 3, 301, dtype)
+    x = to_device(data["logits"])
+    padded = torch.full((3, 50, 3, 317), 50.0, dtype=x.dtype, device=x.device)       # what lies between the rows would win
+    padded[..., 5:5 + 302] = x
+    _check(tb, w, data, logits=padded[..., 5:5 + 302], what="padded")
+    swapped = x.permute(1, 2, 0, 3).contiguous().permute(2, 0, 1, 3)                  # streams innermost of the rows
+    _check(tb, w, data, logits=swapped, what="reordered")
+
+
+@pytest.mark.parametrize("levels", [2, 8])
+@pytest.mark.parametrize("V", [90, 3000])
+def test_ties(tb, levels, V):
+    w, data = _inputs(V + levels, 4, 80, 3, V, "f32", levels=levels, n_phrases=60)
+    _check(tb, w, data, what="ties")
+
+
+@pytest.mark.parametrize("wl", [dict(n_phrases=400, n_shared=2600, len_lo=3, len_hi=10), dict(n_phrases=300, len_hi=4)])
+def test_long_lists_walked_and_resolved(tb, wl):
+    """Lists that are walked along the suffix chain (too large to be resolved), and resolved ones of hundreds of tokens."""
+    w, data = _inputs(8, 4, 200, 3, 700, "bf16", **wl)
+    lists = list(data["phrases"])
+    lists[2] = None
+    _check(tb, w, data, lists=lists, what="long lists")
+
+
+def test_repeating_token_lists_and_extremes(tb):
+    """A phrase that repeats one token keeps a stream in one state; rows without tokens (all -inf but the blank) and rows
+    whose blank is -inf close frames in every way."""
+    w, data = _inputs(21, 4, 120, 3, 64, "f32")
+    x = data["logits"]
+    x[:, ::5, :, :64] = -np.inf
+    x[:, [t for t in range(3, 120, 7) if t % 5], :, 64] = -np.inf
+    x[:, :, :, 15:18] += 1.0
+    lists = [[[15] * 12, [3, 4]], [[15, 16] * 4], data["phrases"][2], None]
+    _check(tb, w, data, lists=lists, what="extremes")
+
+
+@pytest.mark.parametrize("n_dur,S,V,dtype,chunk,phr", [(0, 3, 257, "f32", 8, 40), (5, 3, 1024, "bf16", 8, 100), (3, 2, 2500, "bf16", 16, 60),
+                                                       (5, 4, 100, "f32", 17, 30), (32, 1, 77, "f32", 40, 20), (0, 1, 5000, "f32", 5, 300)])
+def test_chunks(tb, n_dur, S, V, dtype, chunk, phr):
+    """Chunks of every size against the oracle's, streams ending inside chunks, slots re-bound on the way."""
+    n, T = 5, 3 * chunk + 2
+    w, data = _inputs(V + chunk, n, T, S, V, dtype, n_phrases=phr, n_dur=n_dur)
+    lists = list(data["phrases"])
+    lists[3] = None
+    batch, _ = make_batch(tb, w, lists)
+    graphs = [oracle_graph(w, p) for p in lists]
+    st = [O.StreamState() for _ in range(n)]
+    for i in range(n):
+        st[i].state = 0 if lists[i] is not None else -1
+    valid = np.array([T, T - 1, chunk + 1, T, 2 * chunk], dtype=np.int32)
+    dv = torch.from_numpy(valid).to("cuda:0")
+    pad = np.zeros((n, 4 * chunk, S, w.row_width), dtype=data["logits"].dtype)
+    pad[:, :T] = data["logits"]
+    start = [0] * n
+    for c in range(0, 4 * chunk, chunk):
+        x = np.ascontiguousarray(pad[:, c:c + chunk])
+        if c == 2 * chunk:                        # slot 1 starts a new stream, slot 4 loses its list
+            g = tb.tb_graph_compile(lists[0], w.V, case_class=w.vocab.case_class)
+            out = to_host(tb.tb_stream_chunk_binds(batch, [1, 4], [g, None], to_device(x), n_dur, dv))
+            graphs[1], graphs[4] = oracle_graph(w, lists[0]), None
+            for i, s0 in ((1, 0), (4, -1)):
+                st[i] = O.StreamState()
+                st[i].state = s0
+                start[i] = c
+        else:
+            out = to_host(tb.tb_stream_chunk(batch, to_device(x), n_dur, dv))
+        assert tb.tb_batch_status(batch) == 0
+        for i in range(n):
+            ref = O.stream_chunk(graphs[i], x[i], n_dur, c - start[i], int(valid[i]), st[i])
+            k = int(out["counts"][i])
+            assert k == len(ref["tokens"]), (c, i)
+            for name in ("tokens", "frames", "durs"):
+                assert np.array_equal(out[name][i, :k], ref[name]), (c, i, name)
+            assert int(out["states"][i]) == st[i].state and abs(float(out["scores"][i]) - float(st[i].score)) <= SCORE_TOL
