@@ -1123,10 +1123,12 @@ extern "C" int tb_batch_bind_counts(const tb_batch* b, int64_t* out_pulled, int6
 // being captured, or when it cannot be had.
 static void beam_prepass(tb_batch* b, TbBeamParams* p, int32_t T, int32_t E, int64_t frame_stride, int64_t row_stride,
                          const int32_t* n_frames, cudaStream_t stream) {
-  p->top_base = nullptr; p->top_row = nullptr; p->top_m = 0;
+  p->top_base = nullptr; p->top_m = 0;
   if (b->flags & (TB_FLAG_GENERAL_KERNELS | TB_FLAG_BEAM_WHOLE_ROWS)) return;
   if (2 * (b->vocab + 1) > (1 << TB_RS_TOK_BITS) || b->vocab > 0xFFFE) return;   // (the steps' token view has the same limit)
-  const int32_t M = 2 * p->K + 8;
+  // the K picks can all come from one hypothesis; a few more for tokens its state lists (with the entry for the rest, rows
+  // are a multiple of 48 bytes)
+  const int32_t M = ((p->K + 9 + 3) / 4 * 4 < 16 ? 16 : (p->K + 9 + 3) / 4 * 4) - 1;
   const size_t want = static_cast<size_t>(p->B) * T * E * (M + 1) * sizeof(TbTopEnt);
   {
     void* mem = b->d_top;

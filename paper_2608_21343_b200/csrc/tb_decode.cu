@@ -279,43 +279,6 @@ struct BeamKey {  // order: value descending, token key ascending, parent ascend
   int32_t tkey, par;
 };
 // One beam expansion of the block's stream (the body of k_beam_step; k_beam_frames calls it once per row).
-// The K largest of the keys ckey[first], ckey[first + stride], ... (those below n; 0 = no candidate) that this warp's
-// lanes look at, R per lane: out_key[r] / out_idx[r] for r < K, best first (key 0, index -1 once nothing is left).
-// Every lane keeps its keys sorted in registers, so a round is two warp-wide integer maxima over the lanes' heads;
-// the lane that holds the winner finds its index again (one of its R places in the array) and moves up its other keys.
-template <int R>
-__device__ __forceinline__ void warp_top_keys(const unsigned long long* ckey, int n, int first, int stride, int K, int lane,
-                                              unsigned long long* out_key, int32_t* out_idx) {
-  unsigned long long ck[R];
-#pragma unroll
-  for (int j = 0; j < R; ++j) { const int i = first + stride * j; ck[j] = i < n ? ckey[i] : 0ull; }
-  auto ce = [&](int a, int b) { const bool sw = ck[b] > ck[a]; const unsigned long long hi = sw ? ck[b] : ck[a], lo = sw ? ck[a] : ck[b]; ck[a] = hi; ck[b] = lo; };
-  if (R == 2) { ce(0, 1); }
-  if (R == 4) { ce(0, 1); ce(2, 3); ce(0, 2); ce(1, 3); ce(1, 2); }
-  if (R == 8) {
-    ce(0, 1); ce(2, 3); ce(4, 5); ce(6, 7); ce(0, 2); ce(1, 3); ce(4, 6); ce(5, 7); ce(1, 2); ce(5, 6);
-    ce(0, 4); ce(1, 5); ce(2, 6); ce(3, 7); ce(2, 4); ce(3, 5); ce(1, 2); ce(3, 4); ce(5, 6);
-  }
-  for (int r = 0; r < K; ++r) {
-    const unsigned long long a = ck[0];
-    const uint32_t hi = static_cast<uint32_t>(a >> 32), lo = static_cast<uint32_t>(a);
-    const uint32_t mh = __reduce_max_sync(0xffffffffu, hi);
-    const uint32_t ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-    const unsigned long long best = (static_cast<unsigned long long>(mh) << 32) | ml;
-    if (best == 0ull) {
-      if (lane == 0) { out_key[r] = 0ull; out_idx[r] = -1; }
-    } else if (a == best) {
-      int idx = -1;
-#pragma unroll
-      for (int j = 0; j < R; ++j) { const int i = first + stride * j; if (i < n && ckey[i] == best) idx = i; }
-      out_key[r] = best; out_idx[r] = idx;
-#pragma unroll
-      for (int j = 0; j + 1 < R; ++j) ck[j] = ck[j + 1];
-      ck[R - 1] = 0ull;
-    }
-  }
-}
-
 // threads of a beam block: more warps than the general kernel's hide the latencies of its short dependent phases; 17
 // warps take a row of 1025 logits (vocabularies of about a thousand pieces) in two strides instead of three
 constexpr int kBeamThreads = 544;
@@ -324,7 +287,7 @@ constexpr int kBeamPref = 5;   // elements of a shared row each thread may hold 
 // launch; next_row: where the next step's shared row starts (null: none), fetched while this step selects.
 // What a beam block keeps in shared memory besides its candidate arrays: the stream's hypotheses from step to step,
 // and the working set of a step.
-constexpr int kTeamMaxK = 8;   // (= kFastMaxK, needed here already)
+constexpr int kHistBins = 128, kSurvivors = 512;   // of a team step: histogram bins, candidates that may be picks
 struct BeamShared {
   ChainSmem chain;
   // token-view path: per hypothesis a copy of its state's short list, to find the next state of a pick
@@ -340,24 +303,22 @@ struct BeamShared {
   unsigned long long h_hash[TB_MAX_BEAM];   // identity of the hypothesis' token sequence
   int32_t h_len[TB_MAX_BEAM];
   BeamKey sel[TB_MAX_BEAM];
-  int32_t sel_dst[TB_MAX_BEAM];      // compact path: the graph state a selected candidate leads to
-  int32_t cp_n, cp_flag;             // compact path: candidates laid out; 0 = this step cannot take it
-  int32_t cp_off[TB_MAX_BEAM + 1];   // compact path: where each hypothesis' listed candidates start
-  int32_t rec_ready;                 // the hypotheses' list records in h_beg / h_cnt / h_D are those of their current states
-  TbTopEnt ttop[2 * TB_MAX_BEAM + 9]; // this step's reduced row
   float root_wmax;                   // largest |root arc weight| of the stream's graph (filled with the root tables)
-  int32_t fast_done;                 // narrow beams: steps the team has just taken
-  // narrow beams, between the team's warps: the hypotheses a step works on, each worker's picks and bound term
-  float f_sc[kTeamMaxK]; int32_t f_st[kTeamMaxK]; uint8_t f_lv[kTeamMaxK];
-  unsigned long long f_key[kTeamMaxK][kTeamMaxK]; int32_t f_dst[kTeamMaxK][kTeamMaxK];
-  float f_ub[kTeamMaxK];
-  volatile int32_t f_cmd, f_fail;    // 1: the run ends here / a worker met a list it cannot take
+  int32_t team_done;                 // steps the team has just taken
+  // the team's steps (beam_team_run); two copies of what one step still reads while the next one writes
+  float w_ub[2][TB_MAX_BEAM];                            // what the K-th pick has to clear on behalf of each hypothesis
+  __align__(16) int32_t hist[2][kHistBins];              // candidates by value
+  __align__(16) unsigned long long sk[kSurvivors + 64];  // the candidates that may be picks: keys, target states
+  int32_t sd[kSurvivors + 1];
+  int32_t ord[TB_MAX_BEAM];                              // the K best of them, best first
+  int32_t n_surv[2], cmd, done;
+  __align__(16) uint32_t hlow[TB_MAX_BEAM];              // low words of the sequences' hashes
+  uint4 no_rec;                                          // the empty list (unbound streams)
 };
 
 template <typename LT>
 __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared& sh, LT (&xpre)[kBeamPref], bool& xpre_valid,
-                                               const LT* next_row, TbTopEnt& tpre, bool& tpre_valid,
-                                               const TbTopEnt* next_top) {
+                                               const LT* next_row) {
   extern __shared__ __align__(16) unsigned char dyn[];
   const int V = p.V, K = p.K, W = V + 1;
   float* cand = reinterpret_cast<float*>(dyn);                         // [K, V+1]
@@ -371,11 +332,7 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
   auto& h_beg = sh.h_beg; auto& h_cnt = sh.h_cnt; auto& h_D = sh.h_D;
   auto& red64 = sh.red64;
   auto& h_score = sh.h_score; auto& h_state = sh.h_state; auto& h_live = sh.h_live; auto& h_hash = sh.h_hash; auto& h_len = sh.h_len;
-  auto& sel = sh.sel; auto& sel_dst = sh.sel_dst;
-  int32_t& cp_n = sh.cp_n; int32_t& cp_flag = sh.cp_flag;
-  auto& cp_off = sh.cp_off;
-  int32_t& rec_ready = sh.rec_ready;
-  auto& ttop = sh.ttop;
+  auto& sel = sh.sel;
   float& root_wmax = sh.root_wmax;
 
   const int b = blockIdx.x;
@@ -388,7 +345,7 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
   // rows shared by the hypotheses of a stream (hyp_stride 0) depend on nothing that is loaded below: fetch this
   // thread's elements now, so that their latency overlaps the loads of the slot record, states and lists
   constexpr int kPref = kBeamPref;
-  const bool pref = (use_tv || (!bound && p.top_row != nullptr)) && p.hyp_stride == 0 && W <= kPref * kBeamThreads;
+  const bool pref = use_tv && p.hyp_stride == 0 && W <= kPref * kBeamThreads;
   if (pref && !xpre_valid) {
     const LT* row0 = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(b) * p.stream_stride;
 #pragma unroll
@@ -466,337 +423,8 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
   unsigned long long m1 = 0ull, m2 = 0ull;
   bool swept = false;
   auto offer = [&](unsigned long long kk) { if (kk > m1) { m2 = m1; m1 = kk; } else if (kk > m2) m2 = kk; };
-  // ---- the compact path ---------------------------------------------------------------------------------
-  // With the row reduced ahead of time to its top_m root-boosted tokens (k_beam_topm), a hypothesis' candidates are
-  // its blank, the tokens its graph state lists (exact values from their entries) and the first tokens of that
-  // short list which the state does not list (exact values from the list's logits): a few dozen per hypothesis
-  // instead of vocab + 1.  Every token outside the list has y <= y_next, hence a value of at most
-  // score + y_next + lambda * D plus roundings; the step is valid when the K-th selected candidate clears that
-  // bound for every hypothesis by a margin that dominates the roundings.  Otherwise (or with a very long list)
-  // the step is done again the long way below.
-  bool compact_done = false;
-  bool row_staged = false;      // the compact path put this step's row into shared memory and asked for the next one (in xpre)
-  float* xrow_s = reinterpret_cast<float*>(aux + beam_aux_bytes(V, p.C, p.tokview));
-  if (p.top_row != nullptr && p.hyp_stride == 0 && (use_tv || !bound) && p.top_m <= 2 * TB_MAX_BEAM + 8) {
-    unsigned long long* ckey = reinterpret_cast<unsigned long long*>(cand);
-    const int M = p.top_m;
-    float* xrow = xrow_s;                                     // [W] this step's row, staged
-    // the candidate arrays share the whole-row path's value array: keys, target states, then the warps' picks
-    const int wsel_bytes = (kBeamThreads / 32) * TB_MAX_BEAM * 12;
-    const int cap = (static_cast<int>(static_cast<size_t>(K) * W * sizeof(float)) - wsel_bytes - 16) / 12 & ~1;
-    int32_t* cdst = reinterpret_cast<int32_t*>(ckey + cap);
-    const LT* base = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(b) * p.stream_stride;
-    const bool recs_at_hand = p.tv_ready && rec_ready;        // left by the previous step of this launch
-    if (warp == 0) {
-      // lane k: hypothesis k's list record (fetched now unless the previous step left it), then where its listed
-      // candidates start in the candidate array: a prefix sum over the warp (K <= 32)
-      const int k = lane;
-      int cntk = 0;
-      bool lv = false;
-      if (k < K) {
-        if (!recs_at_hand) {
-          int32_t beg = 0;
-          float Dk = 0.0f;
-          if (bound && h_score[k] != -INFINITY) {
-            int32_t st = h_state[k];
-            if (st < 0 || st >= rec.n_states) { atomicOr(p.status, TB_STATUS_BAD_STATE); st = 0; }
-            const TbRsRec r = reinterpret_cast<const TbRsRec*>(blob + rec.off_rsrec)[st];
-            beg = r.begin; cntk = r.count; Dk = r.D;
-          }
-          h_beg[k] = beg; h_cnt[k] = cntk; h_D[k] = Dk;
-        } else {
-          cntk = h_cnt[k];
-        }
-        lv = h_score[k] != -INFINITY && h_live[k];
-        hl_n[k] = !lv ? 0 : (cntk <= kBeamList ? cntk : -1);
-      }
-      const int c = lv ? cntk : 0;
-      int incl = c;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += o;
-      }
-      if (k < K) cp_off[k] = incl - c;
-      const int total = __shfl_sync(0xffffffffu, incl, 31);
-      if (lane == 0) {
-        cp_off[K] = total;
-        cp_flag = total + K * (M + 1) <= cap ? 1 : 0;
-        cp_n = total + K * (M + 1);
-      }
-    }
-    for (int i = threadIdx.x; i < K * WW; i += kBeamThreads) ovr[i] = 0u;
-    // the row and its reduced form, asked for during the previous step (or now), go to shared memory
-    if (pref) {
-#pragma unroll
-      for (int j = 0; j < kPref; ++j) { const int v = threadIdx.x + j * kBeamThreads; if (v < W) xrow[v] = LogitLoad<LT>::widen(xpre[j]); }
-    }
-    if (threadIdx.x <= M) ttop[threadIdx.x] = tpre_valid ? tpre : p.top_row[threadIdx.x];
-    __syncthreads();
-    // the next step's row and reduced row are requested now: their trip overlaps the rest of this step
-    row_staged = pref;
-    xpre_valid = false;
-    if (pref && next_row) {
-#pragma unroll
-      for (int j = 0; j < kPref; ++j) {
-        const int v = threadIdx.x + j * kBeamThreads;
-        if (v < W) xpre[j] = LogitLoad<LT>::raw(next_row + v);      // (the load alone: widened when it is used)
-      }
-      xpre_valid = true;
-    }
-    tpre_valid = false;
-    if (next_top) { if (threadIdx.x <= M) tpre = next_top[threadIdx.x]; tpre_valid = true; }
-    // (one warp doing a narrow beam's few dozen candidates by itself, with warp-wide synchronisation only, was
-    // measured slower than the whole block; narrow beams are taken by a team of warps instead, see beam_fast_run)
-    const int cth = static_cast<int>(threadIdx.x), cnt = kBeamThreads;
-    {
-      if (cp_flag) {
-        const int n_listed = cp_off[K], n = cp_n;
-        // the listed tokens of every hypothesis, all hypotheses at once: exact values; marked, so that the walk over
-        // the reduced row leaves them out.  Candidate slots that stay unused hold key 0 (none).
-        if (bound) {
-          const TbRsEnt* ent = reinterpret_cast<const TbRsEnt*>(blob + rec.off_rsent);
-          // (eight entries per thread are requested before the first is used: one trip to L2 for all of them)
-          for (int q0 = cth; q0 < n_listed; q0 += 8 * cnt) {
-            TbRsEnt e8[8];
-            int k8[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const int q = q0 + j * cnt;
-              int k = 0;
-              if (q < n_listed) {
-                // the hypothesis whose listed candidates include place q: the last k with cp_off[k] <= q (bisection)
-                int hi_k = K;
-                while (hi_k - k > 1) { const int mid = (k + hi_k) >> 1; if (cp_off[mid] <= q) k = mid; else hi_k = mid; }
-                e8[j] = ent[h_beg[k] + (q - cp_off[k])];
-              }
-              k8[j] = k;
-            }
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const int q = q0 + j * cnt;
-              if (q >= n_listed) continue;
-              const int k = k8[j], i = q - cp_off[k];
-              const TbRsEnt e = e8[j];
-              const int tk = static_cast<int>((e.dst_tok & ((1u << TB_RS_TOK_BITS) - 1u)) >> 1);   // padding entries carry token V
-              if (i < kBeamList) { hl_tok[k][i] = static_cast<uint16_t>(tk); hl_dst[k][i] = static_cast<int32_t>(e.dst_tok >> TB_RS_TOK_BITS); }
-              unsigned long long key = 0ull;
-              if (tk < V) {
-                const float x = pref ? xrow[tk] : LogitLoad<LT>::at(base + tk);
-                key = make_key(__fadd_rn(h_score[k], __fadd_rn(x, e.lb)), tk, k);
-                atomicOr(&ovr[k * WW + (tk >> 5)], 1u << (tk & 31));
-              }
-              ckey[q] = key; cdst[q] = static_cast<int32_t>(e.dst_tok >> TB_RS_TOK_BITS);
-            }
-          }
-        }
-        __syncthreads();
-        // blank, the first unlisted tokens of the reduced row, and the frozen hypotheses' carried candidates
-        for (int pr = cth; pr < K * (M + 1); pr += cnt) {
-          const int k = pr / (M + 1), j = pr - k * (M + 1);
-          unsigned long long key = 0ull;
-          int32_t dst = -1;
-          if (h_score[k] != -INFINITY) {
-            const TbTopEnt t = ttop[j];
-            if (!h_live[k]) {
-              if (j == M) { key = make_key(h_score[k], V + 1, k); dst = h_state[k]; }
-            } else if (j == M) {
-              key = make_key(__fadd_rn(h_score[k], t.x), V, k); dst = h_state[k];
-            } else {
-              const int tk = static_cast<int>(t.tok_cls & 0xFFFFu), cl = static_cast<int>(t.tok_cls >> 16);
-              if (tk < V && !((ovr[k * WW + (tk >> 5)] >> (tk & 31)) & 1u)) {     // (tk >= V: the row has fewer tokens)
-                const float val = bound ? __fadd_rn(t.x, __fmul_rn(g.lambda, __fadd_rn(h_D[k], tv.rootcw[cl]))) : t.x;
-                key = make_key(__fadd_rn(h_score[k], val), tk, k);
-                dst = bound ? tv.rootdst[cl] : -1;
-              }
-            }
-          }
-          ckey[n_listed + pr] = key; cdst[n_listed + pr] = dst;
-        }
-        __syncthreads();
-        {
-          // Selection (warp_top_keys).  A thread takes its candidates (indices thread, thread + block size, ...) into
-          // registers once and keeps them sorted; a round is then two warp-wide integer maxima over the lanes' best.
-          // Few candidates (narrow beams): warp 0 alone.  Many: every warp picks the K best of its candidates and
-          // leaves them, best first, in shared memory; warp 0 then merges the warps' lists, one lane per list, the
-          // head of each in a register.
-          unsigned long long* wkey = reinterpret_cast<unsigned long long*>(cdst + cap);            // [warps][K] (key); behind the targets
-          int32_t* widx = reinterpret_cast<int32_t*>(wkey + (kBeamThreads / 32) * TB_MAX_BEAM);   // [warps][K] where in ckey
-          constexpr int kSelRegs = 8;
-          constexpr int kRadixMinK = 9;       // beams at least this wide (wider than the teams of warps take) find their picks by radix selection
-          const bool solo = n <= 32 * kSelRegs;
-          auto put_sel = [&](int r, unsigned long long best, int idx) {
-            const uint32_t mh = static_cast<uint32_t>(best >> 32);
-            const uint32_t l2 = 0xFFFFFFFFu - static_cast<uint32_t>(best & 0xFFFFFFFFull);
-            BeamKey c;
-            c.v = __uint_as_float(mh ^ ((mh >> 31) ? 0x80000000u : 0xFFFFFFFFu));
-            c.tkey = static_cast<int32_t>(l2 >> 5); c.par = static_cast<int32_t>(l2 & 31u);
-            if (best == 0ull) c = BeamKey{-INFINITY, INT32_MAX, INT32_MAX};
-            sel[r] = c; sel_dst[r] = best == 0ull ? -1 : cdst[idx];
-          };
-          if (solo) {
-            if (warp == 0) {
-              if (n <= 32 * 4) warp_top_keys<4>(ckey, n, lane, 32, K, lane, wkey, widx);
-              else warp_top_keys<8>(ckey, n, lane, 32, K, lane, wkey, widx);
-              __syncwarp();
-              if (lane < K) put_sel(lane, wkey[lane], widx[lane]);
-            }
-          } else if (K >= kRadixMinK) {
-            // Wide beams: K rounds at two levels cost more than finding the K-th largest key first.  The keys are 64-bit
-            // numbers, all different; the K-th largest is found digit by digit (8 bits at a time, from the highest
-            // digit in which the candidates differ) with a histogram in shared memory, the keys at or above it are
-            // collected, and one warp orders them by counting, for each, the keys above it.
-            int* hist = reinterpret_cast<int*>(wkey);                     // [256]
-            int* ctl = hist + 256;                                        // digit, its count, rank left, collected
-            unsigned long long* okey = reinterpret_cast<unsigned long long*>(ctl + 8);   // [K] the collected keys
-            int32_t* oidx = reinterpret_cast<int32_t*>(okey + TB_MAX_BEAM);              // [K] where they sit in ckey
-            uint32_t hmax = 0u, hmin = 0xFFFFFFFFu;
-            for (int ii = threadIdx.x; ii < n; ii += kBeamThreads) {
-              const unsigned long long kk = ckey[ii];
-              if (kk != 0ull) { const uint32_t h = static_cast<uint32_t>(kk >> 32); hmax = max(hmax, h); hmin = min(hmin, h); }
-            }
-            hmax = __reduce_max_sync(0xffffffffu, hmax);
-            hmin = __reduce_min_sync(0xffffffffu, hmin);
-            if (lane == 0) { red64[0][warp] = hmax; red64[1][warp] = hmin; }
-            if (threadIdx.x == 0) ctl[3] = 0;
-            __syncthreads();
-#pragma unroll
-            for (int w2 = 0; w2 < kBeamThreads / 32; ++w2) {
-              hmax = max(hmax, static_cast<uint32_t>(red64[0][w2])); hmin = min(hmin, static_cast<uint32_t>(red64[1][w2]));
-            }
-            unsigned long long t_low = 1ull;                               // keys at or above this are the picks
-            if (hmax != 0u) {
-              const uint32_t diff = hmax ^ hmin;
-              int shift = diff == 0u ? 24 : 32 + ((31 - __clz(diff)) >> 3) * 8;
-              unsigned long long prefix = shift + 8 >= 64 ? 0ull : ((static_cast<unsigned long long>(hmax) << 32) >> (shift + 8));
-              int want = K;
-              for (;;) {
-                if (threadIdx.x < 256) hist[threadIdx.x] = 0;
-                __syncthreads();
-                for (int ii = threadIdx.x; ii < n; ii += kBeamThreads) {
-                  const unsigned long long kk = ckey[ii];
-                  if (kk != 0ull && (shift + 8 >= 64 || (kk >> (shift + 8)) == prefix)) atomicAdd(&hist[static_cast<int>((kk >> shift) & 255ull)], 1);
-                }
-                __syncthreads();
-                if (warp == 0) {
-                  // lane l looks at digits 255 - 8 l ... 248 - 8 l; the digit of the K-th key is the first at which
-                  // the count of keys with that digit or a higher one reaches the rank wanted
-                  int c[8], mine_total = 0;
-#pragma unroll
-                  for (int d = 0; d < 8; ++d) { c[d] = hist[255 - (8 * lane + d)]; mine_total += c[d]; }
-                  int incl = mine_total;
-#pragma unroll
-                  for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
-                  const int total = __shfl_sync(0xffffffffu, incl, 31);
-                  const unsigned reach = __ballot_sync(0xffffffffu, incl >= want);
-                  if (total < want) {
-                    if (lane == 0) ctl[0] = -1;                           // fewer candidates than places: all of them
-                  } else if (lane == __ffs(reach) - 1) {
-                    int above = incl - mine_total, d = 0;
-                    while (above + c[d] < want) { above += c[d]; ++d; }
-                    ctl[0] = 255 - (8 * lane + d); ctl[1] = c[d]; ctl[2] = want - above;
-                  }
-                }
-                __syncthreads();
-                const int digit = ctl[0];
-                if (digit < 0) break;
-                const int cD = ctl[1];
-                want = ctl[2];
-                prefix = (prefix << 8) | static_cast<unsigned long long>(digit);
-                if (want == cD || shift == 0) { t_low = prefix << shift; break; }
-                shift -= 8;
-              }
-              for (int ii = threadIdx.x; ii < n; ii += kBeamThreads) {
-                const unsigned long long kk = ckey[ii];
-                if (kk != 0ull && kk >= t_low) {
-                  const int pos = atomicAdd(&ctl[3], 1);
-                  if (pos < TB_MAX_BEAM) { okey[pos] = kk; oidx[pos] = ii; }
-                }
-              }
-            }
-            __syncthreads();
-            if (warp == 0) {
-              const int cnt = min(ctl[3], K);
-              if (lane < cnt) {
-                const unsigned long long mine = okey[lane];
-                int rank = 0;
-                for (int j2 = 0; j2 < cnt; ++j2) rank += okey[j2] > mine ? 1 : 0;
-                put_sel(rank, mine, oidx[lane]);
-              } else if (lane < K) {
-                put_sel(lane, 0ull, -1);
-              }
-            }
-          } else {
-            if (n <= kBeamThreads * 2) {
-              warp_top_keys<2>(ckey, n, static_cast<int>(threadIdx.x), kBeamThreads, K, lane, wkey + warp * TB_MAX_BEAM, widx + warp * TB_MAX_BEAM);
-            } else if (n <= kBeamThreads * 4) {
-              warp_top_keys<4>(ckey, n, static_cast<int>(threadIdx.x), kBeamThreads, K, lane, wkey + warp * TB_MAX_BEAM, widx + warp * TB_MAX_BEAM);
-            } else if (n <= kBeamThreads * 8) {
-              warp_top_keys<8>(ckey, n, static_cast<int>(threadIdx.x), kBeamThreads, K, lane, wkey + warp * TB_MAX_BEAM, widx + warp * TB_MAX_BEAM);
-            } else {
-              // (more candidates than the registers take: rounds over the array in shared memory)
-              unsigned long long lim = ~0ull;
-              for (int r = 0; r < K; ++r) {
-                unsigned long long a = 0ull;
-                int ai = -1;
-                for (int ii = threadIdx.x; ii < n; ii += kBeamThreads) { const unsigned long long kk = ckey[ii]; if (kk < lim && kk > a) { a = kk; ai = ii; } }
-                const uint32_t hi = static_cast<uint32_t>(a >> 32), lo = static_cast<uint32_t>(a);
-                const uint32_t mh = __reduce_max_sync(0xffffffffu, hi);
-                const uint32_t ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-                const unsigned long long best = (static_cast<unsigned long long>(mh) << 32) | ml;
-                if (best != 0ull && a == best) { wkey[warp * TB_MAX_BEAM + r] = best; widx[warp * TB_MAX_BEAM + r] = ai; }
-                if (best == 0ull && lane == 0) { wkey[warp * TB_MAX_BEAM + r] = 0ull; widx[warp * TB_MAX_BEAM + r] = -1; }
-                lim = best;                                       // (0 once nothing is left: the later rounds find nothing either)
-              }
-            }
-            __syncthreads();
-            if (warp == 0) {
-              // lane w walks warp w's list from its head, which it keeps in a register; a round takes the largest head
-              int ptr = 0;
-              unsigned long long hk = lane < kBeamThreads / 32 ? wkey[lane * TB_MAX_BEAM] : 0ull;
-              for (int r = 0; r < K; ++r) {
-                const uint32_t hi = static_cast<uint32_t>(hk >> 32), lo = static_cast<uint32_t>(hk);
-                const uint32_t mh = __reduce_max_sync(0xffffffffu, hi);
-                const uint32_t ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-                const unsigned long long best = (static_cast<unsigned long long>(mh) << 32) | ml;
-                if (best == 0ull) {
-                  if (lane == 0) put_sel(r, 0ull, -1);
-                } else if (hk == best) {
-                  put_sel(r, best, widx[lane * TB_MAX_BEAM + ptr]);
-                  ++ptr;
-                  hk = ptr < K ? wkey[lane * TB_MAX_BEAM + ptr] : 0ull;
-                }
-              }
-            }
-          }
-          if (warp == 0) {
-            // does the K-th pick clear everything that was not looked at?  Lane k answers for hypothesis k.
-            __syncwarp();
-            const float y_next = ttop[M].y;
-            bool okk = true;
-            if (y_next != -INFINITY && lane < K && h_score[lane] != -INFINITY && h_live[lane]) {
-              const int k = lane;
-              const float c_k = sel[K - 1].par != INT32_MAX ? sel[K - 1].v : -INFINITY;
-              const float lamD = bound ? g.lambda * h_D[k] : 0.0f;
-              const float scale = fabsf(h_score[k]) + fabsf(y_next) + 2.0f * (bound ? fabsf(g.lambda) * (fabsf(h_D[k]) + root_wmax) : 0.0f);
-              const float ub = (h_score[k] + y_next) + lamD + scale * 3.814697265625e-6f + 1e-30f;      // 2^-18 of the scale
-              okk = c_k > ub;
-            }
-            const bool all_ok = __all_sync(0xffffffffu, okk);
-            if (lane == 0) cp_flag = all_ok ? 1 : 0;
-          }
-        }
-      }
-    }
-    __syncthreads();
-    compact_done = cp_flag != 0;
-  }
-  if (threadIdx.x == 0) rec_ready = 0;      // (set again below, once the new hypotheses' records have been fetched)
-
   // all candidate values of the live hypotheses
-  if (compact_done) {
-    // (nothing to lay out)
-  } else if (use_tv) {
+  if (use_tv) {
     // every hypothesis at once: its state's record, then all plain values, then the listed tokens on top
     if (threadIdx.x < K) {
       const int k = threadIdx.x;
@@ -836,7 +464,7 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
         const int v = threadIdx.x + j * kBeamThreads;
         if (v < W) {
           const float plain_w = v < V ? tv.rootcw[__ldg(p.cls + v)] : 0.0f;
-          const float x = row_staged ? xrow_s[v] : LogitLoad<LT>::widen(xpre[j]);
+          const float x = LogitLoad<LT>::widen(xpre[j]);
           for (int k = 0; k < K; ++k) {
             if (h_score[k] == -INFINITY || !h_live[k]) continue;
             float c;
@@ -896,18 +524,14 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
   // best key below `limit` among this thread's candidates: tokens v = tid, tid + 256, ... of every live
   // hypothesis, plus (thread k) the carried candidate of a frozen hypothesis k
   // the row of the next step is requested now: its trip from HBM overlaps the selection rounds
-  if (!compact_done && !row_staged) {
-    xpre_valid = false;
-    if (pref && next_row) {
+  xpre_valid = false;
+  if (pref && next_row) {
 #pragma unroll
-      for (int j = 0; j < kPref; ++j) {
-        const int v = threadIdx.x + j * kBeamThreads;
-        if (v < W) xpre[j] = LogitLoad<LT>::raw(next_row + v);
-      }
-      xpre_valid = true;
+    for (int j = 0; j < kPref; ++j) {
+      const int v = threadIdx.x + j * kBeamThreads;
+      if (v < W) xpre[j] = LogitLoad<LT>::raw(next_row + v);
     }
-    tpre_valid = false;
-    if (next_top) { if (threadIdx.x <= p.top_m) tpre = next_top[threadIdx.x]; tpre_valid = true; }
+    xpre_valid = true;
   }
   unsigned long long spare = 0ull;                            // this thread's second best key below the limit of its last scan
   bool have_spare = false;
@@ -929,10 +553,9 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
     return m;
   };
   unsigned long long mine = 0ull;
-  if (compact_done) { /* picked already */ }
-  else if (swept) { mine = m1; spare = m2; have_spare = true; }     // collected during the sweep
+  if (swept) { mine = m1; spare = m2; have_spare = true; }     // collected during the sweep
   else mine = scan_mine(~0ull);
-  for (int r = 0; r < K && !compact_done; ++r) {
+  for (int r = 0; r < K; ++r) {
     // the warp's best key: the largest high word, then the largest low word among the lanes that have it
     const uint32_t hi = static_cast<uint32_t>(mine >> 32), lo = static_cast<uint32_t>(mine);
     const uint32_t mh = __reduce_max_sync(0xffffffffu, hi);
@@ -973,9 +596,7 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
       token = (c.tkey == V + 1) ? -1 : c.tkey;
       state = h_state[parent];
       if (token >= 0 && token != V) {
-        if (compact_done) {
-          state = sel_dst[r];
-        } else if (use_tv && hl_n[parent] >= 0) {
+        if (use_tv && hl_n[parent] >= 0) {
           int nx = tv.rootdst[__ldg(p.cls + token)];          // a pick that the parent's list does not hold is a plain token
           for (int i = 0; i < hl_n[parent]; ++i)
             if (hl_tok[parent][i] == token) { nx = hl_dst[parent][i]; break; }
@@ -1006,56 +627,52 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
       p.tree[at * K + r] = make_int2(parent, token);
     }
   }
-  // the list record of every new hypothesis' state, for the next step's compact path: fetched now, so that its trip
-  // to L2 is over when that step starts
-  TbRsRec nrec{0, 0, 0.0f, 0.0f};
-  int rec_ok = 1;
-  if (threadIdx.x < K && p.top_row != nullptr && use_tv && sc != -INFINITY) {
-    if (state >= 0 && state < rec.n_states) nrec = reinterpret_cast<const TbRsRec*>(blob + rec.off_rsrec)[state];
-    else rec_ok = 0;                                        // (the next step reports it)
-  }
   // ... and in shared memory, for the next step of a launch that runs several (read by every thread above: wait)
-  const int all_ok = __syncthreads_and(rec_ok);
+  __syncthreads();
   if (threadIdx.x < K) {
     h_score[threadIdx.x] = sc; h_state[threadIdx.x] = state; h_live[threadIdx.x] = lv;
     h_hash[threadIdx.x] = nh; h_len[threadIdx.x] = nl;
-    if (p.top_row != nullptr) { h_beg[threadIdx.x] = nrec.begin; h_cnt[threadIdx.x] = nrec.count; h_D[threadIdx.x] = nrec.D; }
   }
-  if (threadIdx.x == 0) rec_ready = (p.top_row != nullptr && (use_tv || !bound) && all_ok) ? 1 : 0;
 }
 
 template <typename LT>
 __global__ void __launch_bounds__(kBeamThreads) k_beam_step(TbBeamParams p) {
   LT xpre[kBeamPref] = {};
   bool xpre_valid = false;
-  TbTopEnt tpre{0.0f, 0.0f, 0u};
-  bool tpre_valid = false;
   __shared__ BeamShared sh;
-  beam_step_body<LT>(p, sh, xpre, xpre_valid, static_cast<const LT*>(nullptr), tpre, tpre_valid, nullptr);
+  beam_step_body<LT>(p, sh, xpre, xpre_valid, static_cast<const LT*>(nullptr));
 }
 
 
-// ---- narrow beams: steps taken by a small team of warps ------------------------------------------------------------
-// With K <= 8 and the rows reduced ahead of the steps, a step has a few dozen candidates, and the block-wide step body
-// spends its time in block-wide barriers between short phases.  beam_fast_run lets K + 1 warps take such steps, one
-// after the other, while the block's other warps wait: warp 0 coordinates (it holds the stream's hypotheses in
-// registers, lane k: hypothesis k), warp k + 1 works for hypothesis k.  Per step
-//   worker k     : the hypothesis' list record, its listed tokens (exact values; logits from the row, which arrives
-//                  in shared memory by asynchronous copies the coordinator issues two steps ahead), blank, the first
-//                  unlisted tokens of the reduced row or the carried hypothesis, every lane keeping the three best
-//                  of those it sees in registers; the K best of them in K rounds of two warp-wide integer maxima;
-//   barrier of the team (a named barrier, not the block's);
-//   coordinator  : the K best of the workers' picks, the same bound check as the block-wide compact path, the new
-//                  hypotheses, and, where the next step begins a frame, merging and pruning;
-//   barrier of the team; then the workers go on while the coordinator writes the step's results to global memory
-//                  and asks for the row after the next.
-// A step the team cannot take (the bound not cleared, more than three picks due to one lane) is left untouched: the
-// run ends before it, the hypotheses go back to shared memory, and the whole block does that step with
-// beam_step_body.  Same arithmetic, same order of candidates, hence the same results bit for bit.
-constexpr int kFastMaxK = 8;      // widest beam of the team's steps
-constexpr int kFastMaxList = 2048; // longest list of boosted tokens a worker takes
-constexpr int kFastRecCache = 48 << 10;   // shared memory for a copy of the stream's list records (graphs of up to 3072 states)
+// ---- steps taken by a team of warps ---------------------------------------------------------------------------------
+// With the rows reduced ahead of the steps (k_beam_topm) a hypothesis' candidates are the tokens its graph state lists
+// (exact values from their entries), its blank, and the first tokens of the reduced row that the state does not list: a
+// few dozen instead of vocab + 1.  Every token outside the reduced row has y <= y_next, hence a value of at most
+// score + y_next + lambda * D plus roundings; a step is valid when its K-th pick clears that bound for every hypothesis
+// by a margin that dominates the roundings (2^-18 of the operands' scale).
+//
+// beam_team_run lets min(K, 16) worker warps (at least four) and a keeper take such steps one after the other; worker w
+// works for hypotheses w and w + 16.  Per step
+//   1. every listed token, the first eight of the reduced row per hypothesis and the blanks go into a histogram of values
+//      (128 bins of 1/8 below a reference above the best hypothesis);
+//   2. every worker finds the bin in which the K-th best of these lies -- a lower bound on the K-th pick -- and notes its
+//      candidates in that bin or above it (over the whole beam K and a few more) with their target states;
+//   3. these are ranked by counting the keys above each (few: by every warp for itself; many: shared out);
+//   4. every warp now knows the K picks and which of them are its hypotheses, asks for their lists and goes on with the
+//      next step, while the keeper checks the bound, writes the tree and fetches rows; its verdict is read at the next
+//      barrier.
+// A step is a chain of short phases, so what counts is the number of dependent instructions on it and its trips to memory:
+// two barriers (three with many candidates), rows and reduced rows by asynchronous copies ahead of time, values kept in
+// registers from 1 to 2, few branches, nothing on the way that divides.  (Guessing the bound from the steps before instead
+// of the histogram needed 1.6 to 2.3 passes per step and was slower.)
+// A step the team cannot take (the bound not cleared, too many candidates in the bin) is left untouched: the run ends
+// before it and the whole block does that step with beam_step_body.  Same arithmetic and order of candidates, hence the
+// same results bit for bit.
+constexpr int kTeamRecCache = 48 << 10;   // shared memory for a copy of the stream's list records (graphs of up to 3072 states)
+constexpr float kHistAbove = 6.0f, kHistPerUnit = 8.0f;   // the reference's distance above score + best plain value; bins per unit
+constexpr int kTeamRows = 3;              // rows (and reduced rows) in shared memory
 
+__host__ __device__ inline int team_warps(int K) { return K > 16 ? 16 : K < 4 ? 4 : K; }
 __device__ __forceinline__ unsigned long long beam_key(float v, int tkey, int k) {
   const uint32_t u = __float_as_uint(v + 0.0f);             // -0 folded into +0: equal values, equal keys
   const uint32_t hi = u ^ ((u >> 31) ? 0xFFFFFFFFu : 0x80000000u);
@@ -1066,17 +683,11 @@ __device__ __forceinline__ float beam_key_value(unsigned long long key) {
   const uint32_t mh = static_cast<uint32_t>(key >> 32);
   return __uint_as_float(mh ^ ((mh >> 31) ? 0x80000000u : 0xFFFFFFFFu));
 }
-__device__ __forceinline__ unsigned long long shfl_u64(unsigned long long v, int src) {
-  const uint32_t lo = __shfl_sync(0xffffffffu, static_cast<uint32_t>(v), src);
-  const uint32_t hi = __shfl_sync(0xffffffffu, static_cast<uint32_t>(v >> 32), src);
-  return (static_cast<unsigned long long>(hi) << 32) | lo;
+__device__ __forceinline__ uint32_t beam_order(float v) {     // order-preserving image of a score
+  const uint32_t u = __float_as_uint(v + 0.0f);
+  return u ^ ((u >> 31) ? 0xFFFFFFFFu : 0x80000000u);
 }
-__device__ __forceinline__ void beam_cp_async16(unsigned char* dst_smem, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst_smem))), "l"(src) : "memory");
-}
-__device__ __forceinline__ void beam_cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void beam_cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ float beam_order_inv(uint32_t k) { return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xFFFFFFFFu)); }
 template <typename LT> __device__ __forceinline__ float beam_smem_logit(const unsigned char* row, int idx);
 template <> __device__ __forceinline__ float beam_smem_logit<uint16_t>(const unsigned char* row, int idx) {
   return __uint_as_float(static_cast<uint32_t>(*reinterpret_cast<const uint16_t*>(row + 2 * idx)) << 16);
@@ -1084,395 +695,582 @@ template <> __device__ __forceinline__ float beam_smem_logit<uint16_t>(const uns
 template <> __device__ __forceinline__ float beam_smem_logit<float>(const unsigned char* row, int idx) {
   return *reinterpret_cast<const float*>(row + 4 * idx);
 }
-// Starts the copy of one row (its 16-byte aligned superset) into buf; a 16-byte piece that is not wholly inside the
-// tensor [lo, hi) is assembled from the elements that are.
+__device__ __forceinline__ void beam_cp_async16(unsigned char* dst_smem, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst_smem))), "l"(src) : "memory");
+}
+// Starts the copy of one row (its 16-byte aligned superset) into buf, n threads sharing the pieces; a 16-byte piece that
+// is not wholly inside the tensor [lo, hi) is assembled from the elements that are.
 template <typename LT>
 __device__ __forceinline__ void beam_fetch_row(unsigned char* buf, const LT* row, int W, const unsigned char* lo,
-                                               const unsigned char* hi, int lane) {
+                                               const unsigned char* hi, int tid, int n) {
   const unsigned char* rp = reinterpret_cast<const unsigned char*>(row);
   const int off = static_cast<int>(reinterpret_cast<uintptr_t>(rp) & 15);
   const unsigned char* a0 = rp - off;
   const int nchunks = (off + W * static_cast<int>(sizeof(LT)) + 15) >> 4;
-  for (int c = lane; c < nchunks; c += 32) {
+#pragma unroll 1
+  for (int c = tid; c < nchunks; c += n) {
     const unsigned char* ac = a0 + 16 * c;
     if (ac >= lo && ac + 16 <= hi) {
       beam_cp_async16(buf + 16 * c, ac);
     } else {
+#pragma unroll 1
       for (int e = 0; e < 16; e += static_cast<int>(sizeof(LT)))
         if (ac + e >= lo && ac + e + sizeof(LT) <= hi) *reinterpret_cast<LT*>(buf + 16 * c + e) = *reinterpret_cast<const LT*>(ac + e);
     }
   }
 }
-__host__ __device__ inline size_t beam_ring_bytes(int V, int elem) {   // two row buffers of the team steps
-  const size_t one = ((static_cast<size_t>(V + 1) * elem + 16 + 15) & ~size_t(15)) + 16;
-  return 2 * one + 16;
+// Shared memory of the team behind the block's other arrays: row buffers, reduced rows, the copy of the list records.
+struct TeamSmem { int row, row_stride, top, top_stride, recs, total; };
+__host__ __device__ inline TeamSmem team_smem(int V, int elem, int top_m, int rec_bytes) {
+  TeamSmem t;
+  t.row_stride = (((V + 1) * elem + 16 + 15) & ~15) + 16;
+  t.row = 0;
+  t.top_stride = ((top_m + 1) * 12 + 15) & ~15;
+  t.top = kTeamRows * t.row_stride;
+  t.recs = t.top + kTeamRows * t.top_stride;
+  t.total = t.recs + rec_bytes;
+  return t;
 }
-
-// Where the team keeps a copy of the stream's list records (16 bytes per graph state), behind the row buffers.
-template <typename LT>
-__device__ __forceinline__ TbRsRec* beam_rec_cache(const TbBeamParams& p, unsigned char* dyn) {
+__device__ __forceinline__ unsigned char* team_base(const TbBeamParams& p, unsigned char* dyn) {
   const int W = p.V + 1, WW = (W + 31) >> 5;
   unsigned char* ovr = dyn + ((static_cast<size_t>(p.K) * W * sizeof(float) + 15) & ~size_t(15));
-  unsigned char* aux = ovr + ((static_cast<size_t>(p.K) * WW * sizeof(uint32_t) + 15) & ~size_t(15));
-  unsigned char* ring = aux + beam_aux_bytes(p.V, p.C, p.tokview) + static_cast<size_t>(W) * sizeof(float);
-  ring += (16 - (reinterpret_cast<uintptr_t>(ring) & 15)) & 15;
-  return reinterpret_cast<TbRsRec*>(ring + beam_ring_bytes(p.V, sizeof(LT)));
+  return ovr + ((static_cast<size_t>(p.K) * WW * sizeof(uint32_t) + 15) & ~size_t(15)) + beam_aux_bytes(p.V, p.C, p.tokview);
 }
-// Block-wide, once per launch: fills that copy if the stream's records fit.  Returns whether they do.
-template <typename LT>
-__device__ __forceinline__ bool beam_rec_cache_fill(const TbBeamParams& p, unsigned char* dyn) {
-  const TbSlotRec& rec = p.slots[blockIdx.x];
-  if (rec.n_states <= 0 || rec.n_rsent < 0 || static_cast<int64_t>(rec.n_states) * 16 > p.rec_cache_bytes) return false;
-  const uint4* src = reinterpret_cast<const uint4*>(p.arena + rec.blob_off + rec.off_rsrec);
-  uint4* dst = reinterpret_cast<uint4*>(beam_rec_cache<LT>(p, dyn));
-  for (int i = threadIdx.x; i < rec.n_states; i += blockDim.x) dst[i] = src[i];
-  return true;                                                  // (the barriers of the launch's first step come before any use)
+// Shared-memory atomics under a predicate, without a branch.
+__device__ __forceinline__ uint32_t beam_smem_addr(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
+__device__ __forceinline__ void shared_or(uint32_t* p, uint32_t v, bool yes) {
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %2, 0; @q red.shared.or.b32 [%0], %1; }" ::"r"(beam_smem_addr(p)), "r"(v), "r"(yes ? 1u : 0u) : "memory");
 }
-
+__device__ __forceinline__ void shared_add(int32_t* p, int v, bool yes) {
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %2, 0; @q red.shared.add.u32 [%0], %1; }" ::"r"(beam_smem_addr(p)), "r"(v), "r"(yes ? 1u : 0u) : "memory");
+}
+__device__ __forceinline__ void shared_put(unsigned long long* pk, unsigned long long key, int32_t* pd, int32_t d, bool yes) {
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %4, 0; @q st.shared.u64 [%0], %1; @q st.shared.u32 [%2], %3; }" ::"r"(beam_smem_addr(pk)), "l"(key),
+               "r"(beam_smem_addr(pd)), "r"(d), "r"(yes ? 1u : 0u) : "memory");
+}
+__device__ __forceinline__ int shared_fetch_add(int32_t* p, int v, bool yes) {
+  int r = 0;
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %3, 0; @q atom.shared.add.u32 %0, [%1], %2; }" : "+r"(r) : "r"(beam_smem_addr(p)), "r"(v), "r"(yes ? 1u : 0u) : "memory");
+  return r;
+}
 __device__ __forceinline__ void beam_team_barrier(int n_threads) { asm volatile("bar.sync 1, %0;" ::"r"(n_threads) : "memory"); }
 
-// Takes the steps sidx, sidx + 1, ... of the block's stream as long as it can; returns (on warp 0) how many it took.
-// Called by warps 0 .. K; the hypotheses are read from and left in sh.h_*.  hashA / hashB, lenA / lenB: the two halves
-// of the sequence records; step s writes half ((par0 + s) & 1 ? A : B).
-template <typename LT>
-__device__ __forceinline__ int beam_fast_run(const TbBeamParams& p, BeamShared& sh, unsigned char* dyn, int32_t sidx, const int32_t n_steps,
-                                             const int32_t E, const int64_t frame_stride, const int64_t row_stride,
-                                             const int32_t rows_per_stream, const int32_t step_base, unsigned long long* hashA,
-                                             unsigned long long* hashB, int32_t* lenA, int32_t* lenB, const int32_t par0,
-                                             const bool recs_cached) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int b = blockIdx.x, K = p.K, V = p.V, W = V + 1, M = p.top_m, WW = (W + 31) >> 5;
-  const int team = 32 * (K + 1);
-  const TbSlotRec rec = p.slots[b];
-  const bool bound = rec.n_states > 0;
-  const GraphPtrs g = graph_of(p.arena, rec);
-  const unsigned char* blob = p.arena + rec.blob_off;
-  uint32_t* ovr = reinterpret_cast<uint32_t*>(dyn + ((static_cast<size_t>(K) * W * sizeof(float) + 15) & ~size_t(15)));
-  unsigned char* aux = reinterpret_cast<unsigned char*>(ovr) + ((static_cast<size_t>(K) * WW * sizeof(uint32_t) + 15) & ~size_t(15));
-  unsigned char* ring = aux + beam_aux_bytes(V, p.C, p.tokview) + static_cast<size_t>(W) * sizeof(float);
-  ring += (16 - (reinterpret_cast<uintptr_t>(ring) & 15)) & 15;
-  const int row_buf = static_cast<int>((beam_ring_bytes(V, sizeof(LT)) - 16) / 2);
-  const LT* stream_base = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(b) * p.stream_stride;
-  auto row_of = [&](int s) -> const LT* {
-    const int t = s / E, e = s - t * E;
-    return stream_base + static_cast<int64_t>(t) * frame_stride + static_cast<int64_t>(e) * row_stride;
-  };
-
-  if (warp > 0) {
-    // ================================ worker: hypothesis k ================================
-    const int k = warp - 1;
-    TokView tv;
-    tokview_attach(tv, aux, V, p.C);
-    const TbTopEnt* top0 = p.top_base + static_cast<int64_t>(b) * rows_per_stream * (M + 1);
-    const TbRsRec* rsrec = recs_cached ? beam_rec_cache<LT>(p, dyn) : reinterpret_cast<const TbRsRec*>(blob + rec.off_rsrec);
-    const TbRsEnt* ent = reinterpret_cast<const TbRsEnt*>(blob + rec.off_rsent);
-    uint32_t* ovr_k = ovr + k * WW;
-    TbTopEnt tnext{-INFINITY, -INFINITY, 0xFFFFu};
-    if (lane <= M) tnext = top0[static_cast<int64_t>(sidx) * (M + 1) + lane];
-    beam_team_barrier(team);                                   // the coordinator has set up the first step
-    for (;; ++sidx) {
-      if (sh.f_cmd != 0) break;
-      const TbTopEnt tt = tnext;                               // (lane j: entry j of this step's reduced row, asked for a step ago)
-      if (sidx + 1 < n_steps && lane <= M) tnext = top0[static_cast<int64_t>(sidx + 1) * (M + 1) + lane];
-      const float sc1 = sh.f_sc[k];
-      const int32_t st1 = sh.f_st[k];
-      const bool lv1 = sh.f_lv[k] != 0;
-      // a lane keeps the three best of the candidates it sees, best first (a step's K picks hardly ever include more
-      // than three of one lane's; if they might, the step is left to the whole block)
-      unsigned long long m0 = 0ull, m1 = 0ull, m2 = 0ull;
-      int32_t e0 = -1, e1 = -1, e2 = -1;
-      int n_seen = 0;
-      auto offer = [&](unsigned long long kk, int32_t dd) {
-        ++n_seen;
-        if (kk > m0) { m2 = m1; e2 = e1; m1 = m0; e1 = e0; m0 = kk; e0 = dd; }
-        else if (kk > m1) { m2 = m1; e2 = e1; m1 = kk; e1 = dd; }
-        else if (kk > m2) { m2 = kk; e2 = dd; }
-      };
-      float D = 0.0f;
-      if (sc1 != -INFINITY) {
-        int32_t beg = 0, cnt = 0;
-        if (bound) {
-          int32_t sx = st1;
-          if (sx < 0 || sx >= rec.n_states) { if (lane == 0) atomicOr(p.status, TB_STATUS_BAD_STATE); sx = 0; }
-          const TbRsRec r = rsrec[sx];
-          beg = r.begin; cnt = r.count; D = r.D;
-        }
-        const unsigned char* rowb = ring + (sidx & 1) * row_buf + (reinterpret_cast<uintptr_t>(row_of(sidx)) & 15);
-        if (lv1) {
-          if (cnt > kFastMaxList) { if (lane == 0) sh.f_fail = 1; cnt = 0; }
-          for (int i = lane; i < WW; i += 32) ovr_k[i] = 0u;
-          __syncwarp();
-          // the listed tokens: exact values
-          for (int i0 = 0; i0 < cnt; i0 += 32) {
-            const int i = i0 + lane;
-            if (i < cnt) {
-              const TbRsEnt en = ent[beg + i];
-              const int tk = static_cast<int>((en.dst_tok & ((1u << TB_RS_TOK_BITS) - 1u)) >> 1);   // padding entries carry token V
-              if (tk < V) {
-                const float x = beam_smem_logit<LT>(rowb, tk);
-                offer(beam_key(__fadd_rn(sc1, __fadd_rn(x, en.lb)), tk, k), static_cast<int32_t>(en.dst_tok >> TB_RS_TOK_BITS));
-                atomicOr(&ovr_k[tk >> 5], 1u << (tk & 31));
-              }
-            }
-          }
-          __syncwarp();
-          // blank and the first unlisted tokens of the reduced row: lane j looks at its entry j
-          if (lane == M) {
-            offer(beam_key(__fadd_rn(sc1, tt.x), V, k), st1);
-          } else if (lane < M) {
-            const int tk = static_cast<int>(tt.tok_cls & 0xFFFFu), cl = static_cast<int>(tt.tok_cls >> 16);
-            if (tk < V && !((ovr_k[tk >> 5] >> (tk & 31)) & 1u)) {     // (tk >= V: the row has fewer tokens)
-              const float val = bound ? __fadd_rn(tt.x, __fmul_rn(g.lambda, __fadd_rn(D, tv.rootcw[cl]))) : tt.x;
-              offer(beam_key(__fadd_rn(sc1, val), tk, k), bound ? tv.rootdst[cl] : -1);
-            }
-          }
-        } else if (lane == M) {
-          offer(beam_key(sc1, V + 1, k), st1);                             // a frozen hypothesis is carried
-        }
-      }
-      // the K best of this hypothesis' candidates: lane r ends up with pick r
-      unsigned long long mykey = 0ull;
-      int32_t mydst = -1;
-      int taken = 0;
-      for (int r = 0; r < K; ++r) {
-        const uint32_t hi = static_cast<uint32_t>(m0 >> 32), lo = static_cast<uint32_t>(m0);
-        const uint32_t mh = __reduce_max_sync(0xffffffffu, hi);
-        const uint32_t ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-        const unsigned long long best = (static_cast<unsigned long long>(mh) << 32) | ml;
-        if (best == 0ull) break;                                  // (uniform: nothing left; the later picks stay empty)
-        const bool mine = m0 == best;
-        const unsigned who = __ballot_sync(0xffffffffu, mine);
-        const int32_t dsel = __shfl_sync(0xffffffffu, e0, __ffs(who) - 1);
-        if (lane == r) { mykey = best; mydst = dsel; }
-        if (mine) { m0 = m1; e0 = e1; m1 = m2; e1 = e2; m2 = 0ull; e2 = -1; ++taken; }
-      }
-      // a lane whose three kept candidates were all picked while it had seen more: a fourth might have been due
-      if (__any_sync(0xffffffffu, taken == 3 && n_seen > 3) && lane == 0) sh.f_fail = 1;
-      if (lane < K) { sh.f_key[k][lane] = mykey; sh.f_dst[k][lane] = mydst; }
-      {
-        // what the K-th pick of the step has to clear on behalf of this hypothesis (-inf: nothing)
-        const float y_next = __shfl_sync(0xffffffffu, tt.y, M);
-        if (lane == 0) {
-          float ub = -INFINITY;
-          if (y_next != -INFINITY && sc1 != -INFINITY && lv1) {
-            const float lamD = bound ? g.lambda * D : 0.0f;
-            const float scale = fabsf(sc1) + fabsf(y_next) + 2.0f * (bound ? fabsf(g.lambda) * (fabsf(D) + sh.root_wmax) : 0.0f);
-            ub = (sc1 + y_next) + lamD + scale * 3.814697265625e-6f + 1e-30f;      // 2^-18 of the scale
-          }
-          sh.f_ub[k] = ub;
-        }
-      }
-      beam_team_barrier(team);                                 // picks are in place
-      beam_team_barrier(team);                                 // the coordinator has set up the next step (or ended the run)
-    }
-    return 0;
-  }
-
-  // ================================ coordinator ================================
-  float sc = -INFINITY;
-  int32_t st = -1, hl = 0;
-  bool lv = false;
-  unsigned long long hh = 0ull;
-  if (lane < K) { sc = sh.h_score[lane]; st = sh.h_state[lane]; lv = sh.h_live[lane] != 0; hh = sh.h_hash[lane]; hl = sh.h_len[lane]; }
-  // the working copy of the hypotheses for step s: after the frame start's liveness, merging and pruning
-  float sc1 = sc;
-  int32_t st1 = st;
-  bool lv1 = lv;
-  auto frame_start = [&](int s) {
-    sc1 = sc; st1 = st; lv1 = lv;
-    if (s % E != 0) return;
-    lv1 = sc1 != -INFINITY;
-    if (p.merge) {
-      bool dup = false;
-      for (int j = 0; j + 1 < K; ++j) {
-        const float sj = __shfl_sync(0xffffffffu, sc, j);
-        const int32_t lj = __shfl_sync(0xffffffffu, hl, j), stj = __shfl_sync(0xffffffffu, st, j);
-        const unsigned long long hj = shfl_u64(hh, j);
-        if (lane > j && lane < K && sc != -INFINITY && sj != -INFINITY && lj == hl && hj == hh && stj == st) dup = true;
-      }
-      if (dup) { sc1 = -INFINITY; st1 = -1; lv1 = false; }
-    }
-    if (p.prune_delta >= 0.0f) {
-      float best = sc1;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-      if (lane < K && sc1 != -INFINITY && sc1 < __fsub_rn(best, p.prune_delta)) { sc1 = -INFINITY; st1 = -1; lv1 = false; }
-    }
-  };
-  auto publish = [&]() { if (lane < K) { sh.f_sc[lane] = sc1; sh.f_st[lane] = st1; sh.f_lv[lane] = lv1 ? 1 : 0; } };
-  frame_start(sidx);
-  publish();
-  if (lane == 0) { sh.f_cmd = 0; sh.f_fail = 0; }
-  beam_fetch_row<LT>(ring + (sidx & 1) * row_buf, row_of(sidx), W, p.tensor_lo, p.tensor_hi, lane);
-  if (sidx + 1 < n_steps) beam_fetch_row<LT>(ring + ((sidx + 1) & 1) * row_buf, row_of(sidx + 1), W, p.tensor_lo, p.tensor_hi, lane);
-  beam_cp_async_commit();
-  beam_cp_async_wait<0>();
-  __syncwarp();
-  beam_team_barrier(team);
-  int done = 0;
-  for (;; ++sidx) {
-    beam_team_barrier(team);                                   // the workers' picks are in place
-    // ---- the K best of K * K picks: lane i looks at picks i and i + 32
-    unsigned long long c0 = 0ull, c1 = 0ull;
-    int32_t d0 = -1, d1 = -1;
-    if (lane < K * K) { c0 = sh.f_key[lane / K][lane % K]; d0 = sh.f_dst[lane / K][lane % K]; }
-    if (lane + 32 < K * K) { c1 = sh.f_key[(lane + 32) / K][(lane + 32) % K]; d1 = sh.f_dst[(lane + 32) / K][(lane + 32) % K]; }
-    unsigned long long mykey = 0ull;
-    int32_t mydst = -1;
-    for (int r = 0; r < K; ++r) {
-      const bool second = c1 > c0;
-      const unsigned long long a = second ? c1 : c0;
-      const uint32_t hi = static_cast<uint32_t>(a >> 32), lo = static_cast<uint32_t>(a);
-      const uint32_t mh = __reduce_max_sync(0xffffffffu, hi);
-      const uint32_t ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-      const unsigned long long best = (static_cast<unsigned long long>(mh) << 32) | ml;
-      if (best == 0ull) break;
-      const bool mine = a == best;
-      const unsigned who = __ballot_sync(0xffffffffu, mine);
-      const int32_t dsel = __shfl_sync(0xffffffffu, second ? d1 : d0, __ffs(who) - 1);
-      if (lane == r) { mykey = best; mydst = dsel; }
-      if (mine) { if (second) c1 = 0ull; else c0 = 0ull; }
-    }
-    // ---- does the K-th pick clear everything that was not looked at?
-    bool ok = sh.f_fail == 0;
-    {
-      const unsigned long long key_last = shfl_u64(mykey, K - 1);
-      const float c_k = key_last != 0ull ? beam_key_value(key_last) : -INFINITY;
-      bool okk = true;
-      if (lane < K) { const float ub = sh.f_ub[lane]; okk = ub == -INFINITY || c_k > ub; }
-      ok = ok && __all_sync(0xffffffffu, okk);
-    }
-    if (!ok) {
-      if (lane == 0) sh.f_cmd = 1;
-      __syncwarp();
-      beam_team_barrier(team);
-      break;
-    }
-    // ---- the new hypotheses
-    int32_t parent = -1, token = -1, nstate = -1, nl = 0;
-    bool nlv = false;
-    float nsc = -INFINITY;
-    unsigned long long nh = 0ull;
-    {
-      const uint32_t l2 = 0xFFFFFFFFu - static_cast<uint32_t>(mykey & 0xFFFFFFFFull);
-      const int par_l = mykey != 0ull ? static_cast<int>(l2 & 31u) : 0;
-      const int32_t pst = __shfl_sync(0xffffffffu, st1, par_l), pl = __shfl_sync(0xffffffffu, hl, par_l);
-      const int plv = __shfl_sync(0xffffffffu, lv1 ? 1 : 0, par_l);
-      const unsigned long long ph = shfl_u64(hh, par_l);
-      if (lane < K && mykey != 0ull) {
-        const int tkey = static_cast<int>(l2 >> 5);
-        parent = par_l; nsc = beam_key_value(mykey);
-        token = tkey == V + 1 ? -1 : tkey;
-        nstate = pst;
-        nh = ph; nl = pl;
-        if (token >= 0 && token != V) {
-          nstate = mydst; nlv = plv != 0;
-          nh = (nh ^ static_cast<unsigned long long>(token + 1)) * 0xff51afd7ed558ccdull;
-          nh ^= nh >> 33;
-          nh += 0x9e3779b97f4a7c15ull;
-          ++nl;
-        }
-      }
-    }
-    sc = nsc; st = nstate; lv = nlv; hh = nh; hl = nl;
-    ++done;
-    const bool last = sidx + 1 >= n_steps;
-    if (!last) { frame_start(sidx + 1); publish(); }
-    if (lane == 0 && last) sh.f_cmd = 1;
-    beam_cp_async_wait<0>();                                   // the next step's row (asked for a step ago) is there
-    __syncwarp();
-    beam_team_barrier(team);                                   // the workers go on
-    // ---- off the critical path: this step's results, the row after the next
-    if (lane < K) {
-      const int64_t o = static_cast<int64_t>(b) * K + lane;
-      p.scores[o] = nsc; p.states[o] = nstate; p.live[o] = nlv ? 1 : 0;
-      p.out_parent[o] = parent; p.out_token[o] = token;
-      const bool odd = ((par0 + sidx) & 1) != 0;
-      (odd ? hashA : hashB)[o] = nh; (odd ? lenA : lenB)[o] = nl;
-      if (p.tree) {
-        const int32_t step = step_base + sidx;
-        const int64_t at = p.tree_cap > 0 ? static_cast<int64_t>(b) * p.tree_cap + (step % p.tree_cap)
-                                          : static_cast<int64_t>(step) * p.B + b;
-        p.tree[at * K + lane] = make_int2(parent, token);
-      }
-    }
-    if (last) break;
-    if (sidx + 2 < n_steps) beam_fetch_row<LT>(ring + (sidx & 1) * row_buf, row_of(sidx + 2), W, p.tensor_lo, p.tensor_hi, lane);
-    beam_cp_async_commit();
-  }
-  beam_cp_async_wait<0>();
-  if (lane < K) { sh.h_score[lane] = sc; sh.h_state[lane] = st; sh.h_live[lane] = lv ? 1 : 0; sh.h_hash[lane] = hh; sh.h_len[lane] = hl; }
-  if (lane == 0) sh.rec_ready = 0;
-  __syncwarp();
-  return done;
-}
-
 // Whether the team's steps apply to this launch and this block's stream.
-template <typename LT>
-__device__ __forceinline__ bool beam_fast_applies(const TbBeamParams& p) {
-  if (p.K > kFastMaxK || p.top_base == nullptr || p.tensor_lo == nullptr || p.top_m + 1 > 32) return false;
+__device__ __forceinline__ bool beam_team_applies(const TbBeamParams& p) {
+  if (p.top_base == nullptr || p.tensor_lo == nullptr) return false;
   const TbSlotRec& rec = p.slots[blockIdx.x];
   return rec.n_states <= 0 || (rec.n_rsent >= 0 && p.tokview);
 }
+// Block-wide, once per launch: the stream's hypotheses and root tables into shared memory, and its list records if they
+// fit (returns whether they do).
+__device__ inline bool beam_begin(const TbBeamParams& p, BeamShared& sh, unsigned char* dyn, const unsigned long long* hash_in,
+                                  const int32_t* len_in, bool team, const TeamSmem& tm) {
+  const int tid = threadIdx.x, K = p.K, b = blockIdx.x;
+  const TbSlotRec& rec = p.slots[b];
+  const bool bound = rec.n_states > 0, use_tv = bound && rec.n_rsent >= 0 && p.tokview;
+  if (tid < K) {
+    const int64_t o = static_cast<int64_t>(b) * K + tid;
+    sh.h_score[tid] = p.scores[o]; sh.h_state[tid] = p.states[o]; sh.h_live[tid] = p.live[o];
+    sh.h_hash[tid] = p.fresh ? 0ull : hash_in[o];
+    sh.h_len[tid] = p.fresh ? 0 : len_in[o];
+  }
+  if (tid == 0) { sh.root_wmax = 0.0f; sh.no_rec = make_uint4(0u, 0u, 0u, 0u); }
+  const int W = p.V + 1, WW = (W + 31) >> 5;
+  unsigned char* aux = dyn + ((static_cast<size_t>(K) * W * sizeof(float) + 15) & ~size_t(15)) + ((static_cast<size_t>(K) * WW * sizeof(uint32_t) + 15) & ~size_t(15));
+  bool cached = false;
+  if (use_tv) {
+    TokView tv;
+    tokview_init(tv, aux, p.V, p.C, graph_of(p.arena, rec));
+    if (tid < 32) {
+      float r = 0.0f;
+      for (int c = tid; c < p.C; c += 32) r = fmaxf(r, fabsf(tv.rootcw[c]));
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, off));
+      if (tid == 0) sh.root_wmax = r;
+    }
+    if (team && static_cast<int64_t>(rec.n_states) * 16 <= p.rec_cache_bytes) {
+      cached = true;
+      const uint4* src = reinterpret_cast<const uint4*>(p.arena + rec.blob_off + rec.off_rsrec);
+      uint4* dst = reinterpret_cast<uint4*>(team_base(p, dyn) + tm.recs);
+      for (int i = tid; i < rec.n_states; i += blockDim.x) dst[i] = src[i];
+    }
+  }
+  __syncthreads();
+  return cached;
+}
 
-// T frames of E rows in one launch: the block loops over the expansions of its stream; every hypothesis of the
-// stream reads row (t, e).  What a step leaves in global memory (scores, states, liveness, sequence records) is read
-// back in the next step by the thread that wrote it.
+// Takes the steps sidx, sidx + 1, ... of the block's stream as long as it can; returns how many it took.  Called by the
+// team's warps; the hypotheses are read from and left in sh.h_*.  H: hypotheses per worker.  hashA / hashB, lenA / lenB: the two halves of the
+// sequence records; step s writes half ((par0 + s) & 1 ? A : B), which only matters for the last one.
+template <typename LT, int H>
+__device__ __forceinline__ int beam_team_run(const TbBeamParams& p, BeamShared& sh, unsigned char* dyn, int32_t sidx, const int32_t n_steps,
+                                             const int32_t E, const int64_t frame_stride, const int64_t row_stride,
+                                             const int32_t rows_per_stream, const int32_t step_base, unsigned long long* hashA,
+                                             unsigned long long* hashB, int32_t* lenA, int32_t* lenB, const int32_t par0,
+                                             const bool recs_cached, const TeamSmem& tm) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = blockIdx.x, K = p.K, V = p.V, W = V + 1, M = p.top_m, WW = (W + 31) >> 5;
+  const int nw = team_warps(K), team = 32 * nw + 32;
+  const bool keeper = warp == nw;                              // the warp that keeps the books
+  const TbSlotRec& rec = p.slots[b];
+  const int n_states = rec.n_states;
+  const bool bound = n_states > 0;
+  const float lam = bound ? rec.lambda : 0.0f;
+  const unsigned char* blob = p.arena + rec.blob_off;
+  uint32_t* ovr = reinterpret_cast<uint32_t*>(dyn + ((static_cast<size_t>(K) * W * sizeof(float) + 15) & ~size_t(15)));
+  unsigned char* aux = reinterpret_cast<unsigned char*>(ovr) + ((static_cast<size_t>(K) * WW * sizeof(uint32_t) + 15) & ~size_t(15));
+  const float* rootcw = reinterpret_cast<const float*>(aux);             // (see tokview_attach)
+  const int32_t* rootdst = reinterpret_cast<const int32_t*>(aux + 4 * static_cast<size_t>(p.C));
+  unsigned char* tb_ = team_base(p, dyn);
+  const uint4* rsrec = !bound ? reinterpret_cast<const uint4*>(&sh.no_rec) : recs_cached ? reinterpret_cast<const uint4*>(tb_ + tm.recs) : reinterpret_cast<const uint4*>(blob + rec.off_rsrec);
+  const uint2* ent = reinterpret_cast<const uint2*>(blob + rec.off_rsent);
+  constexpr uint32_t kTok = (1u << TB_RS_TOK_BITS) - 1u;
+  const float root_wmax = sh.root_wmax;
+  // The rows: fr_* is the row that is fetched next (its frame and row in the frame, its buffer), off0 and off1
+  // are the byte offsets of the current and the next row within their first 16-byte pieces, buf the current row's buffer.
+  int e_cur = sidx % E, e_f = e_cur, buf = 0, buf_f = 0, s_f = sidx;
+  const LT* row_f = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(b) * p.stream_stride +
+                    static_cast<int64_t>(sidx / E) * frame_stride + static_cast<int64_t>(e_cur) * row_stride;
+  const unsigned char* top_f = reinterpret_cast<const unsigned char*>(p.top_base + (static_cast<int64_t>(b) * rows_per_stream + sidx) * (M + 1));
+  const int64_t to_frame = frame_stride - static_cast<int64_t>(E - 1) * row_stride;
+  int off0 = 0, off1 = 0;
+  auto fetch = [&]() {                                         // one row and its reduced row, by the keeper: one group of copies
+    off0 = off1;
+    off1 = static_cast<int>(reinterpret_cast<uintptr_t>(row_f) & 15);
+    if (keeper && s_f < n_steps) {
+      beam_fetch_row<LT>(tb_ + tm.row + buf_f * tm.row_stride, row_f, W, p.tensor_lo, p.tensor_hi, lane, 32);
+      unsigned char* dst = tb_ + tm.top + buf_f * tm.top_stride;
+#pragma unroll 1
+      for (int c = lane; c < ((M + 1) * 12) >> 4; c += 32) beam_cp_async16(dst + 16 * c, top_f + 16 * c);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    ++s_f;
+    buf_f = buf_f == kTeamRows - 1 ? 0 : buf_f + 1;
+    if (++e_f == E) { e_f = 0; row_f += to_frame; } else row_f += row_stride;
+    top_f += (M + 1) * 12;
+  };
+  // This warp's hypotheses, warp and (beams wider than sixteen) warp + 16: score, graph state, list, first 32 * kEnt entries
+  // (kEnt per lane).  live / have: bit k, hypothesis k can be expanded / has a score; best: the best score.
+  constexpr int kEnt = 1;
+  float ws[H], D[H];
+  int st[H], beg[H], cnt[H];
+  uint2 en[H][kEnt];
+  unsigned live, have;
+  bool long_lists = false;                                     // some list of this warp's has more entries than that
+  float best;
+  // lane k: the token sequence of hypothesis k (in the keeper, and in every warp where equal sequences are merged)
+  const bool hashes = keeper || p.merge;
+  unsigned long long hh = 0ull;
+  int32_t hl = 0;
+  // The hypotheses as the next step sees them, from lane r's (all warps alike): at a frame start all with a score are
+  // live, equal sequences are merged (the first stays) and what scores far below the best is dropped.  Then every worker
+  // takes its own and asks for their lists.
+  auto prepare = [&](bool frame_start, float sc, int32_t dst, bool lv) {
+    if (frame_start) {
+      lv = sc != -INFINITY;
+      if (p.merge) {
+        // earlier hypotheses with the same low word of the hash (there is hardly ever one: a compare each, no matching
+        // instruction, which goes value by value)
+        sh.hlow[lane] = lv ? static_cast<uint32_t>(hh) : static_cast<uint32_t>(-1 - lane);      // (all warps write the same)
+        __syncwarp();
+        unsigned same = 0u;
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) {
+          const uint4 q = *reinterpret_cast<const uint4*>(&sh.hlow[j]);
+          const uint32_t me = static_cast<uint32_t>(hh);
+          same |= (q.x == me ? 1u << j : 0u) | (q.y == me ? 2u << j : 0u) | (q.z == me ? 4u << j : 0u) | (q.w == me ? 8u << j : 0u);
+        }
+        same = lv ? same & ((1u << lane) - 1u) : 0u;
+        bool dup = false;
+#pragma unroll 1
+        while (__any_sync(0xffffffffu, same != 0u)) {          // equal hashes: lengths and states as well?
+          const int j = same ? __ffs(same) - 1 : lane;
+          const int32_t lj = __shfl_sync(0xffffffffu, hl, j), sj = __shfl_sync(0xffffffffu, dst, j);
+          const bool vj = __shfl_sync(0xffffffffu, sc != -INFINITY ? 1 : 0, j) != 0;
+          const unsigned long long hj = (static_cast<unsigned long long>(__shfl_sync(0xffffffffu, static_cast<uint32_t>(hh >> 32), j)) << 32) |
+                                        __shfl_sync(0xffffffffu, static_cast<uint32_t>(hh), j);
+          if (same && vj && hj == hh && lj == hl && sj == dst) { dup = true; same = 0u; }
+          same &= same - 1u;
+        }
+        if (dup) { sc = -INFINITY; lv = false; }
+      }
+      if (p.prune_delta >= 0.0f) {
+        const float top1 = beam_order_inv(__reduce_max_sync(0xffffffffu, beam_order(sc)));
+        if (sc != -INFINITY && sc < __fsub_rn(top1, p.prune_delta)) { sc = -INFINITY; lv = false; }
+      }
+    }
+    live = __ballot_sync(0xffffffffu, lv && sc != -INFINITY);
+    have = __ballot_sync(0xffffffffu, sc != -INFINITY);
+    best = beam_order_inv(__reduce_max_sync(0xffffffffu, beam_order(sc)));
+    if (!keeper) {
+      long_lists = false;
+#pragma unroll
+      for (int h = 0; h < H; ++h) {
+        const int k = min(warp + 16 * h, 31);                  // (a warp without a hypothesis: one without a score)
+        ws[h] = __shfl_sync(0xffffffffu, sc, k);
+        st[h] = __shfl_sync(0xffffffffu, dst, k);
+        const uint4 r = rsrec[static_cast<unsigned>(st[h]) < static_cast<unsigned>(n_states) ? st[h] : 0];
+        beg[h] = static_cast<int>(r.x); cnt[h] = static_cast<int>(r.y); D[h] = __uint_as_float(r.z);
+#pragma unroll
+        for (int u = 0; u < kEnt; ++u) {
+          en[h][u] = make_uint2(2u * static_cast<uint32_t>(V), 0u);
+          if (32 * u + lane < cnt[h]) en[h][u] = ent[beg[h] + 32 * u + lane];
+        }
+        long_lists |= cnt[h] > 32 * kEnt && ((live >> k) & 1u);
+      }
+    }
+  };
+
+#pragma unroll 1
+  for (int i = tid; i < K * WW; i += team) ovr[i] = 0u;
+#pragma unroll 1
+  for (int i = tid; i < 2 * kHistBins; i += team) (&sh.hist[0][0])[i] = 0;
+  if (tid < 2) sh.n_surv[tid] = 0;
+  if (tid == 0) sh.cmd = 0;
+  fetch();
+  fetch();
+  {
+    float sc = -INFINITY; int32_t dst = -1; bool lv = false;
+    if (lane < K) { sc = sh.h_score[lane]; dst = sh.h_state[lane]; lv = sh.h_live[lane] != 0; hh = sh.h_hash[lane]; hl = sh.h_len[lane]; }
+    if (keeper && bound && lane < K && sc != -INFINITY && (dst < 0 || dst >= n_states)) atomicOr(p.status, TB_STATUS_BAD_STATE);   // (read as the root)
+    prepare(e_cur == 0, sc, dst, lv);
+  }
+  int32_t tree_at = 0;                                         // where the step's nodes go in a ring
+  if (p.tree_cap > 0) tree_at = (step_base + sidx) % p.tree_cap;
+  asm volatile("cp.async.wait_group 1;" ::: "memory");
+  beam_team_barrier(team);
+  int done = 0;
+#pragma unroll 1
+  for (;; ++sidx) {
+    const int par = sidx & 1;
+    const unsigned char* row = tb_ + tm.row + buf * tm.row_stride + off0;
+    const TbTopEnt* top = reinterpret_cast<const TbTopEnt*>(tb_ + tm.top + buf * tm.top_stride);
+    int32_t* hist = sh.hist[par];
+    const bool over = sidx >= n_steps;                         // (only the last step's verdict is still to come)
+    const int hp = H > 1 ? (lane >> 3) & 1 : 0, kp = warp + 16 * hp, j0 = lane & 7;
+    const bool kp_ok = lane < 8 * H && kp < K && !keeper, alive = kp_ok && ((have >> (kp & 31)) & 1u), lvp = kp_ok && ((live >> (kp & 31)) & 1u);
+    const float scp = H > 1 && hp ? ws[H - 1] : ws[0], Dp = H > 1 && hp ? D[H - 1] : D[0];
+    uint32_t* ovr_p = ovr + min(kp, K - 1) * WW;
+    float ref = 0.0f, vp = -INFINITY, vb = -INFINITY, vl[H][kEnt];
+    bool listed[H][kEnt], pun = false, pin = false;
+    int bl[H][kEnt], bp = 0, bb = 0, ptok = V;
+    uint32_t pcls = 0u;
+    auto bin_of = [&](float v) { return max(0, min(kHistBins - 1, __float2int_rz((ref - v) * kHistPerUnit))); };
+    auto plain_value = [&](float x, uint32_t cl) {
+      return __fadd_rn(scp, bound ? __fadd_rn(x, __fmul_rn(lam, __fadd_rn(Dp, rootcw[cl]))) : x);
+    };
+    auto listed_value = [&](int h, const uint2& e, int tk) {
+      return __fadd_rn(ws[h], __fadd_rn(beam_smem_logit<LT>(row, tk), __uint_as_float(e.y)));
+    };
+    // ---- 1. values into the histogram.  A lane keeps the values of its entries per hypothesis, of its token of the reduced
+    // row (eight lanes per hypothesis: hypothesis kp) and of the blank.  (Written without branches: a lone warp pays about
+    // 45 cycles for each.)
+    if (!keeper && !over) {
+      const float xb = top[M].x, y_next = top[M].y;
+      const TbTopEnt tt = top[j0];                             // (M >= 15)
+      ref = best + fmaxf(xb, top[0].y) + kHistAbove;
+#pragma unroll
+      for (int h = 0; h < H; ++h) {
+        const int k = warp + 16 * h;
+        const bool lk = k < K && ((live >> (k & 31)) & 1u);
+        uint32_t* ov = ovr + min(k, K - 1) * WW;
+#pragma unroll
+        for (int u = 0; u < kEnt; ++u) {
+          const int tk = static_cast<int>((en[h][u].x & kTok) >> 1);       // (padding entries and unused lanes carry token V)
+          listed[h][u] = tk < V && lk;
+          shared_or(&ov[tk >> 5], 1u << (tk & 31), listed[h][u]);
+          vl[h][u] = listed_value(h, en[h][u], tk);
+          bl[h][u] = bin_of(vl[h][u]);
+          shared_add(&hist[bl[h][u]], 1, listed[h][u]);
+        }
+      }
+      if (long_lists) {
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const int k = warp + 16 * h;
+          if (k < K && ((live >> (k & 31)) & 1u))
+#pragma unroll 1
+            for (int i0 = 32 * kEnt; i0 < cnt[h]; i0 += 32) {
+              uint2 e = make_uint2(2u * static_cast<uint32_t>(V), 0u);
+              if (i0 + lane < cnt[h]) e = ent[beg[h] + i0 + lane];
+              const int t2 = static_cast<int>((e.x & kTok) >> 1);
+              shared_or(&ovr[k * WW + (t2 >> 5)], 1u << (t2 & 31), t2 < V);
+              shared_add(&hist[bin_of(listed_value(h, e, t2))], 1, t2 < V);
+            }
+        }
+      }
+      ptok = static_cast<int>(tt.tok_cls & 0xFFFFu); pcls = tt.tok_cls >> 16;
+      pin = lvp && ptok < V;                                   // (token >= V: the row has fewer tokens)
+      vp = plain_value(tt.x, pcls);
+      bp = bin_of(vp);
+      vb = lvp ? __fadd_rn(scp, xb) : scp;                     // the blank, or a frozen hypothesis carried
+      bb = bin_of(vb);
+      shared_add(&hist[bb], 1, alive && j0 == 0);
+      // what the K-th pick has to clear on behalf of this hypothesis (-inf: nothing)
+      const float scale = fabsf(scp) + fabsf(y_next) + 2.0f * fabsf(lam) * (fabsf(Dp) + root_wmax);
+      const float ub = (scp + y_next) + lam * Dp + scale * 3.814697265625e-6f + 1e-30f;     // 2^-18 of the scale
+      if (j0 == 0 && kp_ok) sh.w_ub[par][kp] = lvp && y_next != -INFINITY ? ub : -INFINITY;
+      __syncwarp();
+      const uint32_t bits = ovr_p[min(ptok, V) >> 5];
+      pun = pin & !((bits >> (ptok & 31)) & 1u);
+      shared_add(&hist[bp], 1, pun);
+    }
+    beam_team_barrier(team);                                   // the histogram is complete; the keeper has judged the step before
+    if (sh.cmd != 0) break;
+    fetch();
+    // ---- 2. the bin up to which candidates may be picks
+    if (keeper) {
+      *reinterpret_cast<int4*>(&sh.hist[par ^ 1][4 * lane]) = make_int4(0, 0, 0, 0);
+      if (lane == 0) sh.n_surv[par ^ 1] = 0;
+      asm volatile("cp.async.wait_group 1;" ::: "memory");     // the next step's row and reduced row are there
+    } else {
+      int bstar;
+      {
+        const int4 h4 = *reinterpret_cast<const int4*>(hist + 4 * lane);
+        const int c1 = h4.x, c2 = c1 + h4.y, c3 = c2 + h4.z, mine = c3 + h4.w;
+        int incl;
+        if (K <= 8) {                                          // counts up to K in unary: a ballot per unit instead of a scan
+          incl = 0;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) incl += __popc(__ballot_sync(0xffffffffu, mine > u) & (0xFFFFFFFFu >> (31 - lane)));
+        } else {
+          incl = mine;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); incl += lane >= o ? v : 0; }
+        }
+        const unsigned reach = __ballot_sync(0xffffffffu, incl >= K);
+        const int above = incl - (K <= 8 ? min(mine, 8) : mine);
+        const int d = (above + c1 < K ? 1 : 0) + (above + c2 < K ? 1 : 0) + (above + c3 < K ? 1 : 0);
+        const int at = __shfl_sync(0xffffffffu, 4 * lane + d, reach ? __ffs(reach) - 1 : 0);
+        bstar = reach ? at : kHistBins - 1;                    // (fewer than K: all of them)
+      }
+      // a lane's candidates take places one after the other
+      int mine = 0;
+#pragma unroll
+      for (int h = 0; h < H; ++h)
+#pragma unroll
+        for (int u = 0; u < kEnt; ++u) { listed[h][u] = listed[h][u] && bl[h][u] <= bstar; mine += listed[h][u] ? 1 : 0; }
+      const bool inp = pun && bp <= bstar, inb = alive && j0 == 0 && bb <= bstar;
+      mine += (inp ? 1 : 0) + (inb ? 1 : 0);
+      int at = shared_fetch_add(&sh.n_surv[par], mine, mine > 0);
+      auto put = [&](bool yes, float v, int tkey, int k, int32_t dst) {
+        shared_put(&sh.sk[min(at, kSurvivors)], beam_key(v, tkey, k), &sh.sd[min(at, kSurvivors)], dst, yes);     // (one place for what does not fit)
+        at += yes ? 1 : 0;
+      };
+#pragma unroll
+      for (int h = 0; h < H; ++h)
+#pragma unroll
+        for (int u = 0; u < kEnt; ++u)
+          put(listed[h][u], vl[h][u], static_cast<int>((en[h][u].x & kTok) >> 1), warp + 16 * h, static_cast<int32_t>(en[h][u].x >> TB_RS_TOK_BITS));
+      put(inp, vp, ptok, kp, bound ? rootdst[pcls] : -1);
+      put(inb, vb, lvp ? V : V + 1, kp, H > 1 && hp ? st[H - 1] : st[0]);
+      auto note = [&](bool yes, float v, int tkey, int k, int32_t dst) {
+        yes = yes && bin_of(v) <= bstar;
+        at = shared_fetch_add(&sh.n_surv[par], 1, yes);
+        put(yes, v, tkey, k, dst);
+      };
+      if (long_lists) {
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const int k = warp + 16 * h;
+          if (k < K && ((live >> (k & 31)) & 1u))
+#pragma unroll 1
+            for (int i0 = 32 * kEnt; i0 < cnt[h]; i0 += 32) {
+              uint2 e = make_uint2(2u * static_cast<uint32_t>(V), 0u);
+              if (i0 + lane < cnt[h]) e = ent[beg[h] + i0 + lane];
+              const int t2 = static_cast<int>((e.x & kTok) >> 1);
+              note(t2 < V, listed_value(h, e, t2), t2, k, static_cast<int32_t>(e.x >> TB_RS_TOK_BITS));
+            }
+        }
+      }
+      // further tokens of the reduced row, eight at a time, while the group's last one is still within the bins wanted
+      // (the order of the reduced row holds up to roundings: a margin of 2^-18 of the scale)
+      auto within = [&](float v) { return (ref - v - (fabsf(scp) + 32.0f) * 3.814697265625e-6f) * kHistPerUnit < static_cast<float>(bstar + 1); };
+      unsigned more = __ballot_sync(0xffffffffu, pin && within(vp)) & 0x8080u;
+#pragma unroll 1
+      for (int j = j0 + 8; more != 0u; j += 8) {
+        const bool on = ((more >> (lane | 7)) & 1u) && j < M;
+        const TbTopEnt t = top[min(j, M)];
+        const int tk = static_cast<int>(t.tok_cls & 0xFFFFu);
+        const bool good = on && tk < V;
+        const float v = plain_value(t.x, t.tok_cls >> 16);
+        const uint32_t bits = ovr_p[min(tk, V) >> 5];
+        note(good & !((bits >> (tk & 31)) & 1u), v, tk, kp, bound ? rootdst[t.tok_cls >> 16] : -1);
+        more = __ballot_sync(0xffffffffu, good && within(v)) & 0x8080u;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int h = 0; h < H; ++h)                              // the bitmaps are left clean
+#pragma unroll
+        for (int u = 0; u < kEnt; ++u)
+          if (warp + 16 * h < K) ovr[(warp + 16 * h) * WW + static_cast<int>((en[h][u].x & kTok) >> 6)] = 0u;
+      if (long_lists) {
+#pragma unroll
+        for (int h = 0; h < H; ++h)
+          if (warp + 16 * h < K)
+#pragma unroll 1
+            for (int i = lane; i < WW; i += 32) ovr[(warp + 16 * h) * WW + i] = 0u;
+      }
+    }
+    beam_team_barrier(team);                                   // the candidates are noted
+    // ---- 3. ranks
+    const int n = min(sh.n_surv[par], kSurvivors + 1);
+    if (n <= 32) {
+      // few: every warp ranks all of them by itself (lane i: candidate i)
+      const unsigned long long key = sh.sk[lane];
+      int c = 0;
+#pragma unroll 1
+      for (int i0 = 0; i0 < n; i0 += 8) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { const unsigned long long o = sh.sk[i0 + i]; c += (i0 + i < n) & (o > key) ? 1 : 0; }
+      }
+      if (lane < n && c < K) sh.ord[c] = lane;                 // (all warps write the same)
+      __syncwarp();
+    } else {
+      // eight lanes per candidate count the keys above it
+#pragma unroll 1
+      for (int t0 = 4 * warp; t0 < n && n <= kSurvivors; t0 += 4 * nw + 4) {
+        const int t = min(t0 + (lane >> 3), n - 1);
+        const unsigned long long key = sh.sk[t];
+        int c = 0;
+#pragma unroll 1
+        for (int i0 = j0; i0 - j0 < n; i0 += 64) {
+#pragma unroll
+          for (int i = 0; i < 64; i += 8) { const unsigned long long o = sh.sk[i0 + i]; c += (i0 + i < n) & (o > key) ? 1 : 0; }
+        }
+        c += __shfl_xor_sync(0xffffffffu, c, 1);
+        c += __shfl_xor_sync(0xffffffffu, c, 2);
+        c += __shfl_xor_sync(0xffffffffu, c, 4);
+        if (c < K && j0 == 0) sh.ord[c] = t;                   // (the last candidate may be ranked more than once: the same)
+      }
+      beam_team_barrier(team);
+    }
+    // ---- 4. the picks: lane r, pick r (in every warp)
+    const bool picked = n <= kSurvivors && lane < min(n, K);
+    const int pick = picked ? sh.ord[lane] : 0;
+    const unsigned long long pick_key = sh.sk[pick];
+    const int32_t pick_dst = sh.sd[pick];
+    const unsigned long long key = picked ? pick_key : 0ull;
+    const int32_t dst = picked ? pick_dst : -1;
+    const uint32_t l2 = 0xFFFFFFFFu - static_cast<uint32_t>(key & 0xFFFFFFFFull);
+    const int parent = key != 0ull ? static_cast<int>(l2 & 31u) : -1, tkey = static_cast<int>(l2 >> 5);
+    const float sc = key != 0ull ? beam_key_value(key) : -INFINITY;
+    const bool emits = parent >= 0 && tkey < V;
+    const bool lv = emits && ((live >> (parent & 31)) & 1u);
+    const bool last = sidx + 1 >= n_steps, frame_next = e_cur + 1 == E;
+    if (hashes) {                                              // one more token: a 64-bit mix of the sequence so far and the token
+      const int from = parent >= 0 ? parent : lane;
+      unsigned long long nh = (static_cast<unsigned long long>(__shfl_sync(0xffffffffu, static_cast<uint32_t>(hh >> 32), from)) << 32) |
+                              __shfl_sync(0xffffffffu, static_cast<uint32_t>(hh), from);
+      hl = __shfl_sync(0xffffffffu, hl, from) + (emits ? 1 : 0);
+      unsigned long long mh = (nh ^ static_cast<unsigned long long>(tkey + 1)) * 0xff51afd7ed558ccdull;
+      mh ^= mh >> 33;
+      mh += 0x9e3779b97f4a7c15ull;
+      hh = parent < 0 ? 0ull : emits ? mh : nh;
+      if (parent < 0) hl = 0;
+    }
+    if (keeper) {
+      // does the K-th pick clear everything that was not looked at?
+      const float c_k = __shfl_sync(0xffffffffu, sc, K - 1);
+      const float ub = sh.w_ub[par][lane];
+      const bool okk = (lane >= K) | (ub == -INFINITY) | (c_k > ub);
+      if (__all_sync(0xffffffffu, okk) && n <= kSurvivors) {
+        const int32_t token = parent < 0 || tkey == V + 1 ? -1 : tkey;
+        if (lane < K) {
+          sh.h_score[lane] = sc; sh.h_state[lane] = dst; sh.h_live[lane] = lv ? 1 : 0; sh.h_hash[lane] = hh; sh.h_len[lane] = hl;
+          if (p.tree) {
+            const int64_t at = p.tree_cap > 0 ? static_cast<int64_t>(b) * p.tree_cap + tree_at : static_cast<int64_t>(step_base + sidx) * p.B + b;
+            p.tree[at * K + lane] = make_int2(parent, token);
+          }
+          if (last) {
+            const int64_t o = static_cast<int64_t>(b) * K + lane;
+            p.scores[o] = sc; p.states[o] = dst; p.live[o] = lv ? 1 : 0;
+            p.out_parent[o] = parent; p.out_token[o] = token;
+            const bool odd = ((par0 + sidx) & 1) != 0;
+            (odd ? hashA : hashB)[o] = hh; (odd ? lenA : lenB)[o] = hl;
+          }
+        }
+        if (lane == 0) { sh.done = done + 1; if (last) sh.cmd = 1; }
+      } else if (lane == 0) {
+        sh.done = done; sh.cmd = 2;
+      }
+    }
+    ++done;
+    if (!last) prepare(frame_next, sc, dst, lv);
+    e_cur = frame_next ? 0 : e_cur + 1;
+    buf = buf == kTeamRows - 1 ? 0 : buf + 1;
+    if (++tree_at == p.tree_cap) tree_at = 0;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  return sh.done;
+}
+
+// All steps of one stream of a multi-step launch: the team takes what it can, the block the rest.
 template <typename LT>
-__global__ void __launch_bounds__(kBeamThreads) k_beam_frames(TbBeamParams p, int32_t T, int32_t E, int64_t frame_stride,
-                                                          int64_t row_stride) {
-  __shared__ BeamShared sh;
+__device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared& sh, unsigned char* dyn, const int32_t n_steps, const int32_t E,
+                                               const int64_t frame_stride, const int64_t row_stride, const int32_t rows_per_stream,
+                                               const int32_t step_base, unsigned long long* hashA, unsigned long long* hashB, int32_t* lenA,
+                                               int32_t* lenB, const int32_t par0) {
   LT xpre[kBeamPref] = {};
   bool xpre_valid = false;
-  TbTopEnt tpre{0.0f, 0.0f, 0u};
-  bool tpre_valid = false;
+  const bool fast = beam_team_applies(p);
+  const TeamSmem tm = team_smem(p.V, sizeof(LT), p.top_m, p.rec_cache_bytes);
+  const bool odd0 = (par0 & 1) != 0;
+  const bool recs_cached = beam_begin(p, sh, dyn, odd0 ? hashB : hashA, odd0 ? lenB : lenA, fast, tm);
   const LT* stream_base = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(blockIdx.x) * p.stream_stride;
-  extern __shared__ __align__(16) unsigned char dyn_all[];
-  const bool fast = beam_fast_applies<LT>(p);
-  const bool recs_cached = fast && beam_rec_cache_fill<LT>(p, dyn_all);
   int32_t skip = 0, backoff = 0;              // steps until the team tries again after a step it could not take
-  for (int32_t sidx = 0; sidx < T * E; ++sidx) {
-    if (fast && sidx > 0 && skip-- <= 0) {
-      if (threadIdx.x < 32 * (p.K + 1)) {
-        const int d = beam_fast_run<LT>(p, sh, dyn_all, sidx, T * E, E, frame_stride, row_stride, T * E, p.step,
-                                        const_cast<unsigned long long*>(p.hash_in), p.hash_out, const_cast<int32_t*>(p.len_in), p.len_out, 0,
-                                        recs_cached);
-        if (threadIdx.x == 0) sh.fast_done = d;
+#pragma unroll 1
+  for (int32_t sidx = 0; sidx < n_steps; ++sidx) {
+    if (fast && skip-- <= 0) {
+      if (threadIdx.x < 32 * (team_warps(p.K) + 1)) {
+        const int d = p.K > 16 ? beam_team_run<LT, 2>(p, sh, dyn, sidx, n_steps, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB,
+                                                      lenA, lenB, par0, recs_cached, tm)
+                               : beam_team_run<LT, 1>(p, sh, dyn, sidx, n_steps, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB,
+                                                      lenA, lenB, par0, recs_cached, tm);
+        if (threadIdx.x == 0) sh.team_done = d;
       }
       __syncthreads();
-      const int d = sh.fast_done;
+      const int d = sh.team_done;
       __syncthreads();                          // (read by everyone before a later run writes it again)
       sidx += d;
       backoff = d == 0 ? min(2 * backoff + 1, 32) : 0;
       skip = backoff;
-      xpre_valid = false; tpre_valid = false;
-      if (sidx >= T * E) break;
+      xpre_valid = false;
+      if (sidx >= n_steps) break;
     }
-    {
-      const int32_t t = sidx / E, e = sidx - t * E;
-      TbBeamParams q = p;
-      q.logits = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(t) * frame_stride + static_cast<int64_t>(e) * row_stride;
-      q.hyp_stride = 0;
-      q.new_frame = e == 0 ? 1 : 0;
-      q.merge = e == 0 ? p.merge : 0;
-      q.prune_delta = e == 0 ? p.prune_delta : -1.0f;
-      q.fresh = (p.fresh && sidx == 0) ? 1 : 0;
-      q.tv_ready = sidx > 0 ? 1 : 0;
-      q.step = p.step + sidx;
-      q.top_row = p.top_base ? p.top_base + (static_cast<int64_t>(blockIdx.x) * T * E + sidx) * (p.top_m + 1) : nullptr;
-      if (sidx & 1) { q.hash_in = p.hash_out; q.hash_out = const_cast<unsigned long long*>(p.hash_in); q.len_in = p.len_out; q.len_out = const_cast<int32_t*>(p.len_in); }
-      const int32_t nt = e + 1 < E ? t : t + 1, ne = e + 1 < E ? e + 1 : 0;
-      const LT* next_row = nt < T ? stream_base + static_cast<int64_t>(nt) * frame_stride + static_cast<int64_t>(ne) * row_stride : nullptr;
-      const TbTopEnt* next_top = (nt < T && q.top_row) ? q.top_row + (p.top_m + 1) : nullptr;
-      beam_step_body<LT>(q, sh, xpre, xpre_valid, next_row, tpre, tpre_valid, next_top);
-      __syncthreads();
-    }
+    const int32_t t = sidx / E, e = sidx - t * E;
+    TbBeamParams q = p;
+    q.logits = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(t) * frame_stride + static_cast<int64_t>(e) * row_stride;
+    q.hyp_stride = 0;
+    q.new_frame = e == 0 ? 1 : 0;
+    q.merge = e == 0 ? p.merge : 0;
+    q.prune_delta = e == 0 ? p.prune_delta : -1.0f;
+    q.fresh = 0;
+    q.tv_ready = 1;
+    q.step = step_base + sidx;
+    const bool odd = ((par0 + sidx) & 1) != 0;
+    q.hash_in = odd ? hashB : hashA; q.hash_out = odd ? hashA : hashB; q.len_in = odd ? lenB : lenA; q.len_out = odd ? lenA : lenB;
+    const int32_t nt = e + 1 < E ? t : t + 1, ne = e + 1 < E ? e + 1 : 0;
+    const LT* next_row = sidx + 1 < n_steps ? stream_base + static_cast<int64_t>(nt) * frame_stride + static_cast<int64_t>(ne) * row_stride : nullptr;
+    beam_step_body<LT>(q, sh, xpre, xpre_valid, next_row);
+    __syncthreads();
   }
+}
+
+// T frames of E rows in one launch: the block loops over the expansions of its stream; every hypothesis of the
+// stream reads row (t, e).
+template <typename LT>
+__global__ void __launch_bounds__(kBeamThreads) k_beam_frames(TbBeamParams p, int32_t T, int32_t E, int64_t frame_stride,
+                                                          int64_t row_stride) {
+  __shared__ BeamShared sh;
+  extern __shared__ __align__(16) unsigned char dyn_all[];
+  beam_all_steps<LT>(p, sh, dyn_all, T * E, E, frame_stride, row_stride, T * E, p.step, const_cast<unsigned long long*>(p.hash_in), p.hash_out,
+                     const_cast<int32_t*>(p.len_in), p.len_out, 0);
 }
 
 // Beam pre-pass: one warp per logit row, independent of every hypothesis.  With the rows of a stream shared by its
 // hypotheses, the order of a row's tokens that no hypothesis' state boosts is, up to rounding, the order of their
-// root-boosted values y -- so a step only needs the first few of them (see the compact path of beam_step_body).
+// root-boosted values y -- so a step only needs the first few of them (see beam_team_run).
 constexpr int kTopWarps = 8;
 template <typename LT>
 __global__ void __launch_bounds__(kTopWarps * 32) k_beam_topm(const LT* logits, int32_t B, int32_t T, int32_t E, int32_t V, int32_t C,
@@ -1576,55 +1374,12 @@ __global__ void __launch_bounds__(kBeamThreads) k_beam_chunk(TbBeamParams p, int
                                                          int64_t row_stride, const int32_t* n_frames, int32_t* slot_pos,
                                                          unsigned long long* hash, int32_t* len, size_t n_hyp) {
   __shared__ BeamShared sh;
-  LT xpre[kBeamPref] = {};
-  bool xpre_valid = false;
-  TbTopEnt tpre{0.0f, 0.0f, 0u};
-  bool tpre_valid = false;
+  extern __shared__ __align__(16) unsigned char dyn_all[];
   const int b = blockIdx.x;
   const int32_t nf = n_frames ? max(0, min(T, n_frames[b])) : T;
   const int32_t pos0 = slot_pos[b];
-  const LT* stream_base = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(b) * p.stream_stride;
-  extern __shared__ __align__(16) unsigned char dyn_all[];
-  const bool fast = beam_fast_applies<LT>(p);
-  const bool recs_cached = fast && beam_rec_cache_fill<LT>(p, dyn_all);
-  int32_t skip = 0, backoff = 0;
-  for (int32_t sidx = 0; sidx < nf * E; ++sidx) {
-    if (fast && sidx > 0 && skip-- <= 0) {
-      if (threadIdx.x < 32 * (p.K + 1)) {
-        const int d = beam_fast_run<LT>(p, sh, dyn_all, sidx, nf * E, E, frame_stride, row_stride, T * E, pos0, hash, hash + n_hyp,
-                                        len, len + n_hyp, pos0, recs_cached);
-        if (threadIdx.x == 0) sh.fast_done = d;
-      }
-      __syncthreads();
-      const int d = sh.fast_done;
-      __syncthreads();
-      sidx += d;
-      backoff = d == 0 ? min(2 * backoff + 1, 32) : 0;
-      skip = backoff;
-      xpre_valid = false; tpre_valid = false;
-      if (sidx >= nf * E) break;
-    }
-    {
-      const int32_t t = sidx / E, e = sidx - t * E;
-      TbBeamParams q = p;
-      q.logits = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(t) * frame_stride + static_cast<int64_t>(e) * row_stride;
-      q.hyp_stride = 0;
-      q.new_frame = e == 0 ? 1 : 0;
-      q.merge = e == 0 ? p.merge : 0;
-      q.prune_delta = e == 0 ? p.prune_delta : -1.0f;
-      q.fresh = 0;
-      q.tv_ready = sidx > 0 ? 1 : 0;
-      q.step = pos0 + sidx;
-      q.top_row = p.top_base ? p.top_base + (static_cast<int64_t>(b) * T * E + sidx) * (p.top_m + 1) : nullptr;
-      const size_t in = ((pos0 + sidx) & 1) ? n_hyp : 0, out = ((pos0 + sidx) & 1) ? 0 : n_hyp;
-      q.hash_in = hash + in; q.hash_out = hash + out; q.len_in = len + in; q.len_out = len + out;
-      const int32_t nt = e + 1 < E ? t : t + 1, ne = e + 1 < E ? e + 1 : 0;
-      const LT* next_row = nt < nf ? stream_base + static_cast<int64_t>(nt) * frame_stride + static_cast<int64_t>(ne) * row_stride : nullptr;
-      const TbTopEnt* next_top = (nt < nf && q.top_row) ? q.top_row + (p.top_m + 1) : nullptr;
-      beam_step_body<LT>(q, sh, xpre, xpre_valid, next_row, tpre, tpre_valid, next_top);
-      __syncthreads();
-    }
-  }
+  if (nf > 0)
+    beam_all_steps<LT>(p, sh, dyn_all, nf * E, E, frame_stride, row_stride, T * E, pos0, hash, hash + n_hyp, len, len + n_hyp, pos0);
   if (threadIdx.x == 0) slot_pos[b] = pos0 + nf * E;
 }
 
@@ -1750,9 +1505,9 @@ __global__ void k_publish_slot(TbSlotRec* slots, TbSlotState* sstate, int32_t sl
 
 template <typename F>
 int set_smem(F* fn, size_t bytes) {
-  // (the default limit of 48 KB counts the kernel's static shared memory too -- up to 16 KB here -- so the opt-in
+  // (the default limit of 48 KB counts the kernel's static shared memory too -- up to 24 KB here -- so the opt-in
   //  starts well below it)
-  if (bytes > 24 * 1024) {
+  if (bytes > 16 * 1024) {
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes)) != cudaSuccess) {
       cudaGetLastError();
       return TB_ERR_INVALID_ARG;
@@ -1786,7 +1541,7 @@ int tb_launch_decode_general(const TbDecodeParams& p_in, cudaStream_t stream, co
 int tb_launch_beam_step(const TbBeamParams& p_in, cudaStream_t stream) {
   TbBeamParams p = p_in;
   p.tokview = 2 * (p.V + 1) <= (1 << TB_RS_TOK_BITS) ? 1 : 0;
-  const size_t aux = beam_aux_bytes(p.V, p.C, p.tokview) + static_cast<size_t>(p.V + 1) * sizeof(float);   // + the staged row
+  const size_t aux = beam_aux_bytes(p.V, p.C, p.tokview);
   const size_t smem = ((static_cast<size_t>(p.K) * (p.V + 1) * sizeof(float) + 15) & ~size_t(15)) +
                       ((static_cast<size_t>(p.K) * ((p.V + 1 + 31) >> 5) * sizeof(uint32_t) + 15) & ~size_t(15)) + aux;
   if (smem > 200 * 1024) return TB_ERR_INVALID_ARG;
@@ -1801,17 +1556,18 @@ int tb_launch_beam_step(const TbBeamParams& p_in, cudaStream_t stream) {
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
 
-// The team steps of narrow beams (beam_fast_run) read rows through two buffers behind the block's other shared
-// memory and need the extent of the logits tensor; without either (a wide beam, odd strides) they stay off.
-static void beam_fast_setup(TbBeamParams* p, int32_t T, int32_t E, int64_t frame_stride, int64_t row_stride, size_t* smem) {
+// The team's steps (beam_team_run) read rows through buffers behind the block's other shared memory and need the extent
+// of the logits tensor; without either (odd strides, no room) they stay off.
+static void beam_team_setup(TbBeamParams* p, int32_t T, int32_t E, int64_t frame_stride, int64_t row_stride, size_t* smem) {
+  constexpr size_t kMost = 200 * 1024;
   p->tensor_lo = nullptr; p->tensor_hi = nullptr; p->rec_cache_bytes = 0;
-  if (p->K > kFastMaxK || !p->top_base || p->stream_stride < 0 || frame_stride < 0 || row_stride < 0) return;
-  const size_t elem = p->dtype == TB_BF16 ? 2 : 4;
-  const size_t more = beam_ring_bytes(p->V, static_cast<int>(elem)) + 16;
-  if (*smem + more > 200 * 1024) return;
+  if (!p->top_base || p->stream_stride < 0 || frame_stride < 0 || row_stride < 0) return;
+  const int elem = p->dtype == TB_BF16 ? 2 : 4;
+  const size_t more = team_smem(p->V, elem, p->top_m, 0).total;
+  if (*smem + more > kMost) return;
   *smem += more;
-  p->rec_cache_bytes = 0;
-  if (*smem + kFastRecCache <= 200 * 1024) { p->rec_cache_bytes = kFastRecCache; *smem += kFastRecCache; }
+  p->rec_cache_bytes = static_cast<int32_t>((kMost - *smem < static_cast<size_t>(kTeamRecCache) ? kMost - *smem : static_cast<size_t>(kTeamRecCache)) & ~size_t(15));
+  *smem += p->rec_cache_bytes;
   const int64_t last = static_cast<int64_t>(p->B - 1) * p->stream_stride + static_cast<int64_t>(T - 1) * frame_stride +
                        static_cast<int64_t>(E - 1) * row_stride + p->V;
   p->tensor_lo = static_cast<const unsigned char*>(p->logits);
@@ -1822,10 +1578,10 @@ int tb_launch_beam_frames(const TbBeamParams& p_in, int32_t T, int32_t E, int64_
                           cudaStream_t stream) {
   TbBeamParams p = p_in;
   p.tokview = 2 * (p.V + 1) <= (1 << TB_RS_TOK_BITS) ? 1 : 0;
-  const size_t aux = beam_aux_bytes(p.V, p.C, p.tokview) + static_cast<size_t>(p.V + 1) * sizeof(float);   // + the staged row
+  const size_t aux = beam_aux_bytes(p.V, p.C, p.tokview);
   size_t smem = ((static_cast<size_t>(p.K) * (p.V + 1) * sizeof(float) + 15) & ~size_t(15)) +
                 ((static_cast<size_t>(p.K) * ((p.V + 1 + 31) >> 5) * sizeof(uint32_t) + 15) & ~size_t(15)) + aux;
-  beam_fast_setup(&p, T, E, frame_stride, row_stride, &smem);
+  beam_team_setup(&p, T, E, frame_stride, row_stride, &smem);
   if (smem > 200 * 1024) return TB_ERR_INVALID_ARG;
   int rc;
   if (p.dtype == TB_BF16) {
@@ -1981,10 +1737,10 @@ int tb_launch_beam_chunk(const TbBeamParams& p_in, int32_t T, int32_t E, int64_t
                          cudaStream_t stream) {
   TbBeamParams p = p_in;
   p.tokview = 2 * (p.V + 1) <= (1 << TB_RS_TOK_BITS) ? 1 : 0;
-  const size_t aux = beam_aux_bytes(p.V, p.C, p.tokview) + static_cast<size_t>(p.V + 1) * sizeof(float);   // + the staged row
+  const size_t aux = beam_aux_bytes(p.V, p.C, p.tokview);
   size_t smem = ((static_cast<size_t>(p.K) * (p.V + 1) * sizeof(float) + 15) & ~size_t(15)) +
                 ((static_cast<size_t>(p.K) * ((p.V + 1 + 31) >> 5) * sizeof(uint32_t) + 15) & ~size_t(15)) + aux;
-  beam_fast_setup(&p, T, E, frame_stride, row_stride, &smem);
+  beam_team_setup(&p, T, E, frame_stride, row_stride, &smem);
   if (smem > 200 * 1024) return TB_ERR_INVALID_ARG;
   int rc;
   if (p.dtype == TB_BF16) {

@@ -50,8 +50,6 @@ struct TbBeamParams {
   // tree is [steps, B, K] for the whole batch
   int32_t tree_cap;
   // rows reduced ahead of the steps (tb_launch_beam_topm): per row top_m + 1 entries of 12 bytes, see TbTopEnt; null: none.
-  // top_rows: this step's row (set per step inside a multi-step launch); top_base / strides: where the launch finds them
-  const struct TbTopEnt* top_row;
   const struct TbTopEnt* top_base;
   int32_t top_m;
   const TbSlotRec* slots; const unsigned char* arena; const int32_t* cls; int32_t* status;
