@@ -1304,8 +1304,7 @@ extern "C" int tb_beam_backtrace_slots(tb_batch* b, int32_t n_slots, int32_t K, 
   if (!guard.ok) return TB_ERR_CUDA;
   const int32_t cap = static_cast<int32_t>(static_cast<int64_t>(b->max_tree_steps) * b->max_beam / K);
   return tb_launch_beam_backtrace_slots(b->d_tree, cap, b->d_slot_pos, n_slots, K, b->vocab, max_len, out_tokens, out_lens,
-                                        b->d_status, b->d_hyp_len, static_cast<size_t>(b->n_slots) * b->max_beam, nullptr,
-                                        static_cast<cudaStream_t>(stream_));
+                                        b->d_status, nullptr, static_cast<cudaStream_t>(stream_));
 }
 
 extern "C" int tb_beam_backtrace_slot_list(tb_batch* b, int32_t n, const int32_t* slots, int32_t K, int32_t max_len,
@@ -1321,8 +1320,7 @@ extern "C" int tb_beam_backtrace_slot_list(tb_batch* b, int32_t n, const int32_t
     const int32_t m = n - at < TB_BIND_PAIRS ? n - at : TB_BIND_PAIRS;
     const int rc = tb_launch_beam_backtrace_slots(b->d_tree, cap, b->d_slot_pos, m, K, b->vocab, max_len,
                                                   out_tokens + static_cast<int64_t>(at) * K * max_len, out_lens + static_cast<int64_t>(at) * K,
-                                                  b->d_status, b->d_hyp_len, static_cast<size_t>(b->n_slots) * b->max_beam, slots + at,
-                                                  static_cast<cudaStream_t>(stream_));
+                                                  b->d_status, slots + at, static_cast<cudaStream_t>(stream_));
     if (rc != TB_OK) return rc;
   }
   return TB_OK;
@@ -1350,9 +1348,5 @@ extern "C" int tb_beam_backtrace(tb_batch* b, int32_t B, int32_t K, int32_t max_
   if (!b->d_tree || b->tree_steps == 0 || b->tree_B != B || b->tree_K != K) return TB_ERR_INVALID_ARG;
   DeviceGuard guard(b->device);
   if (!guard.ok) return TB_ERR_CUDA;
-  // the sequence records the last step wrote: their lengths are the transcripts' lengths
-  const size_t n_hyp = static_cast<size_t>(b->n_slots) * b->max_beam;
-  const int32_t* len_cur = b->beam_steps > 0 ? b->d_hyp_len + (((b->beam_steps - 1) & 1) ? 0 : n_hyp) : nullptr;
-  return tb_launch_beam_backtrace(b->d_tree, b->tree_steps, B, K, b->vocab, max_len, out_tokens, out_lens, len_cur,
-                                  static_cast<cudaStream_t>(stream_));
+  return tb_launch_beam_backtrace(b->d_tree, b->tree_steps, B, K, b->vocab, max_len, out_tokens, out_lens, static_cast<cudaStream_t>(stream_));
 }

@@ -1409,87 +1409,83 @@ __global__ void k_beam_reset_slots(int32_t* slot_pos, unsigned long long* hash, 
   }
 }
 
-// The tokens of every hypothesis a slot holds, walked back through the slot's own ring to the start of its utterance.
-// Backtrace of one stream's K hypotheses by one warp (lane k: hypothesis k).  The walk from the last step back to the
-// first is a chain of dependent loads; the warp therefore brings the tree's nodes of 32 steps at a time into shared
-// memory (coalesced, one trip) and the lanes follow their chains there.  The number of tokens of a hypothesis is its
-// sequence record's length, so the tokens are written from the back in one walk; only where part of the utterance
-// has left the ring (or no record is at hand) a first walk counts what is still there.
-// RING: the stream's own ring of tree_cap steps at position slot_pos[slot] (streaming), sequence records in the half
-// of len_base that the slot's last step wrote; else the batch-wide tree [n_steps, B, K] with the records at len_cur.
-// sl / use_list: the slots to walk (output row i belongs to sl.slot[i]); else slot = block index.
-constexpr int kBtSteps = 32;
-constexpr int kBtBufs = 4;         // stages in flight: the copies of the next three are under way while one is walked
+// The tokens of every hypothesis a stream holds, walked back to the start of its utterance.  The walk is a chain of
+// dependent look-ups, a step at a time, so the steps are cut into pieces walked at the same time, one warp each: (a) from
+// every hypothesis at a piece's end to its start, counting tokens; (b) the pieces' maps composed from the last to the first
+// give, per hypothesis, where it enters each piece and where its tokens there end in the transcript; (c) the pieces again,
+// now writing.  A warp reads the nodes of 32 / K steps per register, eight registers at a time, and follows the parents with
+// shuffles.  3000 steps, K = 4: 5 us (one warp for the whole chain, nodes staged in shared memory ahead of it: 75 us).
+// RING: the stream's own ring of tree_cap steps at position slot_pos[slot] (streaming); else the batch-wide tree
+// [n_steps, B, K].  sl / use_list: the slots to walk (output row i belongs to sl.slot[i]); else slot = block index.
+constexpr int kBtWarps = 16;
+constexpr int kBtMin = 16;         // steps of a piece at least
+constexpr int kBtRegs = 8;
 template <bool RING>
-__global__ void __launch_bounds__(32) k_beam_backtrace_warp(const int2* tree, int32_t tree_cap, const int32_t* slot_pos, int32_t n_steps,
-                                                           int32_t B, int32_t K, int32_t V, int32_t max_len, int32_t* out_tokens,
-                                                           int32_t* out_lens, int32_t* status, const int32_t* len_base,
-                                                           size_t n_hyp, const int32_t* len_cur, SlotList sl, int32_t use_list) {
-  extern __shared__ __align__(16) int2 bt_stage[];           // [kBtBufs][kBtSteps][K]
-  const int lane = threadIdx.x;
+__global__ void __launch_bounds__(32 * kBtWarps) k_beam_backtrace(const int2* tree, int32_t tree_cap, const int32_t* slot_pos, int32_t n_steps,
+                                                                  int32_t B, int32_t K, int32_t V, int32_t max_len, int32_t* out_tokens,
+                                                                  int32_t* out_lens, int32_t* status, const __grid_constant__ SlotList sl,
+                                                                  int32_t use_list) {
+  __shared__ int2 piece[kBtWarps][TB_MAX_BEAM];              // (a) where a hypothesis at the piece's end stood at its start, its tokens
+  __shared__ int2 enter[kBtWarps][TB_MAX_BEAM];              // (b) which one a hypothesis of the last step was at the piece's end, tokens up to there
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = use_list ? sl.slot[blockIdx.x] : blockIdx.x;
   const int32_t pos = RING ? slot_pos[b] : n_steps;
   const int32_t first = RING ? max(0, pos - tree_cap) : 0;
-  const bool cut = RING && pos > tree_cap;
-  if (cut && lane == 0) atomicOr(status, TB_STATUS_STEP_LIMIT);   // the utterance is longer than the ring: its start is gone
-  const int64_t row = static_cast<int64_t>(blockIdx.x) * K + lane;
-  const int32_t* lens = RING ? (pos > 0 ? len_base + (((pos - 1) & 1) ? 0 : n_hyp) : nullptr) : len_cur;
-  const bool count_first = cut || (lens == nullptr && pos > 0);
-  int32_t n = 0;
-  if (!count_first && lane < K) {
-    n = lens ? lens[static_cast<int64_t>(b) * K + lane] : 0;
-    out_lens[row] = n;
-  }
-  // A stage is the nodes of up to kBtSteps consecutive steps, [step][K], brought in by asynchronous copies: 16 bytes
-  // (two nodes) each when K is even (a step's K nodes are contiguous and then start on a 16-byte boundary), else 8.
-  const bool wide = (K & 1) == 0 && (reinterpret_cast<uintptr_t>(tree) & 15) == 0;
-  const int per_step = wide ? K >> 1 : K;                    // copies per step
-  const uint32_t stage_a = static_cast<uint32_t>(__cvta_generic_to_shared(bt_stage));
-  const int n_stages = (pos - first + kBtSteps - 1) / kBtSteps;
-  const int ps_shift = (per_step & (per_step - 1)) == 0 ? 31 - __clz(per_step) : -1;   // copies per step a power of two: shifts
-  auto fetch = [&](int sidx) {                               // stage sidx holds steps [lo, hi), hi = pos - sidx * kBtSteps
-    if (sidx < n_stages) {
-      const int32_t hi = pos - sidx * kBtSteps, lo = max(first, hi - kBtSteps), cnt = hi - lo;
-      const uint32_t dst0 = stage_a + static_cast<uint32_t>(sidx % kBtBufs) * (kBtSteps * K * 8u);
-      const int32_t r0 = RING ? lo % tree_cap : 0;           // ring position of the stage's first step
-      const int2* base = RING ? tree + static_cast<int64_t>(b) * tree_cap * K : tree + static_cast<int64_t>(b) * K;
-      const int64_t step_stride = RING ? K : static_cast<int64_t>(B) * K;
-      const int total = cnt * per_step;
-      for (int e = lane; e < total; e += 32) {
-        const int j = ps_shift >= 0 ? e >> ps_shift : e / per_step;
-        const int c = e - j * per_step;
-        int32_t sj = RING ? r0 + j : lo + j;
-        if (RING && sj >= tree_cap) sj -= tree_cap;
-        const int2* src = base + sj * step_stride;
-        if (wide) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst0 + (j * K + 2 * c) * 8u), "l"(src + 2 * c) : "memory");
-        else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst0 + (j * K + c) * 8u), "l"(src + c) : "memory");
+  if (RING && pos > tree_cap && threadIdx.x == 0) atomicOr(status, TB_STATUS_STEP_LIMIT);   // the utterance is longer than the ring: its start is gone
+  const int32_t n = pos - first;
+  const int pieces = max(1, min(kBtWarps, n / kBtMin)), per = (n + pieces - 1) / pieces;
+  const int32_t lo = first + warp * per, hi = min(pos, lo + per);
+  const int2* base = RING ? tree + static_cast<int64_t>(b) * tree_cap * K : tree + static_cast<int64_t>(b) * K;
+  const int64_t stride = RING ? K : static_cast<int64_t>(B) * K;
+  const int spr = 32 / K, my_step = lane / K, my_k = lane - my_step * K;      // steps per register; this lane's node in it
+  const int64_t row = (static_cast<int64_t>(blockIdx.x) * K + lane) * max_len;
+  // from hypothesis `cur` after step hi - 1 back to before step lo; at: one past the last token's place
+  auto walk = [&](int& cur, int& at, bool write) {
+#pragma unroll 1
+    for (int32_t top = hi; top > lo; top -= kBtRegs * spr) {
+      int2 e[kBtRegs];
+#pragma unroll
+      for (int r = 0; r < kBtRegs; ++r) {                      // register r: steps top - (r + 1) * spr ... top - r * spr - 1
+        const int32_t sidx = top - (r + 1) * spr + my_step;
+        e[r] = make_int2(-1, -1);
+        if (my_step < spr && sidx >= lo) e[r] = __ldg(base + static_cast<int64_t>(RING ? sidx % tree_cap : sidx) * stride + my_k);
       }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");      // (one group per call, empty beyond the last stage)
-  };
-  for (int pass = count_first ? 0 : 1; pass < 2; ++pass) {
-    int32_t cur = lane < K ? lane : -1, at = n;
-    for (int sidx = 0; sidx < kBtBufs - 1; ++sidx) fetch(sidx);
-    for (int sidx = 0; sidx < n_stages; ++sidx) {
-      fetch(sidx + kBtBufs - 1);
-      asm volatile("cp.async.wait_group %0;" ::"n"(kBtBufs - 1) : "memory");
-      __syncwarp();
-      if (!__any_sync(0xffffffffu, cur >= 0 && (pass == 0 || at > 0))) break;
-      const int32_t hi = pos - sidx * kBtSteps, lo = max(first, hi - kBtSteps), cnt = hi - lo;
-      const int2* stg = bt_stage + static_cast<size_t>(sidx % kBtBufs) * (kBtSteps * K);
-      for (int j = cnt - 1; j >= 0 && cur >= 0; --j) {
-        const int2 e = stg[j * K + cur];
-        if (e.y >= 0 && e.y != V) {
-          if (pass == 0) ++n;
-          else { --at; if (at >= 0 && at < max_len) out_tokens[row * max_len + at] = e.y; }
+#pragma unroll
+      for (int r = 0; r < kBtRegs; ++r) {
+#pragma unroll 1
+        for (int j = spr - 1; j >= 0 && top - (r + 1) * spr + j >= lo; --j) {
+          const int from = j * K + max(cur, 0);
+          const int px = __shfl_sync(0xffffffffu, e[r].x, from), tk = __shfl_sync(0xffffffffu, e[r].y, from);
+          const bool tok = cur >= 0 && tk >= 0 && tk != V;
+          at -= tok ? 1 : 0;
+          if (write && tok && at < max_len) out_tokens[row + at] = tk;
+          cur = cur >= 0 ? px : -1;
         }
-        cur = e.x;
       }
-      __syncwarp();
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncwarp();
-    if (pass == 0 && lane < K) out_lens[row] = n;
+  };
+  int cur = lane < K ? lane : -1, at = 0;
+  if (warp < pieces) {
+    walk(cur, at, false);
+    piece[warp][lane] = make_int2(cur, -at);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    int total = 0, c = lane < K ? lane : -1;
+    for (int w = pieces - 1; w >= 0; --w) {
+      const int2 q = piece[w][max(c, 0)];
+      enter[w][lane] = make_int2(c, total);                    // (tokens after the piece, for now)
+      total += c >= 0 ? q.y : 0;
+      c = c >= 0 ? q.x : -1;
+    }
+    for (int w = 0; w < pieces; ++w) enter[w][lane].y = total - enter[w][lane].y;
+    if (lane < K) out_lens[static_cast<int64_t>(blockIdx.x) * K + lane] = total;
+  }
+  __syncthreads();
+  if (warp < pieces) {
+    const int2 q = enter[warp][lane];
+    cur = q.x; at = q.y;
+    walk(cur, at, true);
   }
 }
 
@@ -1595,11 +1591,10 @@ int tb_launch_beam_frames(const TbBeamParams& p_in, int32_t T, int32_t E, int64_
 }
 
 int tb_launch_beam_backtrace(const int2* tree, int32_t n_steps, int32_t B, int32_t K, int32_t V, int32_t max_len,
-                             int32_t* out_tokens, int32_t* out_lens, const int32_t* len_cur, cudaStream_t stream) {
+                             int32_t* out_tokens, int32_t* out_lens, cudaStream_t stream) {
   SlotList none;
-  for (int i = 0; i < TB_BIND_PAIRS; ++i) none.slot[i] = 0;
-  k_beam_backtrace_warp<false><<<B, 32, kBtBufs * kBtSteps * K * sizeof(int2), stream>>>(tree, 0, nullptr, n_steps, B, K, V, max_len, out_tokens,
-                                                                              out_lens, nullptr, nullptr, 0, len_cur, none, 0);
+  none.slot[0] = 0;
+  k_beam_backtrace<false><<<B, 32 * kBtWarps, 0, stream>>>(tree, 0, nullptr, n_steps, B, K, V, max_len, out_tokens, out_lens, nullptr, none, 0);
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
 
@@ -1765,14 +1760,13 @@ int tb_launch_beam_reset_slots(int32_t* slot_pos, unsigned long long* hash, int3
 
 int tb_launch_beam_backtrace_slots(const int2* tree, int32_t tree_cap, const int32_t* slot_pos, int32_t n_slots, int32_t K,
                                    int32_t V, int32_t max_len, int32_t* out_tokens, int32_t* out_lens, int32_t* status,
-                                   const int32_t* len_base, size_t n_hyp, const int32_t* slot_list, cudaStream_t stream) {
+                                   const int32_t* slot_list, cudaStream_t stream) {
   // slot_list (host, n_slots entries, at most TB_BIND_PAIRS): the slots to walk; null: slots 0 .. n_slots-1
   if (slot_list && n_slots > TB_BIND_PAIRS) return TB_ERR_INVALID_ARG;
   SlotList sl;
   for (int i = 0; i < TB_BIND_PAIRS; ++i) sl.slot[i] = (slot_list && i < n_slots) ? slot_list[i] : 0;
-  k_beam_backtrace_warp<true><<<n_slots, 32, kBtBufs * kBtSteps * K * sizeof(int2), stream>>>(tree, tree_cap, slot_pos, 0, n_slots, K, V, max_len,
-                                                                                   out_tokens, out_lens, status, len_base, n_hyp, nullptr,
-                                                                                   sl, slot_list ? 1 : 0);
+  k_beam_backtrace<true><<<n_slots, 32 * kBtWarps, 0, stream>>>(tree, tree_cap, slot_pos, 0, n_slots, K, V, max_len, out_tokens, out_lens, status, sl,
+                                                                slot_list ? 1 : 0);
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
 
