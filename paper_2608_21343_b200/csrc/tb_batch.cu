@@ -16,6 +16,7 @@ namespace {
 
 constexpr size_t kArenaAlign = 256;
 constexpr int kStagingRing = 4;
+constexpr int32_t kMaxListClasses = 65536;
 constexpr size_t kGroupBytes = 4u << 20;   // graphs a group bind packs into one copy (larger groups go in parts)
 
 struct DeviceGuard {  // makes the batch's device current for the duration of a call
@@ -277,6 +278,7 @@ struct tb_batch {
   TbSlotRec* d_slots = nullptr;
   TbSlotState* d_sstate = nullptr;
   int32_t* d_cls = nullptr;
+  int32_t* d_class_tok = nullptr;             // [n_classes + 1] ranges, then [vocab] the tokens of every class, ascending
   uint32_t flags = 0;
   int32_t* d_status = nullptr;
   int2* d_tree = nullptr;
@@ -327,10 +329,17 @@ struct tb_batch {
   int64_t n_pulled_binds = 0, n_copied_binds = 0;   // tb_stream_chunk_binds: binds carried out by the chunk's launch / ahead of it
 };
 
+static void query_device(tb_batch* b) {
+  if (b->n_sm != 0) return;
+  cudaDeviceGetAttribute(&b->n_sm, cudaDevAttrMultiProcessorCount, b->device);
+  cudaDeviceGetAttribute(&b->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device);
+  cudaGetLastError();
+}
+
 static void destroy_batch(tb_batch* b) {
   if (!b) return;
   cudaDeviceSynchronize();
-  cudaFree(b->arena); cudaFree(b->d_slots); cudaFree(b->d_sstate); cudaFree(b->d_cls);
+  cudaFree(b->arena); cudaFree(b->d_slots); cudaFree(b->d_sstate); cudaFree(b->d_cls); cudaFree(b->d_class_tok);
   cudaFree(b->d_status); cudaFree(b->d_tree); cudaFree(b->d_hyp_hash); cudaFree(b->d_hyp_len); cudaFree(b->d_model_recs); cudaFree(b->d_slot_pos);
   scratch_give(b->device, b->seg_scratch, b->seg_scratch_bytes); scratch_give(b->device, b->sg_scratch, b->sg_scratch_bytes);
   scratch_give(b->device, b->rows_scratch, b->rows_scratch_bytes); scratch_give(b->device, b->chunk_spill, b->chunk_spill_bytes);
@@ -381,6 +390,9 @@ extern "C" int tb_batch_create(int32_t vocab, const int32_t* case_class, int32_t
   ok = ok && cudaMalloc(&b->d_sstate, sizeof(TbSlotState) * n_slots) == cudaSuccess;
   ok = ok && cudaMalloc(&b->d_cls, sizeof(int32_t) * vocab) == cudaSuccess;
   ok = ok && cudaMalloc(&b->d_status, sizeof(int32_t)) == cudaSuccess;
+  // (no decode kernel has room for the tables of so many classes: such a batch derives no lists either)
+  const bool class_tok = n_classes <= kMaxListClasses;
+  if (class_tok) ok = ok && cudaMalloc(&b->d_class_tok, sizeof(int32_t) * (static_cast<size_t>(n_classes) + 1 + vocab)) == cudaSuccess;
   if (ok && max_tree_steps > 0)
     ok = cudaMalloc(&b->d_tree, sizeof(int2) * static_cast<size_t>(max_tree_steps) * n_slots * max_beam) == cudaSuccess;
   const size_t n_hyp = static_cast<size_t>(n_slots) * max_beam;
@@ -398,6 +410,14 @@ extern "C" int tb_batch_create(int32_t vocab, const int32_t* case_class, int32_t
   ok = ok && cudaMemcpy(b->d_sstate, init.data(), sizeof(TbSlotState) * n_slots, cudaMemcpyHostToDevice) == cudaSuccess;
   ok = ok && cudaMemcpy(b->d_cls, cls.data(), sizeof(int32_t) * vocab, cudaMemcpyHostToDevice) == cudaSuccess;
   ok = ok && cudaMemset(b->d_status, 0, sizeof(int32_t)) == cudaSuccess;
+  if (ok && class_tok) {
+    std::vector<int32_t> t(static_cast<size_t>(n_classes) + 1 + vocab, 0);
+    for (int32_t v = 0; v < vocab; ++v) t[cls[v] + 1]++;
+    for (int32_t c = 0; c < n_classes; ++c) t[c + 1] += t[c];
+    std::vector<int32_t> at(t.begin(), t.begin() + n_classes);
+    for (int32_t v = 0; v < vocab; ++v) t[n_classes + 1 + at[cls[v]]++] = v;
+    ok = cudaMemcpy(b->d_class_tok, t.data(), sizeof(int32_t) * t.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+  }
   for (auto& s : b->staging) ok = ok && cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) == cudaSuccess;
   if (!ok) { cudaGetLastError(); destroy_batch(b); return TB_ERR_CUDA; }
   tb_pinned_pool_arm();   // from now on this process keeps the images of the graphs it compiles in page-locked memory
@@ -412,7 +432,8 @@ extern "C" void tb_batch_destroy(tb_batch* b) {
 }
 
 // The slot record of graph g when its blob sits at byte offset `off` of the arena.
-static void fill_record(const tb_graph* g, size_t off, TbSlotRec* rec_out) {
+// lists_ready: the entries of its resolved lists are derived (resolve_lists) ahead of anything that reads the record.
+static void fill_record(const tb_graph* g, size_t off, int32_t lists_ready, TbSlotRec* rec_out) {
   TbSlotRec& rec = *rec_out;
   std::memset(&rec, 0, sizeof rec);
   rec.blob_off = static_cast<int64_t>(off);
@@ -420,9 +441,30 @@ static void fill_record(const tb_graph* g, size_t off, TbSlotRec* rec_out) {
   rec.off_arc_cls = g->off_arc_cls; rec.off_arc_w = g->off_arc_w; rec.off_arc_dst = g->off_arc_dst;
   rec.off_strec = g->off_strec; rec.off_tokent = g->off_tokent;
   rec.off_final = g->off_final;
-  rec.n_tokent = g->n_tokent; rec.blob_bytes = static_cast<int32_t>(g->blob.size());
+  rec.n_tokent = g->n_tokent; rec.blob_bytes = static_cast<int32_t>(g->arena_bytes());
   rec.off_rsrec = g->off_rsrec; rec.off_rsent = g->off_rsent; rec.n_rsent = g->n_rsent; rec.d_max = g->d_max;
   rec.n_states = g->n_states; rec.n_arcs = g->n_arcs; rec.max_depth = g->max_depth; rec.lambda = g->lambda;
+  rec.lists_ready = g->n_rsent == 0 ? 1 : lists_ready;
+}
+
+// Derives the entries of the resolved lists of graphs whose images and records (of `table`, at `at`) are on their way on
+// `stream`: one launch behind them.
+static int resolve_lists(tb_batch* b, TbSlotRec* table, int32_t n, const int32_t* at, const tb_graph* const* graphs, cudaStream_t stream) {
+  if (!b->d_class_tok) return TB_OK;
+  query_device(b);
+  for (int32_t i = 0; i < n;) {
+    int32_t idx[TB_BIND_PAIRS], m = 0, states = 0, depth = 0;
+    for (; i < n && m < TB_BIND_PAIRS; ++i) {
+      if (!graphs[i] || graphs[i]->n_rsent <= 0) continue;
+      idx[m++] = at[i];
+      states = graphs[i]->n_states > states ? graphs[i]->n_states : states;
+      depth = graphs[i]->max_depth > depth ? graphs[i]->max_depth : depth;
+    }
+    const int rc = tb_launch_resolve_lists(table, b->arena, m, idx, states, depth, b->d_class_tok, b->d_class_tok + b->n_classes + 1,
+                                           b->n_classes, b->vocab, b->n_sm, b->d_status, stream);
+    if (rc != TB_OK) return rc;
+  }
+  return TB_OK;
 }
 
 // Copies a graph's blob into a fresh arena block (through the pinned staging ring, on `stream`) and fills the
@@ -431,7 +473,7 @@ static int upload_graph(tb_batch* b, const tb_graph* g, cudaStream_t stream, siz
                         TbSlotRec* rec_out) {
   if (g->vocab != b->vocab || g->class_map_hash != b->class_map_hash) return TB_ERR_INVALID_ARG;
   size_t off = 0;
-  const size_t bytes = round_up(g->blob.size(), kArenaAlign);
+  const size_t bytes = round_up(g->arena_bytes(), kArenaAlign);
   if (!b->alloc.alloc(bytes, &off)) return TB_ERR_ARENA_FULL;
   // pinned staging: wait only if this ring entry's previous copy has not finished yet
   Staging& s = b->staging[b->next_staging];
@@ -460,14 +502,14 @@ static int upload_graph(tb_batch* b, const tb_graph* g, cudaStream_t stream, siz
     s.pending = ok;
   }
   if (!ok) { cudaGetLastError(); b->alloc.release(off, bytes); return TB_ERR_CUDA; }
-  fill_record(g, off, rec_out);
+  fill_record(g, off, 1, rec_out);
   *off_out = off; *bytes_out = bytes;
   return TB_OK;
 }
 
 // what the pipelined kernel caches in shared memory: the resolved lists, else the state records + token arcs
 static int32_t cache_bytes_of(const tb_graph* g) {
-  return static_cast<int32_t>(g->blob.size()) - (g->n_rsent >= 0 ? g->off_rsrec : g->off_strec);
+  return static_cast<int32_t>(g->arena_bytes()) - (g->n_rsent >= 0 ? g->off_rsrec : g->off_strec);
 }
 
 // The slot lets go of what it was bound to: its own block goes back to the free list (anything that reuses it is
@@ -481,13 +523,14 @@ static void release_slot(tb_batch* b, int32_t slot) {
   b->slot_model[slot] = -1;
 }
 
-static bool prepare_pulled_binds(tb_batch* b, int32_t n, const int32_t* slots, const tb_graph* const* graphs, cudaStream_t stream,
+static bool prepare_pulled_binds(tb_batch* b, int32_t n, const int32_t* slots, const tb_graph* const* graphs, int32_t lists_ready, cudaStream_t stream,
                                  TbInlineBinds* ib, Staging** used, std::vector<tb_graph*>* let_go);
+static void unbind_slots(tb_batch* b, int32_t n, const int32_t* slots, cudaStream_t stream);
 
 // Binds of up to TB_INLINE_BINDS graphs whose images lie in the page-locked pool, carried out by one launch that
 // reads the images in place (no copy is enqueued; the graphs are held until the launch's event).  False, with nothing
-// changed, when the group has to go the ordinary way.
-static bool bind_by_pull(tb_batch* b, int32_t n, const int32_t* slots, const tb_graph* const* graphs, cudaStream_t stream) {
+// changed, when the group has to go the ordinary way; else *rc_out is the result of the binds.
+static bool bind_by_pull(tb_batch* b, int32_t n, const int32_t* slots, const tb_graph* const* graphs, cudaStream_t stream, int* rc_out) {
   if (b->flags & TB_FLAG_COPIED_BINDS) return false;
   bool any = false;
   for (int32_t i = 0; i < n && graphs; ++i) any = any || graphs[i] != nullptr;
@@ -495,7 +538,7 @@ static bool bind_by_pull(tb_batch* b, int32_t n, const int32_t* slots, const tb_
   TbInlineBinds ib;
   Staging* used = nullptr;
   std::vector<tb_graph*> let_go;
-  if (!prepare_pulled_binds(b, n, slots, graphs, stream, &ib, &used, &let_go)) return false;
+  if (!prepare_pulled_binds(b, n, slots, graphs, 1, stream, &ib, &used, &let_go)) return false;
   int rc = tb_launch_pull_binds(ib, b->d_sstate, stream);
   if (rc == TB_OK && cudaEventRecord(used->done, stream) == cudaSuccess) used->pending = true;
   else { cudaGetLastError(); cudaStreamSynchronize(stream); }     // (no event, or no launch: nothing reads the graphs once this returns)
@@ -508,8 +551,20 @@ static bool bind_by_pull(tb_batch* b, int32_t n, const int32_t* slots, const tb_
     if (!ok) cudaGetLastError();
     cudaStreamSynchronize(stream);
   }
+  *rc_out = resolve_lists(b, b->d_slots, n, slots, graphs, stream);
+  if (*rc_out != TB_OK) unbind_slots(b, n, slots, stream);
   for (tb_graph* h : let_go) tb_graph_free(h);
   return true;
+}
+
+// Slots whose binds could not be completed are left unbound, on both sides.
+static void unbind_slots(tb_batch* b, int32_t n, const int32_t* slots, cudaStream_t stream) {
+  for (int32_t i = 0; i < n; ++i) {
+    release_slot(b, slots[i]);
+    b->slot_n_states[slots[i]] = 0; b->slot_cache_bytes[slots[i]] = 0; b->slot_resolved[slots[i]] = 1;
+    cudaMemsetAsync(b->d_slots + slots[i], 0, sizeof(TbSlotRec), stream);
+  }
+  cudaGetLastError();
 }
 
 extern "C" int tb_batch_bind_stream(tb_batch* b, int32_t slot, const tb_graph* g, void* stream_) {
@@ -519,22 +574,25 @@ extern "C" int tb_batch_bind_stream(tb_batch* b, int32_t slot, const tb_graph* g
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
   DeviceGuard guard(b->device);
   if (!guard.ok) return TB_ERR_CUDA;
-  if (g && bind_by_pull(b, 1, &slot, &g, stream)) return TB_OK;
+  int rc = TB_OK;
+  if (g && bind_by_pull(b, 1, &slot, &g, stream, &rc)) return rc;
   TbSlotRec rec;
   std::memset(&rec, 0, sizeof rec);
   size_t off = 0, bytes = 0;
   if (g) {
-    int rc = upload_graph(b, g, stream, &off, &bytes, &rec);
+    rc = upload_graph(b, g, stream, &off, &bytes, &rec);
     if (rc != TB_OK) return rc;
   }
-  int rc = tb_launch_publish_slot(b->d_slots, b->d_sstate, slot, rec, stream);
+  rc = tb_launch_publish_slot(b->d_slots, b->d_sstate, slot, rec, stream);
   if (rc != TB_OK) { if (bytes) b->alloc.release(off, bytes); return rc; }
   release_slot(b, slot);
   b->slot_block[slot] = {off, bytes};
   b->slot_n_states[slot] = g ? g->n_states : 0;
   b->slot_cache_bytes[slot] = !g ? 0 : cache_bytes_of(g);
   b->slot_resolved[slot] = (!g || g->n_rsent >= 0) ? 1 : 0;
-  return TB_OK;
+  rc = resolve_lists(b, b->d_slots, 1, &slot, &g, stream);
+  if (rc != TB_OK) unbind_slots(b, 1, &slot, stream);
+  return rc;
 }
 
 // Several slots at once (the streams that start between two chunks): the graphs go into ONE arena block, packed
@@ -557,8 +615,8 @@ extern "C" int tb_batch_bind_streams(tb_batch* b, int32_t n, const int32_t* slot
     const tb_graph* g = graphs[i];
     if (g && (g->vocab != b->vocab || g->class_map_hash != b->class_map_hash)) return TB_ERR_INVALID_ARG;
     if (g && first_part == n) {
-      if (total > 0 && total + g->blob.size() > kGroupBytes) first_part = i;
-      else total += round_up(g->blob.size(), kArenaAlign);
+      if (total > 0 && total + g->arena_bytes() > kGroupBytes) first_part = i;
+      else total += round_up(g->arena_bytes(), kArenaAlign);
     }
   }
   if (first_part < n) {
@@ -577,7 +635,9 @@ extern "C" int tb_batch_bind_streams(tb_batch* b, int32_t n, const int32_t* slot
     int32_t done = 0;
     while (done < n) {
       const int32_t m = n - done < TB_INLINE_BINDS ? n - done : TB_INLINE_BINDS;
-      if (!bind_by_pull(b, m, slots + done, graphs + done, stream)) break;
+      int rc = TB_OK;
+      if (!bind_by_pull(b, m, slots + done, graphs + done, stream, &rc)) break;
+      if (rc != TB_OK) return rc;
       done += m;
     }
     if (done == n) return TB_OK;
@@ -620,8 +680,8 @@ extern "C" int tb_batch_bind_streams(tb_batch* b, int32_t n, const int32_t* slot
   int32_t* slot_of = reinterpret_cast<int32_t*>(s.host + tail_off + static_cast<size_t>(n) * sizeof(TbSlotRec));
   std::vector<std::pair<size_t, size_t>> blocks(static_cast<size_t>(n), {0, 0});
   size_t at = 0;
-  // page-locked images that lie next to each other in host memory (graphs compiled one after the other sit side by
-  // side in the pool, at the spacing the arena uses) travel in one copy
+  // page-locked images that lie next to each other in host memory at the spacing the arena uses (graphs without resolved
+  // lists that were compiled one after the other) travel in one copy
   const unsigned char* run_src = nullptr;
   size_t run_at = 0, run_span = 0, run_bytes = 0;
   auto flush_run = [&]() {
@@ -638,7 +698,7 @@ extern "C" int tb_batch_bind_streams(tb_batch* b, int32_t n, const int32_t* slot
         run_src = g->blob.data(); run_at = at; run_span = 0;
       }
       run_bytes = run_span + g->blob.size();
-      run_span += round_up(g->blob.size(), kArenaAlign);
+      run_span += round_up(g->arena_bytes(), kArenaAlign);
       if (g->registered) flush_run();                                  // (registered memory ends with the image)
       tb_graph* h = const_cast<tb_graph*>(g); h->refs.fetch_add(1); s.held_more.push_back(h);
     } else {
@@ -647,8 +707,8 @@ extern "C" int tb_batch_bind_streams(tb_batch* b, int32_t n, const int32_t* slot
       if (any_pinned)   // (a mixed group: every staged graph is its own copy)
         ok = ok && cudaMemcpyAsync(b->arena + base + at, s.host + at, g->blob.size(), cudaMemcpyHostToDevice, stream) == cudaSuccess;
     }
-    fill_record(g, base + at, &recs[i]);
-    blocks[i] = {base + at, round_up(g->blob.size(), kArenaAlign)};
+    fill_record(g, base + at, 1, &recs[i]);
+    blocks[i] = {base + at, round_up(g->arena_bytes(), kArenaAlign)};
     at += blocks[i].second;
   }
   flush_run();
@@ -671,7 +731,9 @@ extern "C" int tb_batch_bind_streams(tb_batch* b, int32_t n, const int32_t* slot
     b->slot_cache_bytes[slots[i]] = !g ? 0 : cache_bytes_of(g);
     b->slot_resolved[slots[i]] = (!g || g->n_rsent >= 0) ? 1 : 0;
   }
-  return TB_OK;
+  rc = resolve_lists(b, b->d_slots, n, slots, graphs, stream);
+  if (rc != TB_OK) unbind_slots(b, n, slots, stream);
+  return rc;
 }
 
 // A group of binds prepared for the streaming chunk launch that follows to carry out itself (see TbInlineBinds): room in
@@ -681,7 +743,7 @@ extern "C" int tb_batch_bind_streams(tb_batch* b, int32_t n, const int32_t* slot
 // changed, when the group has to go the ordinary way (tb_batch_bind_streams, which also reports what is wrong with it).
 // *used: the staging entry that holds the graphs until the launch is done; the caller records its event after the
 // launch.  let_go: graphs of that entry's previous use, to be released after the launch has been issued.
-static bool prepare_pulled_binds(tb_batch* b, int32_t n, const int32_t* slots, const tb_graph* const* graphs, cudaStream_t stream,
+static bool prepare_pulled_binds(tb_batch* b, int32_t n, const int32_t* slots, const tb_graph* const* graphs, int32_t lists_ready, cudaStream_t stream,
                                  TbInlineBinds* ib, Staging** used, std::vector<tb_graph*>* let_go) {
   if (n < 1 || n > TB_INLINE_BINDS || !slots || !graphs) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -700,7 +762,7 @@ static bool prepare_pulled_binds(tb_batch* b, int32_t n, const int32_t* slots, c
     ib->src[i] = tb_pinned_device_ptr(g->blob.data());
     if (!ib->src[i]) return false;
     ib->bytes[i] = static_cast<int32_t>(g->blob.size());
-    total += round_up(g->blob.size(), kArenaAlign);
+    total += round_up(g->arena_bytes(), kArenaAlign);
   }
   size_t base = 0;
   if (total > 0 && !b->alloc.alloc(total, &base)) return false;
@@ -717,8 +779,8 @@ static bool prepare_pulled_binds(tb_batch* b, int32_t n, const int32_t* slots, c
     const tb_graph* g = graphs[i];
     std::pair<size_t, size_t> block{0, 0};
     if (g) {
-      fill_record(g, base + at, &ib->rec[i]);
-      block = {base + at, round_up(g->blob.size(), kArenaAlign)};
+      fill_record(g, base + at, lists_ready, &ib->rec[i]);
+      block = {base + at, round_up(g->arena_bytes(), kArenaAlign)};
       at += block.second;
       tb_graph* h = const_cast<tb_graph*>(g); h->refs.fetch_add(1); s.held_more.push_back(h);
     } else {
@@ -773,6 +835,7 @@ extern "C" int tb_batch_register_model(tb_batch* b, const tb_graph* g, int32_t* 
     b->d_model_recs = bigger; b->model_recs_cap = cap;
   }
   rc = tb_launch_publish_model(b->d_model_recs, id, m.rec, static_cast<cudaStream_t>(stream_));
+  if (rc == TB_OK) rc = resolve_lists(b, b->d_model_recs, 1, &id, &g, static_cast<cudaStream_t>(stream_));
   if (rc != TB_OK) { b->alloc.release(m.off, m.bytes); return rc; }
   b->models[id] = m;
   *out_model_id = id;
@@ -877,12 +940,6 @@ static bool is_capturing(cudaStream_t stream) {
   if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) { cudaGetLastError(); return false; }
   return cap != cudaStreamCaptureStatusNone;
 }
-static void query_device(tb_batch* b) {
-  if (b->n_sm != 0) return;
-  cudaDeviceGetAttribute(&b->n_sm, cudaDevAttrMultiProcessorCount, b->device);
-  cudaDeviceGetAttribute(&b->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device);
-  cudaGetLastError();
-}
 struct SlotSummary { int32_t max_cache = 0, max_states = 0, all_resolved = 1; };
 static SlotSummary slot_summary(const tb_batch* b, int32_t n) {
   SlotSummary r;
@@ -905,6 +962,7 @@ static int fill_decode_params(tb_batch* b, const void* logits, int dtype, int32_
   p->sb = strides[0]; p->st = strides[1]; p->ss = strides[2]; p->sv = strides[3];
   p->out_cap = frames * S;
   p->slots = b->d_slots; p->sstate = b->d_sstate; p->arena = b->arena; p->cls = b->d_cls; p->status = b->d_status;
+  p->class_tok = b->d_class_tok;
   return TB_OK;
 }
 
@@ -1041,8 +1099,10 @@ static int launch_chunk(tb_batch* b, const TbDecodeParams& p, cudaStream_t strea
   if (!(b->flags & TB_FLAG_GENERAL_KERNELS)) {
     query_device(b);
     const SlotSummary sl = slot_summary(b, p.n_streams);
-    if (p.n_streams <= b->n_sm) if (sl.all_resolved || grow_scratch(b, &b->chunk_spill, &b->chunk_spill_bytes, tb_chunk_rows_spill_bytes(p), is_capturing(stream))) {
-      const int rc = tb_launch_chunk_rows(p, sl.max_states, b->n_sm, b->max_smem, sl.all_resolved ? nullptr : b->chunk_spill, stream, binds);
+    // (the lists of graphs bound with this launch are derived behind it: until then they are put together by walking)
+    const bool walks = !sl.all_resolved || binds;
+    if (!walks || grow_scratch(b, &b->chunk_spill, &b->chunk_spill_bytes, tb_chunk_rows_spill_bytes(p), is_capturing(stream))) {
+      const int rc = tb_launch_chunk_rows(p, sl.max_states, b->n_sm, b->max_smem, walks ? b->chunk_spill : nullptr, stream, binds);
       if (rc != 1) return rc;
     }
   }
@@ -1086,21 +1146,14 @@ extern "C" int tb_stream_chunk_binds(tb_batch* b, int32_t n_binds, const int32_t
     Staging* used = nullptr;
     std::vector<tb_graph*> let_go;
     if (in_chunk && !(b->flags & TB_FLAG_COPIED_BINDS) &&
-        prepare_pulled_binds(b, n_binds, bind_slots, bind_graphs, stream, &ib, &used, &let_go)) {
+        prepare_pulled_binds(b, n_binds, bind_slots, bind_graphs, 0, stream, &ib, &used, &let_go)) {
       rc = launch_chunk(b, p, stream, &ib);
-      if (rc == TB_OK && cudaEventRecord(used->done, stream) == cudaSuccess) used->pending = true;
-      else if (rc == TB_OK) { cudaGetLastError(); cudaStreamSynchronize(stream); }   // (no event: the graphs are let go only after the launch is done)
-      if (rc != TB_OK) {
-        // the launch did not happen: the slots it would have bound are left unbound, on both sides
-        for (int32_t i = 0; i < n_binds; ++i) {
-          release_slot(b, bind_slots[i]);
-          b->slot_n_states[bind_slots[i]] = 0; b->slot_cache_bytes[bind_slots[i]] = 0; b->slot_resolved[bind_slots[i]] = 1;
-          cudaMemsetAsync(b->d_slots + bind_slots[i], 0, sizeof(TbSlotRec), stream);
-        }
-        cudaGetLastError();
-      } else {
-        b->n_pulled_binds += n_binds;
-      }
+      const bool launched = rc == TB_OK;
+      if (launched) rc = resolve_lists(b, b->d_slots, n_binds, bind_slots, bind_graphs, stream);
+      if (launched && cudaEventRecord(used->done, stream) == cudaSuccess) used->pending = true;
+      else if (launched) { cudaGetLastError(); cudaStreamSynchronize(stream); }   // (no event: the graphs are let go only after the launch is done)
+      if (rc != TB_OK) unbind_slots(b, n_binds, bind_slots, stream);
+      else b->n_pulled_binds += n_binds;
       for (tb_graph* h : let_go) tb_graph_free(h);
       return rc;
     }

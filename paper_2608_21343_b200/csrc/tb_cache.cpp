@@ -83,6 +83,11 @@ extern "C" int tb_graph_save(const tb_graph* g, const char* path) {
     put(payload, g->state_arc_begin); put(payload, g->arc_class); put(payload, g->arc_dst); put(payload, g->arc_w);
     put(payload, g->state_fail); put(payload, g->state_bw); put(payload, g->state_final); put(payload, g->state_depth);
     put(payload, g->case_class); put(payload, g->blob);
+    if (g->n_rsent >= 0) {                                   // (a file holds the lists' entries as well: see tb_graph::arena_bytes)
+      std::vector<TbRsEnt> ents(static_cast<size_t>(g->n_rsent) + 2);
+      tb_resolve_lists_host(g, ents.data());
+      put(payload, ents);
+    }
     FileHeader h;
     std::memset(&h, 0, sizeof h);
     h.magic = kMagic; h.version = kVersion;
@@ -91,7 +96,7 @@ extern "C" int tb_graph_save(const tb_graph* g, const char* path) {
     h.off_arc_begin = g->off_arc_begin; h.off_fail = g->off_fail; h.off_bw = g->off_bw; h.off_arc_cls = g->off_arc_cls;
     h.off_arc_w = g->off_arc_w; h.off_arc_dst = g->off_arc_dst; h.off_strec = g->off_strec; h.off_tokent = g->off_tokent;
     h.n_tokent = g->n_tokent; h.off_rsrec = g->off_rsrec; h.off_rsent = g->off_rsent; h.n_rsent = g->n_rsent;
-    h.d_max = g->d_max; h.off_final = g->off_final; h.blob_bytes = g->blob.size();
+    h.d_max = g->d_max; h.off_final = g->off_final; h.blob_bytes = g->arena_bytes();
     h.payload_hash = 0;
     h.payload_hash = file_hash(h, payload);                  // header (with this field zero) and payload together
     std::FILE* f = std::fopen(path, "wb");
@@ -212,6 +217,11 @@ extern "C" int tb_graph_load(const char* path, tb_graph** out) {
       if (!in) { delete g; return TB_ERR_INVALID_ARG; }
     }
     if (g->class_map_hash != tb_hash_class_map(g->case_class.data(), g->vocab)) { delete g; return TB_ERR_INVALID_ARG; }
+    if (g->n_rsent >= 0) {                                   // the device derives the entries after a bind: the image ends before them
+      if (g->off_rsent != g->off_rsrec + 16 * g->n_states) { delete g; return TB_ERR_INVALID_ARG; }
+      TbImage image(g->blob.begin(), g->blob.begin() + g->off_rsent);
+      g->blob.swap(image);
+    }
     g->pinned = tb_pinned_owns(g->blob.data());
     *out = g;
     return TB_OK;

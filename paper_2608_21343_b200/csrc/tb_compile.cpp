@@ -17,21 +17,7 @@
 
 namespace {
 
-struct Folded {
-  const int32_t* tok;  // into the caller's array
-  const float* w;      // may be null
-  int32_t len;
-};
-
 inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
-
-template <typename T>
-int32_t append_section(std::vector<unsigned char>& blob, const std::vector<T>& v) {
-  size_t off = align16(blob.size());
-  blob.resize(off + v.size() * sizeof(T));
-  if (!v.empty()) std::memcpy(blob.data() + off, v.data(), v.size() * sizeof(T));
-  return static_cast<int32_t>(off);
-}
 
 }  // namespace
 
@@ -65,103 +51,143 @@ struct PoolBypass {
   ~PoolBypass() { if (on) tb_pinned_bypass(false); }
 };
 
-// What every front end shares: from the flat arc / state arrays to the device blob (Sec. 2.2 para. 2), with the
-// per-state records, token-expanded arcs and resolved lists the kernels read.
-static void finalize_graph(tb_graph* g, const int32_t* case_class, int32_t vocab, int32_t n_classes, float lambda) {
-  const int32_t N = g->n_states;
+// The image of a graph for the device: the flat arrays (Sec. 2.2 para. 2), then one of two derived forms.  Graphs whose
+// resolved lists (see TbRsRec) stay small carry the lists' records only -- where each state's list begins and how long it is,
+// found here by counting; the entries themselves, four fifths of what such a graph takes in the arena, are derived on the
+// device from the flat arrays after the bind (k_resolve_lists), so they are neither put together, sorted and held here nor
+// moved across the bus (275 phrases: 0.35 ms and 193 KB an image with the entries, 0.06 ms and 34 KB without).  Larger graphs
+// carry per-state records and token-expanded arcs instead, which the kernels walk.
+// `tree`: the arcs are those of a tree of single-class steps (tb_graph_compile), for which a list's length follows from its
+// suffix state's: an own arc shadows an inherited one exactly when the arc's target has a suffix of two classes or more.
+static void finalize_graph(tb_graph* g, const int32_t* case_class, int32_t vocab, int32_t n_classes, float lambda, bool tree) {
+  const int32_t N = g->n_states, A = g->n_arcs;
   g->case_class.resize(vocab);
   for (int32_t v = 0; v < vocab; ++v) g->case_class[v] = case_class ? case_class[v] : v;
   g->class_map_hash = tb_hash_class_map(case_class, vocab);
 
-  // ---- device blob ---------------------------------------------------------------------------
-  std::vector<unsigned char> blob;   // built here, then moved into its final place in one piece
-  g->off_arc_begin = append_section(blob, g->state_arc_begin);
-  g->off_fail = append_section(blob, g->state_fail);
-  g->off_bw = append_section(blob, g->state_bw);
-  g->off_arc_cls = append_section(blob, g->arc_class);
-  g->off_arc_w = append_section(blob, g->arc_w);
-  g->off_arc_dst = append_section(blob, g->arc_dst);
-  g->off_final = append_section(blob, g->state_final);
-  {  // the tokens of every class, in ascending id order
-    std::vector<int32_t> ctb(n_classes + 1, 0), ctk(vocab);
-    for (int32_t v = 0; v < vocab; ++v) ctb[g->case_class[v] + 1]++;
-    for (int32_t c = 0; c < n_classes; ++c) ctb[c + 1] += ctb[c];
+  std::vector<int32_t> csize(n_classes, 0);    // tokens of every class
+  for (int32_t v = 0; v < vocab; ++v) csize[g->case_class[v]]++;
+  float root_w_max = 0.0f;
+  for (int32_t a = g->state_arc_begin[0]; a < g->state_arc_begin[1]; ++a) root_w_max = std::max(root_w_max, std::fabs(g->arc_w[a]));
+  std::vector<TbRsRec> rrecs(N);
+  std::vector<int32_t> count(N, 0);
+  std::vector<int32_t> seen;                   // class -> state that listed it during the current walk
+  if (!tree) seen.assign(n_classes, -1);
+  bool fits = N < (1 << (32 - tb_rs_tok_bits(vocab)));
+  int64_t total = 0;
+  g->d_max = 0.0f;
+  for (int32_t s = 0; s < N; ++s) {
+    float acc = 0.0f;
+    int32_t c = 0;
+    if (tree && s) {
+      c = count[g->state_fail[s]];
+      for (int32_t a = g->state_arc_begin[s]; a < g->state_arc_begin[s + 1]; ++a)
+        if (g->state_depth[g->state_fail[g->arc_dst[a]]] < 2) c += csize[g->arc_class[a]];
+    }
+    for (int32_t u = s; u != 0; u = g->state_fail[u]) {
+      if (!tree && fits)
+        for (int32_t a = g->state_arc_begin[u]; a < g->state_arc_begin[u + 1]; ++a)
+          if (seen[g->arc_class[a]] != s) { seen[g->arc_class[a]] = s; c += csize[g->arc_class[a]]; }   // (else shadowed by a chain state closer to s)
+      acc = acc + g->state_bw[u];
+    }
+    count[s] = c;
+    g->d_max = std::max(g->d_max, std::fabs(acc));
+    const int32_t padded = (c + 3) & ~3;       // sentinels: the blank column with lb = -inf
+    rrecs[s] = {static_cast<int32_t>(total), padded, acc, std::fabs(lambda) * (std::fabs(acc) + root_w_max)};
+    if (fits) total += padded;
+    if (total > TB_RS_MAX_ENTRIES) fits = false;
+  }
+
+  std::vector<TbStateRec> recs;
+  std::vector<TbTokEnt> ents;
+  if (!fits) {
+    std::vector<int32_t> ctb(n_classes + 1, 0), ctk(vocab);   // the tokens of every class, in ascending id order
+    for (int32_t c = 0; c < n_classes; ++c) ctb[c + 1] = ctb[c] + csize[c];
     std::vector<int32_t> fill(ctb.begin(), ctb.end() - 1);
     for (int32_t v = 0; v < vocab; ++v) ctk[fill[g->case_class[v]]++] = v;
-
-    // resolved lists (see TbRsRec): the walk the kernels would do, done once here in float
-    float root_w_max = 0.0f;
-    for (int32_t a = g->state_arc_begin[0]; a < g->state_arc_begin[1]; ++a) root_w_max = std::max(root_w_max, std::fabs(g->arc_w[a]));
-    std::vector<TbRsRec> rrecs(N);
-    std::vector<TbRsEnt> rents;
-    std::vector<int32_t> seen(n_classes, -1);   // class -> state that listed it during the current walk
-    const int tb = tb_rs_tok_bits(vocab);
-    bool fits = N < (1 << (32 - tb));
-    g->d_max = 0.0f;
-    for (int32_t s = 0; s < N; ++s) {
-      float acc = 0.0f;
-      const size_t first = rents.size();
-      for (int32_t u = s; u != 0; u = g->state_fail[u]) {
-        if (fits) {
-          for (int32_t a = g->state_arc_begin[u]; a < g->state_arc_begin[u + 1]; ++a) {
-            const int32_t c = g->arc_class[a];
-            if (seen[c] == s) continue;           // shadowed by a chain state closer to s
-            seen[c] = s;
-            const float bonus = acc + g->arc_w[a];
-            const float lb = lambda * bonus;
-            for (int32_t j = ctb[c]; j < ctb[c + 1]; ++j)
-              rents.push_back({(static_cast<uint32_t>(g->arc_dst[a]) << tb) | static_cast<uint32_t>(2 * ctk[j]), lb});
-          }
-          if (rents.size() > TB_RS_MAX_ENTRIES) fits = false;
-        }
-        acc = acc + g->state_bw[u];
+    recs.resize(N);
+    for (int32_t u = 0; u < N; ++u) {
+      recs[u].tok_begin = static_cast<int32_t>(ents.size());
+      for (int32_t a = g->state_arc_begin[u]; a < g->state_arc_begin[u + 1]; ++a) {
+        const int32_t c = g->arc_class[a];
+        for (int32_t j = ctb[c]; j < ctb[c + 1]; ++j)
+          ents.push_back({static_cast<uint32_t>(ctk[j]) | (static_cast<uint32_t>(c) << 16), g->arc_w[a], g->arc_dst[a], 0});
       }
-      g->d_max = std::max(g->d_max, std::fabs(acc));
-      if (fits) {
-        std::sort(rents.begin() + first, rents.end(), [tb](const TbRsEnt& x, const TbRsEnt& y) {
-          return (x.dst_tok & ((1u << tb) - 1)) < (y.dst_tok & ((1u << tb) - 1));
-        });
-        while ((rents.size() - first) % 4 != 0)   // sentinels: the blank column with lb = -inf
-          rents.push_back({static_cast<uint32_t>(2 * vocab), -std::numeric_limits<float>::infinity()});
-      }
-      rrecs[s].begin = static_cast<int32_t>(first);
-      rrecs[s].count = static_cast<int32_t>(rents.size() - first);
-      rrecs[s].D = acc;
-      rrecs[s].bmag = std::fabs(lambda) * (std::fabs(acc) + root_w_max);
-    }
-    if (fits) {
-      // (the kernels read these lists and nothing else beyond the flat arrays: the image carries no per-state records)
-      g->off_strec = g->off_tokent = 0;
-      g->n_tokent = 0;
-      g->off_rsrec = append_section(blob, rrecs);
-      g->off_rsent = append_section(blob, rents);
-      g->n_rsent = static_cast<int32_t>(rents.size());
-    } else {
-      // too large for resolved lists: per-state records and token-expanded arcs, which the kernels walk instead
-      std::vector<TbStateRec> recs(N);
-      std::vector<TbTokEnt> ents;
-      for (int32_t u = 0; u < N; ++u) {
-        recs[u].tok_begin = static_cast<int32_t>(ents.size());
-        for (int32_t a = g->state_arc_begin[u]; a < g->state_arc_begin[u + 1]; ++a) {
-          const int32_t c = g->arc_class[a];
-          for (int32_t j = ctb[c]; j < ctb[c + 1]; ++j)
-            ents.push_back({static_cast<uint32_t>(ctk[j]) | (static_cast<uint32_t>(c) << 16), g->arc_w[a], g->arc_dst[a], 0});
-        }
-        recs[u].tok_end = static_cast<int32_t>(ents.size());
-        recs[u].fail = g->state_fail[u];
-        recs[u].bw = g->state_bw[u];
-      }
-      g->off_strec = append_section(blob, recs);
-      g->off_tokent = append_section(blob, ents);
-      g->n_tokent = static_cast<int32_t>(ents.size());
-      g->off_rsrec = g->off_rsent = 0;
-      g->n_rsent = -1;
+      recs[u].tok_end = static_cast<int32_t>(ents.size());
+      recs[u].fail = g->state_fail[u];
+      recs[u].bw = g->state_bw[u];
     }
   }
-  blob.resize(align16(blob.size()) + 16);  // tail padding so vector loads may overrun a section
+  // ---- the image, filled in place
+  size_t size = 0;
+  auto section = [&](size_t bytes) { const size_t off = align16(size); size = off + bytes; return static_cast<int32_t>(off); };
+  g->off_arc_begin = section(4 * (static_cast<size_t>(N) + 1));
+  g->off_fail = section(4 * static_cast<size_t>(N));
+  g->off_bw = section(4 * static_cast<size_t>(N));
+  g->off_arc_cls = section(4 * static_cast<size_t>(A));
+  g->off_arc_w = section(4 * static_cast<size_t>(A));
+  g->off_arc_dst = section(4 * static_cast<size_t>(A));
+  g->off_final = section(4 * static_cast<size_t>(N));
+  g->off_strec = g->off_tokent = g->n_tokent = g->off_rsrec = g->off_rsent = 0;
+  if (fits) {
+    g->off_rsrec = section(16 * static_cast<size_t>(N));
+    g->off_rsent = static_cast<int32_t>(size);         // (behind the image: reserved in the arena, filled on the device)
+    g->n_rsent = static_cast<int32_t>(total);
+  } else {
+    g->off_strec = section(16 * static_cast<size_t>(N));
+    g->off_tokent = section(16 * ents.size());
+    g->n_tokent = static_cast<int32_t>(ents.size());
+    g->n_rsent = -1;
+    size = align16(size) + 16;                         // tail padding so vector loads may overrun a section
+  }
   g->blob = TbImage();
-  g->blob.assign(blob.begin(), blob.end());
-  g->pinned = tb_pinned_owns(g->blob.data());
+  g->blob.resize(size);
+  unsigned char* d = g->blob.data();
+  auto put = [&](int32_t off, const void* src, size_t bytes) { if (bytes) std::memcpy(d + off, src, bytes); };
+  put(g->off_arc_begin, g->state_arc_begin.data(), 4 * (static_cast<size_t>(N) + 1));
+  put(g->off_fail, g->state_fail.data(), 4 * static_cast<size_t>(N));
+  put(g->off_bw, g->state_bw.data(), 4 * static_cast<size_t>(N));
+  put(g->off_arc_cls, g->arc_class.data(), 4 * static_cast<size_t>(A));
+  put(g->off_arc_w, g->arc_w.data(), 4 * static_cast<size_t>(A));
+  put(g->off_arc_dst, g->arc_dst.data(), 4 * static_cast<size_t>(A));
+  put(g->off_final, g->state_final.data(), 4 * static_cast<size_t>(N));
+  if (fits) put(g->off_rsrec, rrecs.data(), 16 * static_cast<size_t>(N));
+  else { put(g->off_strec, recs.data(), 16 * static_cast<size_t>(N)); put(g->off_tokent, ents.data(), 16 * ents.size()); }
+  g->pinned = tb_pinned_owns(d);
+}
+
+void tb_resolve_lists_host(const tb_graph* g, TbRsEnt* out) {
+  const int32_t N = g->n_states, vocab = g->vocab, n_classes = g->n_classes;
+  const int tb = tb_rs_tok_bits(vocab);
+  std::vector<int32_t> ctb(n_classes + 1, 0), ctk(vocab), seen(n_classes, -1);
+  for (int32_t v = 0; v < vocab; ++v) ctb[g->case_class[v] + 1]++;
+  for (int32_t c = 0; c < n_classes; ++c) ctb[c + 1] += ctb[c];
+  std::vector<int32_t> fill(ctb.begin(), ctb.end() - 1);
+  for (int32_t v = 0; v < vocab; ++v) ctk[fill[g->case_class[v]]++] = v;
+  std::vector<TbRsEnt> list;
+  for (int32_t s = 0; s < N; ++s) {
+    TbRsRec r;
+    std::memcpy(&r, g->blob.data() + g->off_rsrec + 16 * static_cast<size_t>(s), 16);
+    list.clear();
+    float acc = 0.0f;
+    for (int32_t u = s; u != 0; u = g->state_fail[u]) {
+      for (int32_t a = g->state_arc_begin[u]; a < g->state_arc_begin[u + 1]; ++a) {
+        const int32_t c = g->arc_class[a];
+        if (seen[c] == s) continue;           // shadowed by a chain state closer to s
+        seen[c] = s;
+        const float bonus = acc + g->arc_w[a];
+        const float lb = g->lambda * bonus;
+        for (int32_t j = ctb[c]; j < ctb[c + 1]; ++j)
+          list.push_back({(static_cast<uint32_t>(g->arc_dst[a]) << tb) | static_cast<uint32_t>(2 * ctk[j]), lb});
+      }
+      acc = acc + g->state_bw[u];
+    }
+    std::sort(list.begin(), list.end(), [tb](const TbRsEnt& x, const TbRsEnt& y) {
+      return (x.dst_tok & ((1u << tb) - 1)) < (y.dst_tok & ((1u << tb) - 1));
+    });
+    for (int32_t i = 0; i < r.count; ++i)
+      out[r.begin + i] = i < static_cast<int32_t>(list.size()) ? list[i] : TbRsEnt{static_cast<uint32_t>(2 * vocab), -std::numeric_limits<float>::infinity()};
+  }
 }
 
 static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offsets, int32_t n_phrases,
@@ -177,45 +203,53 @@ static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offs
     }
   }
   if (n_phrases > 0 && phrase_offsets[0] != 0) return TB_ERR_INVALID_ARG;
+  // folded phrases back to back: the classes of every token, and a sort key of the first four
+  struct Folded {
+    uint64_t key;
+    const int32_t* cls;  // [len]
+    const float* w;      // may be null
+    int32_t len;
+  };
+  if (n_phrases > 0 && (phrase_offsets[n_phrases] < 0 || phrase_offsets[n_phrases] > static_cast<int64_t>(n_phrases) * TB_MAX_PHRASE_LEN)) return TB_ERR_INVALID_ARG;
+  std::vector<int32_t> folded(n_phrases > 0 ? static_cast<size_t>(phrase_offsets[n_phrases]) : 0);
   std::vector<Folded> ph;
   ph.reserve(n_phrases);
   int32_t max_len = 0;
   for (int32_t p = 0; p < n_phrases; ++p) {
     int64_t b = phrase_offsets[p], e = phrase_offsets[p + 1];
-    if (e < b) return TB_ERR_INVALID_ARG;
+    if (e < b || e > static_cast<int64_t>(folded.size())) return TB_ERR_INVALID_ARG;
     if (e - b > TB_MAX_PHRASE_LEN) return TB_ERR_INVALID_ARG;
+    uint64_t key = 0;
     for (int64_t i = b; i < e; ++i) {
       if (phrase_tokens[i] < 0 || phrase_tokens[i] >= vocab) return TB_ERR_INVALID_ARG;
       if (token_weights && !(std::isfinite(token_weights[i]) && token_weights[i] >= 0.0f)) return TB_ERR_INVALID_ARG;
+      const int32_t c = case_class ? case_class[phrase_tokens[i]] : phrase_tokens[i];
+      folded[i] = c;
+      if (i < b + 4) key |= static_cast<uint64_t>(std::min(c, 0xFFFE) + 1) << (48 - 16 * (i - b));
     }
     if (e == b) continue;  // empty phrases are skipped
-    ph.push_back({phrase_tokens + b, token_weights ? token_weights + b : nullptr, static_cast<int32_t>(e - b)});
+    ph.push_back({key, folded.data() + b, token_weights ? token_weights + b : nullptr, static_cast<int32_t>(e - b)});
     max_len = std::max(max_len, static_cast<int32_t>(e - b));
   }
-  auto cls_of = [&](int32_t tok) { return case_class ? case_class[tok] : tok; };
 
   // ---- sort the folded phrases, longest-common-prefix with the predecessor -----------------
   const size_t P = ph.size();
-  std::vector<uint32_t> order(P);
-  std::iota(order.begin(), order.end(), 0u);
-  std::sort(order.begin(), order.end(), [&](uint32_t a, uint32_t b) {
-    const Folded &x = ph[a], &y = ph[b];
-    int32_t n = std::min(x.len, y.len);
-    for (int32_t i = 0; i < n; ++i) {
-      int32_t cx = cls_of(x.tok[i]), cy = cls_of(y.tok[i]);
-      if (cx != cy) return cx < cy;
-    }
+  std::sort(ph.begin(), ph.end(), [](const Folded& x, const Folded& y) {
+    if (x.key != y.key) return x.key < y.key;
+    const int32_t n = std::min(x.len, y.len);
+    for (int32_t i = 0; i < n; ++i)
+      if (x.cls[i] != y.cls[i]) return x.cls[i] < y.cls[i];
     return x.len < y.len;
   });
   std::vector<int32_t> lcp(P, 0);
   std::vector<size_t> node_base(P + 1, 0);  // where phrase i's node ids start in `node_of`
   for (size_t i = 0; i < P; ++i) {
-    const Folded& x = ph[order[i]];
+    const Folded& x = ph[i];
     node_base[i + 1] = node_base[i] + x.len;
     if (i == 0) continue;
-    const Folded& y = ph[order[i - 1]];
+    const Folded& y = ph[i - 1];
     int32_t n = std::min(x.len, y.len), l = 0;
-    while (l < n && cls_of(x.tok[l]) == cls_of(y.tok[l])) ++l;
+    while (l < n && x.cls[l] == y.cls[l]) ++l;
     lcp[i] = l;
   }
 
@@ -224,9 +258,10 @@ static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offs
   std::vector<int32_t> parent(1, -1), cls(1, -1);
   std::vector<uint8_t> depth(1, 0), is_end(1, 0);
   std::vector<double> wt(1, 0.0);
+  parent.reserve(node_base[P] + 1); cls.reserve(node_base[P] + 1); depth.reserve(node_base[P] + 1); is_end.reserve(node_base[P] + 1); wt.reserve(node_base[P] + 1);
   for (int32_t d = 1; d <= max_len; ++d) {
     for (size_t i = 0; i < P; ++i) {
-      const Folded& x = ph[order[i]];
+      const Folded& x = ph[i];
       if (x.len < d) continue;
       double w = x.w ? static_cast<double>(x.w[d - 1]) : 1.0;
       int32_t id;
@@ -236,7 +271,7 @@ static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offs
       } else {
         id = static_cast<int32_t>(parent.size());
         parent.push_back(d == 1 ? 0 : node_of[node_base[i] + d - 2]);
-        cls.push_back(cls_of(x.tok[d - 1]));
+        cls.push_back(x.cls[d - 1]);
         depth.push_back(static_cast<uint8_t>(d));
         is_end.push_back(0);
         wt.push_back(w);
@@ -262,11 +297,15 @@ static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offs
   }
   for (int32_t u = 0; u < N; ++u) g->state_arc_begin[u + 1] += g->state_arc_begin[u];
 
+  std::vector<int32_t> root_arc(n_classes, -1);
+  for (int32_t a = 0; a < g->state_arc_begin[1]; ++a) root_arc[g->arc_class[a]] = a;
   auto find_arc = [&](int32_t u, int32_t c) -> int32_t {
+    if (u == 0) return root_arc[c];
     const int32_t* b = g->arc_class.data() + g->state_arc_begin[u];
     const int32_t* e = g->arc_class.data() + g->state_arc_begin[u + 1];
-    const int32_t* it = std::lower_bound(b, e, c);
-    return (it != e && *it == c) ? static_cast<int32_t>(it - g->arc_class.data()) : -1;
+    if (e - b > 16) b = std::lower_bound(b, e, c);
+    else while (b != e && *b < c) ++b;
+    return (b != e && *b == c) ? static_cast<int32_t>(b - g->arc_class.data()) : -1;
   };
 
   // ---- suffix links (ids ascend breadth-first, so the parent's link is ready) ---------------
@@ -300,7 +339,7 @@ static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offs
       g->arc_w[id - 1] = static_cast<float>(loan[id] - loan[parent[id]] + outp[id]);
     }
   }
-  finalize_graph(g, case_class, vocab, n_classes, lambda);
+  finalize_graph(g, case_class, vocab, n_classes, lambda, true);
   return TB_OK;
 }
 
@@ -517,7 +556,7 @@ int compile_variative_impl(const uint8_t* phrase_chars, const int64_t* phrase_of
     g->state_final[id] = static_cast<float>(-loan[id]);
     if (id) g->state_bw[id] = static_cast<float>(loan[fail[id]] - loan[id]);
   }
-  finalize_graph(g, cls.data(), vocab, n_classes, lambda);
+  finalize_graph(g, cls.data(), vocab, n_classes, lambda, false);
   return TB_OK;
 }
 

@@ -146,7 +146,8 @@ __global__ void __launch_bounds__(kThreads) k_decode_general(TbDecodeParams p, T
   const bool bound = rec.n_states > 0;
   const GraphPtrs g = graph_of(p.arena, rec);
   const unsigned char* blob = p.arena + rec.blob_off;
-  const bool use_tv = bound && rec.n_rsent >= 0 && p.tokview;   // resolved lists: token view instead of a chain walk
+  // resolved lists: token view instead of a chain walk (a graph bound with this launch has its lists derived behind it)
+  const bool use_tv = bound && rec.n_rsent >= 0 && rec.lists_ready && p.tokview;
   TokView tv;
   if (use_tv) tokview_init(tv, dyn, p.V, p.C, g);
   const LT* base = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(b) * p.sb;

@@ -70,6 +70,9 @@ struct tb_graph {
   std::atomic<int32_t> refs{1};                        // holders: the caller's handle, one per cache that keeps the graph, one per copy in flight
   bool pinned = false;                                 // the blob's pages are locked (it sits in the pool, or tb_graph_pin registered it): binds copy straight from it
   bool registered = false;                             // ... by tb_graph_pin: to be unregistered
+  // bytes the graph takes in the arena: the image and, behind it, room for the entries of the resolved lists (which the
+  // device fills; 16 bytes more so that vector loads may overrun)
+  size_t arena_bytes() const { return blob.size() + (n_rsent >= 0 ? 8 * static_cast<size_t>(n_rsent) + 16 : 0); }
   ~tb_graph();
 };
 
@@ -77,6 +80,10 @@ struct tb_graph {
 // page-locked pool already, so that a bind can hand it to the copy engine directly instead of going through the
 // staging ring.  Does nothing without a device.
 void tb_graph_pin(tb_graph* g);
+
+// The entries of g's resolved lists (n_rsent of them), as the device derives them; for files (tb_graph_save).
+struct TbRsEnt;
+void tb_resolve_lists_host(const tb_graph* g, TbRsEnt* out);
 
 // Two derived sections of the blob serve the pipelined kernel.  TbStateRec packs what a
 // suffix-link walk needs from one state into one 16-byte load; TbTokEnt lists, per state, its
@@ -133,11 +140,12 @@ struct TbSlotRec {
   int32_t off_arc_begin, off_fail, off_bw, off_arc_cls, off_arc_w, off_arc_dst, off_strec, off_tokent;  // within the blob
   int32_t n_states, n_arcs, max_depth;
   float lambda;
-  int32_t n_tokent, blob_bytes;
+  int32_t n_tokent, blob_bytes;   // (blob_bytes: with the lists' entries, tb_graph::arena_bytes)
   int32_t off_rsrec, off_rsent, n_rsent;  // resolved lists; n_rsent < 0: the graph has none
   float d_max;
   int32_t off_final;   // per-state final weights (within the blob)
-  int32_t pad[11];
+  int32_t lists_ready; // the entries of the resolved lists have been derived (k_resolve_lists)
+  int32_t pad[10];
 };
 static_assert(sizeof(TbSlotRec) == 128, "slot record is 128 bytes");
 

@@ -21,6 +21,7 @@ struct TbDecodeParams {
   int32_t out_cap;           // tokens per stream the output arrays can hold
   const TbSlotRec* slots; TbSlotState* sstate; const unsigned char* arena;
   const int32_t* cls;        // device [V] token -> class
+  const int32_t* class_tok;  // device [C + 1] ranges, [V] the tokens of every class (null: more classes than any kernel has room for)
   int32_t* status;
 };
 
@@ -73,6 +74,12 @@ struct TbInlineBinds {
   TbSlotRec rec[TB_INLINE_BINDS];
 };
 
+// Derives the resolved lists of n <= TB_BIND_PAIRS graphs, whose records are recs[at[i]], from their images in the arena
+// and marks the records (lists_ready).  max_states / max_depth: the largest among them; ctb [C + 1], ctk [V]: the tokens of
+// every class; n_sm: multiprocessors of the device.
+int tb_launch_resolve_lists(TbSlotRec* recs, unsigned char* arena, int32_t n, const int32_t* at, int32_t max_states, int32_t max_depth,
+                            const int32_t* ctb, const int32_t* ctk, int32_t C, int32_t V, int32_t n_sm, int32_t* status,
+                            cudaStream_t stream);
 int tb_launch_decode_general(const TbDecodeParams& p, cudaStream_t stream, const TbInlineBinds* binds = nullptr);
 // The same binds carried out by a launch of their own (tb_batch_bind_stream(s) for graphs in the page-locked pool).
 int tb_launch_pull_binds(const TbInlineBinds& binds, TbSlotState* sstate, cudaStream_t stream);

@@ -1,0 +1,161 @@
+// The resolved lists of freshly bound graphs (see TbRsRec), derived on the device from the flat arrays their images carry.
+#include "tb_device.cuh"
+#include "tb_launch.h"
+
+namespace {
+
+constexpr int kListWarps = 8;
+
+struct ListSlots { int32_t at[TB_BIND_PAIRS]; };
+
+// shared memory of one warp: bits of the tokens the list holds and of the classes written so far, entries before every word
+// of the first, then per chain state its weights crossed so far, its first arc and the arcs before it
+__host__ __device__ inline int list_words(int V) { return (V + 31) >> 5; }
+__host__ __device__ inline int list_smem(int V, int chain) { return 3 * list_words(V) + 3 * (chain + 1); }
+
+// One warp per state.  Bound by the latency of its dependent reads (the chain is short -- one to six states --, its arcs few),
+// so the chain's suffix links are followed first, alone, then the arcs of all chain states are taken side by side, a lane each:
+// two more trips to L2 whatever the chain's length.  The list has to come out ascending by token: a bitmap of its tokens and the
+// number of bits below each word give every entry its place, so nothing is sorted.
+// Five images of 500 phrases (2300 states each, 20 entries a state): 9 us; put together on the host they took 0.4 ms each and
+// made an image six times as large.
+__global__ void __launch_bounds__(kListWarps * 32) k_resolve_lists(TbSlotRec* recs, unsigned char* arena, const __grid_constant__ ListSlots ls,
+                                                                   const int32_t* __restrict__ ctb, const int32_t* __restrict__ ctk,
+                                                                   int32_t C, int32_t V, int32_t chain, int32_t* status) {
+  extern __shared__ __align__(16) uint32_t dynw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, words = list_words(V), tb = tb_rs_tok_bits(V);
+  uint32_t* seen = dynw + warp * list_smem(V, chain);
+  uint32_t* done = seen + words;
+  uint32_t* below = done + words;
+  float* ch_acc = reinterpret_cast<float*>(below + words);
+  int32_t* ch_arc = reinterpret_cast<int32_t*>(ch_acc + chain + 1);
+  int32_t* ch_before = ch_arc + chain + 1;
+  TbSlotRec* rp = recs + ls.at[blockIdx.y];
+  const TbSlotRec rec = *rp;
+  if (rec.n_states <= 0 || rec.n_rsent < 0) return;
+  unsigned char* blob = arena + rec.blob_off;
+  const GraphPtrs g = graph_of(arena, rec);
+  const TbRsRec* rsrec = reinterpret_cast<const TbRsRec*>(blob + rec.off_rsrec);
+  TbRsEnt* rsent = reinterpret_cast<TbRsEnt*>(blob + rec.off_rsent);
+#pragma unroll 1
+  for (int s = blockIdx.x * kListWarps + warp; s < rec.n_states; s += gridDim.x * kListWarps) {
+    const TbRsRec rr = rsrec[s];
+    if (rr.count == 0) continue;                              // (the root, and states whose chain boosts nothing)
+#pragma unroll 1
+    for (int w = lane; w < words; w += 32) { seen[w] = 0u; done[w] = 0u; }
+    // ---- the chain: s, its suffix state, ... down to the root's neighbour
+    int m = 0;
+    {
+      int u = s;
+      float acc = 0.0f;
+#pragma unroll 1
+      while (u != 0) {
+        if (m >= chain) { if (lane == 0) atomicOr(status, TB_STATUS_WALK_TOO_DEEP); break; }
+        if (lane == 0) { ch_acc[m] = acc; ch_arc[m] = u; }
+        acc = __fadd_rn(acc, g.bw[u]);
+        u = g.fail[u];
+        ++m;
+      }
+    }
+    __syncwarp();
+    int n_arcs = 0;
+#pragma unroll 1
+    for (int j0 = 0; j0 < m; j0 += 32) {
+      const int j = j0 + lane;
+      int first = 0, cnt = 0;
+      if (j < m) { const int u = ch_arc[j]; first = g.arc_begin[u]; cnt = g.arc_begin[u + 1] - first; }
+      int incl = cnt;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) { const int o = __shfl_up_sync(0xffffffffu, incl, off); if (lane >= off) incl += o; }
+      if (j < m) { ch_arc[j] = first; ch_before[j] = n_arcs + incl - cnt; }
+      n_arcs += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    __syncwarp();
+    auto arc_at = [&](int i, int* j_out) {                    // the i-th arc of the chain, and the chain state it leaves
+      int lo = 0, hi = m - 1;
+      while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (ch_before[mid] <= i) lo = mid; else hi = mid - 1; }
+      *j_out = lo;
+      return ch_arc[lo] + i - ch_before[lo];
+    };
+    // ---- which tokens
+#pragma unroll 1
+    for (int i = lane; i < n_arcs; i += 32) {
+      int j;
+      const int c = g.arc_cls[arc_at(i, &j)];
+      if (c < 0 || c >= C) continue;
+      const int q1 = ctb[c + 1];
+#pragma unroll 1
+      for (int q = ctb[c]; q < q1; ++q) { const int tk = ctk[q]; atomicOr(&seen[tk >> 5], 1u << (tk & 31)); }
+    }
+    __syncwarp();
+    int n = 0;
+#pragma unroll 1
+    for (int w0 = 0; w0 < words; w0 += 32) {
+      const int cnt = w0 + lane < words ? __popc(seen[w0 + lane]) : 0;
+      int incl = cnt;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) { const int o = __shfl_up_sync(0xffffffffu, incl, off); if (lane >= off) incl += o; }
+      if (w0 + lane < words) below[w0 + lane] = static_cast<uint32_t>(n + incl - cnt);
+      n += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    __syncwarp();
+    // ---- the entries, chain state by chain state: the first arc of a class wins (it is the closest to s)
+    TbRsEnt* out = rsent + rr.begin;
+#pragma unroll 1
+    for (int i0 = 0; i0 < n_arcs; i0 += 32) {
+      const int i = i0 + lane;
+      int c = -1 - lane, a = 0, j = 0;
+      if (i < n_arcs) { a = arc_at(i, &j); const int cc = g.arc_cls[a]; if (cc >= 0 && cc < C) c = cc; }
+      const int q0 = c >= 0 ? ctb[c] : 0, q1 = c >= 0 ? ctb[c + 1] : 0;
+      const int key = q0 < q1 ? ctk[q0] : -1;                 // (the class's first token stands for it)
+      const unsigned same = __match_any_sync(0xffffffffu, c);
+      const bool mine = key >= 0 && __ffs(same) - 1 == lane && !((done[key >> 5] >> (key & 31)) & 1u);
+      if (mine) {
+        TbRsEnt e;
+        const uint32_t dst = static_cast<uint32_t>(g.arc_dst[a]) << tb;
+        e.lb = __fmul_rn(g.lambda, __fadd_rn(ch_acc[j], g.arc_w[a]));
+#pragma unroll 1
+        for (int q = q0; q < q1; ++q) {
+          const int tk = ctk[q];
+          const int at = static_cast<int>(below[tk >> 5]) + __popc(seen[tk >> 5] & ((1u << (tk & 31)) - 1u));
+          e.dst_tok = dst | (2u * static_cast<uint32_t>(tk));
+          if (at < rr.count) out[at] = e;
+        }
+      }
+      __syncwarp();
+      if (mine) atomicOr(&done[key >> 5], 1u << (key & 31));
+      __syncwarp();
+    }
+#pragma unroll 1
+    for (int i = n + lane; i < rr.count; i += 32) {           // sentinels: the blank column with lb = -inf
+      TbRsEnt e;
+      e.dst_tok = 2u * static_cast<uint32_t>(V); e.lb = -INFINITY;
+      out[i] = e;
+    }
+    __syncwarp();
+  }
+  // (the next launch on the stream is the first to look at this)
+  if (blockIdx.x == 0 && threadIdx.x == 0) rp->lists_ready = 1;
+}
+
+}  // namespace
+
+int tb_launch_resolve_lists(TbSlotRec* recs, unsigned char* arena, int32_t n, const int32_t* at, int32_t max_states, int32_t max_depth,
+                            const int32_t* ctb, const int32_t* ctk, int32_t C, int32_t V, int32_t n_sm, int32_t* status, cudaStream_t stream) {
+  if (n < 1 || max_states < 1) return TB_OK;
+  if (n > TB_BIND_PAIRS || V > TB_MAX_VOCAB || max_depth > TB_MAX_PHRASE_LEN) return TB_ERR_INVALID_ARG;
+  ListSlots ls;
+  for (int32_t i = 0; i < n; ++i) ls.at[i] = at[i];
+  const int chain = max_depth + 1;
+  const size_t smem = static_cast<size_t>(kListWarps) * list_smem(V, chain) * 4;
+  if (smem > 40 * 1024 && cudaFuncSetAttribute(k_resolve_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess) {
+    cudaGetLastError();
+    return TB_ERR_CUDA;
+  }
+  // a state per warp until the GPU is full twice over, then several
+  int per = (max_states + kListWarps - 1) / kListWarps;
+  const int most = (n_sm * 16 + n - 1) / n;
+  if (per > most) per = most;
+  k_resolve_lists<<<dim3(per, n), kListWarps * 32, smem, stream>>>(recs, arena, ls, ctb, ctk, C, V, chain, status);
+  return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
+}

@@ -67,7 +67,7 @@ __device__ __forceinline__ DecideCtx<LT> decide_ctx(const TbDecodeParams& p, con
   c.base = base; c.st = p.st; c.ss = p.ss; c.V = p.V; c.S = p.S; c.n_dur = p.n_dur;
   c.tb = tb_rs_tok_bits(p.V); c.norm = p.normalize != 0;
   c.bound = rec.n_states > 0;
-  c.resolved = !c.bound || rec.n_rsent >= 0;
+  c.resolved = !c.bound || (rec.n_rsent >= 0 && rec.lists_ready);
   c.n_states = rec.n_states; c.max_depth = rec.max_depth;
   c.lam = c.bound ? rec.lambda : 0.0f; c.R = root.stats[2];
   c.rsrec = reinterpret_cast<const TbRsRec*>(blob + rec.off_rsrec);
@@ -76,6 +76,7 @@ __device__ __forceinline__ DecideCtx<LT> decide_ctx(const TbDecodeParams& p, con
   c.tokent = reinterpret_cast<const TbTokEnt*>(blob + rec.off_tokent);
   c.root = root; c.cls = p.cls; c.arc_w = g.arc_w; c.arc_dst = g.arc_dst;
   c.bitmap = bitmap; c.walk_buf = walk_buf; c.spill = spill; c.status = p.status;
+  c.p = &p; c.slot = -1;
   return c;
 }
 
@@ -350,7 +351,8 @@ __global__ void __launch_bounds__(kChunkThreads, 3) k_chunk_rows(const __grid_co
   float* vals = reinterpret_cast<float*>(dyn + so.vals);
   int* cursor_t = reinterpret_cast<int*>(part);              // (free again: the frame cursor, from warp 0 to the others)
 
-  const DecideCtx<LT> c = decide_ctx<LT>(p, rec, g, root, blob, base, bitmap, reinterpret_cast<TbRsEnt*>(dyn + so.walk), spill ? spill + static_cast<int64_t>(b) * (p.V + 32) : nullptr);
+  DecideCtx<LT> c = decide_ctx<LT>(p, rec, g, root, blob, base, bitmap, reinterpret_cast<TbRsEnt*>(dyn + so.walk), spill ? spill + static_cast<int64_t>(b) * (p.V + 32) : nullptr);
+  if (bound && rec.n_rsent >= 0 && !rec.lists_ready) c.slot = b;
   Cursor cu;
   DecideOut o;
   float score = st.score;

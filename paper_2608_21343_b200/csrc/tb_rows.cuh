@@ -24,6 +24,7 @@
 #include <cuda_bf16.h>
 
 #include "tb_device.cuh"
+#include "tb_launch.h"
 
 namespace {
 
@@ -376,6 +377,8 @@ struct DecideCtx {
   uint32_t* bitmap;                // [(V + 32) / 32] shared memory of this warp, zero between uses
   TbRsEnt* walk_buf;               // [kWalkBuf] shared memory of this warp, and
   TbRsEnt* spill;                  // [V + 32] global memory: lists put together by walking (null: the lists are resolved)
+  const TbDecodeParams* p;         // streaming chunks only: where a graph bound with this launch, whose lists are not derived
+  int slot;                        // yet, is walked from (-1: it is not such a graph)
   int32_t* status;
 };
 
@@ -391,8 +394,54 @@ __device__ __forceinline__ uint32_t td_pack(uint32_t dst_tok, int tb) { return _
 __device__ __forceinline__ int td_tok(uint32_t td, int tb) { return static_cast<int>(td >> (33 - tb)); }
 __device__ __forceinline__ int td_dst(uint32_t td, int tb) { return static_cast<int>(td & (0xFFFFFFFFu >> tb)); }
 
-// The list of state s (warp-wide).
+// One more entry of a list that is put together by walking, unless a chain state closer to the start listed the token.
 template <typename LT>
+__device__ __forceinline__ void walk_add(const DecideCtx<LT>& c, bool have, int tk, uint32_t dst, float w, float acc, int& n, int lane) {
+  const bool fresh = have && !((c.bitmap[tk >> 5] >> (tk & 31)) & 1u);
+  const unsigned mask = __ballot_sync(0xffffffffu, fresh);
+  if (fresh) {
+    atomicOr(&c.bitmap[tk >> 5], 1u << (tk & 31));
+    TbRsEnt o;
+    o.dst_tok = (dst << c.tb) | (2u * static_cast<uint32_t>(tk));
+    o.lb = __fmul_rn(c.lam, __fadd_rn(acc, w));
+    const int at = n + __popc(mask & ((1u << lane) - 1u));
+    c.spill[at] = o;
+    if (at < kWalkBuf) c.walk_buf[at] = o;
+  }
+  n += __popc(mask);
+}
+// The walk over a graph's flat arrays; sum: the suffix-link weights of the whole chain, in walk order.
+template <typename LT>
+__device__ __forceinline__ int walk_flat(const DecideCtx<LT>& c, int s, float& sum, int lane) {
+  const GraphPtrs g = graph_of(c.p->arena, c.p->slots[c.slot]);
+  const int32_t* ctb = c.p->class_tok;
+  const int32_t* ctk = ctb + c.p->C + 1;
+  int n = 0, u = s > 0 ? s : 0;
+  float acc = 0.0f;
+#pragma unroll 1
+  for (int it = 0; u != 0; ++it) {
+    if (it > c.max_depth + 1) { if (lane == 0) atomicOr(c.status, TB_STATUS_WALK_TOO_DEEP); break; }
+    const int a1 = g.arc_begin[u + 1], nu = g.fail[u];
+    const float bw = g.bw[u];
+#pragma unroll 1
+    for (int a = g.arc_begin[u] + lane; __any_sync(0xffffffffu, a < a1); a += 32) {
+      int q = 0, q1 = 0;
+      uint32_t dst = 0;
+      float w = 0.0f;
+      if (a < a1) { const int cl = g.arc_cls[a]; q = ctb[cl]; q1 = ctb[cl + 1]; dst = static_cast<uint32_t>(g.arc_dst[a]); w = g.arc_w[a]; }
+#pragma unroll 1
+      for (; __any_sync(0xffffffffu, q < q1); ++q) walk_add(c, q < q1, q < q1 ? ctk[q] : 0, dst, w, acc, n, lane);
+    }
+    __syncwarp();
+    acc = __fadd_rn(acc, bw);
+    u = nu > 0 && nu < c.n_states ? nu : 0;
+  }
+  sum = acc;
+  return n;
+}
+
+// The list of state s (warp-wide).  CHUNK: the graph may be one bound with this launch.
+template <typename LT, bool CHUNK>
 __device__ __forceinline__ TokList list_of(const DecideCtx<LT>& c, int s, int lane) {
   TokList L;
   if (c.resolved) {
@@ -408,6 +457,7 @@ __device__ __forceinline__ TokList list_of(const DecideCtx<LT>& c, int s, int la
   int n = 0;
   float acc = 0.0f;
   int u = s > 0 ? s : 0;
+  if (CHUNK && c.slot >= 0) { n = walk_flat(c, s, acc, lane); u = 0; }
   uint4 rec = make_uint4(0u, 0u, 0u, 0u);                     // TbStateRec
   if (u != 0) rec = *reinterpret_cast<const uint4*>(c.strec + u);
 #pragma unroll 1
@@ -422,19 +472,7 @@ __device__ __forceinline__ TokList list_of(const DecideCtx<LT>& c, int s, int la
     for (int e = static_cast<int>(rec.x) + lane; __any_sync(0xffffffffu, e < e1); e += 32) {
       uint4 ent = make_uint4(0u, 0u, 0u, 0u);                 // TbTokEnt
       if (e < e1) ent = *reinterpret_cast<const uint4*>(c.tokent + e);
-      const int tk = static_cast<int>(ent.x & 0xFFFFu);
-      const bool fresh = e < e1 && !((c.bitmap[tk >> 5] >> (tk & 31)) & 1u);
-      const unsigned mask = __ballot_sync(0xffffffffu, fresh);
-      if (fresh) {
-        atomicOr(&c.bitmap[tk >> 5], 1u << (tk & 31));
-        TbRsEnt o;
-        o.dst_tok = (ent.z << c.tb) | (2u * static_cast<uint32_t>(tk));
-        o.lb = __fmul_rn(c.lam, __fadd_rn(acc, __uint_as_float(ent.y)));
-        const int at = n + __popc(mask & ((1u << lane) - 1u));
-        c.spill[at] = o;
-        if (at < kWalkBuf) c.walk_buf[at] = o;
-      }
-      n += __popc(mask);
+      walk_add(c, e < e1, static_cast<int>(ent.x & 0xFFFFu), ent.z, __uint_as_float(ent.y), acc, n, lane);
     }
     __syncwarp();
     acc = __fadd_rn(acc, __uint_as_float(rec.w));
@@ -582,7 +620,7 @@ __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const
         __syncwarp();
       }
     }
-    if (!listed) { L = list_of(c, s, lane); listed = true; }
+    if (!listed) { L = list_of<LT, !SEG>(c, s, lane); listed = true; }
     // Two kinds of round.  List round: the eight lanes 8 r .. 8 r + 7 take row r of {(t, k), (t + 1, 0), (t + 2, 0),
     // (t + 3, 0)} and share out the list.  Grid round (no boosted tokens, or a state that just repeated itself): lane
     // 4 q + j resolves row (t + q, j) on its own, and the walk goes through tokens too while they leave the state unchanged.

@@ -1,0 +1,64 @@
+"""Parity of the per-state token lists that the device derives from a bound graph's arrays, against the CPU oracle: case
+classes of one to many tokens, chains as deep as a phrase may be, states with more arcs than a warp has lanes, vocabularies
+at the edges of a bitmap word, and every way a graph is bound."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+from paper_2608_21343_b200 import workloads as W
+from helpers import check_greedy, to_device, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+def _lists(rng, V, kind):
+    hot = rng.choice(V, size=min(V, 12), replace=False)
+    if kind == "deep":                            # a phrase of one token and of two in turn: chains of hundreds of states
+        a, b = int(hot[0]), int(hot[-1])
+        return [[a] * 255, [a, b] * 100, [b, a, a], [a, b, b, b]]
+    if kind == "fan":                             # states with arcs to (nearly) every class
+        return [[int(hot[0]), int(v)] for v in range(min(V, 300))] + [[int(hot[1]), int(hot[0]), int(v)] for v in range(0, min(V, 300), 2)]
+    if kind == "root":                            # nothing but the root is left
+        return [[int(v)] for v in hot]
+    return [[int(v) for v in rng.choice(hot, size=rng.integers(1, 7))] for _ in range(60)]
+
+
+@pytest.mark.parametrize("V,siblings,kind,dtype", [
+    (1, 1, "mixed", "f32"), (31, 2, "mixed", "bf16"), (32, 32, "mixed", "f32"), (33, 3, "deep", "bf16"), (64, 1, "deep", "f32"),
+    (300, 1, "fan", "bf16"), (300, 7, "fan", "f32"), (1024, 4, "root", "bf16"), (1025, 5, "mixed", "bf16"), (2047, 40, "fan", "bf16"),
+    (2048, 2, "fan", "f32"), (8192, 3, "mixed", "f32"), (8191, 1, "deep", "bf16")])
+def test_lists(tb, V, siblings, kind, dtype):
+    rng = np.random.default_rng(V + siblings)
+    cc = rng.permutation(V).astype(np.int32) // siblings
+    lists = [_lists(rng, V, kind) for _ in range(4)]
+    T, S = 40, 3
+    x = rng.normal(size=(4, T, S, V + 1)).astype(np.float32)
+    for i in range(4):                            # the phrases' own tokens, in phrase order, stand out
+        said = [t for p in lists[i] for t in p][:T * 2]
+        for j, t in enumerate(said):
+            x[i, j // 2, j % 2, t] += 6.0
+    x[..., V] += 3.0
+    logits = W.to_storage(x, dtype)
+    ref = [O.greedy_rnnt(O.Graph(p, V, case_class=cc, lam=1.3), logits[i]) for i, p in enumerate(lists)]
+    graphs = [tb.tb_graph_compile(p, V, case_class=cc, lam=1.3) for p in lists]
+    batch = tb.tb_batch_create(V, cc, 4, arena_bytes=64 << 20)
+    dev = to_device(logits)
+
+    def bind_one_by_one(gs):
+        for i, g in enumerate(gs):
+            tb.tb_batch_bind_stream(batch, i, g)
+
+    def bind_models(gs):
+        tb.tb_batch_bind_models(batch, list(range(4)), [tb.tb_batch_register_model(batch, g) for g in gs])
+
+    def bind_with_a_chunk(gs):                    # the chunk's own rows are of no interest here
+        n = torch.zeros(4, dtype=torch.int32, device="cuda:0")
+        tb.tb_stream_chunk_binds(batch, list(range(4)), gs, dev[:, :2].contiguous(), 0, n)
+
+    for turn, bind in enumerate((bind_one_by_one, lambda gs: tb.tb_batch_bind_streams(batch, list(range(4)), gs), bind_models, bind_with_a_chunk)):
+        bind(graphs)
+        out = to_host(tb.tb_greedy_decode(batch, dev))
+        assert tb.tb_batch_status(batch) == 0
+        for i in range(4):
+            check_greedy(out, i, ref[i], f"bind {turn}")
