@@ -197,7 +197,7 @@ extern "C" int tb_graph_load(const char* path, tb_graph** out) {
       for (int64_t e = 0; in && e < Te; ++e) {
         TbTokEnt te;
         std::memcpy(&te, bl + g->off_tokent + 16 * e, 16);
-        in = static_cast<int32_t>(te.tok_cls & 0xffffu) < h.vocab && te.dst >= 0 && te.dst < Ns;
+        in = static_cast<int32_t>(te.tok_cls & 0xffffu) < h.vocab && te.dst >= 0 && te.dst < Ns && te.dst_begin >= 0 && te.dst_begin <= Te;
       }
       if (Re >= 0) {
         in = in && Re <= TB_RS_MAX_ENTRIES;

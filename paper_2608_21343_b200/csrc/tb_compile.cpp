@@ -117,6 +117,7 @@ static void finalize_graph(tb_graph* g, const int32_t* case_class, int32_t vocab
       recs[u].fail = g->state_fail[u];
       recs[u].bw = g->state_bw[u];
     }
+    for (TbTokEnt& e : ents) e.dst_begin = recs[e.dst].tok_begin;
   }
   // ---- the image, filled in place
   size_t size = 0;

@@ -98,7 +98,7 @@ struct TbTokEnt {
   uint32_t tok_cls;            // token | class << 16
   float w;                     // arc weight
   int32_t dst;                 // arc target
-  int32_t pad;
+  int32_t dst_begin;           // where the target's own arcs begin
 };
 static_assert(sizeof(TbStateRec) == 16 && sizeof(TbTokEnt) == 16, "16-byte records");
 

@@ -32,16 +32,17 @@ struct RowsParams {
   TbDecodeParams d;
   RowSum* sums;               // [n_streams][frames * S]
   int32_t frames_per_warp;    // step 1: frames whose rows one warp reduces (at most 32)
-  int32_t prefetch;           // the logits do not stay in L2 between the steps
   int32_t nseg;
   int32_t cache_bytes;        // shared memory for a copy of the stream's lists (0: none fits)
   int32_t* log_tok; int32_t* log_frm; float* log_val; int64_t log_stride;   // [n_streams][log_stride]
   int32_t* trace; int2* aux;  // [n_streams][frames + 1]
   TbRsEnt* spill;             // [n_streams][nseg][V + 32] or null
+  // where each stretch's part of a stream's logs begins (tabulated: a division in 64 bits takes as long as a frame)
+  int64_t seg_at[kDecMaxSegs + 1];
 };
 
-// what a segment's region of the logs has to hold, in frames: from its warmed-up start to the end of the stream
-__host__ __device__ inline int64_t seg_frames(int64_t frames, int nseg, int i) {
+// what a stretch's part of the logs has to hold, in frames: from its warmed-up start to the end of the stream
+inline int64_t seg_frames(int64_t frames, int nseg, int i) {
   const int64_t f = (frames * (nseg - i) + nseg - 1) / nseg + kDecWarm + 1;
   return f < frames ? f : frames;
 }
@@ -157,9 +158,7 @@ __global__ void __launch_bounds__(32 * kDecMaxSegs, 1) k_decide_rows(const __gri
   asm volatile("griddepcontrol.wait;" ::: "memory");                        // the rows' summaries are in place
   // stretch results: {tokens, values, state, frame it stopped at}, {met, failed}
   int4* res = reinterpret_cast<int4*>(dyn + so.misc);
-  int64_t seg_off = 0;
-#pragma unroll 1
-  for (int i = 0; i < warp; ++i) seg_off += seg_frames(p.frames, P.nseg, i) * S;
+  const int64_t seg_off = P.seg_at[min(warp, kDecMaxSegs - 1)];
   const int64_t log0 = static_cast<int64_t>(b) * P.log_stride;
   if (warp < nseg) {
     DecideCtx<LT> c = decide_ctx<LT>(p, rec, g, root, blob, reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(b) * p.sb,
@@ -173,12 +172,11 @@ __global__ void __launch_bounds__(32 * kDecMaxSegs, 1) k_decide_rows(const __gri
     o.first = warp * Lf; o.is_last = warp == nseg - 1; o.next = o.is_last ? end : min(end, (warp + 1) * Lf);
     o.tok = P.log_tok + log0 + seg_off; o.frm = P.log_frm + log0 + seg_off; o.dur = nullptr;
     o.vals = P.log_val + log0 + seg_off;
-    o.cap = static_cast<int>(seg_frames(p.frames, P.nseg, warp) * S);
-    o.prefetch = P.prefetch != 0;
+    o.cap = static_cast<int>(P.seg_at[warp + 1] - seg_off);
     o.trace = trace; o.trace_aux = P.aux + static_cast<int64_t>(b) * (p.frames + 1);
     Cursor cu;
     cu.t = max(0, o.first - ((bound && warp > 0) ? kDecWarm : 0)); cu.k = 0; cu.s = bound ? 0 : -1;
-    cu.n_out = cu.nv = 0; cu.stable = false; cu.failed = false; cu.met = -1; cu.listed = false;
+    cu.n_out = cu.nv = 0; cu.failed = false; cu.met = -1; cu.listed = false;
     if (warp == 0) o.first = INT32_MAX;                                     // (nobody needs the first stretch's records)
     decide<LT, true>(c, cu, o, P.sums + static_cast<int64_t>(b) * p.frames * S,
                                shared_u32(dyn + so.ring) + warp * kDecRing * S * 32, kDecRing - 1, 0, end, lane);
@@ -189,20 +187,20 @@ __global__ void __launch_bounds__(32 * kDecMaxSegs, 1) k_decide_rows(const __gri
   }
   __threadfence_block();
   __syncthreads();
-  // ---- the chain of stretches: {stretch, first token, end token, output offset}, {first value, end value}
+  // ---- the chain of stretches: {stretch, first token, end token, output offset}, {first value, end value, values before it}
   int4* hops = res + 2 * kDecMaxSegs;
   int* vars = reinterpret_cast<int*>(hops + 2 * kDecMaxSegs);
   const int2* aux = P.aux + static_cast<int64_t>(b) * (p.frames + 1);
   if (tid == 0) {
-    int seg = 0, ptok = 0, pval = 0, n = 0, cnt = 0, fin_state = bound ? 0 : -1, fin_t = 0, bad = 0;
+    int seg = 0, ptok = 0, pval = 0, n = 0, n_val = 0, cnt = 0, fin_state = bound ? 0 : -1, fin_t = 0, bad = 0;
 #pragma unroll 1
     for (int hop = 0; hop < nseg && !bad && end > 0; ++hop) {
       const int4 ra = res[2 * seg], rb = res[2 * seg + 1];
       if (rb.y || ra.x < ptok || ra.y < pval) { bad = 1; break; }
       hops[2 * cnt] = make_int4(seg, ptok, ra.x, n);
-      hops[2 * cnt + 1] = make_int4(pval, ra.y, 0, 0);
+      hops[2 * cnt + 1] = make_int4(pval, ra.y, n_val, 0);
       ++cnt;
-      n += ra.x - ptok;
+      n += ra.x - ptok; n_val += ra.y - pval;
       fin_state = ra.z; fin_t = ra.w;
       if (!rb.x) break;                                   // decoded to the end of the stream
       const int j = min(ra.w / Lf, nseg - 1);             // the owner of frame start ra.w
@@ -212,55 +210,53 @@ __global__ void __launch_bounds__(32 * kDecMaxSegs, 1) k_decide_rows(const __gri
       if (hop == nseg - 1) bad = 1;                       // a chain longer than the number of stretches
     }
     if (bad) atomicOr(p.status, TB_STATUS_STEP_LIMIT);
-    vars[0] = cnt; vars[1] = n; vars[2] = fin_state; vars[3] = fin_t;
+    vars[0] = cnt; vars[1] = n; vars[2] = fin_state; vars[3] = fin_t; vars[4] = n_val;
   }
   __syncthreads();
   const int cnt = vars[0];
   int32_t* o_tok = p.out_tokens + static_cast<int64_t>(b) * p.out_cap;
   int32_t* o_frm = p.out_frames + static_cast<int64_t>(b) * p.out_cap;
-  // The score is the sum of the visited rows' values in visiting order: the chain's values are brought into shared
-  // memory by all threads, a piece at a time (the rings are free now), and added one by one by a single thread.
+  // A warp per link of the chain copies its tokens out.  The score is the sum of the visited rows' values in visiting order:
+  // they are brought into shared memory (the rings are free now), all links at once, a window of them at a time, and added
+  // one by one by a single thread.
   float* vbuf = reinterpret_cast<float*>(dyn + so.ring);
-  const int vcap = P.nseg * kDecRing * S * 8;
+  const int vcap = P.nseg * kDecRing * S * 8, n_val = vars[4];
   float score = 0.0f;
-  int filled = 0;
-  auto add_up = [&]() {
+#pragma unroll 1
+  for (int w0 = 0; w0 == 0 || w0 < n_val; w0 += vcap) {
+    if (warp < cnt) {
+      const int4 ha = hops[2 * warp], hb = hops[2 * warp + 1];
+      const int64_t off = log0 + P.seg_at[ha.x];
+      const int v0 = max(hb.x, hb.x + w0 - hb.z), v1 = min(hb.y, hb.x + w0 + vcap - hb.z);
+#pragma unroll 4
+      for (int v = v0 + lane; v < v1; v += 32) vbuf[hb.z + v - hb.x - w0] = P.log_val[off + v];
+      if (w0 == 0) {
+#pragma unroll 4
+        for (int j = ha.y + lane; j < ha.z; j += 32) {
+          const int at = ha.w + j - ha.y;
+          if (at < p.out_cap) { o_tok[at] = P.log_tok[off + j]; o_frm[at] = P.log_frm[off + j]; }
+        }
+      }
+    }
     __syncthreads();
     if (tid == 0) {
+      const int filled = min(n_val - w0, vcap);
       int i = 0;
 #pragma unroll 1
-      for (; i + 8 <= filled; i += 8) {
-        const float4 a4 = *reinterpret_cast<const float4*>(vbuf + i), b4 = *reinterpret_cast<const float4*>(vbuf + i + 4);
-        score = __fadd_rn(score, a4.x); score = __fadd_rn(score, a4.y); score = __fadd_rn(score, a4.z); score = __fadd_rn(score, a4.w);
-        score = __fadd_rn(score, b4.x); score = __fadd_rn(score, b4.y); score = __fadd_rn(score, b4.z); score = __fadd_rn(score, b4.w);
+      for (; i + 32 <= filled; i += 32) {
+        float4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = *reinterpret_cast<const float4*>(vbuf + i + 4 * u);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          score = __fadd_rn(score, v[u].x); score = __fadd_rn(score, v[u].y); score = __fadd_rn(score, v[u].z); score = __fadd_rn(score, v[u].w);
+        }
       }
 #pragma unroll 1
       for (; i < filled; ++i) score = __fadd_rn(score, vbuf[i]);
     }
-    __syncthreads();
-    filled = 0;
-  };
-#pragma unroll 1
-  for (int h = 0; h < cnt; ++h) {
-    const int4 ha = hops[2 * h], hb = hops[2 * h + 1];
-    int64_t off = log0;
-#pragma unroll 1
-    for (int i = 0; i < ha.x; ++i) off += seg_frames(p.frames, P.nseg, i) * S;
-#pragma unroll 1
-    for (int j = ha.y + tid; j < ha.z; j += nthreads) {
-      const int at = ha.w + j - ha.y;
-      if (at < p.out_cap) { o_tok[at] = P.log_tok[off + j]; o_frm[at] = P.log_frm[off + j]; }
-    }
-#pragma unroll 1
-    for (int v = hb.x; v < hb.y;) {
-      const int take = min(hb.y - v, vcap - filled);
-#pragma unroll 1
-      for (int j = tid; j < take; j += nthreads) vbuf[filled + j] = P.log_val[off + v + j];
-      filled += take; v += take;
-      if (filled == vcap) add_up();
-    }
+    if (w0 + vcap < n_val) __syncthreads();
   }
-  add_up();
   if (tid == 0) {
     p.out_counts[b] = vars[1]; p.out_scores[b] = score; p.out_states[b] = vars[2];
     if (p.out_cursors) p.out_cursors[b] = vars[3];
@@ -356,12 +352,12 @@ __global__ void __launch_bounds__(kChunkThreads, 3) k_chunk_rows(const __grid_co
   Cursor cu;
   DecideOut o;
   float score = st.score;
-  cu.t = st.t; cu.k = st.k; cu.s = bound ? st.state : -1; cu.n_out = cu.nv = 0; cu.stable = false; cu.failed = false; cu.met = -1; cu.listed = false;
+  cu.t = st.t; cu.k = st.k; cu.s = bound ? st.state : -1; cu.n_out = cu.nv = 0; cu.failed = false; cu.met = -1; cu.listed = false;
   if (warp == 0) {
     if (bound && (cu.s < 0 || cu.s >= rec.n_states)) { if (lane == 0) atomicOr(p.status, TB_STATUS_BAD_STATE); cu.s = 0; }
     const int64_t at = static_cast<int64_t>(b) * p.out_cap;
     o.tok = p.out_tokens + at; o.frm = p.out_frames + at; o.dur = p.out_durs ? p.out_durs + at : nullptr;
-    o.vals = vals; o.cap = p.out_cap; o.trace = nullptr; o.trace_aux = nullptr; o.first = o.next = 0; o.is_last = true; o.prefetch = false;
+    o.vals = vals; o.cap = p.out_cap; o.trace = nullptr; o.trace_aux = nullptr; o.first = o.next = 0; o.is_last = true;
   }
   int t = cu.t;
 #pragma unroll 1
@@ -452,6 +448,8 @@ int tb_launch_rows(const TbDecodeParams& d, const TbRowsPlan& plan, int32_t n_sm
   P.log_frm = reinterpret_cast<int32_t*>(sb + l.log_frm);
   P.log_val = reinterpret_cast<float*>(sb + l.log_val);
   P.log_stride = l.log_stride;
+  P.seg_at[0] = 0;
+  for (int i = 0; i < kDecMaxSegs; ++i) P.seg_at[i + 1] = P.seg_at[i] + (i < plan.nseg ? seg_frames(d.frames, plan.nseg, i) * d.S : 0);
   P.trace = reinterpret_cast<int32_t*>(sb + l.trace);
   P.aux = reinterpret_cast<int2*>(sb + l.aux);
   P.spill = plan.all_resolved ? nullptr : reinterpret_cast<TbRsEnt*>(sb + l.spill);
@@ -461,7 +459,6 @@ int tb_launch_rows(const TbDecodeParams& d, const TbRowsPlan& plan, int32_t n_sm
   int64_t per = all / (static_cast<int64_t>(n_sm) * 8 * kSumThreads / 32);
   per = per < 1 ? 1 : per > 16 ? 16 : per;
   P.frames_per_warp = static_cast<int32_t>(per);
-  P.prefetch = static_cast<int64_t>(d.n_streams) * d.frames * d.S * (d.V + 1) * (d.dtype == TB_BF16 ? 2 : 4) > (static_cast<int64_t>(64) << 20);
   // a row of up to 128 blocks of 16 bytes is one group of four per lane, a wider one takes groups of eight
   const bool narrow = d.V * (d.dtype == TB_BF16 ? 2 : 4) <= 128 * 16 + 15;
   void (*f1)(RowsParams) = d.dtype == TB_BF16 ? (narrow ? k_row_sums<uint16_t, 4> : k_row_sums<uint16_t, 8>)

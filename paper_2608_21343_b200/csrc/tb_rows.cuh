@@ -3,12 +3,16 @@
 //
 // Step 1 (frames_summary, one warp per row, independent of the graph state): the row's best root-boosted token, a bound on
 // all others, its blank logit, and -- where asked for -- its log-softmax normaliser or its best duration.
-// Step 2 (decide, one warp per stretch): the sequential part.  A round looks at the rows (t, k), (t+1, 0), (t+2, 0),
-// (t+3, 0) under the current graph state at once: the lanes share out the state's list of boosted tokens, every lane
-// gathers its tokens' logits from the four rows, two warp-wide integer reductions per row find the best listed token
-// (largest value, then lowest token), lane r compares it with row r's summary, and one ballot gives the run of leading
-// blanks and the row that ends it.  What bounds it is the chain state -> list -> logits -> token -> state: a trip to
-// shared memory or L2 for each arrow and about 200 dependent instructions.
+// Step 2 (decide, one warp per stretch): the sequential part.  What bounds it is the chain state -> list -> logits ->
+// token -> state: a trip to shared memory or L2 for each arrow and some 500 instructions, which a warp that is alone on
+// its scheduler issues one every five to seven cycles; 3300 cycles in all, whatever number of rows are looked at.  So a
+// round takes as many rows as can be foreseen: the summaries alone say which way most rows go, and the rows on that way
+// (up to eight, of several frames) are decided at once, each under the state foreseen for it; three to four hold on
+// average.  Rounds of the rows (t, k), (t+1, 0), .. under the current state only, which end with the first token, took
+// twice as many.  A row the summaries cannot decide is read in full, but only for the tokens past a threshold (V = 8192:
+// 190 000 cycles a row when every token was looked up, 20 000 so).  Nothing is asked into L2 ahead: a stretch's rows
+// amount to more requests than its SM issues in the time (V = 8192: 203 us with it, 143 without).
+// 32 fp32 streams of 500 frames, V = 1024: 197 us before these, 118 after.
 //
 // The code is kept small on purpose (no register-resident lists, loops not unrolled beyond what keeps loads in flight,
 // options as uniform branches instead of instantiations): a chunk or a short utterance runs through it a few dozen times
@@ -472,6 +476,11 @@ __device__ __forceinline__ TokList list_of(const DecideCtx<LT>& c, int s, int la
     for (int e = static_cast<int>(rec.x) + lane; __any_sync(0xffffffffu, e < e1); e += 32) {
       uint4 ent = make_uint4(0u, 0u, 0u, 0u);                 // TbTokEnt
       if (e < e1) ent = *reinterpret_cast<const uint4*>(c.tokent + e);
+      // (where an entry leads: the state's record and its first arcs are asked into L2, in case the entry is taken)
+      if (e < e1) {
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(c.strec + ent.z));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(c.tokent + ent.w));
+      }
       walk_add(c, e < e1, static_cast<int>(ent.x & 0xFFFFu), ent.z, __uint_as_float(ent.y), acc, n, lane);
     }
     __syncwarp();
@@ -492,6 +501,7 @@ struct RowPick { float val; int tok, next, dur; float xdur; };   // tok == V: bl
 // Exact evaluation of one row under the current state by the whole warp.
 template <typename LT>
 __device__ __forceinline__ RowPick exact_row(const DecideCtx<LT>& c, const TokList& L, const LT* row, int s, int lane) {
+  using RB = RowBlock<LT>;
   ValId best{LogitLoad<LT>::at(row + c.V), c.V};
   int bn = s;
 #pragma unroll 1
@@ -504,20 +514,44 @@ __device__ __forceinline__ RowPick exact_row(const DecideCtx<LT>& c, const TokLi
     if (better(o, best)) { best = o; bn = static_cast<int>(e.dst_tok >> c.tb); }
   }
   __syncwarp();
-#pragma unroll 4
-  for (int tk = lane; tk < c.V; tk += 32) {
-    const float x = LogitLoad<LT>::at(row + tk);
-    float v = x;
+  // A token outside the list is worth looking up only where its logit alone could bring it past the best so far (`slack`
+  // covers all roundings): the row is compared with that threshold, 16 bytes at a time.
+  const float B = order_key_inv(__reduce_max_sync(0xffffffffu, order_key(best.v)));
+  const float U = c.bound ? c.lam * L.D + c.root.stats[1] : 0.0f;
+  const float slack = (fabsf(B) + fabsf(U) + L.bmag) * 3.814697265625e-6f + 1e-30f;
+  const float thr = RB::threshold(B == -INFINITY ? -INFINITY : B - U - slack);
+  auto offer = [&](int tk) {
+    float v = LogitLoad<LT>::at(row + tk);
     int nx = -1;
     if (c.bound) {
       const int cl = __ldg(c.cls + tk);
-      v = __fadd_rn(x, __fmul_rn(c.lam, __fadd_rn(L.D, c.root.w[cl])));
+      v = __fadd_rn(v, __fmul_rn(c.lam, __fadd_rn(L.D, c.root.w[cl])));
       nx = c.root.arc[cl];
       nx = nx ? -1 - nx : 0;                                   // (the arc's target is looked up for the winner only)
     }
     const ValId o{v, tk};
     if (!((c.bitmap[tk >> 5] >> (tk & 31)) & 1u) && better(o, best)) { best = o; bn = nx; }
+  };
+  const int hd = min(c.V, static_cast<int>((16u - static_cast<uint32_t>(reinterpret_cast<uintptr_t>(row) & 15)) & 15u) / static_cast<int>(sizeof(LT)));
+  const int nb = (c.V - hd) / RB::E;
+#pragma unroll 1
+  for (int g = lane; __any_sync(0xffffffffu, g < nb); g += 32 * 4) {
+    uint4 q[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      q[u] = make_uint4(RB::kNone, RB::kNone, RB::kNone, RB::kNone);
+      if (g + 32 * u < nb) q[u] = __ldg(reinterpret_cast<const uint4*>(row + hd) + g + 32 * u);
+    }
+    uint32_t hits = RB::template hits<4>(q, 0, thr);
+#pragma unroll 1
+    while (hits) {
+      const int bit = __ffs(hits) - 1, bi = g + 32 * RB::unit(bit);
+      hits &= hits - 1u;
+      if (bi < nb) offer(hd + bi * RB::E + RB::elem(bit));
+    }
   }
+  const int edge = lane < hd ? lane : nb * RB::E + lane;         // this lane's token outside the aligned blocks
+  if (lane < 2 * RB::E && edge < c.V) offer(edge);
   __syncwarp();
 #pragma unroll 1
   for (int i = lane; i < L.n; i += 32) c.bitmap[(L.ent[i].dst_tok & ((1u << c.tb) - 1u)) >> 6] = 0u;
@@ -547,7 +581,6 @@ __device__ __forceinline__ RowPick exact_row(const DecideCtx<LT>& c, const TokLi
 struct Cursor {
   int t, k, s;          // frame, row in frame, graph state
   int n_out, nv;        // tokens emitted, row values logged
-  bool stable;          // the last token left the state unchanged
   bool failed;
   int met;              // frame start at which it met a later stretch of the stream (-1: none)
   bool listed;          // list is that of state s
@@ -562,7 +595,7 @@ struct DecideOut {
   // much it had logged there; past `next` it stops where its state is the one recorded there
   volatile int32_t* trace; int2* trace_aux;
   int first, next;
-  bool is_last, prefetch;
+  bool is_last;
 };
 
 // Decides the rows from the cursor on, up to frame `end` (exclusive).  Summaries of row k of frame f are at shared
@@ -574,7 +607,7 @@ __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const
   const int S = c.S, V = c.V, tb = c.tb;
   const bool tdt = !SEG && c.n_dur > 0;
   int t = cu.t, k = cu.k, s = cu.s, n_out = cu.n_out, nv = cu.nv;
-  bool stable = cu.stable, no_grid = false, listed = cu.listed;
+  bool listed = cu.listed;
   TokList L = cu.list;
   const uint32_t none = (2u * static_cast<uint32_t>(V)) << (32 - tb), tmask = (1u << tb) - 1u;
   // what a row adds to the score: its value less its normaliser, or plus its duration's logit
@@ -583,7 +616,7 @@ __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const
     if (SEG && fs >= o.first && fs < o.next) { o.trace_aux[fs] = make_int2(n_tok, n_val); o.trace[fs] = st_; }
   };
   if (SEG && lane == 0 && k == 0) trace(t, s, n_out, nv);
-  int loaded = t & ~3, refill = t;            // SEG: frames up to `loaded` have been asked for; the next group is due at frame `refill`
+  int loaded = t & ~7, refill = t;            // SEG: frames up to `loaded` have been asked for; the next group is due at frame `refill`
   const int max_rounds = (end - t) * (S + 1) + 8;
 #pragma unroll 1
   for (int it = 0; t < end; ++it) {
@@ -592,193 +625,181 @@ __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const
       if (k == 0 && t >= o.next && !o.is_last) {
         if (!c.bound || o.trace[t] == s) { cu.met = t; break; }     // (unbound: no graph state, the owner's decode from here is this one's)
       }
-      // the ring, in groups of four frames: those up to 12 frames ahead are in place, the next group is on its way; the
-      // rows of the next frames are asked into L2, which this stretch's rows have long left when the call's logits are
-      // larger than it
+      // the ring, in groups of eight frames: the round's window is in place, the next group is on its way
       if (t >= refill) {
         do {
-          if (loaded < end) {
-            const int nq = min(4, end - loaded) * S * 2;
-            const uint4* src = reinterpret_cast<const uint4*>(gsum + static_cast<int64_t>(loaded) * S);
-            const uint32_t dst = sum_a + static_cast<uint32_t>((loaded & mask) * S) * 32u;
-            if (lane < nq) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16u * lane), "l"(src + lane) : "memory");
-          }
+          const int nq = min(8, end - loaded) * S * 2;
+          const uint4* src = reinterpret_cast<const uint4*>(gsum + static_cast<int64_t>(loaded) * S);
+          const uint32_t dst = sum_a + static_cast<uint32_t>((loaded & mask) * S) * 32u;
+#pragma unroll
+          for (int i = 0; i < 8 * kRowsPerFrame * 2; i += 32)
+            if (i + lane < nq) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16u * (i + lane)), "l"(src + i + lane) : "memory");
           asm volatile("cp.async.commit_group;" ::: "memory");
-          loaded += 4;
-        } while (loaded < t + 16);
-        refill = (t & ~3) + 4;
+          loaded += 8;
+        } while (loaded < t + 24);
+        refill = (t & ~7) + 8;
         asm volatile("cp.async.wait_group 1;" ::: "memory");
-        if (o.prefetch && lane < 4 * S) {
-          const int f = refill + 4 + lane / S;
-          if (f < end) {
-            const unsigned char* pr = reinterpret_cast<const unsigned char*>(c.base + static_cast<int64_t>(f) * c.st + static_cast<int64_t>(lane % S) * c.ss);
-            const uintptr_t p0 = (reinterpret_cast<uintptr_t>(pr) + 15) & ~static_cast<uintptr_t>(15);
-            const uint32_t bytes = static_cast<uint32_t>(V) * sizeof(LT) - 16u & ~15u;
-            if (V * sizeof(LT) > 64) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p0), "r"(bytes) : "memory");
-          }
-        }
         __syncwarp();
       }
     }
     if (!listed) { L = list_of<LT, !SEG>(c, s, lane); listed = true; }
-    // Two kinds of round.  List round: the eight lanes 8 r .. 8 r + 7 take row r of {(t, k), (t + 1, 0), (t + 2, 0),
-    // (t + 3, 0)} and share out the list.  Grid round (no boosted tokens, or a state that just repeated itself): lane
-    // 4 q + j resolves row (t + q, j) on its own, and the walk goes through tokens too while they leave the state unchanged.
-    const bool grid = !tdt && !no_grid && (L.n == 0 || (stable && L.n <= 64));
-    no_grid = false;
+    // One round: up to eight rows in the order they are visited in, a group of lanes each.  Which rows those are, and the
+    // graph state each is visited in, is predicted from the summaries alone -- a row selects its best plain token, which
+    // leads to a root arc's target, or blank -- and every group then decides its row exactly under the state predicted for
+    // it.  The round ends with the first row that goes another way (a token of the list, most often) or has to be
+    // evaluated in full.  Longer lists get more lanes per row, and fewer rows.
     const int left = end - 1 - t;              // frames after the current one
-    const int r = grid ? lane >> 2 : lane >> 3;
-    const int rk = grid ? min(lane & 3, S - 1) : r == 0 ? k : 0;
-    const bool valid = r <= left;
-    const LT* row = c.base + static_cast<int64_t>(t - f0 + min(r, left)) * c.st + static_cast<int64_t>(rk) * c.ss;
-    const uint32_t a = sum_a + static_cast<uint32_t>(((t + r - f0) & mask) * S + rk) * 32u;
+    const int sh = L.n <= 32 ? 2 : L.n <= 128 ? 3 : 4, G = 1 << sh;
+    auto summary_at = [&](int q, int j) { return sum_a + static_cast<uint32_t>(((t + q - f0) & mask) * S + j) * 32u; };
+    auto pred_tok = [&](float y1, float xb, bool seen) { return (seen ? y1 : __fadd_rn(y1, __fmul_rn(c.lam, L.D))) >= xb; };   // (after a token most often at the root)
+    // where a row leads, as 4 * frame + row
+    auto next_at = [&](int q, int j, bool tk, int dur) {
+      if (tdt && (!tk || dur > 0)) return 4 * (q + max(dur, 1));
+      return tk && j + 1 < S ? 4 * q + j + 1 : 4 * q + 4;
+    };
+    // ---- the path: lane 4 q + j stands for row (t + q, j); lane 31 is where it leaves the window
+    int sel = 31, tok_before = -1;             // this lane's row on the path, and the lane of the last token before it
+    int plain_a;                               // where the best plain token of row (lane >> 2, lane & 3) leads
+    {
+      const int q = lane >> 2, j = lane & 3;
+      const uint32_t a = summary_at(q, min(j, S - 1));
+      const uint4 h1 = lds128(a + 16u), h0 = lds128(a);
+      plain_a = c.bound ? static_cast<int>(h1.y) : -1;
+      const float y1 = __uint_as_float(h0.x), xb = __uint_as_float(h0.z);
+      const int dur = tdt ? static_cast<int>(h1.z >> 24) : 0;
+      const bool tk_s = pred_tok(y1, xb, false), tk_0 = pred_tok(y1, xb, true);
+      uint32_t step = static_cast<uint32_t>(min(next_at(q, j, tk_s, dur), 31)) << 1 | (tk_s ? 1u : 0u) |
+                      static_cast<uint32_t>(min(next_at(q, j, tk_0, dur), 31)) << 17 | (tk_0 ? 1u << 16 : 0u);
+      if (lane == 31) step = 31u << 1 | 31u << 17;
+      int cur = k, last = -1, half = 0;
+      const int group = lane >> sh;
+#pragma unroll
+      for (int g = 0; g < 8; ++g) {
+        if (group == g) { sel = cur; tok_before = last; }
+        if (g == 7) break;
+        const uint32_t w = __shfl_sync(0xffffffffu, step, cur) >> half;
+        if (w & 1u) { last = cur; half = 16; }
+        cur = static_cast<int>((w >> 1) & 31u);
+      }
+    }
+    // ---- this lane's row, state and list
+    const int rq = sel >> 2, rj = min(sel & 3, S - 1);
+    const bool exists = sel != 31 && rq <= left;
+    const uint32_t a = summary_at(rq, rj);
     const uint4 q1 = lds128(a + 16u), q0 = lds128(a);
+    const int before = __shfl_sync(0xffffffffu, plain_a, tok_before & 31);
+    const int ls = tok_before >= 0 ? before : s;
+    TokList ll = L;
+    bool lane_ok = true;
+    if (ls != s) {
+      ll.n = 0; ll.D = 0.0f; ll.bmag = fabsf(c.lam) * c.R;
+      if (ls > 0) {
+        lane_ok = c.resolved && ls < c.n_states;
+        if (lane_ok) {
+          const uint4 rec = *reinterpret_cast<const uint4*>(c.rsrec + ls);
+          ll.ent = c.rsent + rec.x; ll.n = static_cast<int>(rec.y); ll.D = __uint_as_float(rec.z); ll.bmag = __uint_as_float(rec.w);
+          lane_ok = ll.n <= 8 * G;
+        }
+      }
+    }
+    if (!lane_ok || !exists) ll.n = 0;
+    const LT* row = c.base + static_cast<int64_t>(t - f0 + min(rq, left)) * c.st + static_cast<int64_t>(rj) * c.ss;
+    const float y1 = __uint_as_float(q0.x), y2b = __uint_as_float(q0.y), xb = __uint_as_float(q0.z), x1 = __uint_as_float(q0.w);
     const uint32_t id1x2 = 2u * (q1.z & kRsIdMask);
+    const int plain_next = c.bound ? static_cast<int>(q1.y) : -1;
     float lv = -INFINITY;
     uint32_t lt = none;
     bool in_deep = false;
-    {
-      const int step = grid ? 1 : 8;
 #pragma unroll 1
-      for (int i0 = grid ? 0 : lane & 7; i0 < L.n; i0 += 4 * step) {
-        uint2 e[4];
-        float x[4];
+    for (int i0 = lane & (G - 1); i0 < ll.n; i0 += 4 * G) {
+      uint2 e[4];
+      float x[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          e[u] = make_uint2(2u * static_cast<uint32_t>(V), 0xFF800000u);
-          if (i0 + u * step < L.n) e[u] = *reinterpret_cast<const uint2*>(L.ent + i0 + u * step);
-        }
+      for (int u = 0; u < 4; ++u) {
+        e[u] = make_uint2(2u * static_cast<uint32_t>(V), 0xFF800000u);
+        if (i0 + u * G < ll.n) e[u] = *reinterpret_cast<const uint2*>(ll.ent + i0 + u * G);
+      }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = LogitLoad<LT>::at(row + ((e[u].x & tmask) >> 1));
+      for (int u = 0; u < 4; ++u) x[u] = LogitLoad<LT>::at(row + ((e[u].x & tmask) >> 1));
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const uint32_t td = td_pack(e[u].x, tb);
-          const float v = __fadd_rn(x[u], __uint_as_float(e[u].y));
-          if (v > lv || (v == lv && td < lt)) { lv = v; lt = td; }
-          in_deep |= (e[u].x & tmask) == id1x2;
-        }
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t td = td_pack(e[u].x, tb);
+        const float v = __fadd_rn(x[u], __uint_as_float(e[u].y));
+        if (v > lv || (v == lv && td < lt)) { lv = v; lt = td; }
+        in_deep |= (e[u].x & tmask) == id1x2;
       }
     }
-    if (!grid) {
-      // the group's best (largest value, then lowest token), in all its lanes
-#pragma unroll
-      for (int off = 1; off <= 4; off <<= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, lv, off);
-        const uint32_t ot = __shfl_xor_sync(0xffffffffu, lt, off);
-        if (ov > lv || (ov == lv && ot < lt)) { lv = ov; lt = ot; }
-      }
-      in_deep = ((__ballot_sync(0xffffffffu, in_deep) >> (8 * r)) & 0xFFu) != 0u;
-    }
+    // the group's best (largest value, then lowest token), in all its lanes
+    auto join = [&](int off) {
+      const float ov = __shfl_xor_sync(0xffffffffu, lv, off);
+      const uint32_t ot = __shfl_xor_sync(0xffffffffu, lt, off);
+      if (ov > lv || (ov == lv && ot < lt)) { lv = ov; lt = ot; }
+    };
+    join(1); join(2);
+#pragma unroll 1
+    for (int off = 4; off < G; off <<= 1) join(off);
+    in_deep = ((__ballot_sync(0xffffffffu, in_deep) >> (lane & -G)) & ((1u << G) - 1u)) != 0u;
     // the row's pick: the best plain token is exact when the summary's winner is not listed and clears the others by the
     // rounding margin (at the root it is exact by construction); else it is bounded from above
-    const float y1 = __uint_as_float(q0.x), y2b = __uint_as_float(q0.y), xb = __uint_as_float(q0.z), x1 = __uint_as_float(q0.w);
     const float extra = __uint_as_float(q1.w);
-    const int id1 = static_cast<int>(id1x2 >> 1), dur = static_cast<int>(q1.z >> 24);
+    const int id1 = static_cast<int>(id1x2 >> 1), dur = tdt ? static_cast<int>(q1.z >> 24) : 0;
     float wv = lv;
     int wtok = td_tok(lt, tb), wnext = td_dst(lt, tb);
     bool rescan = (q1.z & (kRsOvf | kRsAbsent)) != 0;
     {
-      const bool plain_ok = !in_deep && ((q1.z & kRsGap) != 0 || s <= 0);
-      const float nd = __fadd_rn(x1, __fmul_rn(c.lam, __fadd_rn(L.D, __uint_as_float(q1.x))));
-      const float ub = (in_deep ? y2b : y1) + c.lam * L.D;
-      const float tau = (fabsf(y1) + 4.0f * L.bmag) * 3.814697265625e-6f + 1e-30f;
+      const bool plain_ok = !in_deep && ((q1.z & kRsGap) != 0 || ls <= 0);
+      const float nd = __fadd_rn(x1, __fmul_rn(c.lam, __fadd_rn(ll.D, __uint_as_float(q1.x))));
+      const float ub = (in_deep ? y2b : y1) + c.lam * ll.D;
+      const float tau = (fabsf(y1) + 4.0f * ll.bmag) * 3.814697265625e-6f + 1e-30f;
       rescan = rescan || (!plain_ok && !(fmaxf(wv, xb) > ub + tau));
-      if (plain_ok && (nd > wv || (nd == wv && id1 < wtok))) { wv = nd; wtok = id1; wnext = c.bound ? static_cast<int>(q1.y) : -1; }
+      if (plain_ok && (nd > wv || (nd == wv && id1 < wtok))) { wv = nd; wtok = id1; wnext = plain_next; }
     }
     const bool blank = !(wv >= xb);                            // (a tie with blank goes to the token)
-
-    int tok = V, tnext = s;                                    // the token that ends the round (V: none) and where it leads
-    if (grid) {
-      const bool ready = (lane & 3) < S && (r > 0 || (lane & 3) >= k) && valid && !rescan;
-      const unsigned ready_all = __ballot_sync(0xffffffffu, ready);
-      const unsigned blank_all = __ballot_sync(0xffffffffu, ready && blank);
-      const unsigned keep_all = __ballot_sync(0xffffffffu, wnext == s);
-      // Which rows the decode visits follows from the blank / token pattern alone while the state stays what it is: in a
-      // frame, row j is visited when rows 0 .. j-1 selected tokens (bit 4 q + j: row j of frame t + q).
-      const unsigned m1 = 0x11111111u;
-      const unsigned smask = S >= 4 ? 0xFFFFFFFFu : (m1 << S) - m1;
-      const unsigned pre = (1u << k) - 1u;
-      const unsigned tok_all = ready_all & ~blank_all;
-      const unsigned tokx = tok_all | pre;
-      const unsigned a0 = tokx & m1, a1 = (tokx >> 1) & m1, a2 = (tokx >> 2) & m1;
-      const unsigned vis = (m1 | (a0 << 1) | ((a0 & a1) << 2) | ((a0 & a1 & a2) << 3)) & smask & ~pre;
-      // the walk ends before a row that is not ready (or needs the exact evaluation) and after a token that changes the state
-      const unsigned bad = vis & (~ready_all | (tok_all & ~keep_all));
-      const int pb = bad ? __ffs(bad) - 1 : 32;
-      const bool last_tok = pb < 32 && ((tok_all >> (pb & 31)) & 1u);
-      const unsigned cm = (vis & (pb < 32 ? (1u << (pb & 31)) - 1u : 0xFFFFFFFFu)) | (last_tok ? 1u << (pb & 31) : 0u);
-      if (cm == 0u) { no_grid = true; continue; }              // (the current row needs the exact evaluation: a list round)
-      const unsigned tm = cm & tok_all, bm = cm & blank_all;
-      // frames closed: by a blank, or by a token in the frame's last row
-      const unsigned cl = bm | (tm & (m1 << (S - 1)));
-      const unsigned clf = (cl | (cl >> 1) | (cl >> 2) | (cl >> 3)) & m1;
-      const int fcl = __popc(clf);
-      const int pos = fcl < 8 ? __popc(((tm | (fcl == 0 ? pre : 0u)) >> (4 * (fcl & 7))) & 0xFu) : 0;
-      const unsigned upto = 0xFFFFFFFFu >> (31 - lane);
-      const bool mine_t = (tm >> lane) & 1u;
+    // ---- as far as the rows went as predicted, and the first that did not
+    const bool lead = (lane & (G - 1)) == 0, ready = lead && exists && lane_ok && !rescan;
+    const bool as_pred = blank ? !pred_tok(y1, xb, tok_before >= 0) : pred_tok(y1, xb, tok_before >= 0) && wnext == plain_next;
+    const unsigned ready_m = __ballot_sync(0xffffffffu, ready), blank_m = __ballot_sync(0xffffffffu, blank);
+    const unsigned bad = __ballot_sync(0xffffffffu, lead && !(ready && as_pred));
+    const unsigned cut = bad & (0u - bad);
+    const unsigned cm = ready_m & ((cut - 1u) | cut);          // (cut == 0: all)
+    int tok = V, tnext = s;                                    // where the round leads (tok == V: the state stays)
+    if (cm != 0u) {
+      const unsigned tm = cm & ~blank_m, upto = 0xFFFFFFFFu >> (31 - lane);
+      const bool mine = (cm >> lane) & 1u;
       const int ntok = n_out + __popc(tm & upto), nval = nv + __popc(cm & upto);
-      if (last_tok) { tok = __shfl_sync(0xffffffffu, wtok, pb & 31); tnext = __shfl_sync(0xffffffffu, wnext, pb & 31); }
-      if ((cm >> lane) & 1u) o.vals[nval - 1] = adjust(mine_t ? wv : xb, extra);
-      if (mine_t && ntok <= o.cap) {
-        o.tok[ntok - 1] = wtok; o.frm[ntok - 1] = t + r;
-        if (!SEG && o.dur) o.dur[ntok - 1] = 0;
+      const int after = blank ? ls : wnext, at = next_at(rq, rj, !blank, dur);
+      if (mine) {
+        o.vals[nval - 1] = adjust(blank ? xb : wv, extra);
+        if (!blank && ntok <= o.cap) {
+          o.tok[ntok - 1] = wtok; o.frm[ntok - 1] = t + rq;
+          if (!SEG && o.dur) o.dur[ntok - 1] = dur;
+        }
+        if ((at & 3) == 0) trace(t + rq + 1, after, ntok, nval);
       }
-      if ((cl >> lane) & 1u) trace(t + r + 1, (last_tok && lane == pb) ? tnext : s, ntok, nval);
       nv += __popc(cm);
       n_out += __popc(tm);
-      k = pos;
-      t += fcl;
-      if (last_tok) stable = false;
-    } else {
-      const unsigned m8 = 0x01010101u;                         // (bit 8 r: row r)
-      const unsigned valid_m = __ballot_sync(0xffffffffu, valid) & m8;
-      const unsigned blank_m = __ballot_sync(0xffffffffu, valid && !rescan && blank) & m8;
-      const unsigned resc_m = __ballot_sync(0xffffffffu, rescan) & m8;
-      // the blank rows visited (vm), and the row after them (frame t + j)
-      unsigned vm = 0u;
-      int j = 0;
-      if (!tdt) { const unsigned stop = ~blank_m & m8; j = stop ? (__ffs(stop) - 1) >> 3 : 4; vm = m8 & ((1u << (8 * j - (j == 4 ? 1 : 0))) - 1u); }
-      else
-#pragma unroll 1
-        while (j < 4 && ((blank_m >> (8 * j)) & 1u)) { vm |= 1u << (8 * j); j += max(__shfl_sync(0xffffffffu, dur, 8 * j), 1); }
-      const bool took = j < 4 && ((valid_m >> (8 * j)) & 1u);
-      const int jl = 8 * min(j, 3);
-      tok = took ? __shfl_sync(0xffffffffu, wtok, jl) : V;
-      tnext = took ? __shfl_sync(0xffffffffu, wnext, jl) : s;
-      float val = __shfl_sync(0xffffffffu, wv, jl);
-      float j_extra = __shfl_sync(0xffffffffu, extra, jl);
-      int j_dur = tdt ? __shfl_sync(0xffffffffu, dur, jl) : 0;
-      if (took && ((resc_m >> jl) & 1u)) {
-        const RowPick pk = exact_row(c, L, c.base + static_cast<int64_t>(t - f0 + j) * c.st + (j == 0 ? static_cast<int64_t>(k) * c.ss : 0), s, lane);
-        tok = pk.tok; tnext = pk.next; val = pk.val;
-        if (tdt) { j_dur = pk.dur; j_extra = pk.xdur; }
-      }
-      if ((vm >> lane) & 1u) {
-        o.vals[nv + __popc(vm & ((1u << lane) - 1u))] = adjust(xb, extra);
-        trace(t + r + 1, s, n_out, nv + r + 1);
-      }
-      nv += __popc(vm);
-      t += j;
-      if (j > 0) k = 0;
-      if (took) {
-        if (lane == 0) o.vals[nv] = adjust(val, j_extra);
-        ++nv;
-        bool closed = false;
-        if (tok == V) {                        // blank after all (exact evaluation)
-          t += tdt ? max(j_dur, 1) : 1;
-          k = 0; closed = true;
-        } else {
-          if (lane == 0 && n_out < o.cap) {
-            o.tok[n_out] = tok; o.frm[n_out] = t;
-            if (!SEG && o.dur) o.dur[n_out] = j_dur;
-          }
-          ++n_out;
-          if (tdt && j_dur > 0) { t += j_dur; k = 0; }
-          else if (++k == S) { ++t; k = 0; closed = true; }
-          stable = tnext == s;
+      const int hi = 31 - __clz(cm);
+      const int pos = __shfl_sync(0xffffffffu, at, hi);
+      tnext = __shfl_sync(0xffffffffu, after, hi);
+      if (tnext != s) tok = 0;
+      t += pos >> 2;
+      k = pos & 3;
+    } else {                                                   // the current row, in full
+      const RowPick pk = exact_row(c, L, c.base + static_cast<int64_t>(t - f0) * c.st + static_cast<int64_t>(k) * c.ss, s, lane);
+      tok = pk.tok; tnext = pk.next;
+      if (lane == 0) o.vals[nv] = adjust(pk.val, tdt ? pk.xdur : extra);
+      ++nv;
+      if (tok != V) {
+        if (lane == 0 && n_out < o.cap) {
+          o.tok[n_out] = tok; o.frm[n_out] = t;
+          if (!SEG && o.dur) o.dur[n_out] = pk.dur;
         }
-        if (closed && lane == 0) trace(t, tnext, n_out, nv);
+        ++n_out;
       }
+      const int at = next_at(0, k, tok != V, pk.dur);
+      if (lane == 0 && (at & 3) == 0) trace(t + 1, tnext, n_out, nv);
+      t += at >> 2;
+      k = at & 3;
     }
     if (tok != V && tnext != s && c.bound) {
       if (tnext < 0 || tnext >= c.n_states) { if (lane == 0) atomicOr(c.status, TB_STATUS_BAD_STATE); tnext = 0; }
@@ -787,7 +808,7 @@ __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const
     }
   }
   if (SEG) asm volatile("cp.async.wait_all;" ::: "memory");
-  cu.t = t; cu.k = k; cu.s = s; cu.n_out = n_out; cu.nv = nv; cu.stable = stable; cu.listed = listed; cu.list = L;
+  cu.t = t; cu.k = k; cu.s = s; cu.n_out = n_out; cu.nv = nv; cu.listed = listed; cu.list = L;
 }
 
 }  // namespace
