@@ -296,6 +296,7 @@ struct tb_batch {
   std::vector<int32_t> slot_cache_bytes;               // bytes of the sections the pipelined kernel caches
   std::vector<uint8_t> slot_resolved;                  // the bound graph carries resolved per-state lists (1 for an unbound slot)
   std::vector<int32_t> slot_n_states;
+  std::vector<float> slot_root_span;                    // tb_graph::root_span of the bound graph
   // models registered ahead of a session (Sec. 2.2 para. 5, decoder-level registration): uploaded once, bound to
   // slots by id without a copy
   struct Model {
@@ -304,6 +305,7 @@ struct tb_batch {
     TbSlotRec rec;
     int32_t n_states = 0, cache_bytes = 0, users = 0;
     uint8_t resolved = 1;
+    float root_span = 0.0f;
   };
   std::vector<Model> models;
   TbSlotRec* d_model_recs = nullptr;                   // the registered models' records on the device, by model id
@@ -383,6 +385,7 @@ extern "C" int tb_batch_create(int32_t vocab, const int32_t* case_class, int32_t
   b->slot_cache_bytes.assign(n_slots, 0);
   b->slot_resolved.assign(n_slots, 1);
   b->slot_n_states.assign(n_slots, 0);
+  b->slot_root_span.assign(n_slots, 0.0f);
   b->slot_model.assign(n_slots, -1);
   bool ok = true;
   ok = ok && cudaMalloc(&b->arena, b->arena_bytes) == cudaSuccess;
@@ -587,7 +590,7 @@ extern "C" int tb_batch_bind_stream(tb_batch* b, int32_t slot, const tb_graph* g
   if (rc != TB_OK) { if (bytes) b->alloc.release(off, bytes); return rc; }
   release_slot(b, slot);
   b->slot_block[slot] = {off, bytes};
-  b->slot_n_states[slot] = g ? g->n_states : 0;
+  b->slot_n_states[slot] = g ? g->n_states : 0; b->slot_root_span[slot] = g ? g->root_span() : 0.0f;
   b->slot_cache_bytes[slot] = !g ? 0 : cache_bytes_of(g);
   b->slot_resolved[slot] = (!g || g->n_rsent >= 0) ? 1 : 0;
   rc = resolve_lists(b, b->d_slots, 1, &slot, &g, stream);
@@ -727,7 +730,7 @@ extern "C" int tb_batch_bind_streams(tb_batch* b, int32_t n, const int32_t* slot
     const tb_graph* g = graphs[i];
     release_slot(b, slots[i]);
     b->slot_block[slots[i]] = blocks[i];
-    b->slot_n_states[slots[i]] = g ? g->n_states : 0;
+    b->slot_n_states[slots[i]] = g ? g->n_states : 0; b->slot_root_span[slots[i]] = g ? g->root_span() : 0.0f;
     b->slot_cache_bytes[slots[i]] = !g ? 0 : cache_bytes_of(g);
     b->slot_resolved[slots[i]] = (!g || g->n_rsent >= 0) ? 1 : 0;
   }
@@ -788,7 +791,7 @@ static bool prepare_pulled_binds(tb_batch* b, int32_t n, const int32_t* slots, c
     }
     release_slot(b, slots[i]);                       // (after the group's room was taken: the new blocks are none of the old)
     b->slot_block[slots[i]] = block;
-    b->slot_n_states[slots[i]] = g ? g->n_states : 0;
+    b->slot_n_states[slots[i]] = g ? g->n_states : 0; b->slot_root_span[slots[i]] = g ? g->root_span() : 0.0f;
     b->slot_cache_bytes[slots[i]] = !g ? 0 : cache_bytes_of(g);
     b->slot_resolved[slots[i]] = (!g || g->n_rsent >= 0) ? 1 : 0;
   }
@@ -807,7 +810,7 @@ extern "C" int tb_batch_register_model(tb_batch* b, const tb_graph* g, int32_t* 
   int rc;
   rc = upload_graph(b, g, static_cast<cudaStream_t>(stream_), &m.off, &m.bytes, &m.rec);
   if (rc != TB_OK) return rc;
-  m.live = true; m.n_states = g->n_states; m.cache_bytes = cache_bytes_of(g); m.resolved = g->n_rsent >= 0 ? 1 : 0;
+  m.live = true; m.n_states = g->n_states; m.cache_bytes = cache_bytes_of(g); m.resolved = g->n_rsent >= 0 ? 1 : 0; m.root_span = g->root_span();
   int32_t id = -1;
   for (size_t i = 0; i < b->models.size(); ++i)
     if (!b->models[i].live) { id = static_cast<int32_t>(i); break; }
@@ -868,7 +871,7 @@ extern "C" int tb_batch_bind_models(tb_batch* b, int32_t n, const int32_t* slots
         b->models[m].users++;
         b->slot_model[slot] = m;
         b->slot_n_states[slot] = b->models[m].n_states; b->slot_cache_bytes[slot] = b->models[m].cache_bytes;
-        b->slot_resolved[slot] = b->models[m].resolved;
+        b->slot_resolved[slot] = b->models[m].resolved; b->slot_root_span[slot] = b->models[m].root_span;
       } else {
         b->slot_n_states[slot] = 0; b->slot_cache_bytes[slot] = 0; b->slot_resolved[slot] = 1;
       }
@@ -894,7 +897,7 @@ extern "C" int tb_batch_bind_model(tb_batch* b, int32_t slot, int32_t model_id, 
     const tb_batch::Model& m = b->models[model_id];
     b->models[model_id].users++;
     b->slot_model[slot] = model_id;
-    b->slot_n_states[slot] = m.n_states; b->slot_cache_bytes[slot] = m.cache_bytes; b->slot_resolved[slot] = m.resolved;
+    b->slot_n_states[slot] = m.n_states; b->slot_cache_bytes[slot] = m.cache_bytes; b->slot_resolved[slot] = m.resolved; b->slot_root_span[slot] = m.root_span;
   } else {
     b->slot_n_states[slot] = 0; b->slot_cache_bytes[slot] = 0; b->slot_resolved[slot] = 1;
   }
@@ -940,13 +943,14 @@ static bool is_capturing(cudaStream_t stream) {
   if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) { cudaGetLastError(); return false; }
   return cap != cudaStreamCaptureStatusNone;
 }
-struct SlotSummary { int32_t max_cache = 0, max_states = 0, all_resolved = 1; };
+struct SlotSummary { int32_t max_cache = 0, max_states = 0, all_resolved = 1; float root_span = 0.0f; };
 static SlotSummary slot_summary(const tb_batch* b, int32_t n) {
   SlotSummary r;
   for (int32_t i = 0; i < n; ++i) {
     r.max_cache = b->slot_cache_bytes[i] > r.max_cache ? b->slot_cache_bytes[i] : r.max_cache;
     r.max_states = b->slot_n_states[i] > r.max_states ? b->slot_n_states[i] : r.max_states;
     if (!b->slot_resolved[i]) r.all_resolved = 0;
+    if (b->slot_n_states[i] && b->slot_root_span[i] > r.root_span) r.root_span = b->slot_root_span[i];
   }
   return r;
 }
@@ -991,7 +995,7 @@ extern "C" int tb_greedy_decode(tb_batch* b, const void* logits, int dtype, int3
     query_device(b);
     TbRowsPlan rplan;
     auto run_rows = [&]() -> bool {
-      if (!tb_rows_plan(p, max_cache, max_states, all_resolved, b->n_sm, b->max_smem, &rplan)) return false;
+      if (!tb_rows_plan(p, max_cache, max_states, all_resolved, sl.root_span, b->n_sm, b->max_smem, &rplan)) return false;
       if (!grow_scratch(b, &b->rows_scratch, &b->rows_scratch_bytes, rplan.scratch_bytes, capturing)) return false;
       rc = tb_launch_rows(p, rplan, b->n_sm, b->rows_scratch, stream);
       if (rc == TB_OK) { b->last_kernel = TB_KERNEL_GENERAL; b->last_NB = 1; b->last_G = 0; }

@@ -70,6 +70,15 @@ struct tb_graph {
   std::atomic<int32_t> refs{1};                        // holders: the caller's handle, one per cache that keeps the graph, one per copy in flight
   bool pinned = false;                                 // the blob's pages are locked (it sits in the pool, or tb_graph_pin registered it): binds copy straight from it
   bool registered = false;                             // ... by tb_graph_pin: to be unregistered
+  // from the lowest to the highest of {0, lambda * root arc weight}
+  float root_span() const {
+    float lo = 0.0f, hi = 0.0f;
+    for (int32_t a = state_arc_begin.empty() ? 0 : state_arc_begin[0]; !state_arc_begin.empty() && a < state_arc_begin[1]; ++a) {
+      const float b = lambda * arc_w[a];
+      lo = b < lo ? b : lo; hi = b > hi ? b : hi;
+    }
+    return hi - lo;
+  }
   // bytes the graph takes in the arena: the image and, behind it, room for the entries of the resolved lists (which the
   // device fills; 16 bytes more so that vector loads may overrun)
   size_t arena_bytes() const { return blob.size() + (n_rsent >= 0 ? 8 * static_cast<size_t>(n_rsent) + 16 : 0); }

@@ -106,10 +106,11 @@ int tb_launch_greedy_seg(const TbDecodeParams& p, int32_t max_cache_bytes, const
 // The two-step kernels (tb_rows.cu): any vocabulary, fp32 or bf16, any strides with contiguous tokens, S <= 4.
 struct TbRowsPlan {
   int32_t nseg = 0, cache_bytes = 0, smem = 0, all_resolved = 0;
+  float root_span = 0.0f;      // largest span of root boosts among the streams' graphs (tb_graph::root_span)
   size_t scratch_bytes = 0;
 };
-bool tb_rows_plan(const TbDecodeParams& p, int32_t max_cache_bytes, int32_t max_states, int32_t all_resolved, int32_t n_sm,
-                  int32_t max_smem, TbRowsPlan* plan);
+bool tb_rows_plan(const TbDecodeParams& p, int32_t max_cache_bytes, int32_t max_states, int32_t all_resolved, float root_span,
+                  int32_t n_sm, int32_t max_smem, TbRowsPlan* plan);
 int tb_launch_rows(const TbDecodeParams& p, const TbRowsPlan& plan, int32_t n_sm, void* scratch, cudaStream_t stream);
 // One streaming chunk.  spill: device memory of tb_chunk_rows_spill_bytes, needed when a slot's graph has no resolved
 // lists (else null).  Returns 1 when the call is outside what the kernel covers.

@@ -58,6 +58,7 @@ __device__ __forceinline__ RowCtx row_ctx(const TbDecodeParams& p, const TbSlotR
   h.boosts = root.stats[2] > 0.0f;
   h.norm = p.normalize != 0;
   h.V = p.V; h.n_dur = p.n_dur;
+  h.boost_a = 0u;
   return h;
 }
 template <typename LT>
@@ -84,8 +85,8 @@ __device__ __forceinline__ DecideCtx<LT> decide_ctx(const TbDecodeParams& p, con
 // ---- step 1 -------------------------------------------------------------------------------------------------------
 // Bound by HBM for wide rows (16 KB a row at V = 8192), by instruction issue for narrow ones.  A block reduces a stretch
 // of frames of one stream, so that its root tables are built once for them; warp w takes frames w, w + 8, ... of it.
-template <typename LT, int G>
-__global__ void __launch_bounds__(kSumThreads) k_row_sums(const __grid_constant__ RowsParams P) {
+template <typename LT, int G, bool TAB>
+__global__ void __launch_bounds__(kSumThreads, G == 4 ? 3 : 2) k_row_sums(const __grid_constant__ RowsParams P) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ float part[3 * kSumThreads / 32];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -100,9 +101,15 @@ __global__ void __launch_bounds__(kSumThreads) k_row_sums(const __grid_constant_
   const GraphPtrs g = graph_of(p.arena, rec);
   const RootTab root = root_tab_at(dyn, p.C);
   root_tab_fill(root, g, rec.n_states > 0, rec.lambda, p.C, part);
-  const RowCtx h = row_ctx(p, rec, g, root);
+  RowCtx h = row_ctx(p, rec, g, root);
+  if (TAB) {
+    unsigned char* tab = dyn + root_tab_bytes(p.C);
+    boost_tab_fill<LT>(tab, root, p.cls, h.lam, p.V);
+    h.boost_a = shared_u32(tab);
+    __syncthreads();
+  }
   if (warp < nf)
-    frames_summary<LT, G>(h, reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(b) * p.sb, p.st, p.ss, p.S, f0 + warp, kWarps,
+    frames_summary<LT, G, TAB>(h, reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(b) * p.sb, p.st, p.ss, p.S, f0 + warp, kWarps,
                           (nf - warp + kWarps - 1) / kWarps, P.sums + static_cast<int64_t>(b) * p.frames * p.S, -1, lane);
 }
 
@@ -364,7 +371,7 @@ __global__ void __launch_bounds__(kChunkThreads, 3) k_chunk_rows(const __grid_co
   for (int f0 = t0; f0 < end; f0 += kPiece) {
     const int f1 = min(f0 + kPiece, end), ff = max(t, f0);   // (frames behind the cursor are not looked at)
     if (ff + warp < f1)
-      frames_summary<LT, 4>(h, base, p.st, p.ss, S, ff - t0 + warp, nwarps, (f1 - ff - warp + nwarps - 1) / nwarps, sums, kPiece - 1, lane);
+      frames_summary<LT, 4, false>(h, base, p.st, p.ss, S, ff - t0 + warp, nwarps, (f1 - ff - warp + nwarps - 1) / nwarps, sums, kPiece - 1, lane);
     __syncthreads();
     if (warp == 0) {
       if (cu.t < f1) {
@@ -422,7 +429,7 @@ RowsLayout rows_layout(const TbDecodeParams& d, int nseg, bool all_resolved) {
 
 }  // namespace
 
-bool tb_rows_plan(const TbDecodeParams& d, int32_t max_cache_bytes, int32_t max_states, int32_t all_resolved, int32_t n_sm,
+bool tb_rows_plan(const TbDecodeParams& d, int32_t max_cache_bytes, int32_t max_states, int32_t all_resolved, float root_span, int32_t n_sm,
                   int32_t max_smem, TbRowsPlan* plan) {
   if (d.persistent || d.n_dur != 0 || n_sm < 1 || !rows_apply(d, max_states)) return false;
   int nseg = static_cast<int>(d.frames / 12);
@@ -433,7 +440,7 @@ bool tb_rows_plan(const TbDecodeParams& d, int32_t max_cache_bytes, int32_t max_
   int smem = dec_smem(d.V, d.C, d.S, d.frames, nseg, cache, all_resolved == 0).total;
   if (smem > max_smem / per_sm - 2048) { cache = 0; smem = dec_smem(d.V, d.C, d.S, d.frames, nseg, 0, all_resolved == 0).total; }
   if (smem > max_smem - 2048) return false;
-  plan->nseg = nseg; plan->cache_bytes = cache; plan->smem = smem; plan->all_resolved = all_resolved;
+  plan->nseg = nseg; plan->cache_bytes = cache; plan->smem = smem; plan->all_resolved = all_resolved; plan->root_span = root_span;
   plan->scratch_bytes = rows_layout(d, nseg, all_resolved != 0).total;
   return true;
 }
@@ -461,10 +468,18 @@ int tb_launch_rows(const TbDecodeParams& d, const TbRowsPlan& plan, int32_t n_sm
   P.frames_per_warp = static_cast<int32_t>(per);
   // a row of up to 128 blocks of 16 bytes is one group of four per lane, a wider one takes groups of eight
   const bool narrow = d.V * (d.dtype == TB_BF16 ? 2 : 4) <= 128 * 16 + 15;
-  void (*f1)(RowsParams) = d.dtype == TB_BF16 ? (narrow ? k_row_sums<uint16_t, 4> : k_row_sums<uint16_t, 8>)
-                                              : (narrow ? k_row_sums<float, 4> : k_row_sums<float, 8>);
+  // The table of root boosts, where boosts beyond a nat or two make candidates of hundreds of tokens (64 x 750 rows of three
+  // with text lists, boosts of 2 to 3 nats, 125 to 440 candidates: 326 us without, 149 with it; boosts of one nat, 18
+  // candidates: 93 without, 118 with it), a block has rows to use it on, and two blocks' tables leave L1 its half of an SM.
+  const size_t tab = d.dtype == TB_BF16 ? BoostTab<uint16_t>::bytes(d.V) : BoostTab<float>::bytes(d.V);
+  const bool with_tab = plan.root_span > 1.5f && per >= 2 && tab <= 40 * 1024;
+  void (*f1)(RowsParams);
+  if (d.dtype == TB_BF16)
+    f1 = narrow ? (with_tab ? k_row_sums<uint16_t, 4, true> : k_row_sums<uint16_t, 4, false>) : with_tab ? k_row_sums<uint16_t, 8, true> : k_row_sums<uint16_t, 8, false>;
+  else
+    f1 = narrow ? (with_tab ? k_row_sums<float, 4, true> : k_row_sums<float, 4, false>) : with_tab ? k_row_sums<float, 8, true> : k_row_sums<float, 8, false>;
   void (*f2)(RowsParams) = d.dtype == TB_BF16 ? k_decide_rows<uint16_t> : k_decide_rows<float>;
-  const size_t smem1 = root_tab_bytes(d.C);
+  const size_t smem1 = root_tab_bytes(d.C) + (with_tab ? tab : 0);
   if (smem1 > 24 * 1024 && cudaFuncSetAttribute(f1, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem1)) != cudaSuccess) {
     cudaGetLastError();
     return TB_ERR_CUDA;

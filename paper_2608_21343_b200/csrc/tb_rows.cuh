@@ -57,6 +57,13 @@ __device__ __forceinline__ float order_key_inv(uint32_t k) {
   return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xFFFFFFFFu));
 }
 
+__device__ __forceinline__ uint4 lds128(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t shared_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
+
 // ---- the graph's root in shared memory: weight and arc per class -------------------------------------------------
 struct RootTab {
   float* w;          // [C] root arc weight (0 if none)
@@ -118,6 +125,7 @@ struct RowCtx {
   const float* arc_w; const int32_t* arc_dst;    // the root's arcs
   float lam, beta_min, beta_max, bmag_max;       // bmag_max: bound on |lambda| * (|D(s)| + largest root weight) over all states s
   bool boosts, norm;                             // the root has arcs; the row's normaliser is wanted
+  uint32_t boost_a;                              // shared address of the table of root boosts per token (BoostTab; TAB only)
   int V, n_dur;
 };
 
@@ -149,6 +157,17 @@ template <> struct RowBlock<uint16_t> {          // eight bf16 each
     }
     return r;
   }
+  // the same for root-boosted values: cb holds a block's boosts, rounded up
+  static __device__ __forceinline__ uint32_t boost(float cb) { return __bfloat16_as_ushort(__float2bfloat16_ru(cb)); }
+  static constexpr float kBoostSlack = 0.0078125f;   // of |value| + largest boost: the roundings of the boost and of the sum
+  static __device__ __forceinline__ uint32_t hits_boosted(const uint4& q, const uint4& cb, int u, float t) {
+    const __nv_bfloat162 t2 = __float2bfloat162_rn(t);
+    uint32_t r = __hge2_mask(__hadd2(h2(q.x), h2(cb.x)), t2) & (0x00010001u << (4 * u));
+    r |= __hge2_mask(__hadd2(h2(q.y), h2(cb.y)), t2) & (0x00010001u << (4 * u + 1));
+    r |= __hge2_mask(__hadd2(h2(q.z), h2(cb.z)), t2) & (0x00010001u << (4 * u + 2));
+    r |= __hge2_mask(__hadd2(h2(q.w), h2(cb.w)), t2) & (0x00010001u << (4 * u + 3));
+    return r;
+  }
   static __device__ __forceinline__ int unit(int bit) { return (bit & 15) >> 2; }
   static __device__ __forceinline__ int elem(int bit) { return (bit & 3) * 2 + (bit >> 4); }
   template <typename F> static __device__ __forceinline__ void each2(const uint4& q, F f) {
@@ -176,6 +195,14 @@ template <> struct RowBlock<float> {             // four floats each
       for (int i = 0; i < 4; ++i) r |= __uint_as_float((&q[u].x)[i]) >= t ? 1u << (4 * u + i) : 0u;
     return r;
   }
+  static __device__ __forceinline__ uint32_t boost(float cb) { return __float_as_uint(cb); }
+  static constexpr float kBoostSlack = 0.0f;
+  static __device__ __forceinline__ uint32_t hits_boosted(const uint4& q, const uint4& cb, int u, float t) {
+    uint32_t r = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r |= __fadd_rn(__uint_as_float((&q.x)[i]), __uint_as_float((&cb.x)[i])) >= t ? 1u << (4 * u + i) : 0u;
+    return r;
+  }
   static __device__ __forceinline__ int unit(int bit) { return bit >> 2; }
   static __device__ __forceinline__ int elem(int bit) { return bit & 3; }
   template <typename F> static __device__ __forceinline__ void each2(const uint4& q, F f) {
@@ -188,6 +215,32 @@ __device__ __forceinline__ float exp2_approx(float x) {
   return y;
 }
 
+// The root boost of every token, in the rows' element type, once for each way a row may be aligned: copy h begins with token
+// h, so that the boosts of a row's aligned 16-byte blocks are aligned blocks themselves.  With it a row's candidates are the
+// tokens whose root-boosted value reaches the row's raw maximum: three or four, where the tokens within the largest boost
+// of the maximum are hundreds when boosts are several nats (lists of text, weighted by the length of a piece).
+template <typename LT>
+struct BoostTab {
+  static __host__ __device__ constexpr size_t copy_bytes(int V) { return (static_cast<size_t>(V) * sizeof(LT) + 31) & ~size_t(15); }
+  static __host__ __device__ constexpr size_t bytes(int V) { return 16 / sizeof(LT) * copy_bytes(V); }
+};
+// Block-wide, after root_tab_fill; the caller's next barrier completes it.
+template <typename LT>
+__device__ __forceinline__ void boost_tab_fill(unsigned char* tab, const RootTab& r, const int32_t* cls, float lam, int V) {
+  using RB = RowBlock<LT>;
+  const size_t stride = BoostTab<LT>::copy_bytes(V);
+#pragma unroll 1
+  for (int v = threadIdx.x; v < V; v += blockDim.x) {
+    const uint32_t cb = RB::boost(__fmul_rn(lam, r.w[__ldg(cls + v)]));
+#pragma unroll
+    for (int h = 0; h < RB::E; ++h)
+      if (v >= h) {
+        if constexpr (sizeof(LT) == 2) reinterpret_cast<uint16_t*>(tab + h * stride)[v - h] = static_cast<uint16_t>(cb);
+        else reinterpret_cast<uint32_t*>(tab + h * stride)[v - h] = cb;
+      }
+  }
+}
+
 // The rows of up to 32 frames by one warp: frames f0, f0 + step, ... (n of them), row k of a frame only when row k - 1 is
 // likely to select a token (its best root-boosted token reaches the blank less a margin); a row left out is marked
 // kRsAbsent, and a decider that gets there after all evaluates it exactly.  About half the rows of three per frame are
@@ -198,7 +251,10 @@ __device__ __forceinline__ float exp2_approx(float x) {
 // after the last aligned block are one per lane; nothing outside the row is read.  The next row's blocks are requested
 // before a row's candidates are looked at, where a row is one group.  What is the same for all lanes is kept by lane i
 // for frame i and finished for all frames of a pass at once (root arcs, normalisers, durations, the store).
-template <typename LT, int G>
+//
+// TAB: the candidates come from the table of root boosts (h.boost_a); else they are the tokens within the largest boost of
+// the row's maximum.
+template <typename LT, int G, bool TAB>
 __device__ __forceinline__ void frames_summary(const RowCtx& h, const LT* base, int64_t st, int64_t ss, int S, int f0, int step, int n,
                                                RowSum* sums, int fmask, int lane) {
   using RB = RowBlock<LT>;
@@ -256,6 +312,10 @@ __device__ __forceinline__ void frames_summary(const RowCtx& h, const LT* base, 
       // keeps a strict margin over all roundings
       const float gamma = (fabsf(mf) + fabsf(h.beta_max) + fabsf(h.beta_min)) * 0.0009765625f + 1e-30f;
       const float thr = RB::threshold(__fsub_rn(__fsub_rn(mf, __fsub_rn(h.beta_max, h.beta_min)), gamma));
+      // tokens that are no candidates have root-boosted values of at most `others`: x < thr, hence <= fl(thr + beta_max); or,
+      // TAB, by their boosted values themselves (some token's reaches mf + beta_min)
+      const float others = TAB ? __fsub_rn(__fadd_rn(mf, h.beta_min), gamma) : __fadd_rn(thr, h.beta_max);
+      const float thr_b = TAB ? RB::threshold(__fsub_rn(others, RB::kBoostSlack * (fabsf(mf) + h.beta_max - h.beta_min))) : 0.0f;
       // L = M + log(sum_v exp(x_v - M)): one fused multiply-add and one exponential per entry, see tb_fast_common.cuh
       float M = 0.0f, acc0 = 0.0f, acc1 = 0.0f;
       if (h.norm) M = fmaxf(mf, LogitLoad<LT>::at(rowi + V));
@@ -278,8 +338,19 @@ __device__ __forceinline__ void frames_summary(const RowCtx& h, const LT* base, 
               acc1 = __fadd_rn(acc1, exp2_approx(__fmaf_rn(x1, kL2e, nc)));
             });
         }
-        uint32_t hits = RB::template hits<G>(q, 0, thr), hits2 = 0u;
-        if constexpr (RB::kUnits < G) hits2 = RB::template hits<G>(q, RB::kUnits, thr);
+        uint32_t hits = 0u, hits2 = 0u;
+        if constexpr (TAB) {
+          const uint32_t at = h.boost_a + static_cast<uint32_t>(hdi) * static_cast<uint32_t>(BoostTab<LT>::copy_bytes(V)) + 16u * (g + lane);
+#pragma unroll
+          for (int u = 0; u < G; ++u)
+            if (g + 32 * u + lane < nbi) {
+              const uint4 cb = lds128(at + 512u * u);
+              if (u < RB::kUnits) hits |= RB::hits_boosted(q[u], cb, u, thr_b); else hits2 |= RB::hits_boosted(q[u], cb, u - RB::kUnits, thr_b);
+            }
+        } else {
+          hits = RB::template hits<G>(q, 0, thr);
+          if constexpr (RB::kUnits < G) hits2 = RB::template hits<G>(q, RB::kUnits, thr);
+        }
         if (g == 0 && inext >= 0) {                            // (q is free: the next row is on its way from here on)
           begin(inext);
           load(0);
@@ -306,13 +377,12 @@ __device__ __forceinline__ void frames_summary(const RowCtx& h, const LT* base, 
         for (int off = 16; off > 0; off >>= 1) acc = __fadd_rn(acc, __shfl_xor_sync(0xffffffffu, acc, off));
         if (lane == i) { m_M = M; m_acc = acc; }
       }
-      // across the warp: best (value, lowest id) and the runner-up value; tokens that are not candidates have x < thr,
-      // hence a root-boosted value <= fl(thr + beta_max)
+      // across the warp: best (value, lowest id) and the runner-up value
       const uint32_t key = order_key(b.v);
       const uint32_t kmax = __reduce_max_sync(0xffffffffu, key);
       const int idmin = static_cast<int>(__reduce_min_sync(0xffffffffu, key == kmax ? static_cast<uint32_t>(b.i) : 0x7FFFFFFFu));
       const uint32_t k2 = __reduce_max_sync(0xffffffffu, order_key((key == kmax && b.i == idmin) ? sec : b.v));
-      if (lane == i) { m_y1 = order_key_inv(kmax); m_id = idmin; m_y2 = fmaxf(order_key_inv(k2), __fadd_rn(thr, h.beta_max)); }
+      if (lane == i) { m_y1 = order_key_inv(kmax); m_id = idmin; m_y2 = fmaxf(order_key_inv(k2), others); }
       i = inext;
     }
     // ---- lane i finishes frame i's row
@@ -356,12 +426,6 @@ __device__ __forceinline__ void frames_summary(const RowCtx& h, const LT* base, 
 }
 
 // ---- step 2: the decider -------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint4 lds128(uint32_t a) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
-  return v;
-}
-__device__ __forceinline__ uint32_t shared_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
 // What a decider needs to know about its stream's graph and rows; the same for all lanes.
 template <typename LT>
