@@ -672,6 +672,7 @@ __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const
   const bool tdt = !SEG && c.n_dur > 0;
   int t = cu.t, k = cu.k, s = cu.s, n_out = cu.n_out, nv = cu.nv;
   bool listed = cu.listed;
+  int still = 0;                               // tokens in a row that left the (non-root) state what it was
   TokList L = cu.list;
   const uint32_t none = (2u * static_cast<uint32_t>(V)) << (32 - tb), tmask = (1u << tb) - 1u;
   // what a row adds to the score: its value less its normaliser, or plus its duration's logit
@@ -715,7 +716,10 @@ __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const
     const int left = end - 1 - t;              // frames after the current one
     const int sh = L.n <= 32 ? 2 : L.n <= 128 ? 3 : 4, G = 1 << sh;
     auto summary_at = [&](int q, int j) { return sum_a + static_cast<uint32_t>(((t + q - f0) & mask) * S + j) * 32u; };
-    auto pred_tok = [&](float y1, float xb, bool seen) { return (seen ? y1 : __fadd_rn(y1, __fmul_rn(c.lam, L.D))) >= xb; };   // (after a token most often at the root)
+    // (after a token the state is the root most often; one that has repeated itself, as lists with repeated tokens make a
+    // state do for hundreds of frames, is taken to go on doing so)
+    const bool stay = still >= 4;
+    auto pred_tok = [&](float y1, float xb, bool seen) { return stay || (seen ? y1 : __fadd_rn(y1, __fmul_rn(c.lam, L.D))) >= xb; };
     // where a row leads, as 4 * frame + row
     auto next_at = [&](int q, int j, bool tk, int dur) {
       if (tdt && (!tk || dur > 0)) return 4 * (q + max(dur, 1));
@@ -752,7 +756,7 @@ __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const
     const uint32_t a = summary_at(rq, rj);
     const uint4 q1 = lds128(a + 16u), q0 = lds128(a);
     const int before = __shfl_sync(0xffffffffu, plain_a, tok_before & 31);
-    const int ls = tok_before >= 0 ? before : s;
+    const int ls = tok_before >= 0 && !stay ? before : s;
     TokList ll = L;
     bool lane_ok = true;
     if (ls != s) {
@@ -770,7 +774,7 @@ __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const
     const LT* row = c.base + static_cast<int64_t>(t - f0 + min(rq, left)) * c.st + static_cast<int64_t>(rj) * c.ss;
     const float y1 = __uint_as_float(q0.x), y2b = __uint_as_float(q0.y), xb = __uint_as_float(q0.z), x1 = __uint_as_float(q0.w);
     const uint32_t id1x2 = 2u * (q1.z & kRsIdMask);
-    const int plain_next = c.bound ? static_cast<int>(q1.y) : -1;
+    const int plain_next = c.bound ? static_cast<int>(q1.y) : -1, pred_next = stay ? s : plain_next;
     float lv = -INFINITY;
     uint32_t lt = none;
     bool in_deep = false;
@@ -821,7 +825,7 @@ __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const
     const bool blank = !(wv >= xb);                            // (a tie with blank goes to the token)
     // ---- as far as the rows went as predicted, and the first that did not
     const bool lead = (lane & (G - 1)) == 0, ready = lead && exists && lane_ok && !rescan;
-    const bool as_pred = blank ? !pred_tok(y1, xb, tok_before >= 0) : pred_tok(y1, xb, tok_before >= 0) && wnext == plain_next;
+    const bool as_pred = blank ? !pred_tok(y1, xb, tok_before >= 0) : pred_tok(y1, xb, tok_before >= 0) && wnext == pred_next;
     const unsigned ready_m = __ballot_sync(0xffffffffu, ready), blank_m = __ballot_sync(0xffffffffu, blank);
     const unsigned bad = __ballot_sync(0xffffffffu, lead && !(ready && as_pred));
     const unsigned cut = bad & (0u - bad);
@@ -845,12 +849,14 @@ __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const
       const int hi = 31 - __clz(cm);
       const int pos = __shfl_sync(0xffffffffu, at, hi);
       tnext = __shfl_sync(0xffffffffu, after, hi);
+      still = s > 0 && tnext == s && ((tm >> hi) & 1u) ? still + __popc(tm) : 0;
       if (tnext != s) tok = 0;
       t += pos >> 2;
       k = pos & 3;
     } else {                                                   // the current row, in full
       const RowPick pk = exact_row(c, L, c.base + static_cast<int64_t>(t - f0) * c.st + static_cast<int64_t>(k) * c.ss, s, lane);
       tok = pk.tok; tnext = pk.next;
+      still = s > 0 && tok != V && tnext == s ? still + 1 : 0;
       if (lane == 0) o.vals[nv] = adjust(pk.val, tdt ? pk.xdur : extra);
       ++nv;
       if (tok != V) {
