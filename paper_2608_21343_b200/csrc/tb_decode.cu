@@ -1278,6 +1278,7 @@ __global__ void __launch_bounds__(kTopWarps * 32) k_beam_topm(const LT* logits, 
                                                             int64_t stream_stride, int64_t frame_stride, int64_t row_stride,
                                                             const int32_t* n_frames, const TbSlotRec* slots, const unsigned char* arena,
                                                             const int32_t* cls, int32_t top_m, TbTopEnt* out) {
+  pdl_chain();
   extern __shared__ __align__(16) unsigned char dyn[];
   float* rootcw = reinterpret_cast<float*>(dyn);                                  // [C] root arc weight per class
   float* ybuf = reinterpret_cast<float*>(dyn) + C;                                // [kTopWarps][V]
@@ -1374,6 +1375,9 @@ template <typename LT>
 __global__ void __launch_bounds__(kBeamThreads) k_beam_chunk(TbBeamParams p, int32_t T, int32_t E, int64_t frame_stride,
                                                          int64_t row_stride, const int32_t* n_frames, int32_t* slot_pos,
                                                          unsigned long long* hash, int32_t* len, size_t n_hyp) {
+  // (chained, but its long steps are not shared with the next launch's blocks: 117 us a chunk of 128 slots with an early start
+  // of what follows, 114 without; k_beam_frames is not chained at all, the wait alone cost its step loop 2 %)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   __shared__ BeamShared sh;
   extern __shared__ __align__(16) unsigned char dyn_all[];
   const int b = blockIdx.x;
@@ -1391,6 +1395,7 @@ struct SlotList { int32_t slot[TB_BIND_PAIRS]; };
 __global__ void k_beam_reset_slots(int32_t* slot_pos, unsigned long long* hash, int32_t* len, size_t n_hyp, int32_t max_beam,   // (max_beam: records per slot)
                                    int32_t n, SlotList sl, int32_t all_slots, const TbSlotRec* slots, int32_t K,
                                    float* scores, int32_t* states, uint8_t* live) {
+  pdl_chain();
   const int i = blockIdx.x;
   if (i >= n) return;
   const int slot = all_slots ? i : sl.slot[i];
@@ -1426,6 +1431,7 @@ __global__ void __launch_bounds__(32 * kBtWarps) k_beam_backtrace(const int2* tr
                                                                   int32_t B, int32_t K, int32_t V, int32_t max_len, int32_t* out_tokens,
                                                                   int32_t* out_lens, int32_t* status, const __grid_constant__ SlotList sl,
                                                                   int32_t use_list) {
+  pdl_chain();
   __shared__ int2 piece[kBtWarps][TB_MAX_BEAM];              // (a) where a hypothesis at the piece's end stood at its start, its tokens
   __shared__ int2 enter[kBtWarps][TB_MAX_BEAM];              // (b) which one a hypothesis of the last step was at the piece's end, tokens up to there
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1595,7 +1601,7 @@ int tb_launch_beam_backtrace(const int2* tree, int32_t n_steps, int32_t B, int32
                              int32_t* out_tokens, int32_t* out_lens, cudaStream_t stream) {
   SlotList none;
   none.slot[0] = 0;
-  k_beam_backtrace<false><<<B, 32 * kBtWarps, 0, stream>>>(tree, 0, nullptr, n_steps, B, K, V, max_len, out_tokens, out_lens, nullptr, none, 0);
+  if (tb_launch_chained(k_beam_backtrace<false>, dim3(B), dim3(32 * kBtWarps), 0, stream, tree, 0, nullptr, n_steps, B, K, V, max_len, out_tokens, out_lens, nullptr, none, 0) != TB_OK) return TB_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
 
@@ -1603,6 +1609,7 @@ int tb_launch_beam_backtrace(const int2* tree, int32_t n_steps, int32_t B, int32
 // score' = fl(score + fl(lambda * final(state))).  Unbound slots, state -1 and empty places (-inf) stay as they are.
 __global__ void k_final_weights(const TbSlotRec* slots, const unsigned char* arena, int32_t B, int32_t K, float* scores,
                                 const int32_t* states, int32_t* status) {
+  pdl_chain();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= B * K) return;
   const TbSlotRec rec = slots[i / K];
@@ -1618,7 +1625,7 @@ __global__ void k_final_weights(const TbSlotRec* slots, const unsigned char* are
 int tb_launch_final_weights(const TbSlotRec* slots, const unsigned char* arena, int32_t B, int32_t K, float* scores,
                             const int32_t* states, int32_t* status, cudaStream_t stream) {
   const int n = B * K;
-  k_final_weights<<<(n + 127) / 128, 128, 0, stream>>>(slots, arena, B, K, scores, states, status);
+  if (tb_launch_chained(k_final_weights, dim3((n + 127) / 128), dim3(128), 0, stream, slots, arena, B, K, scores, states, status) != TB_OK) return TB_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
 
@@ -1677,6 +1684,7 @@ __global__ void k_publish_slots(TbSlotRec* slots, TbSlotState* sstate, int32_t n
 // memory, read in place, into its arena block, then stores the slot's record and starts the slot's stream afresh.
 constexpr int kPullThreads = 512;
 __global__ void __launch_bounds__(kPullThreads) k_pull_binds(TbInlineBinds ib, TbSlotState* sstate) {
+  pdl_chain();
   const int i = blockIdx.x;
   const unsigned char* src = nullptr;
   int32_t bytes = 0, slot = -1;
@@ -1714,6 +1722,7 @@ __global__ void __launch_bounds__(kPullThreads) k_pull_binds(TbInlineBinds ib, T
 
 __global__ void k_final_weights_slots(const TbSlotRec* slots, const unsigned char* arena, int32_t n, SlotList sl, int32_t K,
                                       float* scores, const int32_t* states, int32_t* status) {
+  pdl_chain();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n * K) return;
   const int slot = sl.slot[i / K];
@@ -1741,10 +1750,10 @@ int tb_launch_beam_chunk(const TbBeamParams& p_in, int32_t T, int32_t E, int64_t
   int rc;
   if (p.dtype == TB_BF16) {
     if ((rc = set_smem(k_beam_chunk<uint16_t>, smem)) != TB_OK) return rc;
-    k_beam_chunk<uint16_t><<<p.B, kBeamThreads, smem, stream>>>(p, T, E, frame_stride, row_stride, n_frames, slot_pos, hash, len, n_hyp);
+    if (tb_launch_chained(k_beam_chunk<uint16_t>, dim3(p.B), dim3(kBeamThreads), smem, stream, p, T, E, frame_stride, row_stride, n_frames, slot_pos, hash, len, n_hyp) != TB_OK) return TB_ERR_CUDA;
   } else {
     if ((rc = set_smem(k_beam_chunk<float>, smem)) != TB_OK) return rc;
-    k_beam_chunk<float><<<p.B, kBeamThreads, smem, stream>>>(p, T, E, frame_stride, row_stride, n_frames, slot_pos, hash, len, n_hyp);
+    if (tb_launch_chained(k_beam_chunk<float>, dim3(p.B), dim3(kBeamThreads), smem, stream, p, T, E, frame_stride, row_stride, n_frames, slot_pos, hash, len, n_hyp) != TB_OK) return TB_ERR_CUDA;
   }
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
@@ -1755,7 +1764,7 @@ int tb_launch_beam_reset_slots(int32_t* slot_pos, unsigned long long* hash, int3
   if (n < 1 || (!all_slots && n > TB_BIND_PAIRS)) return TB_ERR_INVALID_ARG;
   SlotList sl;
   for (int i = 0; i < TB_BIND_PAIRS; ++i) sl.slot[i] = (!all_slots && i < n) ? slots[i] : 0;
-  k_beam_reset_slots<<<n, 32, 0, stream>>>(slot_pos, hash, len, n_hyp, max_beam, n, sl, all_slots, slot_recs, K, scores, states, live);
+  if (tb_launch_chained(k_beam_reset_slots, dim3(n), dim3(32), 0, stream, slot_pos, hash, len, n_hyp, max_beam, n, sl, all_slots, slot_recs, K, scores, states, live) != TB_OK) return TB_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
 
@@ -1766,8 +1775,8 @@ int tb_launch_beam_backtrace_slots(const int2* tree, int32_t tree_cap, const int
   if (slot_list && n_slots > TB_BIND_PAIRS) return TB_ERR_INVALID_ARG;
   SlotList sl;
   for (int i = 0; i < TB_BIND_PAIRS; ++i) sl.slot[i] = (slot_list && i < n_slots) ? slot_list[i] : 0;
-  k_beam_backtrace<true><<<n_slots, 32 * kBtWarps, 0, stream>>>(tree, tree_cap, slot_pos, 0, n_slots, K, V, max_len, out_tokens, out_lens, status, sl,
-                                                                slot_list ? 1 : 0);
+  if (tb_launch_chained(k_beam_backtrace<true>, dim3(n_slots), dim3(32 * kBtWarps), 0, stream, tree, tree_cap, slot_pos, 0, n_slots, K, V, max_len, out_tokens, out_lens, status, sl,
+                                                                slot_list ? 1 : 0) != TB_OK) return TB_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
 
@@ -1777,7 +1786,7 @@ int tb_launch_final_weights_slots(const TbSlotRec* slots, const unsigned char* a
   SlotList sl;
   for (int i = 0; i < TB_BIND_PAIRS; ++i) sl.slot[i] = i < n ? slot_list[i] : 0;
   const int total = n * K;
-  k_final_weights_slots<<<(total + 127) / 128, 128, 0, stream>>>(slots, arena, n, sl, K, scores, states, status);
+  if (tb_launch_chained(k_final_weights_slots, dim3((total + 127) / 128), dim3(128), 0, stream, slots, arena, n, sl, K, scores, states, status) != TB_OK) return TB_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
 
@@ -1804,12 +1813,12 @@ int tb_launch_beam_topm(const void* logits, int dtype, int32_t B, int32_t T, int
   int rc;
   if (dtype == TB_BF16) {
     if ((rc = set_smem(k_beam_topm<uint16_t>, smem)) != TB_OK) return rc;
-    k_beam_topm<uint16_t><<<blocks, kTopWarps * 32, smem, stream>>>(static_cast<const uint16_t*>(logits), B, T, E, V, C, stream_stride,
-                                                                  frame_stride, row_stride, n_frames, slots, arena, cls, top_m, out);
+    if (tb_launch_chained(k_beam_topm<uint16_t>, dim3(blocks), dim3(kTopWarps * 32), smem, stream, static_cast<const uint16_t*>(logits), B, T, E, V, C, stream_stride,
+                                                                  frame_stride, row_stride, n_frames, slots, arena, cls, top_m, out) != TB_OK) return TB_ERR_CUDA;
   } else {
     if ((rc = set_smem(k_beam_topm<float>, smem)) != TB_OK) return rc;
-    k_beam_topm<float><<<blocks, kTopWarps * 32, smem, stream>>>(static_cast<const float*>(logits), B, T, E, V, C, stream_stride,
-                                                               frame_stride, row_stride, n_frames, slots, arena, cls, top_m, out);
+    if (tb_launch_chained(k_beam_topm<float>, dim3(blocks), dim3(kTopWarps * 32), smem, stream, static_cast<const float*>(logits), B, T, E, V, C, stream_stride,
+                                                               frame_stride, row_stride, n_frames, slots, arena, cls, top_m, out) != TB_OK) return TB_ERR_CUDA;
   }
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }

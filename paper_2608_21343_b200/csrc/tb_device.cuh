@@ -11,6 +11,13 @@
 
 #define TB_CHAIN_MAX 257  // a walk visits at most max_depth + 1 <= 256 states
 
+// The first statement of every kernel launched by tb_launch_chained: lets the next launch's blocks take their places, then waits
+// for the launch before this one.  Nothing may be read or written ahead of it.
+__device__ __forceinline__ void pdl_chain() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 struct GraphPtrs {
   const int32_t* arc_begin;
   const int32_t* fail;

@@ -7,6 +7,25 @@
 
 #include "tb_internal.h"
 
+// Launches a kernel that begins with pdl_chain() (tb_device.cuh): its blocks may take their places while the launch before
+// it on the stream still runs, and wait there until that has completed and its writes are visible.  Between short
+// launches of one call sequence this takes out most of the gap (a streaming beam chunk of seven launches, two slots at K = 2:
+// 79 us -> 66; a TDT chunk and the derivation of its new streams' lists: 45 -> 43).  While the stream is being captured into a graph, where what comes before may be anything, an ordinary launch.
+#ifdef __CUDACC__
+template <typename... P, typename... A>
+inline int tb_launch_chained(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) cudaGetLastError();
+  cfg.attrs = at; cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...) == cudaSuccess ? 0 : (cudaGetLastError(), TB_ERR_CUDA);
+}
+#endif
+
 struct TbDecodeParams {
   const void* logits;        // device
   int dtype;                 // TB_BF16 / TB_F32

@@ -23,6 +23,7 @@ __global__ void __launch_bounds__(kListWarps * 32) k_resolve_lists(TbSlotRec* re
                                                                    const int32_t* __restrict__ ctb, const int32_t* __restrict__ ctk,
                                                                    int32_t C, int32_t V, int32_t chain, int32_t* status) {
   extern __shared__ __align__(16) uint32_t dynw[];
+  pdl_chain();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, words = list_words(V), tb = tb_rs_tok_bits(V);
   uint32_t* seen = dynw + warp * list_smem(V, chain);
   uint32_t* done = seen + words;
@@ -156,6 +157,5 @@ int tb_launch_resolve_lists(TbSlotRec* recs, unsigned char* arena, int32_t n, co
   int per = (max_states + kListWarps - 1) / kListWarps;
   const int most = (n_sm * 16 + n - 1) / n;
   if (per > most) per = most;
-  k_resolve_lists<<<dim3(per, n), kListWarps * 32, smem, stream>>>(recs, arena, ls, ctb, ctk, C, V, chain, status);
-  return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
+  return tb_launch_chained(k_resolve_lists, dim3(per, n), dim3(kListWarps * 32), smem, stream, recs, arena, ls, ctb, ctk, C, V, chain, status);
 }

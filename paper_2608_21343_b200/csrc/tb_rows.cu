@@ -89,6 +89,8 @@ template <typename LT, int G, bool TAB>
 __global__ void __launch_bounds__(kSumThreads, G == 4 ? 3 : 2) k_row_sums(const __grid_constant__ RowsParams P) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ float part[3 * kSumThreads / 32];
+  // (the second step's blocks read the graphs before their own wait: they may start only once this launch's wait is over)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const TbDecodeParams& p = P.d;
   constexpr int kWarps = kSumThreads / 32;
@@ -133,6 +135,7 @@ template <typename LT>
 __global__ void __launch_bounds__(32 * kDecMaxSegs, 1) k_decide_rows(const __grid_constant__ RowsParams P) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ float part[3 * kDecMaxSegs];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const TbDecodeParams& p = P.d;
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthreads = blockDim.x, S = p.S;
   const DecSmem so = dec_smem(p.V, p.C, S, p.frames, P.nseg, P.cache_bytes, P.spill != nullptr);
@@ -485,7 +488,8 @@ int tb_launch_rows(const TbDecodeParams& d, const TbRowsPlan& plan, int32_t n_sm
     return TB_ERR_CUDA;
   }
   if (cudaFuncSetAttribute(f2, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem) != cudaSuccess) { cudaGetLastError(); return TB_ERR_CUDA; }
-  f1<<<dim3(static_cast<unsigned>((d.frames + per * kSumThreads / 32 - 1) / (per * kSumThreads / 32)), d.n_streams), kSumThreads, smem1, stream>>>(P);
+  if (tb_launch_chained(f1, dim3(static_cast<unsigned>((d.frames + per * kSumThreads / 32 - 1) / (per * kSumThreads / 32)), d.n_streams), dim3(kSumThreads), smem1, stream, P) != TB_OK)
+    return TB_ERR_CUDA;
   if (cudaGetLastError() != cudaSuccess) return TB_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(d.n_streams); cfg.blockDim = dim3(32 * plan.nseg); cfg.dynamicSmemBytes = plan.smem; cfg.stream = stream;
