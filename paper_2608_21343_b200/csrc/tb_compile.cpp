@@ -72,18 +72,18 @@ static void finalize_graph(tb_graph* g, const int32_t* case_class, int32_t vocab
   std::vector<TbRsRec> rrecs(N);
   std::vector<int32_t> count(N, 0);
   std::vector<int32_t> seen;                   // class -> state that listed it during the current walk
+  std::vector<int64_t> own(tree ? static_cast<size_t>(A) + 1 : 0, 0);   // tokens that arcs before this one add to their states' lists
   if (!tree) seen.assign(n_classes, -1);
+  else
+    for (int32_t a = 0; a < A; ++a)            // (arc a leads to state a + 1)
+      own[a + 1] = own[a] + (g->state_depth[g->state_fail[a + 1]] < 2 ? csize[g->arc_class[a]] : 0);
   bool fits = N < (1 << (32 - tb_rs_tok_bits(vocab)));
   int64_t total = 0;
   g->d_max = 0.0f;
   for (int32_t s = 0; s < N; ++s) {
     float acc = 0.0f;
     int32_t c = 0;
-    if (tree && s) {
-      c = count[g->state_fail[s]];
-      for (int32_t a = g->state_arc_begin[s]; a < g->state_arc_begin[s + 1]; ++a)
-        if (g->state_depth[g->state_fail[g->arc_dst[a]]] < 2) c += csize[g->arc_class[a]];
-    }
+    if (tree && s) c = count[g->state_fail[s]] + static_cast<int32_t>(own[g->state_arc_begin[s + 1]] - own[g->state_arc_begin[s]]);
     for (int32_t u = s; u != 0; u = g->state_fail[u]) {
       if (!tree && fits)
         for (int32_t a = g->state_arc_begin[u]; a < g->state_arc_begin[u + 1]; ++a)
@@ -212,6 +212,8 @@ static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offs
     int32_t len;
   };
   if (n_phrases > 0 && (phrase_offsets[n_phrases] < 0 || phrase_offsets[n_phrases] > static_cast<int64_t>(n_phrases) * TB_MAX_PHRASE_LEN)) return TB_ERR_INVALID_ARG;
+  int32_t key_bits = 1;                         // of one class in the sort key (0: the phrase has ended)
+  while (key_bits < 16 && (1 << key_bits) <= n_classes) ++key_bits;
   std::vector<int32_t> folded(n_phrases > 0 ? static_cast<size_t>(phrase_offsets[n_phrases]) : 0);
   std::vector<Folded> ph;
   ph.reserve(n_phrases);
@@ -226,7 +228,7 @@ static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offs
       if (token_weights && !(std::isfinite(token_weights[i]) && token_weights[i] >= 0.0f)) return TB_ERR_INVALID_ARG;
       const int32_t c = case_class ? case_class[phrase_tokens[i]] : phrase_tokens[i];
       folded[i] = c;
-      if (i < b + 4) key |= static_cast<uint64_t>(std::min(c, 0xFFFE) + 1) << (48 - 16 * (i - b));
+      if (i < b + 4) key |= static_cast<uint64_t>(std::min(c, 0xFFFE) + 1) << (key_bits * (3 - (i - b)));
     }
     if (e == b) continue;  // empty phrases are skipped
     ph.push_back({key, folded.data() + b, token_weights ? token_weights + b : nullptr, static_cast<int32_t>(e - b)});
@@ -234,54 +236,72 @@ static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offs
   }
 
   // ---- sort the folded phrases, longest-common-prefix with the predecessor -----------------
-  const size_t P = ph.size();
-  std::sort(ph.begin(), ph.end(), [](const Folded& x, const Folded& y) {
-    if (x.key != y.key) return x.key < y.key;
-    const int32_t n = std::min(x.len, y.len);
-    for (int32_t i = 0; i < n; ++i)
-      if (x.cls[i] != y.cls[i]) return x.cls[i] < y.cls[i];
-    return x.len < y.len;
-  });
-  std::vector<int32_t> lcp(P, 0);
-  std::vector<size_t> node_base(P + 1, 0);  // where phrase i's node ids start in `node_of`
-  for (size_t i = 0; i < P; ++i) {
-    const Folded& x = ph[i];
-    node_base[i + 1] = node_base[i] + x.len;
-    if (i == 0) continue;
-    const Folded& y = ph[i - 1];
-    int32_t n = std::min(x.len, y.len), l = 0;
-    while (l < n && x.cls[l] == y.cls[l]) ++l;
-    lcp[i] = l;
+  const int32_t P = static_cast<int32_t>(ph.size());
+  struct Key { uint64_t key; int32_t at; };
+  std::vector<Key> keys(P);
+  for (int32_t i = 0; i < P; ++i) keys[i] = {ph[i].key, i};
+  // by the key, a byte at a time (275 phrases: 3 us where a comparison sort takes 15), then runs of equal keys by the rest
+  std::vector<Key> keys2(P);
+  for (int32_t shift = 0; shift < 4 * key_bits; shift += 8) {
+    int32_t at[257] = {0};
+    for (const Key& k : keys) at[((k.key >> shift) & 0xFF) + 1]++;
+    for (int32_t i = 0; i < 256; ++i) at[i + 1] += at[i];
+    for (const Key& k : keys) keys2[at[(k.key >> shift) & 0xFF]++] = k;
+    keys.swap(keys2);
+  }
+  for (int32_t i = 0; i < P;) {
+    int32_t j = i + 1;
+    while (j < P && keys[j].key == keys[i].key) ++j;
+    if (j - i > 1)
+      std::sort(keys.begin() + i, keys.begin() + j, [&](const Key& kx, const Key& ky) {
+        const Folded &x = ph[kx.at], &y = ph[ky.at];
+        const int32_t n = std::min(x.len, y.len);
+        for (int32_t k = 0; k < n; ++k)
+          if (x.cls[k] != y.cls[k]) return x.cls[k] < y.cls[k];
+        return x.len < y.len;
+      });
+    i = j;
   }
 
   // ---- states: distinct prefixes, depth by depth = breadth-first order ----------------------
-  std::vector<int32_t> node_of(node_base[P]);   // node id of phrase i's prefix of length d+1
-  std::vector<int32_t> parent(1, -1), cls(1, -1);
-  std::vector<uint8_t> depth(1, 0), is_end(1, 0);
-  std::vector<double> wt(1, 0.0);
-  parent.reserve(node_base[P] + 1); cls.reserve(node_base[P] + 1); depth.reserve(node_base[P] + 1); is_end.reserve(node_base[P] + 1); wt.reserve(node_base[P] + 1);
-  for (int32_t d = 1; d <= max_len; ++d) {
-    for (size_t i = 0; i < P; ++i) {
-      const Folded& x = ph[i];
-      if (x.len < d) continue;
-      double w = x.w ? static_cast<double>(x.w[d - 1]) : 1.0;
-      int32_t id;
-      if (lcp[i] >= d) {  // same prefix as the predecessor, which therefore has this node
-        id = node_of[node_base[i - 1] + d - 1];
-        wt[id] = std::max(wt[id], w);
-      } else {
-        id = static_cast<int32_t>(parent.size());
-        parent.push_back(d == 1 ? 0 : node_of[node_base[i] + d - 2]);
-        cls.push_back(x.cls[d - 1]);
-        depth.push_back(static_cast<uint8_t>(d));
-        is_end.push_back(0);
-        wt.push_back(w);
-      }
-      node_of[node_base[i] + d - 1] = id;
-      if (x.len == d) is_end[id] = 1;
+  // Phrases that reach a depth are taken in sorted order; one that shares its prefix with its predecessor (which then
+  // reaches the depth too) has the state that was numbered last.  No branch depends on the data.
+  struct Reach { const int32_t* cls; const float* w; int32_t len, lcp, node; };
+  std::vector<Reach> reach(P);                  // phrases that reach the depth; node: their state one depth up
+  for (int32_t i = 0; i < P; ++i) {
+    const Folded& x = ph[keys[i].at];
+    int32_t l = 0;
+    if (i > 0) {
+      const Folded& y = ph[keys[i - 1].at];
+      const int32_t n = std::min(x.len, y.len);
+      while (l < n && x.cls[l] == y.cls[l]) ++l;
     }
+    reach[i] = {x.cls, x.w, x.len, l, 0};
   }
-  const int32_t N = static_cast<int32_t>(parent.size());
+  const size_t most = folded.size() + 1;
+  std::vector<int32_t> parent(most), cls(most);
+  std::vector<uint8_t> depth(most), is_end(most);
+  std::vector<double> wt(most);
+  parent[0] = cls[0] = -1;
+  int32_t N = 1;
+  int32_t n_reach = P;
+  for (int32_t d = 1; n_reach > 0; ++d) {
+    int32_t kept = 0;
+    for (int32_t i = 0; i < n_reach; ++i) {
+      Reach x = reach[i];
+      const bool fresh = x.lcp < d;
+      N += fresh ? 1 : 0;
+      const int32_t id = N - 1;
+      const double w = x.w ? static_cast<double>(x.w[d - 1]) : 1.0;
+      parent[id] = x.node; cls[id] = x.cls[d - 1]; depth[id] = static_cast<uint8_t>(d);
+      wt[id] = fresh ? w : std::max(wt[id], w);
+      is_end[id] = static_cast<uint8_t>((fresh ? 0 : is_end[id]) | (x.len == d ? 1 : 0));
+      x.node = id;
+      reach[kept] = x;
+      kept += x.len > d ? 1 : 0;
+    }
+    n_reach = kept;
+  }
   const int32_t A = N - 1;
 
   // ---- arcs: arc a enters state a+1; a state's arcs are contiguous --------------------------
@@ -290,7 +310,7 @@ static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offs
   g->state_arc_begin.assign(N + 1, 0);
   g->arc_class.resize(A); g->arc_dst.resize(A); g->arc_w.resize(A);
   g->state_fail.assign(N, 0); g->state_bw.assign(N, 0.0f); g->state_final.assign(N, 0.0f);
-  g->state_depth.assign(depth.begin(), depth.end());
+  g->state_depth.assign(depth.begin(), depth.begin() + N);
   for (int32_t id = 1; id < N; ++id) {
     g->state_arc_begin[parent[id] + 1]++;
     g->arc_class[id - 1] = cls[id];
