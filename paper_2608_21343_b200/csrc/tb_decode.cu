@@ -1272,7 +1272,17 @@ __global__ void __launch_bounds__(kBeamThreads) k_beam_frames(TbBeamParams p, in
 // Beam pre-pass: one warp per logit row, independent of every hypothesis.  With the rows of a stream shared by its
 // hypotheses, the order of a row's tokens that no hypothesis' state boosts is, up to rounding, the order of their
 // root-boosted values y -- so a step only needs the first few of them (see beam_team_run).
+// Bound by instruction issue.  The top_m + 1 best come without rounds of picking: the (top_m + 1)-th largest of the lanes' best
+// values (two per lane where one is too few) bounds that of the row from below, so the tokens at or above it -- 1.3 times
+// as many as are wanted, on average -- are collected and put in order by counting, for each, those before it.  1000 rows of
+// 1024 for 32 streams: K = 4 (16 entries) 84 us, K = 32 (44 entries) 127 us; a round per pick took 96 and 290.
 constexpr int kTopWarps = 8;
+constexpr int kTopCap = 128;           // tokens collected at a time
+static_assert(kTopCap > TB_MAX_BEAM + 13, "more than any row keeps");
+__device__ __forceinline__ uint32_t top_key(float v) {       // ascending with the value
+  const uint32_t u = __float_as_uint(v + 0.0f);
+  return u ^ ((u >> 31) ? 0xFFFFFFFFu : 0x80000000u);
+}
 template <typename LT>
 __global__ void __launch_bounds__(kTopWarps * 32) k_beam_topm(const LT* logits, int32_t B, int32_t T, int32_t E, int32_t V, int32_t C,
                                                             int64_t stream_stride, int64_t frame_stride, int64_t row_stride,
@@ -1304,66 +1314,92 @@ __global__ void __launch_bounds__(kTopWarps * 32) k_beam_topm(const LT* logits, 
   if (n_frames && t >= n_frames[b]) return;
   const LT* row = logits + static_cast<int64_t>(b) * stream_stride + static_cast<int64_t>(t) * frame_stride + static_cast<int64_t>(e) * row_stride;
   TbTopEnt* o = out + (static_cast<int64_t>(b) * rows_per_stream + r) * (top_m + 1);
-  float* y = ybuf + static_cast<size_t>(warp) * V;
-  // y of every token; on the way every lane keeps the three best of its strip (value descending, token ascending:
-  // the strip is walked in ascending token order, so a strict comparison keeps the lower token among equals)
-  float v0 = -INFINITY, v1 = -INFINITY, v2 = -INFINITY;
-  int i0 = INT32_MAX, i1 = INT32_MAX, i2 = INT32_MAX;
-  int n_strip = 0;
+  uint32_t* y = reinterpret_cast<uint32_t*>(ybuf) + static_cast<size_t>(warp) * V;        // keys of the row's y
+  uint64_t* cand = reinterpret_cast<uint64_t*>(dyn + (((static_cast<size_t>(C) + static_cast<size_t>(kTopWarps) * V) * 4 + 7) & ~size_t(7))) + warp * kTopCap;
+  const int want = top_m + 1;
+  uint32_t k0 = 0u, k1 = 0u;                                  // the lane's best and second best (0: none)
 #pragma unroll 4
   for (int v = lane; v < V; v += 32) {
     const float x = LogitLoad<LT>::at(row + v);
-    const float yv = bound ? __fadd_rn(x, __fmul_rn(g.lambda, rootcw[__ldg(cls + v)])) : x;
-    y[v] = yv;
-    ++n_strip;
-    if (yv > v0 || i0 == INT32_MAX) { v2 = v1; i2 = i1; v1 = v0; i1 = i0; v0 = yv; i0 = v; }
-    else if (yv > v1 || i1 == INT32_MAX) { v2 = v1; i2 = i1; v1 = yv; i1 = v; }
-    else if (yv > v2 || i2 == INT32_MAX) { v2 = yv; i2 = v; }
+    const uint32_t k = top_key(bound ? __fadd_rn(x, __fmul_rn(g.lambda, rootcw[__ldg(cls + v)])) : x);
+    y[v] = k;
+    k1 = max(k1, min(k0, k));
+    k0 = max(k0, k);
   }
   __syncwarp();
-  int n_taken = 0;      // of this lane's strip
-  // The rounds only note which token won and its y (the owner's registers hold both); the logit and the class of the
-  // picks are looked up afterwards by all lanes at once, so that no round waits for a trip to memory.
-  float* pick_y = reinterpret_cast<float*>(ybuf + static_cast<size_t>(kTopWarps) * V) + static_cast<size_t>(warp) * 2 * (top_m + 1);
-  int32_t* pick_i = reinterpret_cast<int32_t*>(pick_y + (top_m + 1));
-  for (int m = 0; m <= top_m; ++m) {
-    // the warp's best: largest value, then lowest token
-    const uint32_t u = __float_as_uint(v0 + 0.0f);
-    const uint32_t key = i0 == INT32_MAX ? 0u : (u ^ ((u >> 31) ? 0xFFFFFFFFu : 0x80000000u));
-    const uint32_t kmax = __reduce_max_sync(0xffffffffu, key);
-    const uint32_t imin = __reduce_min_sync(0xffffffffu, (key == kmax && i0 != INT32_MAX) ? static_cast<uint32_t>(i0) : 0xFFFFFFFFu);
-    const bool none = imin == 0xFFFFFFFFu;                    // fewer than m + 1 tokens in the row
-    if (none) {
-      if (lane == 0) { pick_y[m] = -INFINITY; pick_i[m] = -1; }
-    } else if (static_cast<uint32_t>(i0) == imin) {
-      pick_y[m] = v0; pick_i[m] = i0;
-      if (m < top_m) {
-        // the owner takes it out: its next best moves up; when the three it kept are used up and the strip holds
-        // more, it looks through the strip again
-        y[i0] = __int_as_float(0x7FC00000);                   // (a NaN: never greater than anything, never chosen again)
-        ++n_taken;
-        v0 = v1; i0 = i1; v1 = v2; i1 = i2; v2 = -INFINITY; i2 = INT32_MAX;
-        if (i0 == INT32_MAX && n_taken < n_strip) {
-          for (int v = lane; v < V; v += 32) {
-            const float yv = y[v];
-            if (yv == yv) {
-              if (yv > v0 || i0 == INT32_MAX) { v2 = v1; i2 = i1; v1 = v0; i1 = i0; v0 = yv; i0 = v; }
-              else if (yv > v1 || i1 == INT32_MAX) { v2 = v1; i2 = i1; v1 = yv; i1 = v; }
-              else if (yv > v2 || i2 == INT32_MAX) { v2 = yv; i2 = v; }
-            }
-          }
-        }
+  // at least `want` tokens have thr or more (rows shorter than that: all have)
+  uint32_t thr = 0u;
+  {
+    int n0 = 0, n1 = 0;                                       // how many of the lanes' values come before this lane's
+    const bool both = want > 28;
+#pragma unroll 4
+    for (int j = 0; j < 32; ++j) {
+      const uint32_t o0 = __shfl_sync(0xffffffffu, k0, j);
+      n0 += (o0 > k0 || (o0 == k0 && j < lane)) ? 1 : 0;
+      if (both) {
+        const uint32_t o1 = __shfl_sync(0xffffffffu, k1, j);
+        n0 += o1 > k0 ? 1 : 0;
+        n1 += (o0 >= k1 ? 1 : 0) + ((o1 > k1 || (o1 == k1 && j < lane)) ? 1 : 0);
       }
     }
-    __syncwarp();
+    const unsigned at0 = __ballot_sync(0xffffffffu, n0 == want - 1), at1 = __ballot_sync(0xffffffffu, both && n1 == want - 1);
+    if (at0) thr = __shfl_sync(0xffffffffu, k0, __ffs(at0) - 1);
+    else if (at1) thr = __shfl_sync(0xffffffffu, k1, __ffs(at1) - 1);
   }
-  for (int m = lane; m <= top_m; m += 32) {
-    const int i = pick_i[m];
+  // candidates as value key << 32 | inverted token, all different
+  uint64_t lim = static_cast<uint64_t>(thr) << 32;
+  int n;
+#pragma unroll 1
+  for (;;) {
+    n = 0;
+#pragma unroll 1
+    for (int v0 = 0; v0 < V && n < kTopCap; v0 += 32) {
+      const int v = v0 + lane;
+      const uint64_t k = v < V ? static_cast<uint64_t>(y[v]) << 32 | (0xFFFFFFFFu - static_cast<uint32_t>(v)) : 0ull;
+      const bool hit = v < V && k >= lim;
+      const unsigned mask = __ballot_sync(0xffffffffu, hit);
+      if (mask == 0u) continue;
+      const int at = n + __popc(mask & ((1u << lane) - 1u));
+      if (hit && at < kTopCap) cand[at] = k;
+      n += __popc(mask);
+    }
+    n = min(n, kTopCap);
+    __syncwarp();
+    if (n < kTopCap) break;
+    // more than can be held: the want-th of those that were bounds the row's from below more tightly (and lim rises, as they
+    // are all different and more than are wanted)
+    uint64_t next = 0ull;
+#pragma unroll 1
+    for (int i = lane; i < n; i += 32) {
+      const uint64_t k = cand[i];
+      int before = 0;
+#pragma unroll 4
+      for (int j = 0; j < n; ++j) before += cand[j] > k ? 1 : 0;
+      if (before == want - 1) next = k;
+    }
+    const unsigned who = __ballot_sync(0xffffffffu, next != 0ull);
+    next = __shfl_sync(0xffffffffu, next, __ffs(who) - 1);
+    __syncwarp();
+    lim = next;
+  }
+#pragma unroll 1
+  for (int i = lane; i < n; i += 32) {
+    const uint64_t k = cand[i];
+    int m = 0;
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) m += cand[j] > k ? 1 : 0;
+    if (m > top_m) continue;
+    const int tok = static_cast<int>(0xFFFFFFFFu - static_cast<uint32_t>(k));
+    const uint32_t u = static_cast<uint32_t>(k >> 32);
     TbTopEnt e;
-    e.y = pick_y[m];
+    e.y = __uint_as_float(u ^ ((u >> 31) ? 0x80000000u : 0xFFFFFFFFu));
     if (m == top_m) { e.x = LogitLoad<LT>::at(row + V); e.tok_cls = 0u; }
-    else if (i < 0) { e.x = -INFINITY; e.tok_cls = 0xFFFFu; }
-    else { e.x = LogitLoad<LT>::at(row + i); e.tok_cls = static_cast<uint32_t>(i) | (static_cast<uint32_t>(__ldg(cls + i)) << 16); }
+    else { e.x = LogitLoad<LT>::at(row + tok); e.tok_cls = static_cast<uint32_t>(tok) | (static_cast<uint32_t>(__ldg(cls + tok)) << 16); }
+    o[m] = e;
+  }
+  for (int m = n + lane; m <= top_m; m += 32) {               // fewer tokens in the row
+    TbTopEnt e;
+    e.y = -INFINITY; e.x = m == top_m ? LogitLoad<LT>::at(row + V) : -INFINITY; e.tok_cls = m == top_m ? 0u : 0xFFFFu;
     o[m] = e;
   }
 }
@@ -1807,8 +1843,8 @@ int tb_launch_beam_topm(const void* logits, int dtype, int32_t B, int32_t T, int
                         int64_t stream_stride, int64_t frame_stride, int64_t row_stride, const int32_t* n_frames,
                         const TbSlotRec* slots, const unsigned char* arena, const int32_t* cls, int32_t top_m,
                         TbTopEnt* out, cudaStream_t stream) {
-  // root weights per class, every warp's y values, every warp's picks (value and token, top_m + 1 each)
-  const size_t smem = (static_cast<size_t>(C) + static_cast<size_t>(kTopWarps) * V + static_cast<size_t>(kTopWarps) * 2 * (top_m + 1)) * sizeof(float);
+  // root weights per class, every warp's y values, every warp's candidates
+  const size_t smem = (((static_cast<size_t>(C) + static_cast<size_t>(kTopWarps) * V) * sizeof(float) + 7) & ~size_t(7)) + kTopWarps * kTopCap * sizeof(uint64_t);
   const int blocks = B * ((T * E + kTopWarps - 1) / kTopWarps);
   int rc;
   if (dtype == TB_BF16) {

@@ -1,0 +1,39 @@
+"""Parity of the beam's reduced rows at their edges, against the CPU oracle: rows shorter than what is kept of them, rows
+ascending or descending by token, rows whose large values share one lane's strip of tokens, constant rows, infinities."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2608_21343_b200 import workloads as W
+from helpers import SCORE_TOL, make_batch, oracle_graph
+from test_gpu_beam_stream import run_beam_frames
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("K", [1, 4, 13, 32])
+@pytest.mark.parametrize("V,dtype", [(1, "f32"), (15, "bf16"), (33, "f32"), (45, "bf16"), (300, "f32"), (1024, "bf16"), (1400, "f32")])
+def test_rows(tb, K, V, dtype):
+    w = W.get_workload(4, B=4, T=12, V=V, K=K, dtype=dtype, n_phrases=min(20, V), len_hi=3, n_plants=0)
+    data = W.batch_inputs(w)
+    x = data["logits"] if dtype == "f32" else W.bf16_bits_to_f32(data["logits"])
+    v = np.arange(V, dtype=np.float32)
+    x[:, 0, :, :V] = v / 64
+    x[:, 2, :, :V] = -v / 64
+    x[:, 4, :, :V] += np.where(v % 32 == 5, 6.0, 0.0)
+    x[:, 6, :, :V] = 0.5
+    x[:, 8, :, :V] = np.where(v % 3 == 0, x[:, 8, :, :V], -np.inf)
+    x[:, :, :, V] = x[:, :, :, :V].max(-1) - 0.25
+    data["logits"] = W.to_storage(x, dtype)
+    lists = list(data["phrases"])
+    lists[1] = None
+    batch, _ = make_batch(tb, w, lists, max_beam=K, max_tree_steps=w.T * w.S)
+    out = run_beam_frames(tb, w, data, K, lists, batch, merge=True)
+    for i in range(w.B):
+        ref = O.beam_decode(oracle_graph(w, lists[i]), data["logits"][i], K, merge=True)
+        assert np.array_equal(out["states"][i], ref["states"]) and np.array_equal(out["lens"][i], ref["lens"]), i
+        for k in range(K):
+            assert np.array_equal(out["tokens"][i, k, :ref["lens"][k]], ref["tokens"][k]), (i, k)
+        fin = np.isfinite(ref["scores"])
+        assert np.array_equal(np.isfinite(out["scores"][i]), fin)
+        assert np.all(np.abs(out["scores"][i][fin] - ref["scores"][fin]) <= SCORE_TOL)
