@@ -192,6 +192,7 @@ __device__ __forceinline__ void prog_publish(volatile int* flags, int v) { flags
 
 template <int NIT, bool NORM>
 __global__ void __launch_bounds__(kThreadsF, 1) k_greedy_fast(FastParams P) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");             // (chained: see tb_launch_chained; nothing starts early behind it)
   extern __shared__ __align__(128) unsigned char dyn[];
   const TbDecodeParams& p = P.d;
   const int V = p.V, C = p.C, S = p.S, W = V + 1, nst = P.nst;
@@ -1180,6 +1181,5 @@ int tb_launch_greedy_fast(const TbDecodeParams& d, int32_t max_cache_bytes, int3
     cudaGetLastError();
     return 1;
   }
-  fn<<<d.n_streams, kThreadsF, so.total, stream>>>(P);
-  return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
+  return tb_launch_chained(fn, dim3(d.n_streams), dim3(kThreadsF), static_cast<size_t>(so.total), stream, P);
 }

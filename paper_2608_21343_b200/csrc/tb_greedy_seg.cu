@@ -228,6 +228,7 @@ struct PipeInfo {   // one per pipeline of the block, in shared memory
 
 template <int NIT, bool NORM>
 __global__ void __launch_bounds__(kMaxThreadsS, 1) k_greedy_seg(SegParams P) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");             // (chained: see tb_launch_chained; nothing starts early behind it)
   extern __shared__ __align__(128) unsigned char dyn[];
   const TbDecodeParams& p = P.d;
   const int V = p.V, C = p.C, S = p.S, W = V + 1, G = P.G, H = P.H;
@@ -1115,7 +1116,6 @@ int tb_launch_greedy_seg(const TbDecodeParams& d, int32_t max_cache_bytes, const
     cudaGetLastError();
     return TB_ERR_CUDA;
   }
-  fn<<<d.n_streams * plan.NB, (plan.G + plan.H) * 32, plan.smem, stream>>>(P);
-  return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
+  return tb_launch_chained(fn, dim3(d.n_streams * plan.NB), dim3((plan.G + plan.H) * 32), static_cast<size_t>(plan.smem), stream, P);
 }
 
