@@ -1001,9 +1001,13 @@ extern "C" int tb_greedy_decode(tb_batch* b, const void* logits, int dtype, int3
       if (rc == TB_OK) { b->last_kernel = TB_KERNEL_GENERAL; b->last_NB = 1; b->last_G = 0; }
       return true;
     };
-    // Lists that are walked or too large for the pipelined kernels' caches (48 KB): in two steps, many stretches of a stream
-    // at once, each reading its lists from L2.
-    if (b->plan_G == 0 && !(b->flags & (TB_FLAG_ONE_BLOCK_PER_STREAM | TB_FLAG_TEST_WAIT_TIMEOUT)) && (!all_resolved || max_cache > (48 << 10)))
+    // Lists too large for the pipelined kernels' caches (48 KB): in two steps, many stretches of a stream at once, each reading
+    // its lists from L2 (100 streams of 200 frames, lists of 400 phrases: 230 us against 301).  Lists that are walked: the same
+    // from 256 frames on -- their states are left late, so that a stretch runs on for up to 250 frames before its decode is
+    // the next one's, and shorter streams gain nothing (54 streams of 100 frames: 240 us either way, 60 frames: 178 us
+    // against 135; 16 of 300: 332 us against 519).
+    const bool by_rows = all_resolved ? max_cache > (48 << 10) : T >= 256;
+    if (b->plan_G == 0 && !(b->flags & (TB_FLAG_ONE_BLOCK_PER_STREAM | TB_FLAG_TEST_WAIT_TIMEOUT)) && by_rows)
       if (run_rows()) return rc;
     if (!(b->flags & TB_FLAG_ONE_BLOCK_PER_STREAM)) {
       TbSegPlan plan;
@@ -1103,9 +1107,14 @@ static int launch_chunk(tb_batch* b, const TbDecodeParams& p, cudaStream_t strea
   if (!(b->flags & TB_FLAG_GENERAL_KERNELS)) {
     query_device(b);
     const SlotSummary sl = slot_summary(b, p.n_streams);
+    // A chunk of a few frames is over before the row summaries pay for their set-up: row by row (the general kernel) is as
+    // quick or quicker below four frames (512 slots, one frame of three rows: 13 us against 19) and, with slots for a good
+    // part of the GPU, below eight (128 slots, four frames of one row: 15 against 17; 4 slots: 14 against 13).  It needs
+    // the token view of resolved lists, i.e. vocabularies up to 2047.
+    const bool row_by_row = sl.all_resolved && tb_rs_tok_bits(b->vocab) == TB_RS_TOK_BITS && (p.frames < 4 || (p.frames < 8 && p.n_streams > 32));
     // (the lists of graphs bound with this launch are derived behind it: until then they are put together by walking)
     const bool walks = !sl.all_resolved || binds;
-    if (!walks || grow_scratch(b, &b->chunk_spill, &b->chunk_spill_bytes, tb_chunk_rows_spill_bytes(p), is_capturing(stream))) {
+    if (!row_by_row && (!walks || grow_scratch(b, &b->chunk_spill, &b->chunk_spill_bytes, tb_chunk_rows_spill_bytes(p), is_capturing(stream)))) {
       const int rc = tb_launch_chunk_rows(p, sl.max_states, b->n_sm, b->max_smem, walks ? b->chunk_spill : nullptr, stream, binds);
       if (rc != 1) return rc;
     }

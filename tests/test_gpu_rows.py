@@ -71,7 +71,7 @@ def test_ties(tb, levels, V):
 @pytest.mark.parametrize("wl", [dict(n_phrases=400, n_shared=2600, len_lo=3, len_hi=10), dict(n_phrases=300, len_hi=4)])
 def test_long_lists_walked_and_resolved(tb, wl):
     """Lists that are walked along the suffix chain (too large to be resolved), and resolved ones of hundreds of tokens."""
-    w, data = _inputs(8, 4, 200, 3, 700, "bf16", **wl)
+    w, data = _inputs(8, 4, 260, 3, 700, "bf16", **wl)
     lists = list(data["phrases"])
     lists[2] = None
     _check(tb, w, data, lists=lists, what="long lists")
