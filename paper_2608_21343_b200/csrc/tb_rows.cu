@@ -1,5 +1,5 @@
 // Greedy decode in two steps, for what the pipelined kernels (tb_greedy_fast.cu, tb_greedy_seg.cu) do not cover: fp32
-// logits, vocabularies beyond 2047 tokens, rows that are not packed, graphs without resolved lists in small batches --
+// logits, vocabularies beyond 2047 tokens, rows that are not packed, lists larger than 48 KB or walked along the suffix chain --
 // and streaming chunks, where both steps run in the block of a slot.
 //
 // Offline: k_row_sums reduces every row of the call to a 32-byte summary (one warp per row, all SMs, one pass over HBM),
