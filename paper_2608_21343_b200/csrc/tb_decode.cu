@@ -5,6 +5,7 @@
 // chunk kernels (tb_rows.cu) the rest of what has contiguous tokens, and this one what is left:
 // other token strides, more than four rows a frame, chunks of a few frames.
 #include <cfloat>
+#include <type_traits>
 
 #include "tb_device.cuh"
 #include "tb_launch.h"
@@ -301,6 +302,13 @@ struct BeamShared {
   uint4 no_rec;                                          // the empty list (unbound streams)
 };
 
+// A token sequence's identity with one more token: a 64-bit mix of the sequence so far and the token.
+__device__ __forceinline__ unsigned long long beam_extend(unsigned long long h, int token) {
+  h = (h ^ static_cast<unsigned long long>(token + 1)) * 0xff51afd7ed558ccdull;
+  h ^= h >> 33;
+  return h + 0x9e3779b97f4a7c15ull;
+}
+
 template <typename LT>
 __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared& sh, LT (&xpre)[kBeamPref], bool& xpre_valid,
                                                const LT* next_row) {
@@ -595,12 +603,7 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
     {
       if (parent >= 0) {
         nh = h_hash[parent]; nl = h_len[parent];
-        if (token >= 0 && token != V) {          // one more token: a 64-bit mix of the sequence so far and the token
-          nh = (nh ^ static_cast<unsigned long long>(token + 1)) * 0xff51afd7ed558ccdull;
-          nh ^= nh >> 33;
-          nh += 0x9e3779b97f4a7c15ull;
-          ++nl;
-        }
+        if (token >= 0 && token != V) { nh = beam_extend(nh, token); ++nl; }
       }
       p.hash_out[o] = nh; p.len_out[o] = nl;
     }
@@ -654,6 +657,13 @@ __global__ void __launch_bounds__(kBeamThreads) k_beam_step(TbBeamParams p) {
 constexpr int kTeamRecCache = 48 << 10;   // shared memory for a copy of the stream's list records (graphs of up to 3072 states)
 constexpr float kHistAbove = 6.0f, kHistPerUnit = 8.0f;   // the reference's distance above score + best plain value; bins per unit
 constexpr int kTeamRows = 3;              // rows (and reduced rows) in shared memory
+// Narrow beams take their steps with one warp (tb_beam_solo.cuh); what that cannot take goes to the team.
+constexpr int kSoloBeam = 8;              // hypotheses at most
+constexpr int kSoloRows = 4;              // rows brought at a time (two such groups in shared memory)
+constexpr int kSoloVocab = 64;            // rows of fewer tokens are left to the team
+constexpr int kSoloPlain = 12;            // tokens of a reduced row that are looked at, at most
+__host__ __device__ inline bool beam_solo_width(int K, int V) { return K <= kSoloBeam && V >= kSoloVocab; }
+__host__ __device__ inline int beam_rows_kept(int K, int V) { return beam_solo_width(K, V) ? 2 * kSoloRows : kTeamRows; }
 
 __host__ __device__ inline int team_warps(int K) { return K > 16 ? 16 : K < 4 ? 4 : K; }
 __device__ __forceinline__ unsigned long long beam_key(float v, int tkey, int k) {
@@ -696,13 +706,14 @@ __device__ __forceinline__ void beam_fetch_row(unsigned char* buf, const LT* row
 }
 // Shared memory of the team behind the block's other arrays: row buffers, reduced rows, the copy of the list records.
 struct TeamSmem { int row, row_stride, top, top_stride, recs, total; };
-__host__ __device__ inline TeamSmem team_smem(int V, int elem, int top_m, int rec_bytes) {
+__host__ __device__ inline TeamSmem team_smem(int K, int V, int elem, int top_m, int rec_bytes) {
+  const int rows = beam_rows_kept(K, V);
   TeamSmem t;
   t.row_stride = (((V + 1) * elem + 16 + 15) & ~15) + 16;
   t.row = 0;
   t.top_stride = ((top_m + 1) * 12 + 15) & ~15;
-  t.top = kTeamRows * t.row_stride;
-  t.recs = t.top + kTeamRows * t.top_stride;
+  t.top = rows * t.row_stride;
+  t.recs = t.top + rows * t.top_stride;
   t.total = t.recs + rec_bytes;
   return t;
 }
@@ -1137,15 +1148,12 @@ __device__ __forceinline__ int beam_team_run(const TbBeamParams& p, BeamShared& 
     const bool emits = parent >= 0 && tkey < V;
     const bool lv = emits && ((live >> (parent & 31)) & 1u);
     const bool last = sidx + 1 >= n_steps, frame_next = e_cur + 1 == E;
-    if (hashes) {                                              // one more token: a 64-bit mix of the sequence so far and the token
+    if (hashes) {
       const int from = parent >= 0 ? parent : lane;
       unsigned long long nh = (static_cast<unsigned long long>(__shfl_sync(0xffffffffu, static_cast<uint32_t>(hh >> 32), from)) << 32) |
                               __shfl_sync(0xffffffffu, static_cast<uint32_t>(hh), from);
       hl = __shfl_sync(0xffffffffu, hl, from) + (emits ? 1 : 0);
-      unsigned long long mh = (nh ^ static_cast<unsigned long long>(tkey + 1)) * 0xff51afd7ed558ccdull;
-      mh ^= mh >> 33;
-      mh += 0x9e3779b97f4a7c15ull;
-      hh = parent < 0 ? 0ull : emits ? mh : nh;
+      hh = parent < 0 ? 0ull : emits ? beam_extend(nh, tkey) : nh;
       if (parent < 0) hl = 0;
     }
     if (keeper) {
@@ -1184,8 +1192,12 @@ __device__ __forceinline__ int beam_team_run(const TbBeamParams& p, BeamShared& 
   return sh.done;
 }
 
-// All steps of one stream of a multi-step launch: the team takes what it can, the block the rest.
-template <typename LT>
+#include "tb_beam_solo.cuh"
+
+// All steps of one stream of a multi-step launch: a warp or the team takes what it can, the block the rest.
+// WIDTH: 0 up to kSoloBeam hypotheses, 1 up to 16, 2 more.  (A kernel each: in one kernel the registers and the code of one weighed on the others --
+// 32 streams of 1000 steps, K = 32, 4155 us and 4384 with the single warp's steps beside the team's, 3740 alone; K = 12 2633 and 2406.)
+template <typename LT, int WIDTH>
 __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared& sh, unsigned char* dyn, const int32_t n_steps, const int32_t E,
                                                const int64_t frame_stride, const int64_t row_stride, const int32_t rows_per_stream,
                                                const int32_t step_base, unsigned long long* hashA, unsigned long long* hashB, int32_t* lenA,
@@ -1193,28 +1205,51 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
   LT xpre[kBeamPref] = {};
   bool xpre_valid = false;
   const bool fast = beam_team_applies(p);
-  const TeamSmem tm = team_smem(p.V, sizeof(LT), p.top_m, p.rec_cache_bytes);
+  const TeamSmem tm = team_smem(p.K, p.V, sizeof(LT), p.top_m, p.rec_cache_bytes);
   const bool odd0 = (par0 & 1) != 0;
   const bool recs_cached = beam_begin(p, sh, dyn, odd0 ? hashB : hashA, odd0 ? lenB : lenA, fast, tm);
   const LT* stream_base = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(blockIdx.x) * p.stream_stride;
+  const bool solo = WIDTH == 0 && fast && beam_solo_width(p.K, p.V);
+  __shared__ BeamSolo so;
   int32_t skip = 0, backoff = 0;              // steps until the team tries again after a step it could not take
+  int32_t team_steps = 1;                     // steps the team takes when the warp could not
 #pragma unroll 1
   for (int32_t sidx = 0; sidx < n_steps; ++sidx) {
+    if constexpr (WIDTH == 0) {
+      if (solo && skip <= 0) {
+        if (threadIdx.x < 32) {
+          const int d = p.K > 4 ? beam_solo_run<LT, 8>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm) : beam_solo_run<LT, 4>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm);
+          if (threadIdx.x == 0) sh.team_done = d;
+        } else if (threadIdx.x < 64) {
+          if (p.K > 4)
+            beam_solo_serve<LT, 8>(p, sh, so, dyn, tm, sidx, n_steps, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB, lenA, lenB, par0);
+          else
+            beam_solo_serve<LT, 4>(p, sh, so, dyn, tm, sidx, n_steps, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB, lenA, lenB, par0);
+        }
+        __syncthreads();
+        const int d = sh.team_done;
+        __syncthreads();                          // (read by everyone before a later run writes it again)
+        sidx += d;
+        if (sidx >= n_steps) break;
+        team_steps = d == 0 ? min(2 * team_steps, 32) : 1;
+      }
+    }
     if (fast && skip-- <= 0) {
+      const int32_t stop = solo ? min(n_steps, sidx + team_steps) : n_steps;
       if (threadIdx.x < 32 * (team_warps(p.K) + 1)) {
-        const int d = p.K > 16 ? beam_team_run<LT, 2>(p, sh, dyn, sidx, n_steps, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB,
-                                                      lenA, lenB, par0, recs_cached, tm)
-                               : beam_team_run<LT, 1>(p, sh, dyn, sidx, n_steps, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB,
-                                                      lenA, lenB, par0, recs_cached, tm);
+        const int d = beam_team_run<LT, WIDTH == 2 ? 2 : 1>(p, sh, dyn, sidx, stop, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB, lenA,
+                                                            lenB, par0, recs_cached, tm);
         if (threadIdx.x == 0) sh.team_done = d;
       }
       __syncthreads();
       const int d = sh.team_done;
       __syncthreads();                          // (read by everyone before a later run writes it again)
       sidx += d;
+      if (sidx >= n_steps) break;
+      xpre_valid = false;
+      if (sidx >= stop) { --sidx; continue; }   // (the warp goes on)
       backoff = d == 0 ? min(2 * backoff + 1, 32) : 0;
       skip = backoff;
-      xpre_valid = false;
       if (sidx >= n_steps) break;
     }
     const int32_t t = sidx / E, e = sidx - t * E;
@@ -1238,12 +1273,12 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
 
 // T frames of E rows in one launch: the block loops over the expansions of its stream; every hypothesis of the
 // stream reads row (t, e).
-template <typename LT>
+template <typename LT, int WIDTH>
 __global__ void __launch_bounds__(kBeamThreads) k_beam_frames(TbBeamParams p, int32_t T, int32_t E, int64_t frame_stride,
                                                           int64_t row_stride) {
   __shared__ BeamShared sh;
   extern __shared__ __align__(16) unsigned char dyn_all[];
-  beam_all_steps<LT>(p, sh, dyn_all, T * E, E, frame_stride, row_stride, T * E, p.step, const_cast<unsigned long long*>(p.hash_in), p.hash_out,
+  beam_all_steps<LT, WIDTH>(p, sh, dyn_all, T * E, E, frame_stride, row_stride, T * E, p.step, const_cast<unsigned long long*>(p.hash_in), p.hash_out,
                      const_cast<int32_t*>(p.len_in), p.len_out, 0);
 }
 
@@ -1380,7 +1415,7 @@ __global__ void __launch_bounds__(kTopWarps * 32) k_beam_topm(const LT* logits, 
 // A chunk of streaming beam decoding: slot by slot, n_frames[slot] frames (at most T) of E rows; each slot has its own
 // position in its own tree ring and its own parity of the sequence-record halves, so that slots start, pause and end
 // independently of each other (Sec. 2.3: hypotheses kept across chunks; Sec. 2.2 para. 4: slots re-bound in between).
-template <typename LT>
+template <typename LT, int WIDTH>
 __global__ void __launch_bounds__(kBeamThreads) k_beam_chunk(TbBeamParams p, int32_t T, int32_t E, int64_t frame_stride,
                                                          int64_t row_stride, const int32_t* n_frames, int32_t* slot_pos,
                                                          unsigned long long* hash, int32_t* len, size_t n_hyp) {
@@ -1393,7 +1428,7 @@ __global__ void __launch_bounds__(kBeamThreads) k_beam_chunk(TbBeamParams p, int
   const int32_t nf = n_frames ? max(0, min(T, n_frames[b])) : T;
   const int32_t pos0 = slot_pos[b];
   if (nf > 0)
-    beam_all_steps<LT>(p, sh, dyn_all, nf * E, E, frame_stride, row_stride, T * E, pos0, hash, hash + n_hyp, len, len + n_hyp, pos0);
+    beam_all_steps<LT, WIDTH>(p, sh, dyn_all, nf * E, E, frame_stride, row_stride, T * E, pos0, hash, hash + n_hyp, len, len + n_hyp, pos0);
   if (threadIdx.x == 0) slot_pos[b] = pos0 + nf * E;
 }
 
@@ -1569,6 +1604,14 @@ int tb_launch_beam_step(const TbBeamParams& p_in, cudaStream_t stream) {
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
 
+// Calls f with the width class of beam_all_steps as a compile-time constant.
+template <typename F>
+static int beam_width_class(int K, F f) {
+  if (K <= kSoloBeam) return f(std::integral_constant<int, 0>{});
+  if (K <= 16) return f(std::integral_constant<int, 1>{});
+  return f(std::integral_constant<int, 2>{});
+}
+
 // The team's steps (beam_team_run) read rows through buffers behind the block's other shared memory and need the extent
 // of the logits tensor; without either (odd strides, no room) they stay off.
 static void beam_team_setup(TbBeamParams* p, int32_t T, int32_t E, int64_t frame_stride, int64_t row_stride, size_t* smem) {
@@ -1576,7 +1619,7 @@ static void beam_team_setup(TbBeamParams* p, int32_t T, int32_t E, int64_t frame
   p->tensor_lo = nullptr; p->tensor_hi = nullptr; p->rec_cache_bytes = 0;
   if (!p->top_base || p->stream_stride < 0 || frame_stride < 0 || row_stride < 0) return;
   const int elem = p->dtype == TB_BF16 ? 2 : 4;
-  const size_t more = team_smem(p->V, elem, p->top_m, 0).total;
+  const size_t more = team_smem(p->K, p->V, elem, p->top_m, 0).total;
   if (*smem + more > kMost) return;
   *smem += more;
   p->rec_cache_bytes = static_cast<int32_t>((kMost - *smem < static_cast<size_t>(kTeamRecCache) ? kMost - *smem : static_cast<size_t>(kTeamRecCache)) & ~size_t(15));
@@ -1596,14 +1639,15 @@ int tb_launch_beam_frames(const TbBeamParams& p_in, int32_t T, int32_t E, int64_
                 ((static_cast<size_t>(p.K) * ((p.V + 1 + 31) >> 5) * sizeof(uint32_t) + 15) & ~size_t(15)) + aux;
   beam_team_setup(&p, T, E, frame_stride, row_stride, &smem);
   if (smem > 200 * 1024) return TB_ERR_INVALID_ARG;
-  int rc;
-  if (p.dtype == TB_BF16) {
-    if ((rc = set_smem(k_beam_frames<uint16_t>, smem)) != TB_OK) return rc;
-    k_beam_frames<uint16_t><<<p.B, kBeamThreads, smem, stream>>>(p, T, E, frame_stride, row_stride);
-  } else {
-    if ((rc = set_smem(k_beam_frames<float>, smem)) != TB_OK) return rc;
-    k_beam_frames<float><<<p.B, kBeamThreads, smem, stream>>>(p, T, E, frame_stride, row_stride);
-  }
+  auto launch = [&](auto* fn) -> int {
+    const int rc = set_smem(fn, smem);
+    if (rc == TB_OK) fn<<<p.B, kBeamThreads, smem, stream>>>(p, T, E, frame_stride, row_stride);
+    return rc;
+  };
+  const int rc = beam_width_class(p.K, [&](auto w) {
+    return p.dtype == TB_BF16 ? launch(k_beam_frames<uint16_t, decltype(w)::value>) : launch(k_beam_frames<float, decltype(w)::value>);
+  });
+  if (rc != TB_OK) return rc;
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
 
@@ -1740,14 +1784,15 @@ int tb_launch_beam_chunk(const TbBeamParams& p_in, int32_t T, int32_t E, int64_t
                 ((static_cast<size_t>(p.K) * ((p.V + 1 + 31) >> 5) * sizeof(uint32_t) + 15) & ~size_t(15)) + aux;
   beam_team_setup(&p, T, E, frame_stride, row_stride, &smem);
   if (smem > 200 * 1024) return TB_ERR_INVALID_ARG;
-  int rc;
-  if (p.dtype == TB_BF16) {
-    if ((rc = set_smem(k_beam_chunk<uint16_t>, smem)) != TB_OK) return rc;
-    if (tb_launch_chained(k_beam_chunk<uint16_t>, dim3(p.B), dim3(kBeamThreads), smem, stream, p, T, E, frame_stride, row_stride, n_frames, slot_pos, hash, len, n_hyp) != TB_OK) return TB_ERR_CUDA;
-  } else {
-    if ((rc = set_smem(k_beam_chunk<float>, smem)) != TB_OK) return rc;
-    if (tb_launch_chained(k_beam_chunk<float>, dim3(p.B), dim3(kBeamThreads), smem, stream, p, T, E, frame_stride, row_stride, n_frames, slot_pos, hash, len, n_hyp) != TB_OK) return TB_ERR_CUDA;
-  }
+  auto launch = [&](auto* fn) -> int {
+    const int rc = set_smem(fn, smem);
+    if (rc != TB_OK) return rc;
+    return tb_launch_chained(fn, dim3(p.B), dim3(kBeamThreads), smem, stream, p, T, E, frame_stride, row_stride, n_frames, slot_pos, hash, len, n_hyp) == TB_OK ? TB_OK : TB_ERR_CUDA;
+  };
+  const int rc = beam_width_class(p.K, [&](auto w) {
+    return p.dtype == TB_BF16 ? launch(k_beam_chunk<uint16_t, decltype(w)::value>) : launch(k_beam_chunk<float, decltype(w)::value>);
+  });
+  if (rc != TB_OK) return rc;
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
 
