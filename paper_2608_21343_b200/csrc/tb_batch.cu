@@ -1296,8 +1296,9 @@ static void beam_prepass(tb_batch* b, TbBeamParams* p, int32_t T, int32_t E, int
   const size_t want = static_cast<size_t>(p->B) * T * E * (M + 1) * sizeof(TbTopEnt);
   if (!grow_scratch(b, &b->top, want, is_capturing(stream))) return;
   TbTopEnt* const top = static_cast<TbTopEnt*>(b->top.mem);
+  query_device(b);
   if (tb_launch_beam_topm(p->logits, p->dtype, p->B, T, E, p->V, p->C, p->stream_stride, frame_stride, row_stride, n_frames,
-                          b->d_slots, b->arena, b->d_cls, M, top, stream) != TB_OK)
+                          b->d_slots, b->arena, b->d_cls, M, top, b->n_sm, stream) != TB_OK)
     return;
   p->top_base = top; p->top_m = M;
 }

@@ -31,15 +31,42 @@ struct BeamSolo {
   uint4 plain[2 * kSoloRows][kSoloPlain];                      // per token looked at: logit, its class' root weight, token, the root arc's target
   Row row[2 * kSoloRows];
   uint32_t pick[2 * kSoloRows][kSoloBeam];                     // 32 * token key + parent of every place's pick, all ones: none
+  uint32_t stamp;                                              // the last step's number, in the upper bits (see beam_solo_run)
+};
+
+// Row sidx of the block's stream, the way from a frame's last row to the next frame, and the row's reduced form.
+template <typename LT>
+struct BeamSoloRows {
+  const LT* row;
+  const unsigned char* top;
+  int64_t row_stride, to_frame;
+  int e, E, top_bytes;
+  __device__ __forceinline__ BeamSoloRows(const TbBeamParams& p, int32_t sidx, int32_t E_, int64_t frame_stride, int64_t row_stride_, int32_t rows_per_stream) {
+    const int b = blockIdx.x;
+    E = E_; e = sidx % E; row_stride = row_stride_; to_frame = frame_stride - static_cast<int64_t>(E - 1) * row_stride;
+    row = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(b) * p.stream_stride + static_cast<int64_t>(sidx / E) * frame_stride + static_cast<int64_t>(e) * row_stride;
+    top_bytes = (p.top_m + 1) * 12;
+    top = reinterpret_cast<const unsigned char*>(p.top_base + (static_cast<int64_t>(b) * rows_per_stream + sidx) * (p.top_m + 1));
+  }
+  __device__ __forceinline__ void fetch(const TbBeamParams& p, unsigned char* mem, const TeamSmem& tm, int place) const {      // (by a warp)
+    const int lane = threadIdx.x & 31;
+    beam_fetch_row<LT>(mem + tm.row + place * tm.row_stride, row, p.V + 1, p.tensor_lo, p.tensor_hi, lane, 32);
+    unsigned char* dst = mem + tm.top + place * tm.top_stride;
+#pragma unroll 1
+    for (int c = lane; c < top_bytes >> 4; c += 32) beam_cp_async16(dst + 16 * c, top + 16 * c);
+  }
+  __device__ __forceinline__ void next() {
+    top += top_bytes;
+    if (++e == E) { e = 0; row += to_frame; } else row += row_stride;
+  }
 };
 
 // The second warp: brings rows sidx, sidx + 1, ... into the buffers and keeps the books of the steps before: the tree, and what
-// identifies the hypotheses' token sequences.  sh.cmd holds the number of the barrier that ends the run, sh.done the steps
+// identifies the hypotheses' token sequences.  (fetched: the first rows are on their way already.)  sh.cmd holds the number of the barrier that ends the run, sh.done the steps
 // taken by then.
 template <typename LT, int KG>
 __device__ __forceinline__ void beam_solo_serve(const TbBeamParams& p, BeamShared& sh, BeamSolo& so, unsigned char* dyn, const TeamSmem& tm, int32_t sidx,
-                                                const int32_t n_steps, const int32_t E, const int64_t frame_stride, const int64_t row_stride,
-                                                const int32_t rows_per_stream, const int32_t step_base, unsigned long long* hashA, unsigned long long* hashB,
+                                                const int32_t n_steps, BeamSoloRows<LT> at, bool fetched, const int32_t step_base, unsigned long long* hashA, unsigned long long* hashB,
                                                 int32_t* lenA, int32_t* lenB, const int32_t par0) {
   constexpr int P = KG <= 4 ? 8 : kSoloPlain;
   const int lane = threadIdx.x & 31, b = blockIdx.x, K = p.K, V = p.V, W = V + 1, M = p.top_m;
@@ -49,12 +76,8 @@ __device__ __forceinline__ void beam_solo_serve(const TbBeamParams& p, BeamShare
   const float* rootcw = reinterpret_cast<const float*>(aux);    // (see tokview_attach)
   const int32_t* rootdst = reinterpret_cast<const int32_t*>(aux + 4 * static_cast<size_t>(p.C));
   unsigned char* mem = team_base(p, dyn);
-  int e = sidx % E, step = sidx;                                // step: the next one to be entered in the books
+  int step = sidx;                                              // the next one to be entered in the books
   const int32_t first = sidx;
-  const LT* row = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(b) * p.stream_stride + static_cast<int64_t>(sidx / E) * frame_stride +
-                  static_cast<int64_t>(e) * row_stride;
-  const int64_t to_frame = frame_stride - static_cast<int64_t>(E - 1) * row_stride;
-  const unsigned char* top = reinterpret_cast<const unsigned char*>(p.top_base + (static_cast<int64_t>(b) * rows_per_stream + sidx) * (M + 1));
   int tree_at = p.tree_cap > 0 ? (step_base + sidx) % p.tree_cap : 0;
   unsigned long long hh = 0ull;                                 // lane k: the sequence of hypothesis k
   int32_t hl = 0;
@@ -66,14 +89,11 @@ __device__ __forceinline__ void beam_solo_serve(const TbBeamParams& p, BeamShare
     int rows = 0;
 #pragma unroll 1
     for (; rows < kSoloRows && sidx < n_steps; ++rows, ++sidx) {
-      beam_fetch_row<LT>(mem + tm.row + (buf + rows) * tm.row_stride, row, W, p.tensor_lo, p.tensor_hi, lane, 32);
-      unsigned char* dst = mem + tm.top + (buf + rows) * tm.top_stride;
-#pragma unroll 1
-      for (int c = lane; c < ((M + 1) * 12) >> 4; c += 32) beam_cp_async16(dst + 16 * c, top + 16 * c);
-      if (lane == 0) so.row[buf + rows].at = static_cast<uint32_t>(mem - dyn) + tm.row + (buf + rows) * tm.row_stride + static_cast<uint32_t>(reinterpret_cast<uintptr_t>(row) & 15u);
-      top += (M + 1) * 12;
-      if (++e == E) { e = 0; row += to_frame; } else row += row_stride;
+      if (!fetched) at.fetch(p, mem, tm, buf + rows);
+      if (lane == 0) so.row[buf + rows].at = static_cast<uint32_t>(mem - dyn) + tm.row + (buf + rows) * tm.row_stride + static_cast<uint32_t>(reinterpret_cast<uintptr_t>(at.row) & 15u);
+      at.next();
     }
+    fetched = false;
     // the steps before the last barrier (the rows are on their way)
     const bool end = n > 1 && *cmd == n - 1;
     const int32_t upto = end ? first + *const_cast<volatile int32_t*>(&sh.done) : first + max(n - 2, 0) * kSoloRows;
@@ -148,13 +168,7 @@ __device__ __forceinline__ int beam_solo_run(const TbBeamParams& p, BeamShared& 
   // (which also says whether the hypothesis lists the token).  The block's steps have their candidates there.
   unsigned char* my_lead = dyn + 4 * (mine ? hyp : 0) * W;
   const uint32_t c_own = 0xFFFFFFFFu - static_cast<uint32_t>(hyp);                           // (the lower word of a key: see beam_key)
-  uint32_t stamp = 0u;                                          // this step's number, in the upper bits
-  auto clear = [&]() {
-#pragma unroll 4
-    for (int i = lane; i < K * W; i += 32) reinterpret_cast<uint32_t*>(dyn)[i] = 0u;
-    __syncwarp();
-  };
-  clear();
+  uint32_t stamp = so.stamp;                                    // this step's number, in the upper bits
   int e_cur = sidx % E;
   // this lane's hypothesis: score, state, whether it can be expanded, and (merging) what identifies its token sequence
   float sc = -INFINITY;
@@ -217,7 +231,13 @@ __device__ __forceinline__ int beam_solo_run(const TbBeamParams& p, BeamShared& 
     const BeamSolo::Row ro = so.row[slot];
     const unsigned char* row = dyn + ro.at;
     stamp += 1u << kDstBits;
-    if (stamp == 0u) { clear(); stamp = 1u << kDstBits; }       // (the numbers begin again)
+    if (stamp == 0u) {                                          // (the numbers begin again)
+      __syncwarp();
+#pragma unroll 4
+      for (int i = lane; i < K * W; i += 32) reinterpret_cast<uint32_t*>(dyn)[i] = 0u;
+      __syncwarp();
+      stamp = 1u << kDstBits;
+    }
     // ---- the lane's best candidates: largest value, then lowest token.  A lane's listed tokens come in ascending order, so among
     // them, and for the blank, which comes last of all, a tie stays with what is there.
     float v1 = -INFINITY, v2 = -INFINITY, v3 = -INFINITY, rest = -INFINITY;     // (rest: the best value that is not kept)
@@ -263,13 +283,16 @@ __device__ __forceinline__ int beam_solo_run(const TbBeamParams& p, BeamShared& 
     if (__any_sync(0xffffffffu, n_list > 2 * L)) {
       listed(en[1]);
       if (__any_sync(0xffffffffu, n_list > 4 * L)) {
+        uint4 a = pad, c = pad;
+        if (2 * (j + NE * L) < cnt) a = list[NE * L];
+        if (2 * (j + NE * L + L) < cnt) c = list[NE * L + L];
         listed(en[2]); listed(en[3]);
 #pragma unroll 1
         for (int i = NE * L; __any_sync(0xffffffffu, 2 * i < n_list); i += 2 * L) {
-          uint4 a = pad, c = pad;
-          if (2 * (i + j) < cnt) a = list[i];
-          if (2 * (i + j + L) < cnt) c = list[i + L];
           listed(a); listed(c);
+          a = c = pad;                                         // (the next ones are on their way)
+          if (2 * (i + j + 2 * L) < cnt) a = list[i + 2 * L];
+          if (2 * (i + j + 3 * L) < cnt) c = list[i + 3 * L];
         }
       }
     }
@@ -330,7 +353,7 @@ __device__ __forceinline__ int beam_solo_run(const TbBeamParams& p, BeamShared& 
     e_cur = e_cur + 1 == E ? 0 : e_cur + 1;
     if (sidx + 1 < n_steps) enter(e_cur == 0);
   }
-  if (lane == 0) { *const_cast<volatile int32_t*>(&sh.done) = done; *const_cast<volatile int32_t*>(&sh.cmd) = n_bar + 1; }
+  if (lane == 0) { so.stamp = stamp; *const_cast<volatile int32_t*>(&sh.done) = done; *const_cast<volatile int32_t*>(&sh.cmd) = n_bar + 1; }
   if (mine && j == 0) {
     if (sidx >= n_steps) {
       const int64_t o = static_cast<int64_t>(b) * K + hyp;

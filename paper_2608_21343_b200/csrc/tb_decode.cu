@@ -751,9 +751,19 @@ __device__ __forceinline__ bool beam_team_applies(const TbBeamParams& p) {
 // fit (returns whether they do).
 __device__ inline bool beam_begin(const TbBeamParams& p, BeamShared& sh, unsigned char* dyn, const unsigned long long* hash_in,
                                   const int32_t* len_in, bool team, const TeamSmem& tm) {
-  const int tid = threadIdx.x, K = p.K, b = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, K = p.K, b = blockIdx.x;
   const TbSlotRec& rec = p.slots[b];
   const bool bound = rec.n_states > 0, use_tv = bound && rec.n_rsent >= 0 && p.tokview;
+  const int W = p.V + 1, WW = (W + 31) >> 5;
+  unsigned char* aux = dyn + ((static_cast<size_t>(K) * W * sizeof(float) + 15) & ~size_t(15)) + ((static_cast<size_t>(K) * WW * sizeof(uint32_t) + 15) & ~size_t(15));
+  float* rootcw = reinterpret_cast<float*>(aux);               // (see tokview_attach)
+  int32_t* rootdst = reinterpret_cast<int32_t*>(aux + 4 * static_cast<size_t>(p.C));
+  const bool cached = use_tv && team && static_cast<int64_t>(rec.n_states) * 16 <= p.rec_cache_bytes;
+  if (cached) {
+    const unsigned char* src = p.arena + rec.blob_off + rec.off_rsrec;
+    unsigned char* dst = team_base(p, dyn) + tm.recs;
+    for (int i = tid; i < rec.n_states; i += blockDim.x) beam_cp_async16(dst + 16 * i, src + 16 * i);
+  }
   if (tid < K) {
     const int64_t o = static_cast<int64_t>(b) * K + tid;
     sh.h_score[tid] = p.scores[o]; sh.h_state[tid] = p.states[o]; sh.h_live[tid] = p.live[o];
@@ -761,26 +771,21 @@ __device__ inline bool beam_begin(const TbBeamParams& p, BeamShared& sh, unsigne
     sh.h_len[tid] = p.fresh ? 0 : len_in[o];
   }
   if (tid == 0) { sh.root_wmax = 0.0f; sh.no_rec = make_uint4(0u, 0u, 0u, 0u); }
-  const int W = p.V + 1, WW = (W + 31) >> 5;
-  unsigned char* aux = dyn + ((static_cast<size_t>(K) * W * sizeof(float) + 15) & ~size_t(15)) + ((static_cast<size_t>(K) * WW * sizeof(uint32_t) + 15) & ~size_t(15));
-  bool cached = false;
   if (use_tv) {
-    TokView tv;
-    tokview_init(tv, aux, p.V, p.C, graph_of(p.arena, rec));
-    if (tid < 32) {
-      float r = 0.0f;
-      for (int c = tid; c < p.C; c += 32) r = fmaxf(r, fabsf(tv.rootcw[c]));
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, off));
-      if (tid == 0) sh.root_wmax = r;
+    const GraphPtrs g = graph_of(p.arena, rec);
+    const int a0 = g.arc_begin[0], a1 = g.arc_begin[1];
+    for (int c = tid; c < p.C; c += blockDim.x) { rootcw[c] = 0.0f; rootdst[c] = 0; }
+    __syncthreads();
+    uint32_t r = 0u;                                           // (|w| >= 0: ordered like its bits)
+    for (int a = a0 + tid; a < a1; a += blockDim.x) {
+      const int c = g.arc_cls[a];
+      const float w = __fadd_rn(0.0f, g.arc_w[a]);
+      if (c >= 0 && c < p.C) { rootcw[c] = w; rootdst[c] = g.arc_dst[a]; r = max(r, __float_as_uint(fabsf(w))); }
     }
-    if (team && static_cast<int64_t>(rec.n_states) * 16 <= p.rec_cache_bytes) {
-      cached = true;
-      const uint4* src = reinterpret_cast<const uint4*>(p.arena + rec.blob_off + rec.off_rsrec);
-      uint4* dst = reinterpret_cast<uint4*>(team_base(p, dyn) + tm.recs);
-      for (int i = tid; i < rec.n_states; i += blockDim.x) dst[i] = src[i];
-    }
+    r = __reduce_max_sync(0xffffffffu, r);
+    if (lane == 0 && r != 0u) atomicMax(reinterpret_cast<unsigned int*>(&sh.root_wmax), r);
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   return cached;
 }
@@ -1207,27 +1212,41 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
   const bool fast = beam_team_applies(p);
   const TeamSmem tm = team_smem(p.K, p.V, sizeof(LT), p.top_m, p.rec_cache_bytes);
   const bool odd0 = (par0 & 1) != 0;
-  const bool recs_cached = beam_begin(p, sh, dyn, odd0 ? hashB : hashA, odd0 ? lenB : lenA, fast, tm);
-  const LT* stream_base = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(blockIdx.x) * p.stream_stride;
   const bool solo = WIDTH == 0 && fast && beam_solo_width(p.K, p.V);
   __shared__ BeamSolo so;
+  if constexpr (WIDTH == 0) {                 // the first rows are on their way while the tables are laid out
+    const int row = static_cast<int>(threadIdx.x >> 5) - (kBeamThreads / 32 - kSoloRows);     // (a row each by the block's last warps)
+    if (solo && row >= 0 && row < n_steps) BeamSoloRows<LT>(p, row, E, frame_stride, row_stride, rows_per_stream).fetch(p, team_base(p, dyn), tm, row);
+  }
+  const bool recs_cached = beam_begin(p, sh, dyn, odd0 ? hashB : hashA, odd0 ? lenB : lenA, fast, tm);
+  const LT* stream_base = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(blockIdx.x) * p.stream_stride;
+  // what the warp's steps keep behind dyn begins empty, and again after a step by the block
+  auto clear = [&]() {
+    for (int i = threadIdx.x; i < p.K * (p.V + 1); i += kBeamThreads) reinterpret_cast<uint32_t*>(dyn)[i] = 0u;
+    if (threadIdx.x == 0) so.stamp = 0u;
+    __syncthreads();
+  };
+  bool clean = false, first = true;
   int32_t skip = 0, backoff = 0;              // steps until the team tries again after a step it could not take
   int32_t team_steps = 1;                     // steps the team takes when the warp could not
 #pragma unroll 1
   for (int32_t sidx = 0; sidx < n_steps; ++sidx) {
     if constexpr (WIDTH == 0) {
       if (solo && skip <= 0) {
+        if (!clean) { clear(); clean = true; }
         if (threadIdx.x < 32) {
           const int d = p.K > 4 ? beam_solo_run<LT, 8>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm) : beam_solo_run<LT, 4>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm);
           if (threadIdx.x == 0) sh.team_done = d;
         } else if (threadIdx.x < 64) {
+          const BeamSoloRows<LT> at(p, sidx, E, frame_stride, row_stride, rows_per_stream);
           if (p.K > 4)
-            beam_solo_serve<LT, 8>(p, sh, so, dyn, tm, sidx, n_steps, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB, lenA, lenB, par0);
+            beam_solo_serve<LT, 8>(p, sh, so, dyn, tm, sidx, n_steps, at, sidx == 0 && first, step_base, hashA, hashB, lenA, lenB, par0);
           else
-            beam_solo_serve<LT, 4>(p, sh, so, dyn, tm, sidx, n_steps, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB, lenA, lenB, par0);
+            beam_solo_serve<LT, 4>(p, sh, so, dyn, tm, sidx, n_steps, at, sidx == 0 && first, step_base, hashA, hashB, lenA, lenB, par0);
         }
         __syncthreads();
         const int d = sh.team_done;
+        first = false;
         __syncthreads();                          // (read by everyone before a later run writes it again)
         sidx += d;
         if (sidx >= n_steps) break;
@@ -1252,6 +1271,7 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
       skip = backoff;
       if (sidx >= n_steps) break;
     }
+    clean = false;
     const int32_t t = sidx / E, e = sidx - t * E;
     TbBeamParams q = p;
     q.logits = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(t) * frame_stride + static_cast<int64_t>(e) * row_stride;
@@ -1280,136 +1300,6 @@ __global__ void __launch_bounds__(kBeamThreads) k_beam_frames(TbBeamParams p, in
   extern __shared__ __align__(16) unsigned char dyn_all[];
   beam_all_steps<LT, WIDTH>(p, sh, dyn_all, T * E, E, frame_stride, row_stride, T * E, p.step, const_cast<unsigned long long*>(p.hash_in), p.hash_out,
                      const_cast<int32_t*>(p.len_in), p.len_out, 0);
-}
-
-// Beam pre-pass: one warp per logit row, independent of every hypothesis.  With the rows of a stream shared by its
-// hypotheses, the order of a row's tokens that no hypothesis' state boosts is, up to rounding, the order of their
-// root-boosted values y -- so a step only needs the first few of them (see beam_team_run).
-// Bound by instruction issue.  The top_m + 1 best come without rounds of picking: the (top_m + 1)-th largest of the lanes' best
-// values (two per lane where one is too few) bounds that of the row from below, so the tokens at or above it -- 1.3 times
-// as many as are wanted, on average -- are collected and put in order by counting, for each, those before it.  1000 rows of
-// 1024 for 32 streams: K = 4 (16 entries) 84 us, K = 32 (44 entries) 127 us; a round per pick took 96 and 290.
-constexpr int kTopWarps = 8;
-constexpr int kTopCap = 128;           // tokens collected at a time
-static_assert(kTopCap > TB_MAX_BEAM + 13, "more than any row keeps");
-template <typename LT>
-__global__ void __launch_bounds__(kTopWarps * 32) k_beam_topm(const LT* logits, int32_t B, int32_t T, int32_t E, int32_t V, int32_t C,
-                                                            int64_t stream_stride, int64_t frame_stride, int64_t row_stride,
-                                                            const int32_t* n_frames, const TbSlotRec* slots, const unsigned char* arena,
-                                                            const int32_t* cls, int32_t top_m, TbTopEnt* out) {
-  pdl_chain();
-  extern __shared__ __align__(16) unsigned char dyn[];
-  float* rootcw = reinterpret_cast<float*>(dyn);                                  // [C] root arc weight per class
-  float* ybuf = reinterpret_cast<float*>(dyn) + C;                                // [kTopWarps][V]
-  const int rows_per_stream = T * E, blocks_per_stream = (rows_per_stream + kTopWarps - 1) / kTopWarps;
-  const int b = blockIdx.x / blocks_per_stream, r0 = (blockIdx.x - b * blocks_per_stream) * kTopWarps;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const TbSlotRec rec = slots[b];
-  const bool bound = rec.n_states > 0;
-  const GraphPtrs g = graph_of(arena, rec);
-  for (int c = threadIdx.x; c < C; c += blockDim.x) rootcw[c] = 0.0f;
-  __syncthreads();
-  if (bound) {
-    const int e = g.arc_begin[1];
-    for (int a = g.arc_begin[0] + threadIdx.x; a < e; a += blockDim.x) {
-      const int c = g.arc_cls[a];
-      if (c >= 0 && c < C) rootcw[c] = __fadd_rn(0.0f, g.arc_w[a]);
-    }
-  }
-  __syncthreads();
-  const int r = r0 + warp;
-  if (r >= rows_per_stream) return;
-  const int t = r / E, e = r - t * E;
-  if (n_frames && t >= n_frames[b]) return;
-  const LT* row = logits + static_cast<int64_t>(b) * stream_stride + static_cast<int64_t>(t) * frame_stride + static_cast<int64_t>(e) * row_stride;
-  TbTopEnt* o = out + (static_cast<int64_t>(b) * rows_per_stream + r) * (top_m + 1);
-  uint32_t* y = reinterpret_cast<uint32_t*>(ybuf) + static_cast<size_t>(warp) * V;        // keys of the row's y
-  uint64_t* cand = reinterpret_cast<uint64_t*>(dyn + (((static_cast<size_t>(C) + static_cast<size_t>(kTopWarps) * V) * 4 + 7) & ~size_t(7))) + warp * kTopCap;
-  const int want = top_m + 1;
-  uint32_t k0 = 0u, k1 = 0u;                                  // the lane's best and second best (0: none)
-#pragma unroll 4
-  for (int v = lane; v < V; v += 32) {
-    const float x = LogitLoad<LT>::at(row + v);
-    const uint32_t k = order_key(bound ? __fadd_rn(x, __fmul_rn(g.lambda, rootcw[__ldg(cls + v)])) : x);
-    y[v] = k;
-    k1 = max(k1, min(k0, k));
-    k0 = max(k0, k);
-  }
-  __syncwarp();
-  // at least `want` tokens have thr or more (rows shorter than that: all have)
-  uint32_t thr = 0u;
-  {
-    int n0 = 0, n1 = 0;                                       // how many of the lanes' values come before this lane's
-    const bool both = want > 28;
-#pragma unroll 4
-    for (int j = 0; j < 32; ++j) {
-      const uint32_t o0 = __shfl_sync(0xffffffffu, k0, j);
-      n0 += (o0 > k0 || (o0 == k0 && j < lane)) ? 1 : 0;
-      if (both) {
-        const uint32_t o1 = __shfl_sync(0xffffffffu, k1, j);
-        n0 += o1 > k0 ? 1 : 0;
-        n1 += (o0 >= k1 ? 1 : 0) + ((o1 > k1 || (o1 == k1 && j < lane)) ? 1 : 0);
-      }
-    }
-    const unsigned at0 = __ballot_sync(0xffffffffu, n0 == want - 1), at1 = __ballot_sync(0xffffffffu, both && n1 == want - 1);
-    if (at0) thr = __shfl_sync(0xffffffffu, k0, __ffs(at0) - 1);
-    else if (at1) thr = __shfl_sync(0xffffffffu, k1, __ffs(at1) - 1);
-  }
-  // candidates as value key << 32 | inverted token, all different
-  uint64_t lim = static_cast<uint64_t>(thr) << 32;
-  int n;
-#pragma unroll 1
-  for (;;) {
-    n = 0;
-#pragma unroll 1
-    for (int v0 = 0; v0 < V && n < kTopCap; v0 += 32) {
-      const int v = v0 + lane;
-      const uint64_t k = v < V ? static_cast<uint64_t>(y[v]) << 32 | (0xFFFFFFFFu - static_cast<uint32_t>(v)) : 0ull;
-      const bool hit = v < V && k >= lim;
-      const unsigned mask = __ballot_sync(0xffffffffu, hit);
-      if (mask == 0u) continue;
-      const int at = n + __popc(mask & ((1u << lane) - 1u));
-      if (hit && at < kTopCap) cand[at] = k;
-      n += __popc(mask);
-    }
-    n = min(n, kTopCap);
-    __syncwarp();
-    if (n < kTopCap) break;
-    // more than can be held: the want-th of those that were bounds the row's from below more tightly (and lim rises, as they
-    // are all different and more than are wanted)
-    uint64_t next = 0ull;
-#pragma unroll 1
-    for (int i = lane; i < n; i += 32) {
-      const uint64_t k = cand[i];
-      int before = 0;
-#pragma unroll 4
-      for (int j = 0; j < n; ++j) before += cand[j] > k ? 1 : 0;
-      if (before == want - 1) next = k;
-    }
-    const unsigned who = __ballot_sync(0xffffffffu, next != 0ull);
-    next = __shfl_sync(0xffffffffu, next, __ffs(who) - 1);
-    __syncwarp();
-    lim = next;
-  }
-#pragma unroll 1
-  for (int i = lane; i < n; i += 32) {
-    const uint64_t k = cand[i];
-    int m = 0;
-#pragma unroll 4
-    for (int j = 0; j < n; ++j) m += cand[j] > k ? 1 : 0;
-    if (m > top_m) continue;
-    const int tok = static_cast<int>(0xFFFFFFFFu - static_cast<uint32_t>(k));
-    TbTopEnt e;
-    e.y = order_key_inv(static_cast<uint32_t>(k >> 32));
-    if (m == top_m) { e.x = LogitLoad<LT>::at(row + V); e.tok_cls = 0u; }
-    else { e.x = LogitLoad<LT>::at(row + tok); e.tok_cls = static_cast<uint32_t>(tok) | (static_cast<uint32_t>(__ldg(cls + tok)) << 16); }
-    o[m] = e;
-  }
-  for (int m = n + lane; m <= top_m; m += 32) {               // fewer tokens in the row
-    TbTopEnt e;
-    e.y = -INFINITY; e.x = m == top_m ? LogitLoad<LT>::at(row + V) : -INFINITY; e.tok_cls = m == top_m ? 0u : 0xFFFFu;
-    o[m] = e;
-  }
 }
 
 // A chunk of streaming beam decoding: slot by slot, n_frames[slot] frames (at most T) of E rows; each slot has its own
@@ -1838,25 +1728,5 @@ int tb_launch_publish_slots(TbSlotRec* slots, TbSlotState* sstate, int32_t n, co
 int tb_launch_pull_binds(const TbInlineBinds& ib, TbSlotState* sstate, cudaStream_t stream) {
   if (ib.n < 1 || ib.n > TB_INLINE_BINDS || !ib.arena || !ib.slots || !sstate) return TB_ERR_INVALID_ARG;
   k_pull_binds<<<ib.n, kPullThreads, 0, stream>>>(ib, sstate);
-  return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
-}
-
-int tb_launch_beam_topm(const void* logits, int dtype, int32_t B, int32_t T, int32_t E, int32_t V, int32_t C,
-                        int64_t stream_stride, int64_t frame_stride, int64_t row_stride, const int32_t* n_frames,
-                        const TbSlotRec* slots, const unsigned char* arena, const int32_t* cls, int32_t top_m,
-                        TbTopEnt* out, cudaStream_t stream) {
-  // root weights per class, every warp's y values, every warp's candidates
-  const size_t smem = (((static_cast<size_t>(C) + static_cast<size_t>(kTopWarps) * V) * sizeof(float) + 7) & ~size_t(7)) + kTopWarps * kTopCap * sizeof(uint64_t);
-  const int blocks = B * ((T * E + kTopWarps - 1) / kTopWarps);
-  int rc;
-  if (dtype == TB_BF16) {
-    if ((rc = set_smem(k_beam_topm<uint16_t>, smem)) != TB_OK) return rc;
-    if (tb_launch_chained(k_beam_topm<uint16_t>, dim3(blocks), dim3(kTopWarps * 32), smem, stream, static_cast<const uint16_t*>(logits), B, T, E, V, C, stream_stride,
-                                                                  frame_stride, row_stride, n_frames, slots, arena, cls, top_m, out) != TB_OK) return TB_ERR_CUDA;
-  } else {
-    if ((rc = set_smem(k_beam_topm<float>, smem)) != TB_OK) return rc;
-    if (tb_launch_chained(k_beam_topm<float>, dim3(blocks), dim3(kTopWarps * 32), smem, stream, static_cast<const float*>(logits), B, T, E, V, C, stream_stride,
-                                                               frame_stride, row_stride, n_frames, slots, arena, cls, top_m, out) != TB_OK) return TB_ERR_CUDA;
-  }
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }

@@ -159,7 +159,7 @@ int tb_launch_final_weights_slots(const TbSlotRec* slots, const unsigned char* a
 int tb_launch_beam_topm(const void* logits, int dtype, int32_t B, int32_t T, int32_t E, int32_t V, int32_t C,
                         int64_t stream_stride, int64_t frame_stride, int64_t row_stride, const int32_t* n_frames,
                         const TbSlotRec* slots, const unsigned char* arena, const int32_t* cls, int32_t top_m,
-                        TbTopEnt* out, cudaStream_t stream);
+                        TbTopEnt* out, int32_t n_sm, cudaStream_t stream);
 int tb_launch_beam_backtrace(const int2* tree, int32_t n_steps, int32_t B, int32_t K, int32_t V, int32_t max_len,
                              int32_t* out_tokens, int32_t* out_lens, cudaStream_t stream);
 // Registered models: their records live in a device table; tb_launch_bind_models points up to TB_BIND_PAIRS slots at
