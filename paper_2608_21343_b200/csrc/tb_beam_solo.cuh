@@ -14,7 +14,7 @@
 // beams would have two lanes a hypothesis, which a first step's picks do not fit.)
 // A step is untouched and left to the team when a lane might have held one pick more than it keeps, or when the K-th pick does not
 // clear the bound on the tokens that were not looked at (as in the team's step, with the first token behind those looked at).
-__device__ __forceinline__ void beam_solo_barrier() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
+__device__ __forceinline__ void beam_group_barrier(int n_threads) { asm volatile("bar.sync 2, %0;" ::"r"(n_threads) : "memory"); }
 
 // The logit at 2 * token of a row in shared memory.
 template <typename LT> __device__ __forceinline__ float beam_smem_logit2(const unsigned char* row, uint32_t token2);
@@ -25,14 +25,17 @@ template <> __device__ __forceinline__ float beam_smem_logit2<float>(const unsig
   return *reinterpret_cast<const float*>(row + 2 * token2);
 }
 
-// What the second warp prepares per row, and what the first leaves it per step.
-struct BeamSolo {
+// What the serving warp prepares per row, and what the steps leave it: rows brought R at a time, PLAIN tokens of a reduced row, PLACES hypotheses at most.
+template <int R, int PLAIN, int PLACES>
+struct BeamAhead {
+  static constexpr int kRows = R;
   struct Row { float xb, y_next; uint32_t at, unused; };       // blank, value of the first token not looked at, where the row begins (behind dyn)
-  uint4 plain[2 * kSoloRows][kSoloPlain];                      // per token looked at: logit, its class' root weight, token, the root arc's target
-  Row row[2 * kSoloRows];
-  uint32_t pick[2 * kSoloRows][kSoloBeam];                     // 32 * token key + parent of every place's pick, all ones: none
+  uint4 plain[2 * R][PLAIN];                                   // per token looked at: logit, its class' root weight, token, the root arc's target
+  Row row[2 * R];
+  uint32_t pick[2 * R][PLACES];                                // 32 * token key + parent of every place's pick, all ones: none
   uint32_t stamp;                                              // the last step's number, in the upper bits (see beam_solo_run)
 };
+using BeamSolo = BeamAhead<kSoloRows, kSoloPlain, kSoloBeam>;
 
 // Row sidx of the block's stream, the way from a frame's last row to the next frame, and the row's reduced form.
 template <typename LT>
@@ -63,12 +66,12 @@ struct BeamSoloRows {
 
 // The second warp: brings rows sidx, sidx + 1, ... into the buffers and keeps the books of the steps before: the tree, and what
 // identifies the hypotheses' token sequences.  (fetched: the first rows are on their way already.)  sh.cmd holds the number of the barrier that ends the run, sh.done the steps
-// taken by then.
-template <typename LT, int KG>
-__device__ __forceinline__ void beam_solo_serve(const TbBeamParams& p, BeamShared& sh, BeamSolo& so, unsigned char* dyn, const TeamSmem& tm, int32_t sidx,
+// taken by then.  P: tokens of a reduced row that the steps look at; n_threads: of the group barrier, the steps' warps and this one.
+template <typename LT, int P, typename Ahead>
+__device__ __forceinline__ void beam_serve(const TbBeamParams& p, BeamShared& sh, Ahead& so, unsigned char* dyn, const TeamSmem& tm, int32_t sidx,
                                                 const int32_t n_steps, BeamSoloRows<LT> at, bool fetched, const int32_t step_base, unsigned long long* hashA, unsigned long long* hashB,
-                                                int32_t* lenA, int32_t* lenB, const int32_t par0) {
-  constexpr int P = KG <= 4 ? 8 : kSoloPlain;
+                                                int32_t* lenA, int32_t* lenB, const int32_t par0, const int n_threads) {
+  constexpr int R = Ahead::kRows;
   const int lane = threadIdx.x & 31, b = blockIdx.x, K = p.K, V = p.V, W = V + 1, M = p.top_m;
   const bool bound = p.slots[b].n_states > 0;
   const int WW = (W + 31) >> 5;
@@ -88,7 +91,7 @@ __device__ __forceinline__ void beam_solo_serve(const TbBeamParams& p, BeamShare
   for (int n = 1;; ++n) {
     int rows = 0;
 #pragma unroll 1
-    for (; rows < kSoloRows && sidx < n_steps; ++rows, ++sidx) {
+    for (; rows < R && sidx < n_steps; ++rows, ++sidx) {
       if (!fetched) at.fetch(p, mem, tm, buf + rows);
       if (lane == 0) so.row[buf + rows].at = static_cast<uint32_t>(mem - dyn) + tm.row + (buf + rows) * tm.row_stride + static_cast<uint32_t>(reinterpret_cast<uintptr_t>(at.row) & 15u);
       at.next();
@@ -96,7 +99,7 @@ __device__ __forceinline__ void beam_solo_serve(const TbBeamParams& p, BeamShare
     fetched = false;
     // the steps before the last barrier (the rows are on their way)
     const bool end = n > 1 && *cmd == n - 1;
-    const int32_t upto = end ? first + *const_cast<volatile int32_t*>(&sh.done) : first + max(n - 2, 0) * kSoloRows;
+    const int32_t upto = end ? first + *const_cast<volatile int32_t*>(&sh.done) : first + max(n - 2, 0) * R;
 #pragma unroll 1
     for (; step < upto; ++step) {
       const uint32_t l2 = lane < K ? so.pick[book][lane] : 0xFFFFFFFFu;
@@ -122,7 +125,7 @@ __device__ __forceinline__ void beam_solo_serve(const TbBeamParams& p, BeamShare
         }
       }
       if (++tree_at == p.tree_cap) tree_at = 0;
-      book = (book + 1) & (2 * kSoloRows - 1);
+      book = (book + 1) & (2 * R - 1);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();
@@ -135,8 +138,8 @@ __device__ __forceinline__ void beam_solo_serve(const TbBeamParams& p, BeamShare
       so.plain[r][q] = make_uint4(__float_as_uint(t[q].x), bound ? __float_as_uint(rootcw[cl]) : 0u, tc & 0xFFFFu, bound ? static_cast<uint32_t>(rootdst[cl]) : 0u);
       if (q == 0) { so.row[r].xb = t[M].x; so.row[r].y_next = t[P].y; }
     }
-    beam_solo_barrier();                                       // group n is there, group n - 1 has been read
-    buf ^= kSoloRows;
+    beam_group_barrier(n_threads);                                       // group n is there, group n - 1 has been read
+    buf ^= R;
   }
   if (lane < K) { sh.h_hash[lane] = hh; sh.h_len[lane] = hl; }
 }
@@ -227,7 +230,7 @@ __device__ __forceinline__ int beam_solo_run(const TbBeamParams& p, BeamShared& 
   int done = 0, slot = 0, n_bar = 0;
 #pragma unroll 1
   for (; sidx < n_steps; ++sidx) {
-    if ((slot & (kSoloRows - 1)) == 0) { beam_solo_barrier(); ++n_bar; }
+    if ((slot & (kSoloRows - 1)) == 0) { beam_group_barrier(64); ++n_bar; }
     const BeamSolo::Row ro = so.row[slot];
     const unsigned char* row = dyn + ro.at;
     stamp += 1u << kDstBits;
@@ -363,7 +366,7 @@ __device__ __forceinline__ int beam_solo_run(const TbBeamParams& p, BeamShared& 
     sh.h_score[hyp] = sc; sh.h_state[hyp] = st; sh.h_live[hyp] = lv ? 1 : 0;
   }
   __syncwarp();
-  beam_solo_barrier();
+  beam_group_barrier(64);
   return done;
 }
 

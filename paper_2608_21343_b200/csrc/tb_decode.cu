@@ -662,8 +662,10 @@ constexpr int kSoloBeam = 8;              // hypotheses at most
 constexpr int kSoloRows = 4;              // rows brought at a time (two such groups in shared memory)
 constexpr int kSoloVocab = 64;            // rows of fewer tokens are left to the team
 constexpr int kSoloPlain = 12;            // tokens of a reduced row that are looked at, at most
-__host__ __device__ inline bool beam_solo_width(int K, int V) { return K <= kSoloBeam && V >= kSoloVocab; }
-__host__ __device__ inline int beam_rows_kept(int K, int V) { return beam_solo_width(K, V) ? 2 * kSoloRows : kTeamRows; }
+// Wider ones by a crew of warps, four hypotheses each (tb_beam_crew.cuh); what that cannot take goes to the team as well.
+constexpr int kCrewBeam = 32, kCrewWarps = kCrewBeam / 4;
+constexpr int kCrewRows = 2;              // rows brought at a time (two such groups in shared memory)
+constexpr int kCrewPlain = 16;            // tokens of a reduced row that are looked at
 
 __host__ __device__ inline int team_warps(int K) { return K > 16 ? 16 : K < 4 ? 4 : K; }
 __device__ __forceinline__ unsigned long long beam_key(float v, int tkey, int k) {
@@ -706,8 +708,7 @@ __device__ __forceinline__ void beam_fetch_row(unsigned char* buf, const LT* row
 }
 // Shared memory of the team behind the block's other arrays: row buffers, reduced rows, the copy of the list records.
 struct TeamSmem { int row, row_stride, top, top_stride, recs, total; };
-__host__ __device__ inline TeamSmem team_smem(int K, int V, int elem, int top_m, int rec_bytes) {
-  const int rows = beam_rows_kept(K, V);
+__host__ __device__ inline TeamSmem team_smem(int rows, int V, int elem, int top_m, int rec_bytes) {
   TeamSmem t;
   t.row_stride = (((V + 1) * elem + 16 + 15) & ~15) + 16;
   t.row = 0;
@@ -1198,10 +1199,12 @@ __device__ __forceinline__ int beam_team_run(const TbBeamParams& p, BeamShared& 
 }
 
 #include "tb_beam_solo.cuh"
+using BeamCrewAhead = BeamAhead<kCrewRows, kCrewPlain, kCrewBeam>;
+#include "tb_beam_crew.cuh"
 
 // All steps of one stream of a multi-step launch: a warp or the team takes what it can, the block the rest.
 // WIDTH: 0 up to kSoloBeam hypotheses, 1 up to 16, 2 more.  (A kernel each: in one kernel the registers and the code of one weighed on the others --
-// 32 streams of 1000 steps, K = 32, 4155 us and 4384 with the single warp's steps beside the team's, 3740 alone; K = 12 2633 and 2406.)
+// 32 streams of 1000 steps, K = 32, 4384 us with the single warp's steps beside the team's, 3740 with the team's alone; K = 12 2633 and 2406.)
 template <typename LT, int WIDTH>
 __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared& sh, unsigned char* dyn, const int32_t n_steps, const int32_t E,
                                                const int64_t frame_stride, const int64_t row_stride, const int32_t rows_per_stream,
@@ -1210,12 +1213,13 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
   LT xpre[kBeamPref] = {};
   bool xpre_valid = false;
   const bool fast = beam_team_applies(p);
-  const TeamSmem tm = team_smem(p.K, p.V, sizeof(LT), p.top_m, p.rec_cache_bytes);
+  const TeamSmem tm = team_smem(p.rows_kept, p.V, sizeof(LT), p.top_m, p.rec_cache_bytes);
   const bool odd0 = (par0 & 1) != 0;
-  const bool solo = WIDTH == 0 && fast && beam_solo_width(p.K, p.V);
-  __shared__ BeamSolo so;
-  if constexpr (WIDTH == 0) {                 // the first rows are on their way while the tables are laid out
-    const int row = static_cast<int>(threadIdx.x >> 5) - (kBeamThreads / 32 - kSoloRows);     // (a row each by the block's last warps)
+  const bool solo = fast && p.rows_kept > kTeamRows;            // steps by a warp or a crew (the launcher made room for their rows)
+  using Ahead = typename std::conditional<WIDTH == 0, BeamSolo, BeamCrewAhead>::type;
+  __shared__ Ahead so;
+  {                                           // the first rows are on their way while the tables are laid out
+    const int row = static_cast<int>(threadIdx.x >> 5) - (kBeamThreads / 32 - Ahead::kRows);     // (a row each by the block's last warps)
     if (solo && row >= 0 && row < n_steps) BeamSoloRows<LT>(p, row, E, frame_stride, row_stride, rows_per_stream).fetch(p, team_base(p, dyn), tm, row);
   }
   const bool recs_cached = beam_begin(p, sh, dyn, odd0 ? hashB : hashA, odd0 ? lenB : lenA, fast, tm);
@@ -1231,27 +1235,35 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
   int32_t team_steps = 1;                     // steps the team takes when the warp could not
 #pragma unroll 1
   for (int32_t sidx = 0; sidx < n_steps; ++sidx) {
-    if constexpr (WIDTH == 0) {
-      if (solo && skip <= 0) {
-        if (!clean) { clear(); clean = true; }
-        if (threadIdx.x < 32) {
-          const int d = p.K > 4 ? beam_solo_run<LT, 8>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm) : beam_solo_run<LT, 4>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm);
-          if (threadIdx.x == 0) sh.team_done = d;
-        } else if (threadIdx.x < 64) {
-          const BeamSoloRows<LT> at(p, sidx, E, frame_stride, row_stride, rows_per_stream);
-          if (p.K > 4)
-            beam_solo_serve<LT, 8>(p, sh, so, dyn, tm, sidx, n_steps, at, sidx == 0 && first, step_base, hashA, hashB, lenA, lenB, par0);
-          else
-            beam_solo_serve<LT, 4>(p, sh, so, dyn, tm, sidx, n_steps, at, sidx == 0 && first, step_base, hashA, hashB, lenA, lenB, par0);
-        }
-        __syncthreads();
-        const int d = sh.team_done;
-        first = false;
-        __syncthreads();                          // (read by everyone before a later run writes it again)
-        sidx += d;
-        if (sidx >= n_steps) break;
-        team_steps = d == 0 ? min(2 * team_steps, 32) : 1;
+    if (solo && skip <= 0) {
+      if (!clean) { clear(); clean = true; }
+      const BeamSoloRows<LT> at(p, sidx, E, frame_stride, row_stride, rows_per_stream);
+      const bool fetched = sidx == 0 && first;
+      const int warp = threadIdx.x >> 5;
+      int d = 0;
+      if constexpr (WIDTH == 0) {
+        if (warp == 0)
+          d = p.K > 4 ? beam_solo_run<LT, 8>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm) : beam_solo_run<LT, 4>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm);
+        else if (warp == 1 && p.K > 4)
+          beam_serve<LT, kSoloPlain>(p, sh, so, dyn, tm, sidx, n_steps, at, fetched, step_base, hashA, hashB, lenA, lenB, par0, 64);
+        else if (warp == 1)
+          beam_serve<LT, 8>(p, sh, so, dyn, tm, sidx, n_steps, at, fetched, step_base, hashA, hashB, lenA, lenB, par0, 64);
+      } else {
+        __shared__ BeamCrew cr;
+        const int n_warps = (p.K + 3) >> 2;
+        if (warp < n_warps)
+          d = beam_crew_run<LT>(p, sh, so, cr, dyn, sidx, n_steps, E, recs_cached, tm);
+        else if (warp == n_warps)
+          beam_serve<LT, kCrewPlain>(p, sh, so, dyn, tm, sidx, n_steps, at, fetched, step_base, hashA, hashB, lenA, lenB, par0, 32 * n_warps + 32);
       }
+      if (threadIdx.x == 0) sh.team_done = d;
+      __syncthreads();
+      d = sh.team_done;
+      first = false;
+      __syncthreads();                          // (read by everyone before a later run writes it again)
+      sidx += d;
+      if (sidx >= n_steps) break;
+      team_steps = d == 0 ? min(2 * team_steps, 32) : 1;
     }
     if (fast && skip-- <= 0) {
       const int32_t stop = solo ? min(n_steps, sidx + team_steps) : n_steps;
@@ -1506,10 +1518,15 @@ static int beam_width_class(int K, F f) {
 // of the logits tensor; without either (odd strides, no room) they stay off.
 static void beam_team_setup(TbBeamParams* p, int32_t T, int32_t E, int64_t frame_stride, int64_t row_stride, size_t* smem) {
   constexpr size_t kMost = 200 * 1024;
-  p->tensor_lo = nullptr; p->tensor_hi = nullptr; p->rec_cache_bytes = 0;
+  p->tensor_lo = nullptr; p->tensor_hi = nullptr; p->rec_cache_bytes = 0; p->rows_kept = 0;
   if (!p->top_base || p->stream_stride < 0 || frame_stride < 0 || row_stride < 0) return;
   const int elem = p->dtype == TB_BF16 ? 2 : 4;
-  const size_t more = team_smem(p->K, p->V, elem, p->top_m, 0).total;
+  p->rows_kept = p->K <= kSoloBeam ? 2 * kSoloRows : 2 * kCrewRows;
+  size_t more = team_smem(p->rows_kept, p->V, elem, p->top_m, 0).total;
+  if (p->V < kSoloVocab || *smem + more > kMost) {
+    p->rows_kept = kTeamRows;
+    more = team_smem(kTeamRows, p->V, elem, p->top_m, 0).total;
+  }
   if (*smem + more > kMost) return;
   *smem += more;
   p->rec_cache_bytes = static_cast<int32_t>((kMost - *smem < static_cast<size_t>(kTeamRecCache) ? kMost - *smem : static_cast<size_t>(kTeamRecCache)) & ~size_t(15));
