@@ -135,7 +135,7 @@ __host__ __device__ inline DecSmem dec_smem(int V, int C, int S, int frames, int
   return s;
 }
 
-template <typename LT>
+template <typename LT, bool WALK>
 __global__ void __launch_bounds__(32 * kDecMaxSegs, 1) k_decide_rows(const __grid_constant__ RowsParams P) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ float part[3 * kDecMaxSegs];
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(32 * kDecMaxSegs, 1) k_decide_rows(const __gri
     cu.t = max(0, o.first - ((bound && warp > 0) ? kDecWarm : 0)); cu.k = 0; cu.s = bound ? 0 : -1;
     cu.n_out = cu.nv = 0; cu.failed = false; cu.met = -1; cu.listed = false;
     if (warp == 0) o.first = INT32_MAX;                                     // (nobody needs the first stretch's records)
-    decide<LT, true>(c, cu, o, P.sums + static_cast<int64_t>(b) * p.frames * S,
+    decide<LT, true, WALK>(c, cu, o, P.sums + static_cast<int64_t>(b) * p.frames * S,
                                shared_u32(dyn + so.ring) + warp * kDecRing * S * 32, kDecRing - 1, 0, end, lane);
     if (lane == 0) {
       res[2 * warp] = make_int4(cu.n_out, cu.nv, cu.s, cu.met >= 0 ? cu.met : cu.t);
@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(kChunkThreads, 3) k_chunk_rows(const __grid_co
     if (warp == 0) {
       if (cu.t < f1) {
         cu.nv = 0;
-        decide<LT, false>(c, cu, o, nullptr, shared_u32(sums), kPiece - 1, t0, f1, lane);
+        decide<LT, false, false>(c, cu, o, nullptr, shared_u32(sums), kPiece - 1, t0, f1, lane);
         __syncwarp();
         if (lane == 0) {
 #pragma unroll 4
@@ -478,7 +478,8 @@ int tb_launch_rows(const TbDecodeParams& d, const TbRowsPlan& plan, int32_t n_sm
     f1 = narrow ? (with_tab ? k_row_sums<uint16_t, 4, true> : k_row_sums<uint16_t, 4, false>) : with_tab ? k_row_sums<uint16_t, 8, true> : k_row_sums<uint16_t, 8, false>;
   else
     f1 = narrow ? (with_tab ? k_row_sums<float, 4, true> : k_row_sums<float, 4, false>) : with_tab ? k_row_sums<float, 8, true> : k_row_sums<float, 8, false>;
-  void (*f2)(RowsParams) = d.dtype == TB_BF16 ? k_decide_rows<uint16_t> : k_decide_rows<float>;
+  void (*f2)(RowsParams) = plan.all_resolved ? (d.dtype == TB_BF16 ? k_decide_rows<uint16_t, false> : k_decide_rows<float, false>)
+                                             : d.dtype == TB_BF16 ? k_decide_rows<uint16_t, true> : k_decide_rows<float, true>;
   const size_t smem1 = root_tab_bytes(d.C) + (with_tab ? tab : 0);
   if (smem1 > 24 * 1024 && cudaFuncSetAttribute(f1, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem1)) != cudaSuccess) {
     cudaGetLastError();

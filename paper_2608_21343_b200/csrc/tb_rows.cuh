@@ -503,8 +503,8 @@ __device__ __forceinline__ int walk_flat(const DecideCtx<LT>& c, int s, float& s
   return n;
 }
 
-// The list of state s (warp-wide).
-template <typename LT>
+// The list of state s (warp-wide); W: groups of 32 entries of a chain state that are asked for at once.
+template <typename LT, int W>
 __device__ __forceinline__ TokList list_of(const DecideCtx<LT>& c, int s, int lane) {
   TokList L;
   if (c.resolved) {
@@ -531,16 +531,37 @@ __device__ __forceinline__ TokList list_of(const DecideCtx<LT>& c, int s, int la
     uint4 nrec = rec;
     if (nu > 0) nrec = *reinterpret_cast<const uint4*>(c.strec + nu);
     const int e1 = static_cast<int>(rec.y);
-#pragma unroll 2
-    for (int e = static_cast<int>(rec.x) + lane; __any_sync(0xffffffffu, e < e1); e += 32) {
-      uint4 ent = make_uint4(0u, 0u, 0u, 0u);                 // TbTokEnt
-      if (e < e1) ent = *reinterpret_cast<const uint4*>(c.tokent + e);
-      // (where an entry leads: the state's record and its first arcs are asked into L2, in case the entry is taken)
-      if (e < e1) {
+    // (where an entry leads: the state's record and its first arcs are asked into L2, in case the entry is taken)
+    auto take = [&](bool have, const uint4& ent) {            // TbTokEnt
+      if (have) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(c.strec + ent.z));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(c.tokent + ent.w));
       }
-      walk_add(c, e < e1, static_cast<int>(ent.x & 0xFFFFu), ent.z, __uint_as_float(ent.y), acc, n, lane);
+      walk_add(c, have, static_cast<int>(ent.x & 0xFFFFu), ent.z, __uint_as_float(ent.y), acc, n, lane);
+    };
+    if constexpr (W > 1) {
+#pragma unroll 1
+      for (int e0 = static_cast<int>(rec.x); e0 < e1; e0 += 32 * W) {
+        uint4 ent[W];
+#pragma unroll
+        for (int u = 0; u < W; ++u) {
+          const int e = e0 + 32 * u + lane;
+          ent[u] = make_uint4(0u, 0u, 0u, 0u);
+          if (e < e1) ent[u] = *reinterpret_cast<const uint4*>(c.tokent + e);
+        }
+#pragma unroll
+        for (int u = 0; u < W; ++u) {
+          if (u > 0 && e0 + 32 * u >= e1) break;
+          take(e0 + 32 * u + lane < e1, ent[u]);
+        }
+      }
+    } else {
+#pragma unroll 2
+      for (int e = static_cast<int>(rec.x) + lane; __any_sync(0xffffffffu, e < e1); e += 32) {
+        uint4 ent = make_uint4(0u, 0u, 0u, 0u);
+        if (e < e1) ent = *reinterpret_cast<const uint4*>(c.tokent + e);
+        take(e < e1, ent);
+      }
     }
     __syncwarp();
     acc = __fadd_rn(acc, __uint_as_float(rec.w));
@@ -662,10 +683,16 @@ struct DecideOut {
 // Decides the rows from the cursor on, up to frame `end` (exclusive).  Summaries of row k of frame f are at shared
 // address sum_a + (((f - f0) & mask) * S + k) * 32; SEG: that is a ring of mask + 1 frames which the decider fills itself
 // from gsum (the summary of row 0 of frame 0), else they are all in place.  f0: the frame the rows (c.base) start at.
-template <typename LT, bool SEG>
+// WALK: for lists that are put together by walking.  A lane's entries of a list whose logits are on their way at once, and groups of a chain state's entries,
+// are more then: a state of 64 streams with lists of 1000 own phrases and 4000 shared ones has about 140 entries, of which the logits, all over their row, took
+// 4400 of a round's 9500 cycles and the walk 3600.  A call took 1283 us with 4 entries and 2 groups, 1169 with 8 and 2, 1119 with 8 and 4, 1096 with 12 and 4,
+// 1117 with 16 and 4, 1203 with 8 and 8.  (Resolved lists are shorter: 32 fp32 streams of 500 frames 152 us with 4 entries, 162 with 12.  Rows
+// brought into shared memory ahead of their rounds leave L1 too little: 1369.)
+template <typename LT, bool SEG, bool WALK>
 __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const DecideOut& o, const RowSum* gsum,
                                        uint32_t sum_a, int mask, int f0, int end, int lane) {
   const int S = c.S, V = c.V, tb = c.tb;
+  constexpr int kIn = WALK ? 12 : 4, kWalk = WALK ? 4 : 1;
   const bool tdt = !SEG && c.n_dur > 0;
   int t = cu.t, k = cu.k, s = cu.s, n_out = cu.n_out, nv = cu.nv;
   bool listed = cu.listed;
@@ -704,7 +731,7 @@ __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const
         __syncwarp();
       }
     }
-    if (!listed) { L = list_of<LT>(c, s, lane); listed = true; }
+    if (!listed) { L = list_of<LT, kWalk>(c, s, lane); listed = true; }
     // One round: up to eight rows in the order they are visited in, a group of lanes each.  Which rows those are, and the
     // graph state each is visited in, is predicted from the summaries alone -- a row selects its best plain token, which
     // leads to a root arc's target, or blank -- and every group then decides its row exactly under the state predicted for
@@ -776,18 +803,18 @@ __device__ __forceinline__ void decide(const DecideCtx<LT>& c, Cursor& cu, const
     uint32_t lt = none;
     bool in_deep = false;
 #pragma unroll 1
-    for (int i0 = lane & (G - 1); i0 < ll.n; i0 += 4 * G) {
-      uint2 e[4];
-      float x[4];
+    for (int i0 = lane & (G - 1); i0 < ll.n; i0 += kIn * G) {
+      uint2 e[kIn];
+      float x[kIn];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < kIn; ++u) {
         e[u] = make_uint2(2u * static_cast<uint32_t>(V), 0xFF800000u);
         if (i0 + u * G < ll.n) e[u] = *reinterpret_cast<const uint2*>(ll.ent + i0 + u * G);
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) x[u] = LogitLoad<LT>::at(row + ((e[u].x & tmask) >> 1));
+      for (int u = 0; u < kIn; ++u) x[u] = LogitLoad<LT>::at(row + ((e[u].x & tmask) >> 1));
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < kIn; ++u) {
         const uint32_t td = td_pack(e[u].x, tb);
         const float v = __fadd_rn(x[u], __uint_as_float(e[u].y));
         if (v > lv || (v == lv && td < lt)) { lv = v; lt = td; }
