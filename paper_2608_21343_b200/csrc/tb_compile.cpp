@@ -59,7 +59,9 @@ struct PoolBypass {
 // carry per-state records and token-expanded arcs instead, which the kernels walk.
 // `tree`: the arcs are those of a tree of single-class steps (tb_graph_compile), for which a list's length follows from its
 // suffix state's: an own arc shadows an inherited one exactly when the arc's target has a suffix of two classes or more.
-static void finalize_graph(tb_graph* g, const int32_t* case_class, int32_t vocab, int32_t n_classes, float lambda, bool tree) {
+// `whole`: the suffix links' weights are whole numbers far below 2^24 (every token weighs 1), so their sums along a chain do not depend on the order and
+// follow from the suffix state's as well.
+static void finalize_graph(tb_graph* g, const int32_t* case_class, int32_t vocab, int32_t n_classes, float lambda, bool tree, bool whole) {
   const int32_t N = g->n_states, A = g->n_arcs;
   g->case_class.resize(vocab);
   for (int32_t v = 0; v < vocab; ++v) g->case_class[v] = case_class ? case_class[v] : v;
@@ -80,11 +82,13 @@ static void finalize_graph(tb_graph* g, const int32_t* case_class, int32_t vocab
   bool fits = N < (1 << (32 - tb_rs_tok_bits(vocab)));
   int64_t total = 0;
   g->d_max = 0.0f;
+  // (lists of 970 tokens on average, this part of a compile: 9.7 us with a walk per state, 6.5 with the suffix states' sums)
   for (int32_t s = 0; s < N; ++s) {
     float acc = 0.0f;
     int32_t c = 0;
+    if (whole && s) acc = rrecs[g->state_fail[s]].D + g->state_bw[s];
     if (tree && s) c = count[g->state_fail[s]] + static_cast<int32_t>(own[g->state_arc_begin[s + 1]] - own[g->state_arc_begin[s]]);
-    for (int32_t u = s; u != 0; u = g->state_fail[u]) {
+    for (int32_t u = whole ? 0 : s; u != 0; u = g->state_fail[u]) {
       if (!tree && fits)
         for (int32_t a = g->state_arc_begin[u]; a < g->state_arc_begin[u + 1]; ++a)
           if (seen[g->arc_class[a]] != s) { seen[g->arc_class[a]] = s; c += csize[g->arc_class[a]]; }   // (else shadowed by a chain state closer to s)
@@ -314,8 +318,10 @@ static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offs
   g->arc_class.resize(A); g->arc_dst.resize(A); g->arc_w.resize(A);
   g->state_fail.assign(N, 0); g->state_bw.assign(N, 0.0f); g->state_final.assign(N, 0.0f);
   g->state_depth.assign(depth.begin(), depth.begin() + N);
+  std::vector<uint64_t> has(N, 0);              // bit c mod 64: the state may have an arc of class c
   for (int32_t id = 1; id < N; ++id) {
     g->state_arc_begin[parent[id] + 1]++;
+    has[parent[id]] |= uint64_t(1) << (cls[id] & 63);
     g->arc_class[id - 1] = cls[id];
     g->arc_dst[id - 1] = id;
   }
@@ -323,8 +329,7 @@ static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offs
 
   std::vector<int32_t> root_arc(n_classes, -1);
   for (int32_t a = 0; a < g->state_arc_begin[1]; ++a) root_arc[g->arc_class[a]] = a;
-  auto find_arc = [&](int32_t u, int32_t c) -> int32_t {
-    if (u == 0) return root_arc[c];
+  auto find_arc = [&](int32_t u, int32_t c) -> int32_t {      // (not the root's)
     const int32_t* b = g->arc_class.data() + g->state_arc_begin[u];
     const int32_t* e = g->arc_class.data() + g->state_arc_begin[u + 1];
     if (e - b > 16) b = std::lower_bound(b, e, c);
@@ -333,16 +338,16 @@ static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offs
   };
 
   // ---- suffix links (ids ascend breadth-first, so the parent's link is ready) ---------------
+  // Most states on the way have no such arc, which their bits say without a look at the arcs, whose number no branch
+  // foresees (the same lists: 15.6 us and 8.3).
   for (int32_t id = 1; id < N; ++id) {
     int32_t f = 0;
     if (parent[id] != 0) {
-      int32_t q = g->state_fail[parent[id]];
-      for (;;) {
-        int32_t a = find_arc(q, cls[id]);
-        if (a >= 0) { f = g->arc_dst[a]; break; }
-        if (q == 0) break;
-        q = g->state_fail[q];
-      }
+      const int32_t c = cls[id];
+      int32_t q = g->state_fail[parent[id]], a = -1;
+      for (; q != 0; q = g->state_fail[q])
+        if ((has[q] >> (c & 63)) & 1u && (a = find_arc(q, c)) >= 0) break;
+      f = (q == 0 ? root_arc[c] : a) + 1;                     // (arc a enters state a + 1; none: the root)
     }
     g->state_fail[id] = f;
   }
@@ -363,7 +368,7 @@ static int compile_impl(const int32_t* phrase_tokens, const int64_t* phrase_offs
       g->arc_w[id - 1] = static_cast<float>(loan[id] - loan[parent[id]] + outp[id]);
     }
   }
-  finalize_graph(g, case_class, vocab, n_classes, lambda, true);
+  finalize_graph(g, case_class, vocab, n_classes, lambda, true, token_weights == nullptr);
   return TB_OK;
 }
 
@@ -580,7 +585,7 @@ int compile_variative_impl(const uint8_t* phrase_chars, const int64_t* phrase_of
     g->state_final[id] = static_cast<float>(-loan[id]);
     if (id) g->state_bw[id] = static_cast<float>(loan[fail[id]] - loan[id]);
   }
-  finalize_graph(g, cls.data(), vocab, n_classes, lambda, false);
+  finalize_graph(g, cls.data(), vocab, n_classes, lambda, false, false);
   return TB_OK;
 }
 
