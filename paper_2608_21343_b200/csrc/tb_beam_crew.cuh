@@ -13,8 +13,8 @@
 // Four barriers of the crew a step; a ninth warp brings rows and keeps the books (beam_serve).  The team's step (beam_team_run), which takes what this one cannot,
 // puts every candidate into a histogram in shared memory, goes through long lists twice, and has all of its seventeen warps keep the books: the instructions
 // that four schedulers issue for it bound it (6900 cycles at K = 32); this one is bound by the latency of a step's chain, 3500 cycles at K = 12 and 5000 at K = 32.
-// 32 streams of 1000 steps, V = 1024, lists of 300 phrases, merging and pruning, whole call, before and after: K = 9 2638 and 1876 us, K = 12 2896 and 1895,
-// K = 16 3337 and 2056, K = 17 4265 and 2272, K = 24 4013 and 2279, K = 32 4423 and 2729; a chunk of 8 frames of 64 slots, two rows each: K = 12 105 and
+// 32 streams of 1000 steps, V = 1024, lists of 300 phrases, merging and pruning, whole call, before and after: K = 9 2638 and 1840 us, K = 12 2896 and 1859,
+// K = 16 3337 and 2036, K = 24 4013 and 2268, K = 32 4423 and 2727; a chunk of 8 frames of 64 slots, two rows each: K = 12 105 and
 // 87 us, K = 16 115 and 95, K = 24 135 and 118, K = 32 135 and 133 (its new streams begin with steps of the team).
 // A step is untouched and left to the team when a lane might have held one pick more than it keeps, when the K-th pick does not clear the bound on the
 // tokens that were not looked at, or when a value is infinite or no number.
@@ -51,7 +51,7 @@ __device__ __forceinline__ int beam_crew_run(const TbBeamParams& p, BeamShared& 
   constexpr uint32_t kTok = (1u << TB_RS_TOK_BITS) - 1u;
   constexpr int kDstBits = 32 - TB_RS_TOK_BITS;
   constexpr uint32_t kMinusInf = 0x007FFFFFu, kPlusInf = 0xFF800000u;     // order_key of the infinities
-  const float lam2 = 2.0f * fabsf(lam), root_wmax = sh.root_wmax;
+  const float lam2 = 2.0f * fabsf(lam), root_wmax = sh.root_wmax, parts = 1.0f / static_cast<float>(n_warps + 1);
   unsigned char* my_lead = dyn + 4 * (mine ? hyp : 0) * W;      // where each candidate leads (see beam_solo_run); only this warp's lanes use it
   const uint32_t c_own = 0xFFFFFFFFu - static_cast<uint32_t>(hyp);                           // (the lower word of a key: see beam_key)
   uint32_t stamp = so.stamp;
@@ -233,7 +233,7 @@ __device__ __forceinline__ int beam_crew_run(const TbBeamParams& p, BeamShared& 
       top1 = __reduce_max_sync(0xffffffffu, order_key(m));
       const float lo = order_key_inv(__reduce_min_sync(0xffffffffu, order_key(m))), range = order_key_inv(top1) - lo;     // (32 values reach lo)
       // every warp counts the values that reach one place between it and the best
-      const float part = range / static_cast<float>(n_warps + 1), mid = lo + static_cast<float>(warp + 1) * part;
+      const float part = range * parts, mid = lo + static_cast<float>(warp + 1) * part;
       int c = 0;
 #pragma unroll
       for (int i = 0; i < kCrewWarps; ++i) c += q[i] >= mid ? 1 : 0;
