@@ -138,16 +138,15 @@ __device__ __forceinline__ int beam_crew_run(const TbBeamParams& p, BeamShared& 
       stamp = 1u << kDstBits;
     }
     // ---- the lane's best candidates (see beam_solo_run)
-    float v1 = -INFINITY, v2 = -INFINITY, v3 = -INFINITY, rest = -INFINITY, sum = 0.0f;     // (sum: no number if any value is none)
+    float v1 = -INFINITY, v2 = -INFINITY, v3 = -INFINITY, rest = -INFINITY;
     uint32_t c1 = 0u, c2 = 0u, c3 = 0u;
     auto keep = [&](float v, uint32_t c, bool g1, bool g2, bool g3) {
-      sum += v;
       if (kThree) {
-        rest = fmaxf(rest, fminf(v3, v));
+        rest = max_nan(rest, min_nan(v3, v));
         v3 = fmaxf(v3, fminf(v2, v));
         c3 = g2 ? c2 : g3 ? c : c3;
       } else {
-        rest = fmaxf(rest, fminf(v2, v));
+        rest = max_nan(rest, min_nan(v2, v));
       }
       v2 = fmaxf(v2, fminf(v1, v));
       v1 = fmaxf(v1, v);
@@ -212,7 +211,7 @@ __device__ __forceinline__ int beam_crew_run(const TbBeamParams& p, BeamShared& 
     cr.best[32 * warp + lane] = v1;
     {
       const uint32_t l = max(lv ? order_key(ub) : 0u, rest > -INFINITY ? order_key(rest) : 0u);
-      const uint32_t lim = __reduce_max_sync(0xffffffffu, sum != sum ? 0xFFFFFFFFu : l);
+      const uint32_t lim = __reduce_max_sync(0xffffffffu, rest != rest ? 0xFFFFFFFFu : l);
       if (lane == 0) cr.limit[sidx & 1][warp] = lim;
     }
     // (where the lane's candidates lead: tokens through the table, others stay)

@@ -13,8 +13,12 @@
 // whole call, before and after: K = 1 1864 and 872 us, K = 2 1911 and 881, K = 4 2029 and 978, K = 5 2088 and 1294, K = 8 2177 and 1278.  (Wider
 // beams would have two lanes a hypothesis, which a first step's picks do not fit.)
 // A step is untouched and left to the team when a lane might have held one pick more than it keeps, or when the K-th pick does not
-// clear the bound on the tokens that were not looked at (as in the team's step, with the first token behind those looked at).
+// clear the bound on the tokens that were not looked at (as in the team's step, with the first token behind those looked at), and when a value is no number.
 __device__ __forceinline__ void beam_group_barrier(int n_threads) { asm volatile("bar.sync 2, %0;" ::"r"(n_threads) : "memory"); }
+
+// The larger and the smaller of two values, no number if either is none.
+__device__ __forceinline__ float max_nan(float a, float b) { float r; asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
+__device__ __forceinline__ float min_nan(float a, float b) { float r; asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
 
 // The logit at 2 * token of a row in shared memory.
 template <typename LT> __device__ __forceinline__ float beam_smem_logit2(const unsigned char* row, uint32_t token2);
@@ -243,15 +247,15 @@ __device__ __forceinline__ int beam_solo_run(const TbBeamParams& p, BeamShared& 
     }
     // ---- the lane's best candidates: largest value, then lowest token.  A lane's listed tokens come in ascending order, so among
     // them, and for the blank, which comes last of all, a tie stays with what is there.
-    float v1 = -INFINITY, v2 = -INFINITY, v3 = -INFINITY, rest = -INFINITY;     // (rest: the best value that is not kept)
+    float v1 = -INFINITY, v2 = -INFINITY, v3 = -INFINITY, rest = -INFINITY;     // (rest: the best value that is not kept; no number if any value is none)
     uint32_t c1 = 0u, c2 = 0u, c3 = 0u;                        // the lower words of the keys
     auto keep = [&](float v, uint32_t c, bool g1, bool g2, bool g3) {           // (g: comes before the first, second, third)
       if (kThree) {
-        rest = fmaxf(rest, fminf(v3, v));
+        rest = max_nan(rest, min_nan(v3, v));
         v3 = fmaxf(v3, fminf(v2, v));
         c3 = g2 ? c2 : g3 ? c : c3;
       } else {
-        rest = fmaxf(rest, fminf(v2, v));
+        rest = max_nan(rest, min_nan(v2, v));
       }
       v2 = fmaxf(v2, fminf(v1, v));
       v1 = fmaxf(v1, v);
@@ -333,12 +337,12 @@ __device__ __forceinline__ int beam_solo_run(const TbBeamParams& p, BeamShared& 
     const uint32_t l2 = some ? ~pl : 0xFFFFFFFFu;
     const int tkey = static_cast<int>(l2 >> 5), parent = some ? static_cast<int>(l2 & 31u) : 0, from = some ? parent * L : lane;
     const bool emits = some && tkey < V;
-    const int32_t goes = static_cast<int32_t>(reinterpret_cast<const uint32_t*>(dyn)[parent * W + min(tkey, V)] & ((1u << kDstBits) - 1u)), stays = __shfl_sync(0xffffffffu, st, from);
+    const int32_t goes = static_cast<int32_t>(reinterpret_cast<const uint32_t*>(dyn)[min(parent, K - 1) * W + min(tkey, V)] & ((1u << kDstBits) - 1u)), stays = __shfl_sync(0xffffffffu, st, from);
     const bool plv = __shfl_sync(0xffffffffu, lv ? 1 : 0, from) != 0;
     const float c_k = order_key_inv(kth);
     const bool out = h1 == kMinusInf && rest >= c_k && rest > -INFINITY;   // (this lane's are used up, and it had one more)
-    // (infinite values: differences with them are no numbers)
-    if (__any_sync(0xffffffffu, out || (lv && !(c_k > ub)) || top1 >= kPlusInf)) break;
+    // (infinite values: differences with them are no numbers.  A value that is none leaves a kept value without its token.)
+    if (__any_sync(0xffffffffu, out || (lv && !(c_k > ub)) || top1 >= kPlusInf || rest != rest)) break;
     st = !some || !bound ? -1 : emits ? goes : stays;
     ask(st);
     if (mine && j == 0) so.pick[slot][hyp] = l2;
