@@ -1250,6 +1250,7 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
           beam_serve<LT, 8>(p, sh, so, dyn, tm, sidx, n_steps, at, fetched, step_base, hashA, hashB, lenA, lenB, par0, 64);
       } else {
         __shared__ BeamCrew cr;
+        static_assert(sizeof(BeamShared) + sizeof(BeamCrewAhead) + sizeof(BeamCrew) + 200 * 1024 <= 227 * 1024, "beside the launcher's 200 KB");
         const int n_warps = (p.K + 3) >> 2;
         if (warp < n_warps)
           d = beam_crew_run<LT>(p, sh, so, cr, dyn, sidx, n_steps, E, recs_cached, tm);
