@@ -10,7 +10,8 @@
 // Bound by the latency of a step's dependent instructions (one issued every four to five cycles): about 1500 cycles at K = 4 -- values of the plain
 // tokens 110, of up to two listed tokens a lane 120 and of longer lists 230 on average, what is kept of the plain ones and the blank 220, picks 245 (60 each),
 // where they lead 125, their records and lists 330 -- where the team's step took 3500.  32 streams of 1000 steps, V = 1024, lists of 300 phrases,
-// whole call, before and after: K = 1 1864 and 872 us, K = 2 1911 and 881, K = 4 2029 and 978, K = 5 2088 and 1294, K = 8 2177 and 1278.  (Wider
+// whole call, before and after: K = 1 1864 and 872 us, K = 2 1911 and 881, K = 4 2029 and 978, K = 5 2088 and 1294, K = 8 2177 and 1278 (with twelve tokens
+// of a reduced row; merging and pruning, with twelve and with eight: K = 5 1360 and 1307, K = 8 1335 and 1296).  (Wider
 // beams would have two lanes a hypothesis, which a first step's picks do not fit.)
 // A step is untouched and left to the team when a lane might have held one pick more than it keeps, or when the K-th pick does not
 // clear the bound on the tokens that were not looked at (as in the team's step, with the first token behind those looked at), and when a value is no number.
@@ -152,7 +153,7 @@ __device__ __forceinline__ void beam_serve(const TbBeamParams& p, BeamShared& sh
 template <typename LT, int KG>
 __device__ __forceinline__ int beam_solo_run(const TbBeamParams& p, BeamShared& sh, BeamSolo& so, unsigned char* dyn, int32_t sidx, const int32_t n_steps,
                                              const int32_t E, const bool recs_cached, const TeamSmem& tm) {
-  constexpr int L = 32 / KG, NP = KG <= 4 ? 1 : 3;              // lanes per hypothesis; tokens of the reduced row per lane
+  constexpr int L = 32 / KG, NP = kSoloPlain / L;              // lanes per hypothesis; tokens of the reduced row per lane
   constexpr int NE = 4;                                         // 16-byte pieces (two entries) of a list that a lane has at hand
   constexpr bool kThree = KG > 4;                               // a lane keeps three candidates (else two)
   const int lane = threadIdx.x & 31, b = blockIdx.x, K = p.K, V = p.V, W = V + 1;

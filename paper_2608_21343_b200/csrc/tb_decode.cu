@@ -661,7 +661,7 @@ constexpr int kTeamRows = 3;              // rows (and reduced rows) in shared m
 constexpr int kSoloBeam = 8;              // hypotheses at most
 constexpr int kSoloRows = 4;              // rows brought at a time (two such groups in shared memory)
 constexpr int kSoloVocab = 64;            // rows of fewer tokens are left to the team
-constexpr int kSoloPlain = 12;            // tokens of a reduced row that are looked at, at most
+constexpr int kSoloPlain = 8;             // tokens of a reduced row that are looked at (with twelve K = 5 1360 us a call, 1307 with eight, K = 8 1335 and 1296)
 // Wider ones by a crew of warps, four hypotheses each (tb_beam_crew.cuh); what that cannot take goes to the team as well.
 constexpr int kCrewBeam = 32, kCrewWarps = kCrewBeam / 4;
 constexpr int kCrewRows = 2;              // rows brought at a time (two such groups in shared memory)
@@ -1244,10 +1244,8 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
       if constexpr (WIDTH == 0) {
         if (warp == 0)
           d = p.K > 4 ? beam_solo_run<LT, 8>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm) : beam_solo_run<LT, 4>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm);
-        else if (warp == 1 && p.K > 4)
-          beam_serve<LT, kSoloPlain>(p, sh, so, dyn, tm, sidx, n_steps, at, fetched, step_base, hashA, hashB, lenA, lenB, par0, 64);
         else if (warp == 1)
-          beam_serve<LT, 8>(p, sh, so, dyn, tm, sidx, n_steps, at, fetched, step_base, hashA, hashB, lenA, lenB, par0, 64);
+          beam_serve<LT, kSoloPlain>(p, sh, so, dyn, tm, sidx, n_steps, at, fetched, step_base, hashA, hashB, lenA, lenB, par0, 64);
       } else {
         __shared__ BeamCrew cr;
         static_assert(sizeof(BeamShared) + sizeof(BeamCrewAhead) + sizeof(BeamCrew) + 200 * 1024 <= 227 * 1024, "beside the launcher's 200 KB");
