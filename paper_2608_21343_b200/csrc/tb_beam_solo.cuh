@@ -141,7 +141,8 @@ __device__ __forceinline__ void beam_serve(const TbBeamParams& p, BeamShared& sh
       const TbTopEnt* t = reinterpret_cast<const TbTopEnt*>(mem + tm.top + r * tm.top_stride);
       const uint32_t tc = t[q].tok_cls, cl = tc >> 16;
       so.plain[r][q] = make_uint4(__float_as_uint(t[q].x), bound ? __float_as_uint(rootcw[cl]) : 0u, tc & 0xFFFFu, bound ? static_cast<uint32_t>(rootdst[cl]) : 0u);
-      if (q == 0) { so.row[r].xb = t[M].x; so.row[r].y_next = t[P].y; }
+      // (no finite value left: nothing was left out.  The steps' bound is then below any finite pick, where -inf would make it no number)
+      if (q == 0) { so.row[r].xb = t[M].x; so.row[r].y_next = t[P].y == -INFINITY ? -FLT_MAX : t[P].y; }
     }
     beam_group_barrier(n_threads);                                       // group n is there, group n - 1 has been read
     buf ^= R;
