@@ -17,10 +17,6 @@
 // clear the bound on the tokens that were not looked at (as in the team's step, with the first token behind those looked at), and when a value is no number.
 __device__ __forceinline__ void beam_group_barrier(int n_threads) { asm volatile("bar.sync 2, %0;" ::"r"(n_threads) : "memory"); }
 
-// The larger and the smaller of two values, no number if either is none.
-__device__ __forceinline__ float max_nan(float a, float b) { float r; asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
-__device__ __forceinline__ float min_nan(float a, float b) { float r; asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
-
 // The logit at 2 * token of a row in shared memory.
 template <typename LT> __device__ __forceinline__ float beam_smem_logit2(const unsigned char* row, uint32_t token2);
 template <> __device__ __forceinline__ float beam_smem_logit2<uint16_t>(const unsigned char* row, uint32_t token2) {

@@ -9,7 +9,7 @@ namespace {
 // copies, the h-th beginning with token h, so that the boosts of a row's aligned 16-byte pieces are aligned as well); a row's
 // values then take one addition each.  The top_m + 1 best come without rounds of picking: a threshold that as many of the lanes' best values
 // (two per lane where one is too few) reach bounds the last of them from below; the row's tokens at or above that -- 1.3 times as many as are wanted, on average -- are collected and put in order by counting, for
-// each, those before it.  32 x 1000 rows of 1024 bf16, K = 4 (16 entries): 84 us token by token with a class and a root weight looked up for
+// each, those before it.  Values that are no numbers come first, as their keys do, wherever in the row they are.  32 x 1000 rows of 1024 bf16, K = 4 (16 entries): 84 us token by token with a class and a root weight looked up for
 // each, 53 so (10 by their bytes); 32 x 200 rows, K = 32 (44 entries): 26 us; 128 x 16 rows, K = 4: 11 to 21 us, 10 so.
 constexpr int kTopWarps = 8;
 constexpr int kTopGroup = 4;           // 16-byte pieces of a row a lane has at hand
@@ -101,12 +101,12 @@ __global__ void __launch_bounds__(kTopWarps * 32, 3) k_beam_topm(const LT* logit
         }
       }
     };
-    // the lane's best and second best value
+    // the lane's best and second best value (of those that are numbers)
     float m1 = -INFINITY, m2 = -INFINITY;
     auto best_of = [&]() {
       if (both) {
 #pragma unroll
-        for (int i = 0; i < G * EB; ++i) { m2 = fmaxf(m2, fminf(m1, y[i])); m1 = fmaxf(m1, y[i]); }
+        for (int i = 0; i < G * EB; ++i) { m2 = fmaxf(m2, min_nan(m1, y[i])); m1 = fmaxf(m1, y[i]); }
       } else {
 #pragma unroll
         for (int i = 0; i < G * EB; ++i) m1 = fmaxf(m1, y[i]);
@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kTopWarps * 32, 3) k_beam_topm(const LT* logit
     const float* boost0 = reinterpret_cast<const float*>(tab);
     float ys = -INFINITY;
     if (sok) ys = __fadd_rn(LogitLoad<LT>::at(rowi + sidx), boost0[sidx]);
-    m1 = ys;
+    m1 = fmaxf(m1, ys);
     int g_last = 0;
     values(0);
     best_of();
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(kTopWarps * 32, 3) k_beam_topm(const LT* logit
 #pragma unroll
         for (int u = 0; u < G; ++u)
 #pragma unroll
-          for (int e = 0; e < EB; ++e) hits |= y[u * EB + e] >= lim_v ? 1u << (u * EB + e) : 0u;
+          for (int e = 0; e < EB; ++e) hits |= !(y[u * EB + e] < lim_v) ? 1u << (u * EB + e) : 0u;     // (what is no number, too: its key decides)
 #pragma unroll 1
         while (__any_sync(0xffffffffu, hits != 0u) && n < kTopCap) {
           const int bit = max(__ffs(hits) - 1, 0), bi = g0 + 32 * (bit / EB) + lane, tok = hdi + bi * EB + bit % EB;

@@ -27,6 +27,10 @@ __device__ __forceinline__ float order_key_inv(uint32_t k) {
   return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xFFFFFFFFu));
 }
 
+// The larger and the smaller of two values, no number if either is none.
+__device__ __forceinline__ float max_nan(float a, float b) { float r; asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
+__device__ __forceinline__ float min_nan(float a, float b) { float r; asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
+
 // A bind that a launch carries out itself: the block brings the graph's image from page-locked host memory, read in place, into
 // the arena, U 16-byte loads a thread on their way across the bus at once.  (Both places are padded to the arena's granule.)
 template <int U>
