@@ -410,9 +410,8 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
     const uint32_t lo = 0xFFFFFFFFu - (static_cast<uint32_t>(tkey) * 32u + static_cast<uint32_t>(k));
     return (static_cast<unsigned long long>(order_key(v)) << 32) | lo;
   };
-  // this thread's two best candidates, when the sweep below has already looked at all of them
+  // this thread's two best candidates, collected by the sweep below
   unsigned long long m1 = 0ull, m2 = 0ull;
-  bool swept = false;
   auto offer = [&](unsigned long long kk) { if (kk > m1) { m2 = m1; m1 = kk; } else if (kk > m2) m2 = kk; };
   // all candidate values of the live hypotheses
   if (use_tv) {
@@ -488,9 +487,6 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
         }
       }
     }
-    // a frozen hypothesis is carried as one candidate (thread k offers it)
-    if (threadIdx.x < K && h_score[threadIdx.x] != -INFINITY && !h_live[threadIdx.x]) offer(make_key(h_score[threadIdx.x], V + 1, threadIdx.x));
-    swept = true;
     __syncthreads();
   } else {
     for (int k = 0; k < K; ++k) {
@@ -502,18 +498,21 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
       for (int v = threadIdx.x; v < W; v += kBeamThreads) {
         float x = LogitLoad<LT>::at(row + v);
         float val = (bound && v < V) ? __fadd_rn(x, __fmul_rn(g.lambda, bvec[__ldg(p.cls + v)])) : x;
-        cand[static_cast<size_t>(k) * W + v] = __fadd_rn(sc, val);
+        const float c = __fadd_rn(sc, val);
+        cand[static_cast<size_t>(k) * W + v] = c;
+        offer(make_key(c, v, k));
       }
       __syncthreads();
     }
   }
+  // a frozen hypothesis is carried as one candidate (thread k offers it)
+  if (threadIdx.x < K && h_score[threadIdx.x] != -INFINITY && !h_live[threadIdx.x]) offer(make_key(h_score[threadIdx.x], V + 1, threadIdx.x));
 
   // K rounds of selection.  A candidate's place in the order (value descending, token key ascending,
   // parent ascending) is one 64-bit key: the order-preserving image of the value above the inverted
-  // (token key, parent) pair; keys are distinct, 0 means "none".  Every thread keeps the best key among
-  // its own candidates that has not been picked yet; after a round only the owner of the pick rescans.
-  // best key below `limit` among this thread's candidates: tokens v = tid, tid + 256, ... of every live
-  // hypothesis, plus (thread k) the carried candidate of a frozen hypothesis k
+  // (token key, parent) pair; keys are distinct, 0 means "none".  Every thread keeps the two best keys among its own
+  // candidates -- tokens v = tid, tid + kBeamThreads, ... of every live hypothesis, plus (thread k) the carried candidate of a
+  // frozen hypothesis k -- that have not been picked yet.
   // the row of the next step is requested now: its trip from HBM overlaps the selection rounds
   xpre_valid = false;
   if (pref && next_row) {
@@ -524,34 +523,37 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
     }
     xpre_valid = true;
   }
-  unsigned long long spare = 0ull;                            // this thread's second best key below the limit of its last scan
-  bool have_spare = false;
-  auto scan_mine = [&](unsigned long long limit) -> unsigned long long {
-    unsigned long long m = 0ull, m2 = 0ull;
-    for (int k = 0; k < K; ++k) {
-      if (h_score[k] == -INFINITY) continue;
-      if (!h_live[k]) {
-        if (threadIdx.x == k) { const unsigned long long kk = make_key(h_score[k], V + 1, k); if (kk < limit) { if (kk > m) { m2 = m; m = kk; } else if (kk > m2) m2 = kk; } }
-        continue;
-      }
-      const float* ck = cand + static_cast<size_t>(k) * W;
-      for (int v = threadIdx.x; v < W; v += kBeamThreads) {
-        const unsigned long long kk = make_key(ck[v], v, k);
-        if (kk < limit) { if (kk > m) { m2 = m; m = kk; } else if (kk > m2) m2 = kk; }
+  unsigned long long mine = m1, spare = m2;
+  bool have_spare = true;
+  // The largest of the lanes' keys.
+  auto warp_best = [](unsigned long long k) -> unsigned long long {
+    const uint32_t hi = static_cast<uint32_t>(k >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+    const uint32_t ml = __reduce_max_sync(0xffffffffu, hi == mh ? static_cast<uint32_t>(k) : 0u);
+    return (static_cast<unsigned long long>(mh) << 32) | ml;
+  };
+  // When a thread's two are used up, its warp looks for the next two, a hypothesis a lane: all others wait for it.  (By the thread alone, hypothesis after
+  // hypothesis, this was most of a step: 8 streams of 120 steps, V = 1024, K = 4 932 us, K = 12 3100, K = 32
+  // 14 020; so 877, 2064 and 5010.)
+  static_assert(TB_MAX_BEAM <= 32, "a lane each");
+  auto look_again = [&](unsigned long long limit, int thread, unsigned long long& first, unsigned long long& second) {
+    unsigned long long m = 0ull, n = 0ull;
+    if (lane < K && h_score[lane] != -INFINITY) {
+      if (!h_live[lane]) {
+        if (thread == lane) { const unsigned long long kk = make_key(h_score[lane], V + 1, lane); m = kk < limit ? kk : 0ull; }
+      } else {
+        const float* ck = cand + static_cast<size_t>(lane) * W;
+        for (int v = thread; v < W; v += kBeamThreads) {
+          const unsigned long long kk = make_key(ck[v], v, lane);
+          if (kk < limit) { if (kk > m) { n = m; m = kk; } else if (kk > n) n = kk; }
+        }
       }
     }
-    spare = m2; have_spare = true;
-    return m;
+    first = warp_best(m);
+    second = warp_best(m == first ? n : m);
   };
-  unsigned long long mine = 0ull;
-  if (swept) { mine = m1; spare = m2; have_spare = true; }     // collected during the sweep
-  else mine = scan_mine(~0ull);
   for (int r = 0; r < K; ++r) {
-    // the warp's best key: the largest high word, then the largest low word among the lanes that have it
-    const uint32_t hi = static_cast<uint32_t>(mine >> 32), lo = static_cast<uint32_t>(mine);
-    const uint32_t mh = __reduce_max_sync(0xffffffffu, hi);
-    const uint32_t ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-    if (lane == 0) red64[r & 1][warp] = (static_cast<unsigned long long>(mh) << 32) | ml;
+    const unsigned long long wb = warp_best(mine);
+    if (lane == 0) red64[r & 1][warp] = wb;
     __syncthreads();                     // (one barrier per round: the next round writes the other copy)
     unsigned long long best = red64[r & 1][0];
 #pragma unroll
@@ -565,9 +567,16 @@ __device__ __forceinline__ void beam_step_body(const TbBeamParams& p, BeamShared
       }
       sel[r] = c;
     }
-    if (best != 0ull && mine == best) {                          // this thread owned the pick: its next best
-      if (have_spare) { mine = spare; have_spare = false; }
-      else mine = scan_mine(best);
+    const unsigned own = __ballot_sync(0xffffffffu, best != 0ull && mine == best);
+    if (own != 0u) {                                             // one of this warp's threads owned the pick: its next best
+      const int src = __ffs(own) - 1;
+      if (__shfl_sync(0xffffffffu, have_spare ? 1 : 0, src)) {
+        if (lane == src) { mine = spare; have_spare = false; }
+      } else {
+        unsigned long long m, n;
+        look_again(best, 32 * warp + src, m, n);
+        if (lane == src) { mine = m; spare = n; have_spare = true; }
+      }
     }
   }
   __syncthreads();
@@ -666,6 +675,7 @@ constexpr int kSoloPlain = 8;             // tokens of a reduced row that are lo
 constexpr int kCrewBeam = 32, kCrewWarps = kCrewBeam / 4;
 constexpr int kCrewRows = 2;              // rows brought at a time (two such groups in shared memory)
 constexpr int kCrewPlain = 16;            // tokens of a reduced row that are looked at
+constexpr int kWholeRows = 3;             // (in the place of a width class) neither: steps by the whole block only
 
 __host__ __device__ inline int team_warps(int K) { return K > 16 ? 16 : K < 4 ? 4 : K; }
 __device__ __forceinline__ unsigned long long beam_key(float v, int tkey, int k) {
@@ -1198,91 +1208,16 @@ __device__ __forceinline__ int beam_team_run(const TbBeamParams& p, BeamShared& 
   return sh.done;
 }
 
-#include "tb_beam_solo.cuh"
-using BeamCrewAhead = BeamAhead<kCrewRows, kCrewPlain, kCrewBeam>;
-#include "tb_beam_crew.cuh"
-
-// All steps of one stream of a multi-step launch: a warp or the team takes what it can, the block the rest.
-// WIDTH: 0 up to kSoloBeam hypotheses, 1 up to 16, 2 more.  (A kernel each: in one kernel the registers and the code of one weighed on the others --
-// 32 streams of 1000 steps, K = 32, 4384 us with the single warp's steps beside the team's, 3740 with the team's alone; K = 12 2633 and 2406.)
-template <typename LT, int WIDTH>
-__device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared& sh, unsigned char* dyn, const int32_t n_steps, const int32_t E,
-                                               const int64_t frame_stride, const int64_t row_stride, const int32_t rows_per_stream,
-                                               const int32_t step_base, unsigned long long* hashA, unsigned long long* hashB, int32_t* lenA,
-                                               int32_t* lenB, const int32_t par0) {
+// Steps sidx to end - 1 of a launch's n_steps by the whole block.
+template <typename LT>
+__device__ __forceinline__ void beam_block_steps(const TbBeamParams& p, BeamShared& sh, int32_t sidx, const int32_t end, const int32_t n_steps, const int32_t E,
+                                                 const int64_t frame_stride, const int64_t row_stride, const int32_t step_base, unsigned long long* hashA,
+                                                 unsigned long long* hashB, int32_t* lenA, int32_t* lenB, const int32_t par0) {
   LT xpre[kBeamPref] = {};
   bool xpre_valid = false;
-  const bool fast = beam_team_applies(p);
-  const TeamSmem tm = team_smem(p.rows_kept, p.V, sizeof(LT), p.top_m, p.rec_cache_bytes);
-  const bool odd0 = (par0 & 1) != 0;
-  const bool solo = fast && p.rows_kept > kTeamRows;            // steps by a warp or a crew (the launcher made room for their rows)
-  using Ahead = typename std::conditional<WIDTH == 0, BeamSolo, BeamCrewAhead>::type;
-  __shared__ Ahead so;
-  {                                           // the first rows are on their way while the tables are laid out
-    const int row = static_cast<int>(threadIdx.x >> 5) - (kBeamThreads / 32 - Ahead::kRows);     // (a row each by the block's last warps)
-    if (solo && row >= 0 && row < n_steps) BeamSoloRows<LT>(p, row, E, frame_stride, row_stride, rows_per_stream).fetch(p, team_base(p, dyn), tm, row);
-  }
-  const bool recs_cached = beam_begin(p, sh, dyn, odd0 ? hashB : hashA, odd0 ? lenB : lenA, fast, tm);
   const LT* stream_base = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(blockIdx.x) * p.stream_stride;
-  // what the warp's steps keep behind dyn begins empty, and again after a step by the block
-  auto clear = [&]() {
-    for (int i = threadIdx.x; i < p.K * (p.V + 1); i += kBeamThreads) reinterpret_cast<uint32_t*>(dyn)[i] = 0u;
-    if (threadIdx.x == 0) so.stamp = 0u;
-    __syncthreads();
-  };
-  bool clean = false, first = true;
-  int32_t skip = 0, backoff = 0;              // steps until the team tries again after a step it could not take
-  int32_t team_steps = 1;                     // steps the team takes when the warp could not
 #pragma unroll 1
-  for (int32_t sidx = 0; sidx < n_steps; ++sidx) {
-    if (solo && skip <= 0) {
-      if (!clean) { clear(); clean = true; }
-      const BeamSoloRows<LT> at(p, sidx, E, frame_stride, row_stride, rows_per_stream);
-      const bool fetched = sidx == 0 && first;
-      const int warp = threadIdx.x >> 5;
-      int d = 0;
-      if constexpr (WIDTH == 0) {
-        if (warp == 0)
-          d = p.K > 4 ? beam_solo_run<LT, 8>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm) : beam_solo_run<LT, 4>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm);
-        else if (warp == 1)
-          beam_serve<LT, kSoloPlain>(p, sh, so, dyn, tm, sidx, n_steps, at, fetched, step_base, hashA, hashB, lenA, lenB, par0, 64);
-      } else {
-        __shared__ BeamCrew cr;
-        static_assert(sizeof(BeamShared) + sizeof(BeamCrewAhead) + sizeof(BeamCrew) + 200 * 1024 <= 227 * 1024, "beside the launcher's 200 KB");
-        const int n_warps = (p.K + 3) >> 2;
-        if (warp < n_warps)
-          d = beam_crew_run<LT>(p, sh, so, cr, dyn, sidx, n_steps, E, recs_cached, tm);
-        else if (warp == n_warps)
-          beam_serve<LT, kCrewPlain>(p, sh, so, dyn, tm, sidx, n_steps, at, fetched, step_base, hashA, hashB, lenA, lenB, par0, 32 * n_warps + 32);
-      }
-      if (threadIdx.x == 0) sh.team_done = d;
-      __syncthreads();
-      d = sh.team_done;
-      first = false;
-      __syncthreads();                          // (read by everyone before a later run writes it again)
-      sidx += d;
-      if (sidx >= n_steps) break;
-      team_steps = d == 0 ? min(2 * team_steps, 32) : 1;
-    }
-    if (fast && skip-- <= 0) {
-      const int32_t stop = solo ? min(n_steps, sidx + team_steps) : n_steps;
-      if (threadIdx.x < 32 * (team_warps(p.K) + 1)) {
-        const int d = beam_team_run<LT, WIDTH == 2 ? 2 : 1>(p, sh, dyn, sidx, stop, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB, lenA,
-                                                            lenB, par0, recs_cached, tm);
-        if (threadIdx.x == 0) sh.team_done = d;
-      }
-      __syncthreads();
-      const int d = sh.team_done;
-      __syncthreads();                          // (read by everyone before a later run writes it again)
-      sidx += d;
-      if (sidx >= n_steps) break;
-      xpre_valid = false;
-      if (sidx >= stop) { --sidx; continue; }   // (the warp goes on)
-      backoff = d == 0 ? min(2 * backoff + 1, 32) : 0;
-      skip = backoff;
-      if (sidx >= n_steps) break;
-    }
-    clean = false;
+  for (; sidx < end; ++sidx) {
     const int32_t t = sidx / E, e = sidx - t * E;
     TbBeamParams q = p;
     q.logits = reinterpret_cast<const LT*>(p.logits) + static_cast<int64_t>(t) * frame_stride + static_cast<int64_t>(e) * row_stride;
@@ -1302,22 +1237,130 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
   }
 }
 
+// The same in a function of its own, for launches that seldom come to it: its registers do not weigh on the other steps', nor theirs on its.
+template <typename LT>
+__device__ __noinline__ void beam_block_steps_apart(const TbBeamParams& p, BeamShared& sh, const int32_t sidx, const int32_t end, const int32_t n_steps, const int32_t E,
+                                                    const int64_t frame_stride, const int64_t row_stride, const int32_t step_base, unsigned long long* hashA,
+                                                    unsigned long long* hashB, int32_t* lenA, int32_t* lenB, const int32_t par0) {
+  __builtin_assume(__isShared(&sh));
+  beam_block_steps<LT>(p, sh, sidx, end, n_steps, E, frame_stride, row_stride, step_base, hashA, hashB, lenA, lenB, par0);
+}
+
+// All steps of one stream of a launch without reduced rows, or without room for the team's (large vocabularies, odd strides).  A kernel of its own:
+// what the other steps keep in shared memory and in registers is not there.
+template <typename LT>
+__device__ __forceinline__ void beam_whole_steps(const TbBeamParams& p, BeamShared& sh, unsigned char* dyn, const int32_t n_steps, const int32_t E,
+                                                 const int64_t frame_stride, const int64_t row_stride, const int32_t step_base, unsigned long long* hashA,
+                                                 unsigned long long* hashB, int32_t* lenA, int32_t* lenB, const int32_t par0) {
+  const bool odd0 = (par0 & 1) != 0;
+  beam_begin(p, sh, dyn, odd0 ? hashB : hashA, odd0 ? lenB : lenA, false, TeamSmem());
+  beam_block_steps<LT>(p, sh, 0, n_steps, n_steps, E, frame_stride, row_stride, step_base, hashA, hashB, lenA, lenB, par0);
+}
+
+#include "tb_beam_solo.cuh"
+using BeamCrewAhead = BeamAhead<kCrewRows, kCrewPlain, kCrewBeam>;
+#include "tb_beam_crew.cuh"
+
+// All steps of one stream of a multi-step launch: a warp or the team takes what it can, the block the rest.
+// WIDTH: 0 up to kSoloBeam hypotheses, 1 up to 16, 2 more.  (A kernel each: in one kernel the registers and the code of one weighed on the others --
+// 32 streams of 1000 steps, K = 32, 4384 us with the single warp's steps beside the team's, 3740 with the team's alone; K = 12 2633 and 2406.)
+template <typename LT, int WIDTH>
+__device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared& sh, unsigned char* dyn, const int32_t n_steps, const int32_t E,
+                                               const int64_t frame_stride, const int64_t row_stride, const int32_t rows_per_stream,
+                                               const int32_t step_base, unsigned long long* hashA, unsigned long long* hashB, int32_t* lenA,
+                                               int32_t* lenB, const int32_t par0) {
+  const bool fast = beam_team_applies(p);
+  const TeamSmem tm = team_smem(p.rows_kept, p.V, sizeof(LT), p.top_m, p.rec_cache_bytes);
+  const bool odd0 = (par0 & 1) != 0;
+  const bool solo = fast && p.rows_kept > kTeamRows;            // steps by a warp or a crew (the launcher made room for their rows)
+  using Ahead = typename std::conditional<WIDTH == 0, BeamSolo, BeamCrewAhead>::type;
+  __shared__ Ahead so;
+  {                                           // the first rows are on their way while the tables are laid out
+    const int row = static_cast<int>(threadIdx.x >> 5) - (kBeamThreads / 32 - Ahead::kRows);     // (a row each by the block's last warps)
+    if (solo && row >= 0 && row < n_steps) BeamSoloRows<LT>(p, row, E, frame_stride, row_stride, rows_per_stream).fetch(p, team_base(p, dyn), tm, row);
+  }
+  const bool recs_cached = beam_begin(p, sh, dyn, odd0 ? hashB : hashA, odd0 ? lenB : lenA, fast, tm);
+  // what the warp's steps keep behind dyn begins empty, and again after a step by the block
+  auto clear = [&]() {
+    for (int i = threadIdx.x; i < p.K * (p.V + 1); i += kBeamThreads) reinterpret_cast<uint32_t*>(dyn)[i] = 0u;
+    if (threadIdx.x == 0) so.stamp = 0u;
+    __syncthreads();
+  };
+  bool clean = false;
+  int32_t backoff = 0;                        // steps the block takes beside one that the team could not take
+  int32_t team_steps = 1;                     // steps the team takes when the warp could not
+  int32_t sidx = 0;
+#pragma unroll 1
+  while (sidx < n_steps) {
+    if (solo && backoff == 0) {               // (after the block's steps the team tries first)
+      if (!clean) { clear(); clean = true; }
+      const BeamSoloRows<LT> at(p, sidx, E, frame_stride, row_stride, rows_per_stream);
+      const bool fetched = sidx == 0;
+      const int warp = threadIdx.x >> 5;
+      int d = 0;
+      if constexpr (WIDTH == 0) {
+        if (warp == 0)
+          d = p.K > 4 ? beam_solo_run<LT, 8>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm) : beam_solo_run<LT, 4>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm);
+        else if (warp == 1)
+          beam_serve<LT, kSoloPlain>(p, sh, so, dyn, tm, sidx, n_steps, at, fetched, step_base, hashA, hashB, lenA, lenB, par0, 64);
+      } else {
+        __shared__ BeamCrew cr;
+        static_assert(sizeof(BeamShared) + sizeof(BeamCrewAhead) + sizeof(BeamCrew) + 200 * 1024 <= 227 * 1024, "beside the launcher's 200 KB");
+        const int n_warps = (p.K + 3) >> 2;
+        if (warp < n_warps)
+          d = beam_crew_run<LT>(p, sh, so, cr, dyn, sidx, n_steps, E, recs_cached, tm);
+        else if (warp == n_warps)
+          beam_serve<LT, kCrewPlain>(p, sh, so, dyn, tm, sidx, n_steps, at, fetched, step_base, hashA, hashB, lenA, lenB, par0, 32 * n_warps + 32);
+      }
+      if (threadIdx.x == 0) sh.team_done = d;
+      __syncthreads();
+      d = sh.team_done;
+      __syncthreads();                          // (read by everyone before a later run writes it again)
+      sidx += d;
+      if (sidx >= n_steps) break;
+      team_steps = d == 0 ? min(2 * team_steps, 32) : 1;
+    }
+    if (fast) {
+      const int32_t stop = solo ? min(n_steps, sidx + team_steps) : n_steps;
+      if (threadIdx.x < 32 * (team_warps(p.K) + 1)) {
+        const int d = beam_team_run<LT, WIDTH == 2 ? 2 : 1>(p, sh, dyn, sidx, stop, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB, lenA,
+                                                            lenB, par0, recs_cached, tm);
+        if (threadIdx.x == 0) sh.team_done = d;
+      }
+      __syncthreads();
+      const int d = sh.team_done;
+      __syncthreads();                          // (read by everyone before a later run writes it again)
+      sidx += d;
+      if (sidx >= n_steps) break;
+      backoff = d == 0 ? min(2 * backoff + 1, 32) : 0;
+      if (sidx >= stop) continue;               // (the warp goes on)
+    }
+    clean = false;
+    const int32_t end = fast ? min(n_steps, sidx + backoff + 1) : n_steps;
+    beam_block_steps_apart<LT>(p, sh, sidx, end, n_steps, E, frame_stride, row_stride, step_base, hashA, hashB, lenA, lenB, par0);
+    sidx = end;
+  }
+}
+
 // T frames of E rows in one launch: the block loops over the expansions of its stream; every hypothesis of the
 // stream reads row (t, e).
 template <typename LT, int WIDTH>
-__global__ void __launch_bounds__(kBeamThreads) k_beam_frames(TbBeamParams p, int32_t T, int32_t E, int64_t frame_stride,
+__global__ void __launch_bounds__(kBeamThreads, 1) k_beam_frames(const __grid_constant__ TbBeamParams p, int32_t T, int32_t E, int64_t frame_stride,
                                                           int64_t row_stride) {
   __shared__ BeamShared sh;
   extern __shared__ __align__(16) unsigned char dyn_all[];
-  beam_all_steps<LT, WIDTH>(p, sh, dyn_all, T * E, E, frame_stride, row_stride, T * E, p.step, const_cast<unsigned long long*>(p.hash_in), p.hash_out,
-                     const_cast<int32_t*>(p.len_in), p.len_out, 0);
+  if constexpr (WIDTH == kWholeRows)
+    beam_whole_steps<LT>(p, sh, dyn_all, T * E, E, frame_stride, row_stride, p.step, const_cast<unsigned long long*>(p.hash_in), p.hash_out, const_cast<int32_t*>(p.len_in), p.len_out, 0);
+  else
+    beam_all_steps<LT, WIDTH>(p, sh, dyn_all, T * E, E, frame_stride, row_stride, T * E, p.step, const_cast<unsigned long long*>(p.hash_in), p.hash_out,
+                       const_cast<int32_t*>(p.len_in), p.len_out, 0);
 }
 
 // A chunk of streaming beam decoding: slot by slot, n_frames[slot] frames (at most T) of E rows; each slot has its own
 // position in its own tree ring and its own parity of the sequence-record halves, so that slots start, pause and end
 // independently of each other (Sec. 2.3: hypotheses kept across chunks; Sec. 2.2 para. 4: slots re-bound in between).
 template <typename LT, int WIDTH>
-__global__ void __launch_bounds__(kBeamThreads) k_beam_chunk(TbBeamParams p, int32_t T, int32_t E, int64_t frame_stride,
+__global__ void __launch_bounds__(kBeamThreads, 1) k_beam_chunk(const __grid_constant__ TbBeamParams p, int32_t T, int32_t E, int64_t frame_stride,
                                                          int64_t row_stride, const int32_t* n_frames, int32_t* slot_pos,
                                                          unsigned long long* hash, int32_t* len, size_t n_hyp) {
   // (chained, but its long steps are not shared with the next launch's blocks: 117 us a chunk of 128 slots with an early start
@@ -1328,8 +1371,12 @@ __global__ void __launch_bounds__(kBeamThreads) k_beam_chunk(TbBeamParams p, int
   const int b = blockIdx.x;
   const int32_t nf = n_frames ? max(0, min(T, n_frames[b])) : T;
   const int32_t pos0 = slot_pos[b];
-  if (nf > 0)
-    beam_all_steps<LT, WIDTH>(p, sh, dyn_all, nf * E, E, frame_stride, row_stride, T * E, pos0, hash, hash + n_hyp, len, len + n_hyp, pos0);
+  if (nf > 0) {
+    if constexpr (WIDTH == kWholeRows)
+      beam_whole_steps<LT>(p, sh, dyn_all, nf * E, E, frame_stride, row_stride, pos0, hash, hash + n_hyp, len, len + n_hyp, pos0);
+    else
+      beam_all_steps<LT, WIDTH>(p, sh, dyn_all, nf * E, E, frame_stride, row_stride, T * E, pos0, hash, hash + n_hyp, len, len + n_hyp, pos0);
+  }
   if (threadIdx.x == 0) slot_pos[b] = pos0 + nf * E;
 }
 
@@ -1505,9 +1552,11 @@ int tb_launch_beam_step(const TbBeamParams& p_in, cudaStream_t stream) {
   return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
 
-// Calls f with the width class of beam_all_steps as a compile-time constant.
+// Calls f with the width class of beam_all_steps, or kWholeRows, as a compile-time constant.
 template <typename F>
-static int beam_width_class(int K, F f) {
+static int beam_width_class(const TbBeamParams& p, F f) {
+  if (!p.tensor_lo) return f(std::integral_constant<int, kWholeRows>{});     // (see beam_team_setup)
+  const int K = p.K;
   if (K <= kSoloBeam) return f(std::integral_constant<int, 0>{});
   if (K <= 16) return f(std::integral_constant<int, 1>{});
   return f(std::integral_constant<int, 2>{});
@@ -1550,7 +1599,7 @@ int tb_launch_beam_frames(const TbBeamParams& p_in, int32_t T, int32_t E, int64_
     if (rc == TB_OK) fn<<<p.B, kBeamThreads, smem, stream>>>(p, T, E, frame_stride, row_stride);
     return rc;
   };
-  const int rc = beam_width_class(p.K, [&](auto w) {
+  const int rc = beam_width_class(p, [&](auto w) {
     return p.dtype == TB_BF16 ? launch(k_beam_frames<uint16_t, decltype(w)::value>) : launch(k_beam_frames<float, decltype(w)::value>);
   });
   if (rc != TB_OK) return rc;
@@ -1695,7 +1744,7 @@ int tb_launch_beam_chunk(const TbBeamParams& p_in, int32_t T, int32_t E, int64_t
     if (rc != TB_OK) return rc;
     return tb_launch_chained(fn, dim3(p.B), dim3(kBeamThreads), smem, stream, p, T, E, frame_stride, row_stride, n_frames, slot_pos, hash, len, n_hyp) == TB_OK ? TB_OK : TB_ERR_CUDA;
   };
-  const int rc = beam_width_class(p.K, [&](auto w) {
+  const int rc = beam_width_class(p, [&](auto w) {
     return p.dtype == TB_BF16 ? launch(k_beam_chunk<uint16_t, decltype(w)::value>) : launch(k_beam_chunk<float, decltype(w)::value>);
   });
   if (rc != TB_OK) return rc;
