@@ -371,6 +371,13 @@ int tb_batch_last_greedy_kernel(const tb_batch *b, int32_t *kernel, int32_t *blo
 int tb_batch_status(tb_batch *b, int32_t *device_status, void *stream);
 
 /*
+ * How many steps of this batch's tb_beam_frames and tb_beam_chunk calls so far, summed over the streams, were taken by a warp or a crew of
+ * warps / by a team of warps / by a whole block: out[3] (host), after synchronising `stream`.  All give identical results; a caller that depends on
+ * the speed of one can assert it here.
+ */
+int tb_batch_beam_steps(tb_batch *b, int64_t *out, void *stream);
+
+/*
  * Greedy RNNT decoding of B streams, slot i serving stream i, all on the device with no
  * host synchronisation per frame (Sec. 2.2 para. 3 for the boosted scores, Sec. 3.4 for greedy
  * label-looping decoding, Sec. 2.3 for GPU-resident execution).

@@ -74,6 +74,7 @@ _SIGS = {
     "tb_batch_bind_stream": (C.c_int, [_vp, _i32, _vp, _vp]),
     "tb_batch_bind_streams": (C.c_int, [_vp, _i32, _vp, _vp, _vp]),
     "tb_batch_status": (C.c_int, [_vp, C.POINTER(_i32), _vp]),
+    "tb_batch_beam_steps": (C.c_int, [_vp, C.POINTER(_i64), _vp]),
     "tb_batch_set_flags": (C.c_int, [_vp, C.c_uint32]),
     "tb_batch_set_greedy_plan": (C.c_int, [_vp, _i32, _i32, _i32]),
     "tb_batch_last_greedy_kernel": (C.c_int, [_vp, C.POINTER(_i32), C.POINTER(_i32), C.POINTER(_i32)]),
@@ -418,6 +419,13 @@ def tb_batch_bind_counts(batch: Batch) -> dict:
     pulled, copied = _i64(0), _i64(0)
     _check(_lib.tb_batch_bind_counts(batch.handle, C.byref(pulled), C.byref(copied)), "tb_batch_bind_counts")
     return dict(pulled=pulled.value, copied=copied.value)
+
+
+def tb_batch_beam_steps(batch: Batch, stream=None) -> dict:
+    """Steps of tb_beam_frames and tb_beam_chunk so far, over all streams: taken by a warp or a crew / by a team / by a whole block."""
+    n = (_i64 * 3)()
+    _check(_lib.tb_batch_beam_steps(batch.handle, n, _stream(stream)), "tb_batch_beam_steps")
+    return dict(warps=n[0], team=n[1], block=n[2])
 
 
 def tb_batch_status(batch: Batch, stream=None) -> int:

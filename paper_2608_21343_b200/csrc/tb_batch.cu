@@ -288,6 +288,7 @@ struct tb_batch {
   int32_t* d_class_tok = nullptr;             // [n_classes + 1] ranges, then [vocab] the tokens of every class, ascending
   uint32_t flags = 0;
   int32_t* d_status = nullptr;
+  unsigned long long* d_taken = nullptr;               // [3], behind the status word (TbBeamParams::taken)
   int2* d_tree = nullptr;
   unsigned long long* d_hyp_hash = nullptr;   // [2][n_slots * max_beam]: token-sequence hash of every beam hypothesis, ping-pong
   int32_t* d_hyp_len = nullptr;               // [2][n_slots * max_beam]: its length
@@ -405,7 +406,7 @@ extern "C" int tb_batch_create(int32_t vocab, const int32_t* case_class, int32_t
   size_t total = 0;
   auto room = [&](size_t bytes) { const size_t off = total; total += round_up(bytes, kArenaAlign); return off; };
   const size_t at_slots = room(sizeof(TbSlotRec) * n), at_hash = room(2 * n_hyp * sizeof(unsigned long long)), at_len = room(2 * n_hyp * sizeof(int32_t));
-  const size_t at_pos = room(sizeof(int32_t) * n), at_status = room(sizeof(int32_t)), zeros = total;
+  const size_t at_pos = room(sizeof(int32_t) * n), at_status = room(8 + 3 * sizeof(unsigned long long)), zeros = total;
   const size_t at_sstate = room(sizeof(TbSlotState) * n), at_cls = room(sizeof(int32_t) * vocab);
   const size_t at_class_tok = room(class_tok ? sizeof(int32_t) * (static_cast<size_t>(n_classes) + 1 + vocab) : 0), uploaded = total;
   const size_t at_tree = room(sizeof(int2) * static_cast<size_t>(max_tree_steps) * n_hyp), at_arena = room(b->arena_bytes);
@@ -429,6 +430,7 @@ extern "C" int tb_batch_create(int32_t vocab, const int32_t* case_class, int32_t
   b->d_slots = reinterpret_cast<TbSlotRec*>(m + at_slots); b->d_sstate = reinterpret_cast<TbSlotState*>(m + at_sstate);
   b->d_hyp_hash = reinterpret_cast<unsigned long long*>(m + at_hash); b->d_hyp_len = reinterpret_cast<int32_t*>(m + at_len);
   b->d_slot_pos = reinterpret_cast<int32_t*>(m + at_pos); b->d_status = reinterpret_cast<int32_t*>(m + at_status);
+  b->d_taken = reinterpret_cast<unsigned long long*>(m + at_status + 8);
   b->d_cls = reinterpret_cast<int32_t*>(m + at_cls);
   if (class_tok) b->d_class_tok = reinterpret_cast<int32_t*>(m + at_class_tok);
   if (max_tree_steps > 0) b->d_tree = reinterpret_cast<int2*>(m + at_tree);
@@ -988,6 +990,16 @@ extern "C" int tb_batch_status(tb_batch* b, int32_t* device_status, void* stream
   return st == 0 ? TB_OK : TB_ERR_DEVICE_STATUS;
 }
 
+extern "C" int tb_batch_beam_steps(tb_batch* b, int64_t* out, void* stream_) {
+  if (!b || !out) return TB_ERR_INVALID_ARG;
+  cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+  DeviceGuard guard(b->device);
+  if (!guard.ok) return TB_ERR_CUDA;
+  if (cudaMemcpyAsync(out, b->d_taken, 3 * sizeof *out, cudaMemcpyDeviceToHost, stream) == cudaSuccess && cudaStreamSynchronize(stream) == cudaSuccess) return TB_OK;
+  cudaGetLastError();
+  return TB_ERR_CUDA;
+}
+
 // Working memory of at least `want` bytes; never allocated while the caller's stream is being captured into a graph
 // (growing frees the old block first, which waits for earlier work: one decode per batch at a time).  A block that a captured
 // call has used is set aside instead of freed: each replay writes to it, whatever larger calls came in between.
@@ -1380,7 +1392,7 @@ extern "C" int tb_beam_frames(tb_batch* b, const void* logits, int dtype, int32_
   }
   p.new_frame = 1; p.step = b->tree_steps; p.stream_stride = stream_stride; p.hyp_stride = 0;
   p.scores = scores; p.states = states; p.live = live; p.out_parent = out_parent; p.out_token = out_token;
-  p.tree = b->d_tree; p.slots = b->d_slots; p.arena = b->arena; p.cls = b->d_cls; p.status = b->d_status;
+  p.tree = b->d_tree; p.slots = b->d_slots; p.arena = b->arena; p.cls = b->d_cls; p.status = b->d_status; p.taken = b->d_taken;
   DeviceGuard guard(b->device);
   if (!guard.ok) return TB_ERR_CUDA;
   beam_prepass(b, &p, T, E, frame_stride, row_stride, nullptr, static_cast<cudaStream_t>(stream_));
@@ -1449,7 +1461,7 @@ extern "C" int tb_beam_chunk(tb_batch* b, const void* logits, int dtype, int32_t
   // each slot's ring: the tree buffer holds max_tree_steps * n_slots * max_beam entries, i.e. per slot
   // max_tree_steps * max_beam / K steps of K entries (an entry index never leaves the slot's share)
   p.tree_cap = static_cast<int32_t>(static_cast<int64_t>(b->max_tree_steps) * b->max_beam / K);
-  p.slots = b->d_slots; p.arena = b->arena; p.cls = b->d_cls; p.status = b->d_status;
+  p.slots = b->d_slots; p.arena = b->arena; p.cls = b->d_cls; p.status = b->d_status; p.taken = b->d_taken;
   DeviceGuard guard(b->device);
   if (!guard.ok) return TB_ERR_CUDA;
   const size_t n_hyp = static_cast<size_t>(b->n_slots) * b->max_beam;

@@ -291,6 +291,7 @@ struct BeamShared {
   BeamKey sel[TB_MAX_BEAM];
   float root_wmax;                   // largest |root arc weight| of the stream's graph (filled with the root tables)
   int32_t team_done;                 // steps the team has just taken
+  int32_t taken[3];                  // steps of this launch so far, by kind (TbBeamParams::taken)
   // the team's steps (beam_team_run); two copies of what one step still reads while the next one writes
   float w_ub[2][TB_MAX_BEAM];                            // what the K-th pick has to clear on behalf of each hypothesis
   __align__(16) int32_t hist[2][kHistBins];              // candidates by value
@@ -781,7 +782,7 @@ __device__ inline bool beam_begin(const TbBeamParams& p, BeamShared& sh, unsigne
     sh.h_hash[tid] = p.fresh ? 0ull : hash_in[o];
     sh.h_len[tid] = p.fresh ? 0 : len_in[o];
   }
-  if (tid == 0) { sh.root_wmax = 0.0f; sh.no_rec = make_uint4(0u, 0u, 0u, 0u); }
+  if (tid == 0) { sh.root_wmax = 0.0f; sh.no_rec = make_uint4(0u, 0u, 0u, 0u); sh.taken[0] = sh.taken[1] = sh.taken[2] = 0; }
   if (use_tv) {
     const GraphPtrs g = graph_of(p.arena, rec);
     const int a0 = g.arc_begin[0], a1 = g.arc_begin[1];
@@ -1208,6 +1209,15 @@ __device__ __forceinline__ int beam_team_run(const TbBeamParams& p, BeamShared& 
   return sh.done;
 }
 
+// The steps of this launch go to the batch's counts (thread 0 has written them).
+__device__ __forceinline__ void beam_count(const TbBeamParams& p, const BeamShared& sh) {
+  if (threadIdx.x == 0 && p.taken) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      if (sh.taken[i] > 0) atomicAdd(p.taken + i, static_cast<unsigned long long>(sh.taken[i]));
+  }
+}
+
 // Steps sidx to end - 1 of a launch's n_steps by the whole block.
 template <typename LT>
 __device__ __forceinline__ void beam_block_steps(const TbBeamParams& p, BeamShared& sh, int32_t sidx, const int32_t end, const int32_t n_steps, const int32_t E,
@@ -1255,6 +1265,8 @@ __device__ __forceinline__ void beam_whole_steps(const TbBeamParams& p, BeamShar
   const bool odd0 = (par0 & 1) != 0;
   beam_begin(p, sh, dyn, odd0 ? hashB : hashA, odd0 ? lenB : lenA, false, TeamSmem());
   beam_block_steps<LT>(p, sh, 0, n_steps, n_steps, E, frame_stride, row_stride, step_base, hashA, hashB, lenA, lenB, par0);
+  if (threadIdx.x == 0) sh.taken[2] = n_steps;
+  beam_count(p, sh);
 }
 
 #include "tb_beam_solo.cuh"
@@ -1312,7 +1324,7 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
         else if (warp == n_warps)
           beam_serve<LT, kCrewPlain>(p, sh, so, dyn, tm, sidx, n_steps, at, fetched, step_base, hashA, hashB, lenA, lenB, par0, 32 * n_warps + 32);
       }
-      if (threadIdx.x == 0) sh.team_done = d;
+      if (threadIdx.x == 0) { sh.team_done = d; sh.taken[0] += d; }
       __syncthreads();
       d = sh.team_done;
       __syncthreads();                          // (read by everyone before a later run writes it again)
@@ -1325,7 +1337,7 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
       if (threadIdx.x < 32 * (team_warps(p.K) + 1)) {
         const int d = beam_team_run<LT, WIDTH == 2 ? 2 : 1>(p, sh, dyn, sidx, stop, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB, lenA,
                                                             lenB, par0, recs_cached, tm);
-        if (threadIdx.x == 0) sh.team_done = d;
+        if (threadIdx.x == 0) { sh.team_done = d; sh.taken[1] += d; }
       }
       __syncthreads();
       const int d = sh.team_done;
@@ -1338,8 +1350,10 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
     clean = false;
     const int32_t end = fast ? min(n_steps, sidx + backoff + 1) : n_steps;
     beam_block_steps_apart<LT>(p, sh, sidx, end, n_steps, E, frame_stride, row_stride, step_base, hashA, hashB, lenA, lenB, par0);
+    if (threadIdx.x == 0) sh.taken[2] += end - sidx;
     sidx = end;
   }
+  beam_count(p, sh);
 }
 
 // T frames of E rows in one launch: the block loops over the expansions of its stream; every hypothesis of the

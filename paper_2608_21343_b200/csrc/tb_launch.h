@@ -77,6 +77,7 @@ struct TbBeamParams {
   const unsigned char* tensor_lo; const unsigned char* tensor_hi;
   int32_t rows_kept;         // rows of a multi-step launch in shared memory (set by the launcher; see beam_team_setup)
   int32_t rec_cache_bytes;   // shared memory set aside for a copy of the stream's list records (narrow beams; 0: none)
+  unsigned long long* taken; // steps of multi-step launches so far: by a warp or a crew, by the team, by the whole block
 };
 
 // Binds that a streaming chunk launch carries out itself (tb_stream_chunk_binds): the block of slot[i] first copies
