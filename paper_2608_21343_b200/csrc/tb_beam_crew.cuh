@@ -2,8 +2,8 @@
 #ifndef TB_BEAM_CREW_CUH_
 #define TB_BEAM_CREW_CUH_
 
-// Eight lanes weigh a hypothesis' candidates as the single warp's steps do (tb_beam_solo.cuh) and keep their best three (with two the steps are shorter, but
-// the slowest of 32 streams leaves 30 of 1000 to the team, at 13 000 cycles each: K = 32 3325 us a call, 2729 with three).  What is left is to find the K
+// Eight lanes weigh a hypothesis' candidates as the single warp's steps do (tb_beam_solo.cuh) and keep their best three (with two the first look is shorter, but
+// settles 30 of 1000 steps less in the slowest of 32 streams).  What is left is to find the K
 // best of up to 3 * 256 candidates that eight warps hold in registers:
 //   A. every lane's best value goes to shared memory.  The least of 32 groups' best values is a lower bound on the K-th pick; every warp counts the values that
 //      reach one of as many places between it and the best, and the highest place that K reach is the bound (a search by all warps for themselves, each over
@@ -13,11 +13,11 @@
 // Four barriers of the crew a step; a ninth warp brings rows and keeps the books (beam_serve).  The team's step (beam_team_run), which takes what this one cannot,
 // puts every candidate into a histogram in shared memory, goes through long lists twice, and has all of its seventeen warps keep the books: the instructions
 // that four schedulers issue for it bound it (6900 cycles at K = 32); this one is bound by the latency of a step's chain, 3500 cycles at K = 12 and 5000 at K = 32.
-// 32 streams of 1000 steps, V = 1024, lists of 300 phrases, merging and pruning, whole call, before and after: K = 9 2638 and 1840 us, K = 12 2896 and 1859,
-// K = 16 3337 and 2036, K = 24 4013 and 2268, K = 32 4423 and 2727; a chunk of 8 frames of 64 slots, two rows each: K = 12 105 and
-// 87 us, K = 16 115 and 95, K = 24 135 and 118, K = 32 135 and 133 (its new streams begin with steps of the team).
-// A step is untouched and left to the team when a lane might have held one pick more than it keeps, when the K-th pick does not clear the bound on the
-// tokens that were not looked at, or when a value is infinite or no number.
+// 32 streams of 1000 steps, V = 1024, lists of 300 phrases of two to five tokens, merging and pruning, whole call, by the team and so: K = 9 2295 and 1544 us,
+// K = 12 2571 and 1539, K = 16 2943 and 1609, K = 24 3398 and 1837, K = 32 3541 and 1947; a chunk of 8 frames of 64 slots, one of them new, two rows
+// each: K = 12 62.9 and 42.4 us, K = 16 72.7 and 45.5, K = 24 77.1 and 49.4, K = 32 79.8 and 54.7.
+// Where a lane might have held one pick more than it keeps, or the K-th pick does not clear the bound on the tokens that were not looked at, the crew takes a second look
+// (beam_crew_look).  A step that this does not settle, or with a value that is infinite or no number in it, is untouched and left to the team.
 __device__ __forceinline__ void beam_crew_barrier(int n_threads) { asm volatile("bar.sync 1, %0;" ::"r"(n_threads) : "memory"); }
 
 struct BeamCrew {
@@ -26,15 +26,123 @@ struct BeamCrew {
   int32_t goes[kCrewBeam];                                     // and where they lead
   uint32_t limit[2][kCrewWarps];                                // order_key of what the K-th pick has to clear on behalf of the warp's hypotheses (0: nothing)
   int32_t reach[kCrewWarps];                                   // how many of the lanes' best values reach the warp's place
-  int32_t n_found;
+  uint32_t limit_more[kCrewWarps];                              // the same of a second look
+  int32_t n_found, n_more;
 };
+
+// The places of the n candidates in sh.sk, for those that have one: each is ranked by counting the keys above it, four lanes a candidate.
+__device__ __forceinline__ void beam_crew_rank(BeamShared& sh, BeamCrew& cr, const int n, const int K, const int n_warps) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (n > kSurvivors) return;
+#pragma unroll 1
+  for (int t0 = 8 * warp; t0 < n; t0 += 8 * n_warps) {
+    const int t = min(t0 + (lane >> 2), n - 1);
+    const unsigned long long key = sh.sk[t];
+    int c = 0;
+#pragma unroll 2
+    for (int i0 = 0; i0 < n; i0 += 16) {
+      const int i = i0 + 4 * (lane & 3);
+      const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(&sh.sk[i]), u = *reinterpret_cast<const ulonglong2*>(&sh.sk[i + 2]);
+      c += (i < n) & (o.x > key) ? 1 : 0;
+      c += (i + 1 < n) & (o.y > key) ? 1 : 0;
+      c += (i + 2 < n) & (u.x > key) ? 1 : 0;
+      c += (i + 3 < n) & (u.y > key) ? 1 : 0;
+    }
+    c += __shfl_xor_sync(0xffffffffu, c, 1);
+    c += __shfl_xor_sync(0xffffffffu, c, 2);
+    if (c < K && (lane & 3) == 0) { cr.place[c] = key; cr.goes[c] = sh.sd[t]; }      // (the last candidate may be ranked more than once: the same)
+  }
+}
+
+// A second look at a step that the first one could not settle, when a lane might have held one pick more than it keeps or the K-th pick (kth, its order_key, of those
+// that were looked at; K or more have it, or it is that of -inf) does not clear the bound: all candidates of every hypothesis that reach kth -- listed tokens,
+// blank, all tokens of the reduced row -- are noted and ranked, a warp a hypothesis.  The places are in cr.place then; returns how many candidates there
+// were, or -1 if the step is not settled (the K-th does not clear the bound on the tokens behind the reduced row, fewer than K finite ones, too many, a value that is no
+// number).
+// Steps of which one hypothesis has most of the picks need it: nearly all of a beam that is pruned to one at every frame, a new stream's first, one of a hundred
+// elsewhere.  They went to the team, whose run starts cold: 32 streams of 400 frames, one row each, peaked, pruned to within 1 of the best: K = 17 2170 us a call, K = 32
+// 2320 (1745 and 2050 by the team alone), so 1074 and 1490; a chunk of 4 frames of 128 slots, two rows each, K = 32: 58.6 and 39.8 us.
+// A function of its own: its registers do not weigh on the first look's.
+template <typename LT>
+__device__ __noinline__ int beam_crew_look(const TbBeamParams& p, BeamShared& sh, BeamCrew& cr, unsigned char* dyn, const unsigned char* row, const unsigned char* reduced,
+                                           const uint4* recs, const uint2* ent, const float psc, const int pst, const bool plv, const uint32_t kth, const uint32_t stamp, const float lam,
+                                           const float lam2, const int n_states) {
+  __builtin_assume(__isShared(&sh)); __builtin_assume(__isShared(&cr)); __builtin_assume(__isShared(dyn)); __builtin_assume(__isShared(row)); __builtin_assume(__isShared(reduced));
+  constexpr uint32_t kTok = (1u << TB_RS_TOK_BITS) - 1u, kMinusInf = 0x007FFFFFu;
+  constexpr int kDstBits = 32 - TB_RS_TOK_BITS;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, K = p.K, V = p.V, W = V + 1, M = p.top_m;
+  const int n_warps = (K + 3) >> 2, crew = 32 * n_warps;
+  const bool bound = n_states > 0;
+  const TbTopEnt* top = reinterpret_cast<const TbTopEnt*>(reduced);
+  const unsigned char* aux = dyn + ((static_cast<size_t>(K) * W * sizeof(float) + 15) & ~size_t(15)) + ((static_cast<size_t>(K) * ((W + 31) >> 5) * sizeof(uint32_t) + 15) & ~size_t(15));
+  const float* rootcw = reinterpret_cast<const float*>(aux);    // (see tokview_attach)
+  const int32_t* rootdst = reinterpret_cast<const int32_t*>(aux + 4 * static_cast<size_t>(p.C));
+  const float least = order_key_inv(kth), xb = top[M].x, y_next = top[M].y;
+  uint32_t limit = 0u;
+  bool none = false;                                           // a value that is no number
+#pragma unroll 1
+  for (int k = warp; k < K; k += n_warps) {
+    const float sc = __shfl_sync(0xffffffffu, psc, k);
+    const int st = __shfl_sync(0xffffffffu, pst, k);
+    const bool lv = __shfl_sync(0xffffffffu, plv ? 1 : 0, k) != 0;
+    if (sc == -INFINITY) continue;
+    const uint32_t c_own = 0xFFFFFFFFu - static_cast<uint32_t>(k);
+    const uint32_t* lead = reinterpret_cast<const uint32_t*>(dyn) + static_cast<size_t>(k) * W;
+    auto offer = [&](bool have, float v, uint32_t c, int32_t d) {
+      none |= have && v != v;
+      const bool yes = have && v >= least && v > -INFINITY;
+      const unsigned who = __ballot_sync(0xffffffffu, yes);
+      if (who == 0u) return;
+      int at = shared_fetch_add(&cr.n_more, __popc(who), lane == 0);
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(who & ((1u << lane) - 1u));
+      at = min(at, kSurvivors);
+      const unsigned long long key = (static_cast<unsigned long long>(order_key(v)) << 32) | c;
+      shared_put(&sh.sk[at], key, &sh.sd[at], d, yes);
+    };
+    offer(lane == 0, lv ? __fadd_rn(sc, xb) : sc, c_own - 32u * static_cast<uint32_t>(lv ? V : V + 1), st);
+    if (!lv) continue;
+    const uint4 r = recs[static_cast<unsigned>(st) < static_cast<unsigned>(n_states) ? st : 0];
+    const float D = __uint_as_float(r.z);
+#pragma unroll 1
+    for (int q0 = 0; q0 < M; q0 += 32) {
+      const int q = min(q0 + lane, M - 1);
+      const uint32_t tc = top[q].tok_cls, tok = tc & 0xFFFFu, cl = tc >> 16;
+      const float x = top[q].x, w = bound ? rootcw[cl] : 0.0f;
+      const bool have = q0 + lane < M && tok < static_cast<uint32_t>(V) && (lead[min(tok, static_cast<uint32_t>(V))] >> kDstBits) != (stamp >> kDstBits);
+      offer(have, __fadd_rn(sc, bound ? __fadd_rn(x, __fmul_rn(lam, __fadd_rn(D, w))) : x), c_own - 32u * tok, bound ? rootdst[cl] : 0);
+    }
+    const uint4* list = reinterpret_cast<const uint4*>(ent + r.x);
+    const int pieces = static_cast<int>(r.y) >> 1;
+#pragma unroll 1
+    for (int i0 = 0; i0 < pieces; i0 += 32) {
+      const bool have = i0 + lane < pieces;
+      uint4 e = make_uint4(2u * static_cast<uint32_t>(V), 0xFF800000u, 2u * static_cast<uint32_t>(V), 0xFF800000u);
+      if (have) e = list[i0 + lane];
+      const uint32_t t0 = e.x & kTok, t1 = e.z & kTok;
+      offer(have, __fadd_rn(sc, __fadd_rn(beam_smem_logit2<LT>(row, t0), __uint_as_float(e.y))), c_own - 16u * t0, static_cast<int32_t>(e.x >> TB_RS_TOK_BITS));
+      offer(have, __fadd_rn(sc, __fadd_rn(beam_smem_logit2<LT>(row, t1), __uint_as_float(e.w))), c_own - 16u * t1, static_cast<int32_t>(e.z >> TB_RS_TOK_BITS));
+    }
+    limit = max(limit, kMinusInf);                             // (places that no finite value is left for are the general step's)
+    if (y_next != -INFINITY) {
+      const float scale = fabsf(sc) + fabsf(y_next) + lam2 * (fabsf(D) + sh.root_wmax);
+      limit = max(limit, order_key((sc + y_next) + lam * D + scale * 3.814697265625e-6f + 1e-30f));     // (see beam_crew_run)
+    }
+  }
+  if (__any_sync(0xffffffffu, none)) limit = 0xFFFFFFFFu;
+  if (lane == 0) cr.limit_more[warp] = limit;
+  beam_crew_barrier(crew);
+  const int n = *const_cast<volatile int32_t*>(&cr.n_more);
+  beam_crew_rank(sh, cr, n, K, n_warps);
+  beam_crew_barrier(crew);
+  const uint32_t last = n >= K ? static_cast<uint32_t>(cr.place[K - 1] >> 32) : kMinusInf;
+  return n > kSurvivors || __any_sync(0xffffffffu, lane < n_warps && cr.limit_more[lane & (kCrewWarps - 1)] >= last) ? -1 : n;
+}
 
 // Takes the steps sidx, sidx + 1, ... like beam_team_run; returns how many.  Called by the first (K + 3) / 4 warps (the next one serves them).
 template <typename LT>
 __device__ __forceinline__ int beam_crew_run(const TbBeamParams& p, BeamShared& sh, BeamCrewAhead& so, BeamCrew& cr, unsigned char* dyn, int32_t sidx,
                                              const int32_t n_steps, const int32_t E, const bool recs_cached, const TeamSmem& tm) {
   constexpr int L = 8, NP = kCrewPlain / L;                     // lanes per hypothesis; tokens of the reduced row per lane
-  constexpr bool kThree = true;                                 // (a lane keeps three candidates, else two)
   constexpr int NE = 4;                                         // 16-byte pieces (two entries) of a list that a lane has at hand
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, b = blockIdx.x, K = p.K, V = p.V, W = V + 1;
   const int n_warps = (K + 3) >> 2, crew = 32 * n_warps;
@@ -119,7 +227,7 @@ __device__ __forceinline__ int beam_crew_run(const TbBeamParams& p, BeamShared& 
     lv = __shfl_sync(0xffffffffu, plv ? 1 : 0, hyp) != 0 && mine;
     if (!mine) sc = -INFINITY;
   };
-  if (warp == 0 && lane == 0) { *const_cast<volatile int32_t*>(&sh.cmd) = 0; cr.n_found = 0; }     // (seen by all after the first group barrier)
+  if (warp == 0 && lane == 0) { *const_cast<volatile int32_t*>(&sh.cmd) = 0; cr.n_found = cr.n_more = 0; }     // (seen by all after the first group barrier)
   __syncwarp();
   ask();
   enter(e_cur == 0, true);
@@ -129,25 +237,21 @@ __device__ __forceinline__ int beam_crew_run(const TbBeamParams& p, BeamShared& 
     if ((slot & (kCrewRows - 1)) == 0) { beam_group_barrier(crew + 32); ++n_bar; }
     const BeamCrewAhead::Row ro = so.row[slot];
     const unsigned char* row = dyn + ro.at;
-    stamp += 1u << kDstBits;
+    stamp += 2u << kDstBits;                                    // (the next number marks the plain tokens)
     if (stamp == 0u) {                                          // (the numbers begin again)
       __syncwarp();
 #pragma unroll 4
       for (int i = lane; i < min(4, K - 4 * warp) * W; i += 32) reinterpret_cast<uint32_t*>(dyn)[4 * warp * W + i] = 0u;
       __syncwarp();
-      stamp = 1u << kDstBits;
+      stamp = 2u << kDstBits;
     }
     // ---- the lane's best candidates (see beam_solo_run)
     float v1 = -INFINITY, v2 = -INFINITY, v3 = -INFINITY, rest = -INFINITY;
     uint32_t c1 = 0u, c2 = 0u, c3 = 0u;
     auto keep = [&](float v, uint32_t c, bool g1, bool g2, bool g3) {
-      if (kThree) {
-        rest = max_nan(rest, min_nan(v3, v));
-        v3 = fmaxf(v3, fminf(v2, v));
-        c3 = g2 ? c2 : g3 ? c : c3;
-      } else {
-        rest = max_nan(rest, min_nan(v2, v));
-      }
+      rest = max_nan(rest, min_nan(v3, v));
+      v3 = fmaxf(v3, fminf(v2, v));
+      c3 = g2 ? c2 : g3 ? c : c3;
       v2 = fmaxf(v2, fminf(v1, v));
       v1 = fmaxf(v1, v);
       c2 = g1 ? c1 : g2 ? c : c2;
@@ -198,10 +302,10 @@ __device__ __forceinline__ int beam_crew_run(const TbBeamParams& p, BeamShared& 
     for (int u = 0; u < NP; ++u) {
       uint32_t* at = reinterpret_cast<uint32_t*>(my_lead + 4 * min(ptk[u], static_cast<uint32_t>(V)));
       const bool ok = (ptk[u] < static_cast<uint32_t>(V)) & ((*at >> kDstBits) != (stamp >> kDstBits)) & lv;
-      *(ok ? at : reinterpret_cast<uint32_t*>(my_lead + 4 * V)) = stamp | pdst[u];           // (nobody reads the blank's)
+      *(ok ? at : reinterpret_cast<uint32_t*>(my_lead + 4 * V)) = (stamp + (1u << kDstBits)) | pdst[u];           // (nobody reads the blank's)
       const float v = ok ? pv[u] : -INFINITY;
       const uint32_t c = c_own - 32u * ptk[u];
-      keep(v, c, v > v1 || (v == v1 && c > c1), v > v2 || (v == v2 && c > c2), kThree && (v > v3 || (v == v3 && c > c3)));
+      keep(v, c, v > v1 || (v == v1 && c > c1), v > v2 || (v == v2 && c > c2), v > v3 || (v == v3 && c > c3));
     }
     {
       const float v = j == L - 1 ? (lv ? __fadd_rn(sc, ro.xb) : sc) : -INFINITY;              // the blank, or a frozen hypothesis carried
@@ -221,7 +325,7 @@ __device__ __forceinline__ int beam_crew_run(const TbBeamParams& p, BeamShared& 
       return tkey < static_cast<uint32_t>(V) ? to : st;
     };
     __syncwarp();
-    const int32_t d1 = leads(c1), d2 = leads(c2), d3 = kThree ? leads(c3) : 0;
+    const int32_t d1 = leads(c1), d2 = leads(c2), d3 = leads(c3);
     beam_crew_barrier(crew);
     float floor_v;
     uint32_t top1;
@@ -244,7 +348,7 @@ __device__ __forceinline__ int beam_crew_run(const TbBeamParams& p, BeamShared& 
     }
     // ---- B. the candidates that reach it
     const unsigned b1 = __ballot_sync(0xffffffffu, v1 >= floor_v && v1 > -INFINITY), b2 = __ballot_sync(0xffffffffu, v2 >= floor_v && v2 > -INFINITY),
-                   b3 = kThree ? __ballot_sync(0xffffffffu, v3 >= floor_v && v3 > -INFINITY) : 0u;
+                   b3 = __ballot_sync(0xffffffffu, v3 >= floor_v && v3 > -INFINITY);
     const int n1 = __popc(b1), n2 = __popc(b2), n_mine = n1 + n2 + __popc(b3);
     int at = shared_fetch_add(&cr.n_found, n_mine, lane == 0);
     at = __shfl_sync(0xffffffffu, at, 0);
@@ -256,42 +360,29 @@ __device__ __forceinline__ int beam_crew_run(const TbBeamParams& p, BeamShared& 
     };
     note(b1, at, v1, c1, d1);
     note(b2, at + n1, v2, c2, d2);
-    if (kThree) note(b3, at + n1 + n2, v3, c3, d3);
+    note(b3, at + n1 + n2, v3, c3, d3);
     beam_crew_barrier(crew);
     // ---- C. their ranks
-    const int n = *const_cast<volatile int32_t*>(&cr.n_found);
-    if (n <= kSurvivors) {
-#pragma unroll 1
-      for (int t0 = 8 * warp; t0 < n; t0 += 8 * n_warps) {
-        const int t = min(t0 + (lane >> 2), n - 1);
-        const unsigned long long key = sh.sk[t];
-        int c = 0;
-#pragma unroll 2
-        for (int i0 = 0; i0 < n; i0 += 16) {
-          const int i = i0 + 4 * (lane & 3);
-          const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(&sh.sk[i]), u = *reinterpret_cast<const ulonglong2*>(&sh.sk[i + 2]);
-          c += (i < n) & (o.x > key) ? 1 : 0;
-          c += (i + 1 < n) & (o.y > key) ? 1 : 0;
-          c += (i + 2 < n) & (u.x > key) ? 1 : 0;
-          c += (i + 3 < n) & (u.y > key) ? 1 : 0;
-        }
-        c += __shfl_xor_sync(0xffffffffu, c, 1);
-        c += __shfl_xor_sync(0xffffffffu, c, 2);
-        if (c < K && (lane & 3) == 0) { cr.place[c] = key; cr.goes[c] = sh.sd[t]; }      // (the last candidate may be ranked more than once: the same)
-      }
-    }
+    int n = *const_cast<volatile int32_t*>(&cr.n_found);
+    beam_crew_rank(sh, cr, n, K, n_warps);
     beam_crew_barrier(crew);
     // ---- the next step's hypotheses and their lists
+    unsigned long long key = lane < min(n, K) ? cr.place[lane] : 0ull;
+    // (infinite values: differences with them are no numbers; limit 0: nothing was left out)
+    const uint32_t kth = n >= K ? __shfl_sync(0xffffffffu, static_cast<uint32_t>(key >> 32), K - 1) : kMinusInf;
+    const uint32_t limit = __reduce_max_sync(0xffffffffu, lane < n_warps ? cr.limit[sidx & 1][lane & (kCrewWarps - 1)] : 0u);
+    if (n > kSurvivors || max(top1, limit) >= kPlusInf) break;
+    if (limit >= kth) {
+      n = beam_crew_look<LT>(p, sh, cr, dyn, row, mem + tm.top + slot * tm.top_stride, recs, ent, psc, pst, plv, kth, stamp, lam, lam2, bound ? n_states : 0);
+      if (n < 0) break;
+      key = lane < min(n, K) ? cr.place[lane] : 0ull;
+    }
     const bool some = lane < min(n, K);
-    const unsigned long long key = some ? cr.place[lane] : 0ull;
     const uint32_t l2 = some ? ~static_cast<uint32_t>(key) : 0xFFFFFFFFu;
     const int tkey = static_cast<int>(l2 >> 5), from = some ? static_cast<int>(l2 & 31u) : lane;
     const bool emits = some && tkey < V;
-    // (infinite values: differences with them are no numbers; limit 0: nothing was left out)
-    const uint32_t kth = n >= K ? __shfl_sync(0xffffffffu, static_cast<uint32_t>(key >> 32), K - 1) : kMinusInf;
-    if (__any_sync(0xffffffffu, (lane < n_warps && cr.limit[sidx & 1][lane & (kCrewWarps - 1)] >= kth) || n > kSurvivors || top1 >= kPlusInf)) break;
     if (warp == 0) {
-      if (lane == 0) cr.n_found = 0;
+      if (lane == 0) cr.n_found = cr.n_more = 0;
       if (lane < K) so.pick[slot][lane] = l2;
     }
     pst = some && bound ? cr.goes[lane] : -1;

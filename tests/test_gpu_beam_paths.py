@@ -53,3 +53,19 @@ def test_what_goes_by_the_block(tb, K):
     assert _steps(tb, x, "bf16", K, lists, flags=tb.TB_FLAG_BEAM_WHOLE_ROWS)["block"] == 1.0
     assert _steps(tb, x, "bf16", K, [_walked_list(1100, rng), _walked_list(1100, rng)])["block"] == 1.0
     assert _steps(tb, x, "bf16", K, [_walked_list(1100, rng), lists[0]])["block"] == pytest.approx(0.5, abs=0.05)
+
+
+@pytest.mark.parametrize("K", [9, 17, 24, 32])
+@pytest.mark.parametrize("prune", [0.0, 1.0])
+def test_frames_that_begin_with_one_hypothesis_go_by_a_crew(tb, K, prune):
+    rng = np.random.default_rng(K)
+    lists = [None] + _hub_lists(300, [9, 40], rng)
+    x = _logits(rng, 3, 100, 1, 300, lists[1:] + lists[1:2], False)
+    x[..., 300] += 5.0
+    assert _steps(tb, x, "bf16", K, lists, prune=prune)["warps"] > 0.95
+
+
+def test_new_streams_of_wide_beams_go_by_a_crew(tb):
+    rng = np.random.default_rng(3)
+    lists = [None] + _hub_lists(300, [9, 40], rng)
+    assert _steps(tb, _logits(rng, 3, 1, 2, 300, lists[1:] + lists[1:2], False), "bf16", 32, lists)["warps"] == 1.0

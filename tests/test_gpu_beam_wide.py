@@ -55,3 +55,30 @@ def test_more_steps_than_the_step_numbers_count(tb):
     w = W.get_workload(4, B=2, T=4200, V=70, S=1, K=9, dtype="f32")
     w.vocab.case_class[:] = np.arange(70)
     _check(tb, w, x, "f32", 9, lists, merge=True)
+
+
+@pytest.mark.parametrize("K", [9, 17, 25, 32])
+@pytest.mark.parametrize("V,dtype", [(64, "bf16"), (300, "f32"), (1100, "bf16")])
+@pytest.mark.parametrize("prune,coarse", [(0.0, False), (0.0, True), (0.5, False), (1.0, True)])
+def test_frames_of_few_hypotheses(tb, K, V, dtype, prune, coarse):
+    """One hypothesis, or a few, with most of a step's picks: lists around a warp's share of a second look (64 entries), rows of few finite tokens, and rows without."""
+    rng = np.random.default_rng([K, V, coarse])
+    sizes = [n for n in (1, 17, 62, 63, 66, 130, 260) if n < V - 1]
+    lists = _hub_lists(V, sizes, rng)
+    x = _logits(rng, len(sizes), 24, 1, V, lists, coarse)
+    x[:, 1::3, :, V] += 6.0
+    x[:, 4::5, :, :V][rng.random(x[:, 4::5, :, :V].shape) < 0.8] = -np.inf
+    w = W.get_workload(4, B=len(sizes), T=24, V=V, S=1, K=K, dtype=dtype)
+    w.vocab.case_class[:] = np.arange(V)
+    _check(tb, w, x, dtype, K, lists, merge=True, prune=prune)
+
+
+def test_more_equal_candidates_than_a_second_look_ranks(tb):
+    rng = np.random.default_rng(4)
+    lists = _hub_lists(1100, [500, 511, 640, 900], rng)
+    x = np.zeros((4, 12, 1, 1101), np.float32)
+    for b, p in enumerate(lists):
+        x[b, ::2, 0, p[0][0]] = 9.0                           # the hub, and then every listed token alike
+    w = W.get_workload(4, B=4, T=12, V=1100, S=1, K=32, dtype="f32")
+    w.vocab.case_class[:] = np.arange(1100)
+    _check(tb, w, x, "f32", 32, lists, merge=True, prune=0.0)
