@@ -670,12 +670,12 @@ constexpr int kTeamRows = 3;              // rows (and reduced rows) in shared m
 // Narrow beams take their steps with one warp (tb_beam_solo.cuh); what that cannot take goes to the team.
 constexpr int kSoloBeam = 8;              // hypotheses at most
 constexpr int kSoloRows = 4;              // rows brought at a time (two such groups in shared memory)
-constexpr int kSoloVocab = 64;            // rows of fewer tokens are left to the team
 constexpr int kSoloPlain = 8;             // tokens of a reduced row that are looked at (with twelve K = 5 1360 us a call, 1307 with eight, K = 8 1335 and 1296)
 // Wider ones by a crew of warps, four hypotheses each (tb_beam_crew.cuh); what that cannot take goes to the team as well.
 constexpr int kCrewBeam = 32, kCrewWarps = kCrewBeam / 4;
 constexpr int kCrewRows = 2;              // rows brought at a time (two such groups in shared memory)
 constexpr int kCrewPlain = 16;            // tokens of a reduced row that are looked at
+constexpr int kCrewVocab = 16;            // rows of fewer tokens are left to the team (see beam_team_setup)
 constexpr int kWholeRows = 3;             // (in the place of a width class) neither: steps by the whole block only
 
 __host__ __device__ inline int team_warps(int K) { return K > 16 ? 16 : K < 4 ? 4 : K; }
@@ -1585,7 +1585,9 @@ static void beam_team_setup(TbBeamParams* p, int32_t T, int32_t E, int64_t frame
   const int elem = p->dtype == TB_BF16 ? 2 : 4;
   p->rows_kept = p->K <= kSoloBeam ? 2 * kSoloRows : 2 * kCrewRows;
   size_t more = team_smem(p->rows_kept, p->V, elem, p->top_m, 0).total;
-  if (p->V < kSoloVocab || *smem + more > kMost) {
+  // (Steps of nearly as many places as there are tokens and hypotheses to fill them need a second look each: 32 streams of 200 steps, V = 8: K = 9 427 us by the
+  // team, 440 by a crew, K = 24 648 and 632, K = 32 607 and 723; V = 17: 425 and 355, 649 and 458, 606 and 468.  A single warp: V = 8, K = 8 399 and 207.)
+  if ((p->K > kSoloBeam && p->V < kCrewVocab) || *smem + more > kMost) {
     p->rows_kept = kTeamRows;
     more = team_smem(kTeamRows, p->V, elem, p->top_m, 0).total;
   }
