@@ -250,7 +250,7 @@ int tb_launch_beam_topm(const void* logits, int dtype, int32_t B, int32_t T, int
   const size_t smem = 4 * boost_copy_bytes(V) + kTopWarps * kTopCap * sizeof(uint64_t) + static_cast<size_t>(C) * 4;
   // rows per warp: enough blocks for every SM's three places twice over, before a block's table serves more rows
   const int64_t rows = static_cast<int64_t>(T) * E, all = rows * B;
-  int64_t per = all / (static_cast<int64_t>(n_sm) * 6 * kTopWarps);
+  int64_t per = all / (static_cast<int64_t>(n_sm > 0 ? n_sm : 1) * 6 * kTopWarps);     // (0: the device did not tell)
   per = per < 1 ? 1 : per > 16 ? 16 : per;
   const int blocks = static_cast<int>((rows + per * kTopWarps - 1) / (per * kTopWarps));
   auto launch = [&](auto* fn, auto* x) -> int {
