@@ -12,10 +12,10 @@
 //   C. each is ranked by counting the keys above it, four lanes a candidate, and goes to its place.
 // Four barriers of the crew a step; a ninth warp brings rows and keeps the books (beam_serve).  The team's step (beam_team_run), which takes what this one cannot,
 // puts every candidate into a histogram in shared memory, goes through long lists twice, and has all of its seventeen warps keep the books: the instructions
-// that four schedulers issue for it bound it (6900 cycles at K = 32); this one is bound by the latency of a step's chain, 3500 cycles at K = 12 and 5000 at K = 32.
-// 32 streams of 1000 steps, V = 1024, lists of 300 phrases of two to five tokens, merging and pruning, whole call, by the team and so: K = 9 2295 and 1544 us,
-// K = 12 2571 and 1539, K = 16 2943 and 1609, K = 24 3398 and 1837, K = 32 3541 and 1947; a chunk of 8 frames of 64 slots, one of them new, two rows
-// each: K = 12 62.9 and 42.4 us, K = 16 72.7 and 45.5, K = 24 77.1 and 49.4, K = 32 79.8 and 54.7.
+// that four schedulers issue for it bound it (6900 cycles at K = 32); this one is bound by the latency of a step's chain, 3400 cycles at K = 12 and 4600 at K = 32.
+// 32 streams of 1000 steps, V = 1024, lists of 300 phrases, merging and pruning, whole call with transcripts, by the team and so: K = 9 2617 and 1801 us,
+// K = 12 2922 and 1817, K = 16 3360 and 1948, K = 24 4042 and 2163, K = 32 4442 and 2447; a chunk of 8 frames of 64 slots, two rows each, one of them
+// new and one ending, with all its calls: K = 12 115 and 92 us, K = 16 126 and 97, K = 24 151 and 117, K = 32 154 and 125.
 // Where a lane might have held one pick more than it keeps, or the K-th pick does not clear the bound on the tokens that were not looked at, the crew takes a second look
 // (beam_crew_look).  A step that this does not settle, or with a value that is infinite or no number in it, is untouched and left to the team.
 __device__ __forceinline__ void beam_crew_barrier(int n_threads) { asm volatile("bar.sync 1, %0;" ::"r"(n_threads) : "memory"); }

@@ -3,18 +3,19 @@
 #define TB_BEAM_SOLO_CUH_
 
 // The candidates of a team's step -- listed tokens, blank, the first tokens of the reduced row -- of a beam of up to KG hypotheses fit
-// one warp: 32 / KG lanes per hypothesis.  A lane keeps its two or three best candidates as 64-bit keys (the order of the general step), the
-// picks are the largest of the lanes' best, one after the other by two warp reductions each, and the next step starts from
+// one warp: 32 / KG lanes per hypothesis.  A lane keeps the values of its two or three best candidates and the lower words of their keys (the order of the
+// general step), the picks are the largest of the lanes' best, one after the other by two warp reductions each, and the next step starts from
 // registers: no barriers, no shared counters, no candidates written out and read back.  A second warp brings rows and
 // reduced rows into shared memory and keeps the books, kSoloRows steps at a time, one barrier of two warps for as many steps.
-// Bound by the latency of a step's dependent instructions (one issued every four to five cycles): about 1500 cycles at K = 4 -- values of the plain
-// tokens 110, of up to two listed tokens a lane 120 and of longer lists 230 on average, what is kept of the plain ones and the blank 220, picks 245 (60 each),
-// where they lead 125, their records and lists 330 -- where the team's step took 3500.  32 streams of 1000 steps, V = 1024, lists of 300 phrases,
-// whole call, before and after: K = 1 1864 and 872 us, K = 2 1911 and 881, K = 4 2029 and 978, K = 5 2088 and 1294, K = 8 2177 and 1278 (with twelve tokens
-// of a reduced row; merging and pruning, with twelve and with eight: K = 5 1360 and 1307, K = 8 1335 and 1296).  (Wider
+// Bound by the latency of a step's dependent instructions (one issued every four to five cycles): about 1650 cycles at K = 4 by a call's time; when counted, of 1500 of
+// an average step the values of the plain tokens took 110, of up to two listed tokens a lane 120 and of longer lists 230 on average, what is kept of the plain
+// ones and the blank 220, picks 245 (60 each), where they lead 125, their records and lists 330.  The team's step took 3500.  32 streams of 1000 steps,
+// V = 1024, lists of 300 phrases, whole call with transcripts, by the team and so: K = 1 1869 and 792 us, K = 2 1901 and 791, K = 4 1950 and 894, K = 5 2083
+// and 1193, K = 8 2191 and 1253; merging and pruning K = 4 2091 and 923, K = 5 2241 and 1295, K = 8 2388 and 1345.  (Wider
 // beams would have two lanes a hypothesis, which a first step's picks do not fit.)
-// A step is untouched and left to the team when a lane might have held one pick more than it keeps, or when the K-th pick does not
-// clear the bound on the tokens that were not looked at (as in the team's step, with the first token behind those looked at), and when a value is no number.
+// A step is untouched and left to the team when a lane might have held one pick more than it keeps, when the K-th pick does not
+// clear the bound on the tokens that were not looked at (as in the team's step, with the first token behind those looked at), and when a value that it weighs is
+// no number (a row's tokens with such values are the first of its reduced form, so that one of them is weighed).
 __device__ __forceinline__ void beam_group_barrier(int n_threads) { asm volatile("bar.sync 2, %0;" ::"r"(n_threads) : "memory"); }
 
 // The logit at 2 * token of a row in shared memory.

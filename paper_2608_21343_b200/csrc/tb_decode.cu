@@ -670,7 +670,7 @@ constexpr int kTeamRows = 3;              // rows (and reduced rows) in shared m
 // Narrow beams take their steps with one warp (tb_beam_solo.cuh); what that cannot take goes to the team.
 constexpr int kSoloBeam = 8;              // hypotheses at most
 constexpr int kSoloRows = 4;              // rows brought at a time (two such groups in shared memory)
-constexpr int kSoloPlain = 8;             // tokens of a reduced row that are looked at (with twelve K = 5 1360 us a call, 1307 with eight, K = 8 1335 and 1296)
+constexpr int kSoloPlain = 8;             // tokens of a reduced row that are looked at (merging and pruning, with twelve K = 5 1360 us a call, 1307 with eight, K = 8 1335 and 1296)
 // Wider ones by a crew of warps, four hypotheses each (tb_beam_crew.cuh); what that cannot take goes to the team as well.
 constexpr int kCrewBeam = 32, kCrewWarps = kCrewBeam / 4;
 constexpr int kCrewRows = 2;              // rows brought at a time (two such groups in shared memory)
@@ -1515,7 +1515,7 @@ __global__ void k_publish_slot(TbSlotRec* slots, TbSlotState* sstate, int32_t sl
 
 template <typename F>
 int set_smem(F* fn, size_t bytes) {
-  // (the default limit of 48 KB counts the kernel's static shared memory too -- up to 24 KB here -- so the opt-in
+  // (the default limit of 48 KB counts the kernel's static shared memory too -- up to 28 KB here -- so the opt-in
   //  starts well below it)
   if (bytes > 16 * 1024) {
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes)) != cudaSuccess) {
