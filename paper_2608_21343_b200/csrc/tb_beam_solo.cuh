@@ -10,8 +10,8 @@
 // Bound by the latency of a step's dependent instructions (one issued every four to five cycles): about 1650 cycles at K = 4 by a call's time; when counted, of 1500 of
 // an average step the values of the plain tokens took 110, of up to two listed tokens a lane 120 and of longer lists 230 on average, what is kept of the plain
 // ones and the blank 220, picks 245 (60 each), where they lead 125, their records and lists 330.  The team's step took 3500.  32 streams of 1000 steps,
-// V = 1024, lists of 300 phrases, whole call with transcripts, by the team and so: K = 1 1869 and 792 us, K = 2 1901 and 791, K = 4 1950 and 894, K = 5 2083
-// and 1193, K = 8 2191 and 1253; merging and pruning K = 4 2091 and 923, K = 5 2241 and 1295, K = 8 2388 and 1345.  (Wider
+// V = 1024, lists of 300 phrases, whole call with transcripts, by the team and so: K = 1 1869 and 802 us, K = 2 1901 and 809, K = 4 1950 and 881, K = 5 2083
+// and 1172, K = 8 2191 and 1243; merging and pruning K = 4 2091 and 912, K = 5 2241 and 1273, K = 8 2388 and 1330.  (Wider
 // beams would have two lanes a hypothesis, which a first step's picks do not fit.)
 // A step is untouched and left to the team when a lane might have held one pick more than it keeps, when the K-th pick does not
 // clear the bound on the tokens that were not looked at (as in the team's step, with the first token behind those looked at), and when a value that it weighs is

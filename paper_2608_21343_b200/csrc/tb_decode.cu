@@ -676,7 +676,7 @@ constexpr int kCrewBeam = 32, kCrewWarps = kCrewBeam / 4;
 constexpr int kCrewRows = 2;              // rows brought at a time (two such groups in shared memory)
 constexpr int kCrewPlain = 16;            // tokens of a reduced row that are looked at
 constexpr int kCrewVocab = 16;            // rows of fewer tokens are left to the team (see beam_team_setup)
-constexpr int kWholeRows = 3;             // (in the place of a width class) neither: steps by the whole block only
+constexpr int kWholeRows = 4;             // (in the place of a width class) neither: steps by the whole block only
 
 __host__ __device__ inline int team_warps(int K) { return K > 16 ? 16 : K < 4 ? 4 : K; }
 __device__ __forceinline__ unsigned long long beam_key(float v, int tkey, int k) {
@@ -1247,7 +1247,7 @@ __device__ __forceinline__ void beam_block_steps(const TbBeamParams& p, BeamShar
   }
 }
 
-// The same in a function of its own, for launches that seldom come to it: its registers do not weigh on the other steps', nor theirs on its.
+// The same in a function of its own: its registers do not weigh on the other steps', nor theirs on its (see beam_all_steps).
 template <typename LT>
 __device__ __noinline__ void beam_block_steps_apart(const TbBeamParams& p, BeamShared& sh, const int32_t sidx, const int32_t end, const int32_t n_steps, const int32_t E,
                                                     const int64_t frame_stride, const int64_t row_stride, const int32_t step_base, unsigned long long* hashA,
@@ -1274,8 +1274,10 @@ using BeamCrewAhead = BeamAhead<kCrewRows, kCrewPlain, kCrewBeam>;
 #include "tb_beam_crew.cuh"
 
 // All steps of one stream of a multi-step launch: a warp or the team takes what it can, the block the rest.
-// WIDTH: 0 up to kSoloBeam hypotheses, 1 up to 16, 2 more.  (A kernel each: in one kernel the registers and the code of one weighed on the others --
+// WIDTH: 0 up to kSoloBeam / 2 hypotheses, 1 up to kSoloBeam, 2 up to 16, 3 more.  (A kernel each: in one kernel the registers and the code of one weighed on the others --
 // 32 streams of 1000 steps, K = 32, 4384 us with the single warp's steps beside the team's, 3740 with the team's alone; K = 12 2633 and 2406.)
+// The block's steps are a function apart but for WIDTH 1, whose own leave the compiler with no spilled registers: K = 5 1185 us apart and 1172 in place, K = 8 1256
+// and 1243; K = 4 875 apart and 982 in place.
 template <typename LT, int WIDTH>
 __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared& sh, unsigned char* dyn, const int32_t n_steps, const int32_t E,
                                                const int64_t frame_stride, const int64_t row_stride, const int32_t rows_per_stream,
@@ -1285,7 +1287,7 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
   const TeamSmem tm = team_smem(p.rows_kept, p.V, sizeof(LT), p.top_m, p.rec_cache_bytes);
   const bool odd0 = (par0 & 1) != 0;
   const bool solo = fast && p.rows_kept > kTeamRows;            // steps by a warp or a crew (the launcher made room for their rows)
-  using Ahead = typename std::conditional<WIDTH == 0, BeamSolo, BeamCrewAhead>::type;
+  using Ahead = typename std::conditional<WIDTH <= 1, BeamSolo, BeamCrewAhead>::type;
   __shared__ Ahead so;
   {                                           // the first rows are on their way while the tables are laid out
     const int row = static_cast<int>(threadIdx.x >> 5) - (kBeamThreads / 32 - Ahead::kRows);     // (a row each by the block's last warps)
@@ -1310,9 +1312,9 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
       const bool fetched = sidx == 0;
       const int warp = threadIdx.x >> 5;
       int d = 0;
-      if constexpr (WIDTH == 0) {
+      if constexpr (WIDTH <= 1) {
         if (warp == 0)
-          d = p.K > 4 ? beam_solo_run<LT, 8>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm) : beam_solo_run<LT, 4>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm);
+          d = beam_solo_run<LT, WIDTH == 0 ? 4 : 8>(p, sh, so, dyn, sidx, n_steps, E, recs_cached, tm);
         else if (warp == 1)
           beam_serve<LT, kSoloPlain>(p, sh, so, dyn, tm, sidx, n_steps, at, fetched, step_base, hashA, hashB, lenA, lenB, par0, 64);
       } else {
@@ -1335,7 +1337,7 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
     if (fast) {
       const int32_t stop = solo ? min(n_steps, sidx + team_steps) : n_steps;
       if (threadIdx.x < 32 * (team_warps(p.K) + 1)) {
-        const int d = beam_team_run<LT, WIDTH == 2 ? 2 : 1>(p, sh, dyn, sidx, stop, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB, lenA,
+        const int d = beam_team_run<LT, WIDTH == 3 ? 2 : 1>(p, sh, dyn, sidx, stop, E, frame_stride, row_stride, rows_per_stream, step_base, hashA, hashB, lenA,
                                                             lenB, par0, recs_cached, tm);
         if (threadIdx.x == 0) { sh.team_done = d; sh.taken[1] += d; }
       }
@@ -1349,7 +1351,10 @@ __device__ __forceinline__ void beam_all_steps(const TbBeamParams& p, BeamShared
     }
     clean = false;
     const int32_t end = fast ? min(n_steps, sidx + backoff + 1) : n_steps;
-    beam_block_steps_apart<LT>(p, sh, sidx, end, n_steps, E, frame_stride, row_stride, step_base, hashA, hashB, lenA, lenB, par0);
+    if constexpr (WIDTH == 1)
+      beam_block_steps<LT>(p, sh, sidx, end, n_steps, E, frame_stride, row_stride, step_base, hashA, hashB, lenA, lenB, par0);
+    else
+      beam_block_steps_apart<LT>(p, sh, sidx, end, n_steps, E, frame_stride, row_stride, step_base, hashA, hashB, lenA, lenB, par0);
     if (threadIdx.x == 0) sh.taken[2] += end - sidx;
     sidx = end;
   }
@@ -1571,9 +1576,10 @@ template <typename F>
 static int beam_width_class(const TbBeamParams& p, F f) {
   if (!p.tensor_lo) return f(std::integral_constant<int, kWholeRows>{});     // (see beam_team_setup)
   const int K = p.K;
-  if (K <= kSoloBeam) return f(std::integral_constant<int, 0>{});
-  if (K <= 16) return f(std::integral_constant<int, 1>{});
-  return f(std::integral_constant<int, 2>{});
+  if (K <= kSoloBeam / 2) return f(std::integral_constant<int, 0>{});
+  if (K <= kSoloBeam) return f(std::integral_constant<int, 1>{});
+  if (K <= 16) return f(std::integral_constant<int, 2>{});
+  return f(std::integral_constant<int, 3>{});
 }
 
 // The team's steps (beam_team_run) read rows through buffers behind the block's other shared memory and need the extent
